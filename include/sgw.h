@@ -8,11 +8,13 @@
  * accumulation, and the transform of Sigma to frequency and the QP solve.
  *
  * Conventions (all entry points):
- *  - Grids are cubic, n^3 points with spacing h (bohr); n in {16, 32, 64, 128} (plane path: one
- *    xy plane per CTA, two HBM passes per H application) or n in {48, 96, 288} (row path:
- *    n = 2^a 3^b, units of 8 x rows per CTA plus y- and z-line passes, four HBM passes per H
- *    application; the 288^2 plane does not fit one CTA's shared memory).  Results agree between
- *    the paths to FP32 rounding; the split-operator entries need the plane path (SGW_EINVAL).
+ *  - Grids are cubic, n^3 points with spacing h (bohr); n in {16, 32, 64, 128} or {48, 96, 288}.
+ *    Without an energy cutoff the kinetic energy is applied axis by axis: two HBM passes per H
+ *    application (z lines, xy planes), three at n = 288 (z lines, y lines, x rows; the 288^2 plane
+ *    does not fit one CTA's shared memory).  With a cutoff it is applied through the 3D transform,
+ *    in two passes (one xy plane per CTA) or, on grids whose side is not a power of two, in four
+ *    (units of x rows per CTA plus y- and z-line passes).  Results agree between these forms to FP32
+ *    rounding; the split-operator entries need n in {16, 32, 64, 128} (SGW_EINVAL).
  *    A grid function is stored with x fastest: index g = (z*n + y)*n + x.
  *  - A complex vector is interleaved complex64 ("c64": float re, float im), N_g
  *    elements; a batch of B vectors is B contiguous vectors [B][N_g].
@@ -90,7 +92,8 @@ sgw_status sgw_set_graph_mode(sgw_ctx* ctx, int enable);
 /*
  * Launch tuning (the paper's GPU port batches all vectors of a step into each launch, Sec. 2.3;
  * these keys refine how those launches use the memory system).  Every key is a performance hint:
- * no result depends on it.
+ * no result depends on it.  They act on the passes of contexts with an energy cutoff; without one
+ * the kernels take no launch hints, the keys are accepted and the autotuner keeps their values.
  *   SGW_TUNE_PLANE_OPERANDS   : bit 0 (1) = each xy-plane pass block starts by prefetching into L2
  *                               the operands of its pointwise step (b_{k+1}, psi, b_{k+2},
  *                               potential rows), so they arrive while its inverse transform runs;

@@ -22,6 +22,7 @@ struct sgw_ctx {
     int n = 0;
     int64_t ng = 0;
     double h = 0, dV = 0, L = 0, ecut = 0;
+    bool sep = false;          // no cutoff: the kinetic energy is a sum over the axes (kernels_sep.cu)
     int device = 0;
     cudaStream_t stream = nullptr;
     int max_batch = 0;
@@ -326,21 +327,75 @@ void set_kb_args(const sgw_ctx* ctx, sgw::StepArgs& a) {
     a.n_proj = kb.n_proj;
 }
 
+// The fused step's arguments that do not depend on the kinetic path.
+sgw::StepArgs step_args(const sgw_ctx* ctx, const Step& s, const float2* b1, const float2* b2, const float2* psi,
+                        float2* out, const float* vpot, const float* dvpot, const sgw::VecInfo* info) {
+    sgw::StepArgs a{};
+    a.W = ctx->W;
+    a.b1 = b1;
+    a.b2 = b2;
+    a.psi = psi;
+    a.out = out;
+    a.vpot = vpot;
+    a.dvpot = dvpot;
+    a.info = info;
+    a.kbc = ctx->kb.n_atoms > 0 ? ctx->kbc : nullptr;
+    set_kb_args(ctx, a);
+    a.ebar = (float)(0.5 * (ctx->emax + ctx->emin));
+    a.alpha = (float)(2.0 / (0.5 * (ctx->emax - ctx->emin)));
+    a.pf_ahead = ctx->tune[SGW_TUNE_PLANE_LOOKAHEAD];
+    a.pf_operands = ctx->tune[SGW_TUNE_PLANE_OPERANDS];
+    for (int q = 0; q < 2; ++q) {
+        a.coef.cpsi[q] = f2(s.cpsi[q]);
+        a.coef.ch[q] = f2(s.ch[q]);
+        a.coef.c2[q] = f2(s.c2[q]);
+    }
+    return a;
+}
+
+// One H application and recurrence update with the separable kinetic energy: the z lines (with the
+// reduction of the KB partials that the previous step left, when `reduce`), at 288 the y lines, and
+// the step on planes or rows.
+sgw_status sep_term(sgw_ctx* ctx, const sgw::StepArgs& a, int batch, bool reduce, int vrows) {
+    cudaStream_t st = ctx->stream;
+    const int n = ctx->n;
+    const float kscale = (float)std::pow(2.0 * M_PI / ctx->L, 2);
+    const double vp = (double)ctx->ng * batch;
+    {
+        sgw::KbReduceArgs kr;
+        if (reduce) kr = sgw::kb_reduce_args(ctx->kb, ctx->kbp, (float)ctx->dV, ctx->kbc);
+        Launch L(ctx, SGW_PROF_PENCIL, 1, 16.0 * vp + (reduce ? 32.0 * (double)ctx->kb.total_slots * batch : 0.0));
+        sgw::sep_z(n, a.b1, ctx->W, batch, kscale, ctx->tw, kr, st);
+        CKL();
+    }
+    if (sgw::cluster_plane(n)) {
+        Launch L(ctx, SGW_PROF_LINES, 1, 24.0 * vp);
+        sgw::sep_y288(a.b1, ctx->W, batch, kscale, ctx->tw, st);
+        CKL();
+    }
+    double bytes = 8.0 * (3 + (a.psi ? 1 : 0) + (a.b2 ? 1 : 0)) * vp + 4.0 * (double)ctx->ng * vrows * (a.dvpot ? 2 : 1);
+    if (a.kbc) bytes += 4.0 * (double)ctx->ng + 20.0 * (double)ctx->kb.n_sup;
+    Launch L(ctx, SGW_PROF_PLANE_STEP, 1, bytes);
+    sgw::sep_step(n, a, batch, kscale, ctx->tw, st);
+    CKL();
+    return SGW_OK;
+}
+
 // Run one Chebyshev sum over a batch.  psi_in: real-space input; out: result (may alias psi_in).
-// W must hold the forward xy transform of psi_in on entry when w_ready; on exit it holds the
-// transform of the output when want_wout.
+// ready: the context holds what a previous sum with want_next left for psi_in (its KB partials, and
+// with a cutoff the forward xy transform in W); on exit it holds the same for the output when
+// want_next.
 sgw_status run_series(sgw_ctx* ctx, const std::vector<Step>& plan, const float2* psi_in, float2* out, int batch,
-                      const float* vpot, const float* dvpot, const sgw::VecInfo* info, bool w_ready, bool want_wout,
+                      const float* vpot, const float* dvpot, const sgw::VecInfo* info, bool ready, bool want_next,
                       int vrows = 1) {
     cudaStream_t st = ctx->stream;
     const int n = ctx->n;
     const float kscale = (float)std::pow(2.0 * M_PI / ctx->L, 2);
-    const double ebar = 0.5 * (ctx->emax + ctx->emin), de = 0.5 * (ctx->emax - ctx->emin);
     if (plan.empty()) {
         if (out != psi_in) CK(cudaMemcpyAsync(out, psi_in, sizeof(float2) * ctx->ng * batch, cudaMemcpyDeviceToDevice, st));
         return SGW_OK;
     }
-    if (!w_ready) {
+    if (!ready && !ctx->sep) {
         Launch L(ctx, SGW_PROF_PLANE_FWD, 1, 16.0 * (double)ctx->ng * batch);
         sgw::launch_plane_fwd(n, psi_in, ctx->W, batch, ctx->tw, st);
         CKL();
@@ -352,16 +407,23 @@ sgw_status run_series(sgw_ctx* ctx, const std::vector<Step>& plan, const float2*
         const Step& s = plan[i];
         const float2* b1 = buf(s.b1);
         if (ctx->kb.n_atoms > 0) {
-            if (i == 0 && !w_ready) {
+            if (i == 0 && !ready) {
                 // gathered psi (8 B) per support point and vector, plus the support index and beta (20 B)
                 Launch L(ctx, SGW_PROF_KB, 1, (double)ctx->kb.n_sup * (8.0 * batch + 20.0));
                 sgw::launch_kb_project(n, ctx->kb, b1, batch, (float)ctx->dV, ctx->kbc, st);
-            } else {
+            } else if (!ctx->sep) {
                 // the previous plane pass left per-plane partial projections of b1
                 Launch L(ctx, SGW_PROF_KB, 1, 32.0 * (double)ctx->kb.total_slots * batch);
                 sgw::launch_kb_reduce(ctx->kb, ctx->kbp, batch, (float)ctx->dV, ctx->kbc, st);
             }
             CKL();
+        }
+        sgw::StepArgs a = step_args(ctx, s, b1, s.b2 >= 0 ? buf(s.b2) : nullptr, psi_in, buf(s.out), vpot, dvpot, info);
+        const bool next = i + 1 < plan.size() || want_next;
+        a.kbp = (ctx->kb.n_atoms > 0 && next) ? ctx->kbp : nullptr;
+        if (ctx->sep) {
+            if (sgw_status r = sep_term(ctx, a, batch, ctx->kb.n_atoms > 0 && (i > 0 || ready), vrows)) return r;
+            continue;
         }
         {
             Launch L(ctx, SGW_PROF_PENCIL, 1, 16.0 * (double)ctx->ng * batch);
@@ -369,31 +431,7 @@ sgw_status run_series(sgw_ctx* ctx, const std::vector<Step>& plan, const float2*
                                ctx->tune[SGW_TUNE_PENCIL_LOOKAHEAD], nullptr, 0.f, ctx->tune[SGW_TUNE_LINE_FORM]);
             CKL();
         }
-        sgw::StepArgs a{};
-        a.W = ctx->W;
-        const bool last = (i + 1 == plan.size());
-        a.Wout = (!last || want_wout) ? ctx->W : nullptr;
-        a.b1 = b1;
-        a.b2 = s.b2 >= 0 ? buf(s.b2) : nullptr;
-        a.psi = psi_in;
-        a.out = buf(s.out);
-        a.vpot = vpot;
-        a.dvpot = dvpot;
-        a.info = info;
-        a.kbc = ctx->kb.n_atoms > 0 ? ctx->kbc : nullptr;
-        a.kbp = (ctx->kb.n_atoms > 0 && a.Wout != nullptr) ? ctx->kbp : nullptr;
-        set_kb_args(ctx, a);
-        a.total_slots = ctx->kb.total_slots;
-        a.n_proj = ctx->kb.n_proj;
-        a.ebar = (float)ebar;
-        a.alpha = (float)(2.0 / de);
-        a.pf_ahead = ctx->tune[SGW_TUNE_PLANE_LOOKAHEAD];
-        a.pf_operands = ctx->tune[SGW_TUNE_PLANE_OPERANDS];
-        for (int q = 0; q < 2; ++q) {
-            a.coef.cpsi[q] = f2(s.cpsi[q]);
-            a.coef.ch[q] = f2(s.ch[q]);
-            a.coef.c2[q] = f2(s.c2[q]);
-        }
+        a.Wout = next ? ctx->W : nullptr;
         {
             // per vector-point: W, b1 in; psi, b2 in when used; out and Wout written; plus the
             // potential rows (and tangent rows) shared by the vectors, and the KB point index.
@@ -541,6 +579,7 @@ sgw_status sgw_setup_grid(sgw_ctx** out, int nx, int ny, int nz, double h, doubl
     ctx->dV = h * h * h;
     ctx->L = nx * h;
     ctx->ecut = ecut > 0 ? ecut : 0.0;
+    ctx->sep = !(ecut > 0);
     ctx->device = device;
     ctx->stream = (cudaStream_t)stream;
     ctx->max_batch = max_batch;
@@ -560,6 +599,7 @@ sgw_status sgw_setup_grid(sgw_ctx** out, int nx, int ny, int nz, double h, doubl
     }
     e = cudaMemcpy(ctx->tw, tw.data(), sizeof(float2) * nx, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = sgw::grid_init_attributes(nx);
+    if (e == cudaSuccess && ctx->sep) e = sgw::sep_init_attributes(nx);
     if (e == cudaSuccess) e = cudaMemset(ctx->vloc, 0, sizeof(float) * ctx->ng);
     if (e != cudaSuccess) {
         std::string m = std::string("setup: ") + cudaGetErrorString(e);
@@ -837,6 +877,8 @@ sgw_status sgw_autotune(sgw_ctx* ctx, int batch, int reps, int* chosen_host) {
         else if (key == SGW_TUNE_PLANE_VARIANT && sgw::cluster_plane(ctx->n)) cand = {0, 1, 2};
         else if (key == SGW_TUNE_PLANE_OPERANDS && sgw::cluster_plane(ctx->n)) cand = {0, 1, 2, 3};
         else if (sgw::rows_path(ctx->n)) cand = {ctx->tune[key]};   // the row kernels take no other launch hints
+        if (ctx->sep) cand = {ctx->tune[key]};                      // the separable kernels take no launch hints
+        if (cand.size() == 1 && cand[0] == ctx->tune[key]) continue;
         int best_v = 0;
         float best = 1e30f;
         for (int v : cand) {
@@ -867,6 +909,7 @@ sgw_status sgw_set_potential(sgw_ctx* ctx, const float* vloc_dev, int n_atoms, c
     if (!vloc_dev) return fail(ctx, SGW_EINVAL, "vloc_dev is null");
     if (n_atoms < 0) return fail(ctx, SGW_EINVAL, "n_atoms < 0");
     clear_graphs(ctx);
+    ctx->sep = !(ctx->ecut > 0);
     CK(cudaMemcpyAsync(ctx->vloc, vloc_dev, sizeof(float) * ctx->ng, cudaMemcpyDeviceToDevice, ctx->stream));
     // drop any previous KB data
     CK(cudaStreamSynchronize(ctx->stream));
@@ -902,36 +945,48 @@ sgw_status sgw_set_potential(sgw_ctx* ctx, const float* vloc_dev, int n_atoms, c
         // plane on the plane path, 8 x rows on the row path: unit_points consecutive points); atom a's
         // points in unit z are one contiguous run of its sorted support: [run_beg, run_end)
         const int n = ctx->n;
-        const int64_t plane_sz = sgw::unit_points(n);
-        const int nu = (int)(ctx->ng / plane_sz);
-        if (plane_sz > 65536) return fail(ctx, SGW_EINVAL, "in-unit offsets must fit 16 bits");
-        std::vector<std::vector<int>> plane_atoms(nu);
-        std::vector<std::vector<std::pair<int64_t, int64_t>>> plane_runs(nu);
-        for (int a = 0; a < n_atoms; ++a) {
-            int64_t i = sup_off_host[a];
-            while (i < sup_off_host[a + 1]) {
-                const int z = (int)(sup_idx_host[i] / plane_sz);
-                int64_t j = i;
-                while (j < sup_off_host[a + 1] && sup_idx_host[j] / plane_sz == z) ++j;
-                plane_atoms[z].push_back(a);
-                plane_runs[z].push_back({i, j});
-                i = j;
-            }
-        }
-        std::vector<int> plane_off(nu + 1, 0);
-        int max_slots = 0;
-        for (int z = 0; z < nu; ++z) {
-            plane_off[z + 1] = plane_off[z] + (int)plane_atoms[z].size();
-            max_slots = std::max(max_slots, (int)plane_atoms[z].size());
-        }
-        const int total_slots = plane_off[nu];
-        if (max_slots >= 65536) return fail(ctx, SGW_EINVAL, "too many projector supports meet one plane");
-        const size_t smem = sgw::plane_step_smem(n, max_slots);
         int optin = 0;
         CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device));
-        if (smem > (size_t)optin || (sgw::plane_pipe_supported(n) && sgw::plane_pipe_smem(n, max_slots) > (size_t)optin))
-            return fail(ctx, SGW_EINVAL, "the projector slots of one plane do not fit in shared memory");
-        CK(sgw::plane_step_reserve_smem(n, max_slots));
+        int64_t plane_sz = 0;
+        int nu = 0, max_slots = 0;
+        std::vector<std::vector<int>> plane_atoms;
+        std::vector<std::vector<std::pair<int64_t, int64_t>>> plane_runs;
+        auto build_slots = [&](int64_t unit) {
+            plane_sz = unit;
+            nu = (int)(ctx->ng / unit);
+            max_slots = 0;
+            plane_atoms.assign(nu, {});
+            plane_runs.assign(nu, {});
+            for (int a = 0; a < n_atoms; ++a) {
+                int64_t i = sup_off_host[a];
+                while (i < sup_off_host[a + 1]) {
+                    const int z = (int)(sup_idx_host[i] / unit);
+                    int64_t j = i;
+                    while (j < sup_off_host[a + 1] && sup_idx_host[j] / unit == z) ++j;
+                    plane_atoms[z].push_back(a);
+                    plane_runs[z].push_back({i, j});
+                    i = j;
+                }
+            }
+            for (int z = 0; z < nu; ++z) max_slots = std::max(max_slots, (int)plane_atoms[z].size());
+        };
+        if (ctx->sep) {
+            build_slots(sgw::sep_unit_points(n));
+            // more slots than a plane's block has room for: the transform path's smaller units may fit
+            ctx->sep = sgw::sep_step_smem(n, max_slots) <= (size_t)optin;
+        }
+        if (!ctx->sep) {
+            build_slots(sgw::unit_points(n));
+            if (sgw::plane_step_smem(n, max_slots) > (size_t)optin ||
+                (sgw::plane_pipe_supported(n) && sgw::plane_pipe_smem(n, max_slots) > (size_t)optin))
+                return fail(ctx, SGW_EINVAL, "the projector slots of one plane do not fit in shared memory");
+        }
+        if (plane_sz > 65536) return fail(ctx, SGW_EINVAL, "in-unit offsets must fit 16 bits");
+        if (max_slots >= 65536) return fail(ctx, SGW_EINVAL, "too many projector supports meet one plane");
+        std::vector<int> plane_off(nu + 1, 0);
+        for (int z = 0; z < nu; ++z) plane_off[z + 1] = plane_off[z] + (int)plane_atoms[z].size();
+        const int total_slots = plane_off[nu];
+        if (!ctx->sep) CK(sgw::plane_step_reserve_smem(n, max_slots));
         std::vector<int> slot_atom(std::max(total_slots, 1));
         std::vector<std::vector<int>> atom_slots(n_atoms);
         for (int z = 0; z < nu; ++z)
@@ -1045,43 +1100,32 @@ sgw_status sgw_apply_h(sgw_ctx* ctx, const void* in_dev, void* out_dev, int batc
     SGW_ALIGNED(ctx, in_dev, out_dev);
     std::vector<sgw::VecInfo> info(batch, sgw::VecInfo{0, -1, -1, 0});
     if ((s = upload_info(ctx, info))) return s;
-    const float kscale = (float)std::pow(2.0 * M_PI / ctx->L, 2);
     const float2* in = (const float2*)in_dev;
-    {
-        Launch L(ctx, SGW_PROF_PLANE_FWD);
-        sgw::launch_plane_fwd(ctx->n, in, ctx->W, batch, ctx->tw, ctx->stream);
-        CKL();
-    }
     if (ctx->kb.n_atoms > 0) {
         Launch L(ctx, SGW_PROF_KB);
         sgw::launch_kb_project(ctx->n, ctx->kb, in, batch, (float)ctx->dV, ctx->kbc, ctx->stream);
         CKL();
     }
-    {
-        Launch L(ctx, SGW_PROF_PENCIL);
-        sgw::launch_pencil(ctx->n, ctx->W, batch, 0, kscale, (float)ctx->ecut, ctx->tw, ctx->stream,
-                           ctx->tune[SGW_TUNE_PENCIL_LOOKAHEAD], nullptr, 0.f, ctx->tune[SGW_TUNE_LINE_FORM]);
-        CKL();
+    Step one;                                    // out = H in: no shift, no scale, no recurrence
+    for (int q = 0; q < 2; ++q) {
+        one.cpsi[q] = one.c2[q] = 0.0;
+        one.ch[q] = 1.0;
     }
-    sgw::StepArgs a{};
-    a.W = ctx->W;
-    a.Wout = nullptr;
-    a.b1 = in;
-    a.out = (float2*)out_dev;
-    a.vpot = ctx->vloc;
-    a.info = ctx->info;
-    a.kbc = ctx->kb.n_atoms > 0 ? ctx->kbc : nullptr;
-    set_kb_args(ctx, a);
-    a.kbp = nullptr;
-    a.n_proj = ctx->kb.n_proj;
+    sgw::StepArgs a = step_args(ctx, one, in, nullptr, nullptr, (float2*)out_dev, ctx->vloc, nullptr, ctx->info);
     a.ebar = 0.f;
     a.alpha = 1.f;
-    a.pf_ahead = ctx->tune[SGW_TUNE_PLANE_LOOKAHEAD];
-    a.pf_operands = ctx->tune[SGW_TUNE_PLANE_OPERANDS];
-    for (int q = 0; q < 2; ++q) {
-        a.coef.cpsi[q] = make_float2(0.f, 0.f);
-        a.coef.ch[q] = make_float2(1.f, 0.f);
-        a.coef.c2[q] = make_float2(0.f, 0.f);
+    if (ctx->sep) return sep_term(ctx, a, batch, false, 1);
+    {
+        Launch L(ctx, SGW_PROF_PLANE_FWD);
+        sgw::launch_plane_fwd(ctx->n, in, ctx->W, batch, ctx->tw, ctx->stream);
+        CKL();
+    }
+    {
+        Launch L(ctx, SGW_PROF_PENCIL);
+        sgw::launch_pencil(ctx->n, ctx->W, batch, 0, (float)std::pow(2.0 * M_PI / ctx->L, 2), (float)ctx->ecut, ctx->tw,
+                           ctx->stream, ctx->tune[SGW_TUNE_PENCIL_LOOKAHEAD], nullptr, 0.f,
+                           ctx->tune[SGW_TUNE_LINE_FORM]);
+        CKL();
     }
     {
         Launch L(ctx, SGW_PROF_PLANE_STEP);

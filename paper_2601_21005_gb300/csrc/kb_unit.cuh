@@ -11,6 +11,8 @@
 
 namespace sgw {
 
+constexpr int KB_B = 4;    // KB entries per lane whose loads are in flight together
+
 // Position in shared memory of unit point o = y N + x (row y, column x) at row pitch P.  LAYOUT 0:
 // natural, y P + x.  LAYOUT 1 (N = 288, the two-stage row transforms): a row is 16 groups of 19
 // slots, column x at 19 (x mod 16) + x div 16, the order in which the 16 x 18 transforms leave it.
@@ -26,6 +28,32 @@ __device__ __forceinline__ int unit_pos_yx(int y, int x) {
 template <int N, int P, int LAYOUT>
 __device__ __forceinline__ int unit_pos(int o) {
     return unit_pos_yx<N, P, LAYOUT>(o / N, o % N);
+}
+
+// kbc[b][4a + p] = E_ap dV sum_{slots of a} kbp[b][slot][p] by one warp: lane l takes projector p =
+// l % 4 of the atom's slots l / 4, l / 4 + 8, ... (in increasing unit), then the eight lanes of each p
+// are summed by a fixed shuffle tree.  The whole warp calls it with one (a, b); a >= n_atoms does nothing.
+__device__ __forceinline__ void kb_reduce_warp(const KbReduceArgs& kr, int a, int b, int lane) {
+    if (a >= kr.n_atoms) return;
+    const int p = lane & 3;
+    const int q0 = __ldg(kr.atom_pos_off + a), q1 = __ldg(kr.atom_pos_off + a + 1);
+    const float2* kb = kr.kbp + (size_t)b * kr.total_slots * 4;
+    float2 acc = make_float2(0.f, 0.f);
+    for (int q = q0 + (lane >> 2); q < q1; q += 8) {
+        const float2 v = __ldg(kb + (size_t)__ldg(kr.atom_pos + q) * 4 + p);
+        acc.x += v.x;
+        acc.y += v.y;
+    }
+#pragma unroll
+    for (int off = 4; off < 32; off <<= 1) {
+        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, off);
+        acc.y += __shfl_xor_sync(0xffffffffu, acc.y, off);
+    }
+    if (lane < 4) {
+        const float4 e = __ldg(kr.atom_e + a);
+        const float ep = (p == 0 ? e.x : (p == 1 ? e.y : (p == 2 ? e.z : e.w))) * kr.dV;
+        kr.kbc[(size_t)b * kr.n_proj + a * 4 + p] = make_float2(ep * acc.x, ep * acc.y);
+    }
 }
 
 // E-weighted projector coefficients of the unit's slots into shared memory: kcs[4 s + p] for the
@@ -45,15 +73,27 @@ __device__ __forceinline__ void kb_apply_unit(const StepArgs& a, int u, const fl
     for (int c = 0; c < a.max_colors; ++c) {
         const int e0 = __ldg(col + c), e1 = __ldg(col + c + 1);
         if (e0 == e1) break;                  // a unit's colours are used from 0 upwards
-        for (int e = e0 + threadIdx.x; e < e1; e += NT) {
-            const unsigned os = __ldg(a.kbe_os + e);
-            const float4 be = __ldg(a.kbe_beta + e);
-            const int o = (int)(os & 0xffffu), sl = (int)(os >> 16);
-            const float4 c01 = *reinterpret_cast<const float4*>(kcs + 4 * sl);
-            const float4 c23 = *reinterpret_cast<const float4*>(kcs + 4 * sl + 2);
-            float2& hv = sm[unit_pos<N, P, LAYOUT>(o)];
-            hv.x += be.x * c01.x + be.y * c01.z + be.z * c23.x + be.w * c23.z;
-            hv.y += be.x * c01.y + be.y * c01.w + be.z * c23.y + be.w * c23.w;
+        // batches of KB_B entries whose loads are all in flight at once, the last one padded: the
+        // loads' latency is paid per batch, and a remainder taken entry by entry would pay it each time
+        for (int eb = e0 + threadIdx.x; eb < e1; eb += KB_B * NT) {
+            unsigned os[KB_B];
+            float4 be[KB_B];
+#pragma unroll
+            for (int i = 0; i < KB_B; ++i) {
+                const int e = min(eb + i * NT, e1 - 1);
+                os[i] = __ldg(a.kbe_os + e);
+                be[i] = __ldg(a.kbe_beta + e);
+            }
+#pragma unroll
+            for (int i = 0; i < KB_B; ++i) {
+                if (eb + i * NT >= e1) break;
+                const int o = (int)(os[i] & 0xffffu), sl = (int)(os[i] >> 16);
+                const float4 c01 = *reinterpret_cast<const float4*>(kcs + 4 * sl);
+                const float4 c23 = *reinterpret_cast<const float4*>(kcs + 4 * sl + 2);
+                float2& hv = sm[unit_pos<N, P, LAYOUT>(o)];
+                hv.x += be[i].x * c01.x + be[i].y * c01.z + be[i].z * c23.x + be[i].w * c23.z;
+                hv.y += be[i].x * c01.y + be[i].y * c01.w + be[i].z * c23.y + be[i].w * c23.w;
+            }
         }
         __syncthreads();
     }
@@ -68,14 +108,24 @@ __device__ __forceinline__ void kb_project_unit(const StepArgs& a, int u, int b,
     for (int k = sb + warp; k < s1; k += NT / 32) {
         float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
         const int e1 = __ldg(a.kbe_slot_end + k);
-        for (int e = __ldg(a.kbe_slot_beg + k) + lane; e < e1; e += 32) {
-            const int o = (int)(__ldg(a.kbe_os + e) & 0xffffu);
-            const float2 v = sm[unit_pos<N, P, LAYOUT>(o)];
-            const float4 be = __ldg(a.kbe_beta + e);
-            acc[0] += be.x * v.x; acc[1] += be.x * v.y;
-            acc[2] += be.y * v.x; acc[3] += be.y * v.y;
-            acc[4] += be.z * v.x; acc[5] += be.z * v.y;
-            acc[6] += be.w * v.x; acc[7] += be.w * v.y;
+        for (int eb = __ldg(a.kbe_slot_beg + k) + lane; eb < e1; eb += KB_B * 32) {
+            unsigned os[KB_B];
+            float4 be[KB_B];
+#pragma unroll
+            for (int i = 0; i < KB_B; ++i) {
+                const int e = min(eb + 32 * i, e1 - 1);
+                os[i] = __ldg(a.kbe_os + e);
+                be[i] = __ldg(a.kbe_beta + e);
+            }
+#pragma unroll
+            for (int i = 0; i < KB_B; ++i) {
+                if (eb + 32 * i >= e1) break;
+                const float2 v = sm[unit_pos<N, P, LAYOUT>((int)(os[i] & 0xffffu))];
+                acc[0] += be[i].x * v.x; acc[1] += be[i].x * v.y;
+                acc[2] += be[i].y * v.x; acc[3] += be[i].y * v.y;
+                acc[4] += be[i].z * v.x; acc[5] += be[i].z * v.y;
+                acc[6] += be[i].w * v.x; acc[7] += be[i].w * v.y;
+            }
         }
         const float r = warp_reduce_scatter8(acc, lane);
         if ((lane & 3) == 0) reinterpret_cast<float*>(a.kbp + ((size_t)b * a.total_slots + k) * 4)[lane >> 2] = r;

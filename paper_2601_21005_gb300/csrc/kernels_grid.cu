@@ -10,6 +10,7 @@
 // H application is dominated by the FFTs; the potential multiply is fused into them).
 #include "fft_smem.cuh"
 #include "grid_common.cuh"
+#include "kb_unit.cuh"
 #include "sgw_internal.cuh"
 
 namespace sgw {
@@ -760,42 +761,31 @@ k_kb_project(const int64_t* __restrict__ atom_off, const int* __restrict__ sup_i
     }
 }
 
-// kbc[b][4a + p] = E_ap dV sum_{slots of a} kbp[b][slot][p].  One warp per (b, a): lane l takes
-// projector p = l % 4 of the atom's slots l / 4, l / 4 + 8, ... (in increasing plane), then the
-// eight lanes of each p are summed by a fixed shuffle tree.
-__global__ void __launch_bounds__(256)
-k_kb_reduce(const int* __restrict__ atom_pos_off, const int* __restrict__ atom_pos, const float4* __restrict__ atom_e,
-            const float2* __restrict__ kbp, int n_atoms, int batch, int total_slots, int n_proj, float dV,
-            float2* __restrict__ kbc) {
-    const int w = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-    if (w >= batch * n_atoms) return;                     // whole warps leave together
-    const int a = w % n_atoms, b = w / n_atoms, p = lane & 3;
-    const int q0 = __ldg(atom_pos_off + a), q1 = __ldg(atom_pos_off + a + 1);
-    const float2* kb = kbp + (size_t)b * total_slots * 4;
-    float2 acc = make_float2(0.f, 0.f);
-    for (int q = q0 + (lane >> 2); q < q1; q += 8) {
-        const float2 v = __ldg(kb + (size_t)__ldg(atom_pos + q) * 4 + p);
-        acc.x += v.x;
-        acc.y += v.y;
-    }
-#pragma unroll
-    for (int off = 4; off < 32; off <<= 1) {
-        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, off);
-        acc.y += __shfl_xor_sync(0xffffffffu, acc.y, off);
-    }
-    if (lane < 4) {
-        const float4 e = __ldg(atom_e + a);
-        const float ep = (p == 0 ? e.x : (p == 1 ? e.y : (p == 2 ? e.z : e.w))) * dV;
-        kbc[(size_t)b * n_proj + a * 4 + p] = make_float2(ep * acc.x, ep * acc.y);
-    }
+// One warp per (b, a), see kb_reduce_warp.
+__global__ void __launch_bounds__(256) k_kb_reduce(KbReduceArgs kr, int batch) {
+    const int w = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5);
+    if (w >= batch * kr.n_atoms) return;                     // whole warps leave together
+    kb_reduce_warp(kr, w % kr.n_atoms, w / kr.n_atoms, threadIdx.x & 31);
+}
+
+KbReduceArgs kb_reduce_args(const KBDev& kb, const float2* kbp, float dV, float2* kbc) {
+    KbReduceArgs r;
+    r.atom_pos_off = kb.atom_pos_off;
+    r.atom_pos = kb.atom_pos;
+    r.atom_e = kb.atom_e;
+    r.kbp = kbp;
+    r.kbc = kbc;
+    r.n_atoms = kb.n_atoms;
+    r.total_slots = kb.total_slots;
+    r.n_proj = kb.n_proj;
+    r.dV = dV;
+    return r;
 }
 
 void launch_kb_reduce(const KBDev& kb, const float2* kbp, int batch, float dV, float2* kbc, cudaStream_t st) {
     const long warps = (long)batch * kb.n_atoms;
     if (warps == 0) return;
-    k_kb_reduce<<<(unsigned)((warps * 32 + 255) / 256), 256, 0, st>>>(kb.atom_pos_off, kb.atom_pos, kb.atom_e, kbp,
-                                                                     kb.n_atoms, batch, kb.total_slots, kb.n_proj, dV,
-                                                                     kbc);
+    k_kb_reduce<<<(unsigned)((warps * 32 + 255) / 256), 256, 0, st>>>(kb_reduce_args(kb, kbp, dV, kbc), batch);
 }
 
 // ------------------------------------------------------------------ launchers

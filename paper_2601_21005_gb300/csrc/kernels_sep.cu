@@ -1,0 +1,398 @@
+// The Chebyshev term with a separable kinetic energy.
+//
+// Without an energy cutoff T(k) = |k|^2 / 2 is a sum of one-dimensional symbols, so T psi is the sum
+// of three line operations: along each axis a forward transform, times k_a^2 / 2, an inverse
+// transform.  None of them needs another axis transformed, so a term reads and writes only
+// real-space arrays and carries no transformed copy of its vector:
+//   n <= 128:  z lines   W = T_z b                                          (16 B per vector-point)
+//              planes    out = c psi + 2 H~ b - b2, H b = W + (T_x + T_y + V + V_NL) b     (40 B)
+//   n = 288:   z lines   W = T_z b (16 B),  y lines  W += T_y b (24 B),  rows of x: the rest (40 B)
+// against 64 B and 96 B when the vector's 3D transform is carried through the passes.  With a
+// cutoff T is not separable: those contexts keep the transforms of the other grid kernels.
+//
+// Traffic bounds both passes at batches larger than L2; below that the planes' serial phases.  Every
+// line is held in the registers of 2 or 4 lanes (reg_dft.cuh), so a transform takes no barrier; a
+// plane's block meets one barrier per axis and per KB colour, where radix stages through shared
+// memory take two per stage.  Measured per term, the transform path -> this one (h = 0.5 clusters with
+// KB): 64^3 x 64 vectors 240 -> 203 us (z 43 us = 6.3 TB/s, planes 162 us, 129 us without KB); 64^3 x 8
+// 41 -> 36 us; 96^3 x 8 208 -> 114 us; 32^3 x 64 38 -> 32 us; 288^3 x 16 (1963 KB atoms) 8.9 -> 6.1 ms.
+#include <algorithm>
+
+#include "grid_common.cuh"
+#include "kb_unit.cuh"
+#include "reg_dft.cuh"
+#include "sgw_internal.cuh"
+
+namespace sgw {
+
+// ------------------------------------------------------------------ shared pieces
+
+__device__ __forceinline__ void sep_cp16(void* smem, const void* gmem) {
+    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(s), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void sep_cp_wait() {
+    asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+}
+
+// c m^2 for k = k1 + (N / T) i, m the signed frequency of k
+template <int N, int T>
+__device__ __forceinline__ float axis_factor(int k1, int i, float c) {
+    const float m = (float)(k1 + (N / T) * i - (2 * i >= T ? N : 0));
+    return c * m * m;
+}
+
+// The step's pointwise part on ROWS x N points of the unit at global offset `off` (unit points o = y N +
+// x at sm[y PITCH + x], which holds H b but for W and the local potential):
+//   out = cpsi psi + ch alpha (sm + W + (V - Ebar) b1 [+ dv b1_partner]) + c2 b2,
+// to global memory and back into sm.
+template <int N, int ROWS, int PITCH, int NT, int UNROLL>
+__device__ __forceinline__ void sep_pointwise(const StepArgs& a, const VecInfo& inf, size_t off, size_t uoff,
+                                              float2* sm) {
+    static_assert(PITCH % 2 == 0, "rows start on 16 bytes");
+    constexpr size_t NG = (size_t)N * N * N;
+    const float* V = a.vpot + (size_t)inf.vrow * NG + uoff;
+    const float* dV = (a.dvpot != nullptr && inf.dvrow >= 0) ? a.dvpot + (size_t)inf.dvrow * NG + uoff : nullptr;
+    const float2* bp = (dV != nullptr) ? a.b1 + (size_t)inf.partner * NG + uoff : nullptr;
+    const float2 cpsi = a.coef.cpsi[inf.cset], ch = cscale(a.coef.ch[inf.cset], a.alpha), c2 = a.coef.c2[inf.cset];
+    const float ebar = a.ebar;
+#pragma unroll UNROLL
+    for (int q = threadIdx.x; q < ROWS * N / 2; q += NT) {
+        const int y = q / (N / 2), x = 2 * (q % (N / 2));
+        const int o = y * N + x, sp = y * PITCH + x;
+        const float4 bb = ld4(a.b1 + off + o), w = ldcs4(a.W + off + o);
+        const float2 v = __ldg(reinterpret_cast<const float2*>(V + o));
+        float4& sv = *reinterpret_cast<float4*>(sm + sp);
+        float2 h0 = make_float2(sv.x, sv.y), h1 = make_float2(sv.z, sv.w);
+        // the two kinetic parts first: (V - Ebar) b is the largest term, and this way one rounding of
+        // its size is made, in the multiply-add
+        h0 = make_float2(fmaf(v.x - ebar, bb.x, h0.x + w.x), fmaf(v.x - ebar, bb.y, h0.y + w.y));
+        h1 = make_float2(fmaf(v.y - ebar, bb.z, h1.x + w.z), fmaf(v.y - ebar, bb.w, h1.y + w.w));
+        if (dV != nullptr) {
+            const float2 d = __ldg(reinterpret_cast<const float2*>(dV + o));
+            const float4 pb = ld4(bp + o);
+            h0.x += d.x * pb.x;
+            h0.y += d.x * pb.y;
+            h1.x += d.y * pb.z;
+            h1.y += d.y * pb.w;
+        }
+        float2 o0 = cmul(ch, h0), o1 = cmul(ch, h1);
+        if (a.psi != nullptr) {
+            const float4 pp = ldcs4(a.psi + off + o);
+            o0 = cadd(o0, cmul(cpsi, make_float2(pp.x, pp.y)));
+            o1 = cadd(o1, cmul(cpsi, make_float2(pp.z, pp.w)));
+        }
+        if (a.b2 != nullptr) {
+            const float4 b2 = ldcs4(a.b2 + off + o);
+            o0 = cadd(o0, cmul(c2, make_float2(b2.x, b2.y)));
+            o1 = cadd(o1, cmul(c2, make_float2(b2.z, b2.w)));
+        }
+        st4(a.out + off + o, o0, o1);
+        sv = make_float4(o0.x, o0.y, o1.x, o1.y);
+    }
+}
+
+// L2 prefetch of a unit's pointwise operands (one thread), PTS points at offset off
+template <int N, int PTS>
+__device__ __forceinline__ void sep_prefetch(const StepArgs& a, const VecInfo& inf, size_t off, size_t uoff) {
+    constexpr size_t NG = (size_t)N * N * N;
+    constexpr unsigned CB = PTS * sizeof(float2), VB = PTS * sizeof(float);
+    l2_prefetch(a.W + off, CB);
+    if (a.psi != nullptr) l2_prefetch(a.psi + off, CB);
+    if (a.b2 != nullptr) l2_prefetch(a.b2 + off, CB);
+    l2_prefetch(a.vpot + (size_t)inf.vrow * NG + uoff, VB);
+    if (a.dvpot != nullptr && inf.dvrow >= 0) {
+        l2_prefetch(a.dvpot + (size_t)inf.dvrow * NG + uoff, VB);
+        l2_prefetch(a.b1 + (size_t)inf.partner * NG + uoff, CB);
+    }
+}
+
+// ------------------------------------------------------------------ z lines, n <= 128
+// W = T_z b: a warp takes CPW neighbouring columns, each in the registers of T lanes (two lanes up to
+// 64 points: four measured the same, 43 us at 64^3 x 64).  The blocks
+// past the columns' reduce the vector's KB partials (k_kb_reduce's work, which the plane pass needs
+// and which nothing here depends on), so that the term has no launch of its own for it.
+constexpr int ZS_NT = 128;
+template <int N> struct ZsCfg {
+    static constexpr int T = N <= 64 ? 2 : 4;
+    static constexpr int BLOCKS = N * N / (32 / T * (ZS_NT / 32));
+    static constexpr int MINB = N <= 32 ? 8 : (N == 64 || N == 128 ? 4 : 5);
+};
+
+template <int N>
+__global__ void __launch_bounds__(ZS_NT, (ZsCfg<N>::MINB))
+k_sep_z(const float2* __restrict__ in, float2* __restrict__ W, float c, const float2* __restrict__ tw, KbReduceArgs kr) {
+    constexpr int T = ZsCfg<N>::T, P = N / T, CPW = 32 / T;
+    __shared__ float2 tws[N];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // vectors in descending order: the plane pass before left the last ones in L2, and this pass
+    // leaves the first ones there for the plane pass after it
+    const int b = gridDim.y - 1 - blockIdx.y;
+    if (blockIdx.x >= ZsCfg<N>::BLOCKS) {
+        kb_reduce_warp(kr, (blockIdx.x - ZsCfg<N>::BLOCKS) * (ZS_NT / 32) + warp, b, lane);
+        return;
+    }
+    for (int i = threadIdx.x; i < N; i += ZS_NT) tws[i] = __ldg(tw + i);
+    const int t = lane / CPW;
+    const size_t off = (size_t)b * N * N * N + (blockIdx.x * (ZS_NT / 32) + warp) * CPW + lane % CPW + (size_t)t * N * N;
+    float2 v[P];
+#pragma unroll
+    for (int a = 0; a < P; ++a) v[a] = __ldg(in + off + (size_t)(T * a) * N * N);
+    __syncthreads();
+    line_op<N, T>(v, lane, tws, [&](int k1, int i) { return axis_factor<N, T>(k1, i, c); });
+#pragma unroll
+    for (int a = 0; a < P; ++a) W[off + (size_t)(T * a) * N * N] = v[a];
+}
+
+// ------------------------------------------------------------------ planes, n <= 128
+// A block per plane: the plane comes into shared memory by cp.async, T_x row by row in place, the KB
+// apply, T_y of the columns (read again from L2) added, then the pointwise part.  Four lanes per
+// line: two lanes hold twice the points and half the warps, and the same pass took 195 us instead
+// of 169 at 64^3 x 64 (of one SM's four blocks the phases of the others hide one's latency).  The operands
+// of the pointwise part are asked into L2 once the plane has landed, and read evict-first: asked at
+// the block's start they were evicted before use (a third more DRAM traffic than the algorithm's).
+template <int N> struct SpCfg {
+    static constexpr int T = 4;
+    static constexpr int NT = N * T;
+    // row pitch of the plane in shared memory: a half-warp reads 8 rows at two neighbouring points
+    // without bank conflicts, and rows start on 16 bytes
+    static constexpr int PITCH = N + 2;
+    static constexpr int MINB = N == 16 ? 16 : (N == 32 ? 8 : (N == 48 ? 5 : (N == 64 ? 4 : (N == 96 ? 2 : 1))));
+};
+
+template <int N>
+__global__ void __launch_bounds__(SpCfg<N>::NT, (SpCfg<N>::MINB)) k_sep_plane(StepArgs a, float c, const float2* __restrict__ tw) {
+    constexpr int T = SpCfg<N>::T, P = N / T, CPW = 32 / T, NT = SpCfg<N>::NT, PITCH = SpCfg<N>::PITCH;
+    extern __shared__ __align__(16) float2 sm[];
+    float2* tws = sm + N * PITCH;
+    float2* kcs = tws + N;
+    const int z = blockIdx.x, b = blockIdx.y;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const size_t uoff = (size_t)z * N * N, off = (size_t)b * N * N * N + uoff;
+    const VecInfo inf = a.info[b];
+    {
+        const float2* src = a.b1 + off;
+#pragma unroll 4
+        for (int q = threadIdx.x; q < N * N / 2; q += NT) sep_cp16(sm + (q / (N / 2)) * PITCH + 2 * (q % (N / 2)), src + 2 * q);
+    }
+    for (int i = threadIdx.x; i < N; i += NT) tws[i] = __ldg(tw + i);
+    const float2* kc = a.kbc != nullptr ? a.kbc + (size_t)b * a.n_proj : nullptr;
+    if (kc != nullptr) kb_stage_coeffs<NT>(a, kc, z, kcs);
+    sep_cp_wait();
+    __syncthreads();
+    if (threadIdx.x == 0) sep_prefetch<N, N * N>(a, inf, off, uoff);
+    const int l = warp * CPW + lane % CPW, t = lane / CPW;
+    const auto f = [&](int k1, int i) { return axis_factor<N, T>(k1, i, c); };
+    {
+        // T_x b of row l, in place (a lane writes the points it has read)
+        float2 v[P];
+        float2* row = sm + l * PITCH + t;
+#pragma unroll
+        for (int i = 0; i < P; ++i) v[i] = row[T * i];
+        line_op<N, T>(v, lane, tws, f);
+#pragma unroll
+        for (int i = 0; i < P; ++i) row[T * i] = v[i];
+    }
+    __syncthreads();
+    if (kc != nullptr) kb_apply_unit<N, PITCH, NT>(a, z, kcs, sm);
+    {
+        // + T_y b of column l (its points come from L2: the block has just copied the plane)
+        float2 v[P];
+        const float2* src = a.b1 + off + (size_t)t * N + l;
+        float2* col = sm + t * PITCH + l;
+#pragma unroll
+        for (int i = 0; i < P; ++i) v[i] = __ldg(src + T * i * N);
+        line_op<N, T>(v, lane, tws, f);
+#pragma unroll
+        for (int i = 0; i < P; ++i) col[T * i * PITCH] = cadd(col[T * i * PITCH], v[i]);
+    }
+    __syncthreads();
+    sep_pointwise<N, N, PITCH, NT, 4>(a, inf, off, uoff, sm);
+    if (a.kbp == nullptr) return;
+    __syncthreads();
+    kb_project_unit<N, PITCH, NT>(a, z, b, sm);
+}
+
+// ------------------------------------------------------------------ n = 288
+// A 288-point line in the registers of 12 threads, 24 points each: x[t + 12 a] -> DFT24 over a,
+// exchange through shared memory, two DFT12 over t for k1 = t' + 12 i (times W288^(t k1) on the way
+// in and its conjugate on the way out), the factor between the DFT12 and its inverse, exchange back
+// in place, inverse DFT24.  One round trip through shared memory each way.
+constexpr int S2N = 288, S2T = 12, S2P = 24;
+
+// slot(k1, t): position of stage-1 output k1 of thread t in the line's exchange buffer
+template <class SLOT, class SYNC>
+__device__ __forceinline__ void line288(float2 (&v)[S2P], int t, float c, const float2* tws, float2* ex, SLOT slot, SYNC sync) {
+    RegDft<S2P, -1>::run(v);
+#pragma unroll
+    for (int k = 0; k < S2P; ++k) ex[slot(k, t)] = v[k];
+    sync();
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int k1 = t + S2T * i;
+        float2 r[S2T];
+        r[0] = ex[slot(k1, 0)];
+#pragma unroll
+        for (int s = 1; s < S2T; ++s) r[s] = cmul(ex[slot(k1, s)], tws[s * k1]);
+        RegDft<S2T, -1>::run(r);
+#pragma unroll
+        for (int k2 = 0; k2 < S2T; ++k2) {
+            const float m = (float)(k1 + S2P * k2 - (k2 >= S2T / 2 ? S2N : 0));
+            r[k2] = cscale(r[k2], c * m * m);
+        }
+        RegDft<S2T, +1>::run(r);
+        ex[slot(k1, 0)] = r[0];
+#pragma unroll
+        for (int s = 1; s < S2T; ++s) ex[slot(k1, s)] = cmul(r[s], cconj(tws[s * k1]));
+    }
+    sync();
+#pragma unroll
+    for (int k = 0; k < S2P; ++k) v[k] = ex[slot(k, t)];
+    RegDft<S2P, +1>::run(v);
+}
+
+// z lines (AXIS 0: W = T_z b) and y lines (AXIS 1: W += T_y b) of tiles of 16 x-columns; AXIS 0's
+// blocks past the columns' reduce the KB partials.
+constexpr int SL_TX = 16, SL_NT = SL_TX * S2T;
+template <int AXIS>
+__global__ void __launch_bounds__(SL_NT, 4)
+k_sep_lines288(const float2* __restrict__ in, float2* __restrict__ W, float c, const float2* __restrict__ tw, KbReduceArgs kr) {
+    constexpr int NXT = S2N / SL_TX, BLOCKS = NXT * S2N;
+    constexpr size_t NN = (size_t)S2N * S2N, ST = AXIS == 0 ? NN : S2N;
+    extern __shared__ __align__(16) float2 sm[];
+    float2* tws = sm + S2N * SL_TX;
+    const int b = blockIdx.y;
+    if (AXIS == 0 && blockIdx.x >= BLOCKS) {
+        kb_reduce_warp(kr, (blockIdx.x - BLOCKS) * (SL_NT / 32) + (threadIdx.x >> 5), b, threadIdx.x & 31);
+        return;
+    }
+    for (int i = threadIdx.x; i < S2N; i += SL_NT) tws[i] = __ldg(tw + i);
+    const int l = threadIdx.x % SL_TX, t = threadIdx.x / SL_TX;
+    const int xt = blockIdx.x % NXT, o = blockIdx.x / NXT;
+    const size_t off = (size_t)b * S2N * NN + (size_t)o * (AXIS == 0 ? S2N : NN) + xt * SL_TX + l + (size_t)t * ST;
+    float2 v[S2P];
+#pragma unroll
+    for (int a = 0; a < S2P; ++a) v[a] = __ldg(in + off + (size_t)(S2T * a) * ST);
+    line288(v, t, c, tws, sm + l, [](int k, int s) { return (k * S2T + s) * SL_TX; }, [] { __syncthreads(); });
+    if constexpr (AXIS == 1) {
+        float2 w[S2P];
+#pragma unroll
+        for (int a = 0; a < S2P; ++a) w[a] = W[off + (size_t)(S2T * a) * ST];
+#pragma unroll
+        for (int a = 0; a < S2P; ++a) v[a] = cadd(v[a], w[a]);
+    }
+#pragma unroll
+    for (int a = 0; a < S2P; ++a) W[off + (size_t)(S2T * a) * ST] = v[a];
+}
+
+// The rows of x: units of 16 rows (192 threads, four blocks per SM), vectors fastest in launch
+// order so that a unit's potential rows and KB entries come from DRAM once for all of them.  The
+// exchange buffer's pitches (13 per k1, 316 per row) keep every half-warp access free of bank
+// conflicts: 12 is the row pitch mod 16 and 13 x 12 mod 16, so the lanes of the next row continue
+// the banks of this one.
+constexpr int SR_R = 16, SR_NT = SR_R * S2T, SR_PITCH = 316;
+__global__ void __launch_bounds__(SR_NT, 4) k_sep_rows288(StepArgs a, float c, const float2* __restrict__ tw) {
+    constexpr size_t NG = (size_t)S2N * S2N * S2N;
+    extern __shared__ __align__(16) float2 sm[];
+    float2* tws = sm + SR_R * SR_PITCH;
+    float2* kcs = tws + S2N;
+    const int b = blockIdx.x, u = blockIdx.y;
+    const size_t uoff = (size_t)u * SR_R * S2N, off = (size_t)b * NG + uoff;
+    const VecInfo inf = a.info[b];
+    const int r = threadIdx.x / S2T, t = threadIdx.x % S2T;
+    float2 v[S2P];
+    const float2* src = a.b1 + off + (size_t)r * S2N + t;
+#pragma unroll
+    for (int i = 0; i < S2P; ++i) v[i] = __ldg(src + S2T * i);
+    for (int i = threadIdx.x; i < S2N; i += SR_NT) tws[i] = __ldg(tw + i);
+    const float2* kc = a.kbc != nullptr ? a.kbc + (size_t)b * a.n_proj : nullptr;
+    if (kc != nullptr) kb_stage_coeffs<SR_NT>(a, kc, u, kcs);
+    float2* row = sm + r * SR_PITCH;
+    line288(v, t, c, tws, row, [](int k, int s) { return k * 13 + s; }, [] { __syncthreads(); });
+    __syncthreads();
+    if (threadIdx.x == 0) sep_prefetch<S2N, SR_R * S2N>(a, inf, off, uoff);
+#pragma unroll
+    for (int i = 0; i < S2P; ++i) row[t + S2T * i] = v[i];
+    __syncthreads();
+    if (kc != nullptr) kb_apply_unit<S2N, SR_PITCH, SR_NT>(a, u, kcs, sm);
+    sep_pointwise<S2N, SR_R, SR_PITCH, SR_NT, 4>(a, inf, off, uoff, sm);
+    if (a.kbp == nullptr) return;
+    __syncthreads();
+    kb_project_unit<S2N, SR_PITCH, SR_NT>(a, u, b, sm);
+}
+
+// ------------------------------------------------------------------ launchers
+#define SGW_DISPATCH_SEP(n, ...)                         \
+    switch (n) {                                         \
+        case 16: { constexpr int N = 16; __VA_ARGS__; } break;   \
+        case 32: { constexpr int N = 32; __VA_ARGS__; } break;   \
+        case 48: { constexpr int N = 48; __VA_ARGS__; } break;   \
+        case 64: { constexpr int N = 64; __VA_ARGS__; } break;   \
+        case 96: { constexpr int N = 96; __VA_ARGS__; } break;   \
+        case 128: { constexpr int N = 128; __VA_ARGS__; } break; \
+        default: break;                                  \
+    }
+
+int64_t sep_unit_points(int n) { return n == S2N ? (int64_t)SR_R * S2N : (int64_t)n * n; }
+
+size_t sep_step_smem(int n, int max_unit_slots) {
+    size_t pts = (size_t)SR_R * SR_PITCH;
+    SGW_DISPATCH_SEP(n, pts = (size_t)N * SpCfg<N>::PITCH);
+    return sizeof(float2) * (pts + n + 4 * (size_t)max_unit_slots);
+}
+
+static size_t sep_lines_smem() { return sizeof(float2) * ((size_t)S2N * SL_TX + S2N); }
+
+// Every step kernel may use all the shared memory a block can have: the limit does not depend on
+// one context's KB slots, so contexts with different potentials do not disturb each other.
+template <class K> static cudaError_t sep_attr(K kern, int bytes) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                         (int)cudaSharedmemCarveoutMaxShared);
+    return e != cudaSuccess ? e : cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
+
+cudaError_t sep_init_attributes(int n) {
+    int dev = 0, optin = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e != cudaSuccess) return e;
+    if (n == S2N) {
+        if ((e = sep_attr(k_sep_lines288<0>, (int)sep_lines_smem()))) return e;
+        if ((e = sep_attr(k_sep_lines288<1>, (int)sep_lines_smem()))) return e;
+        return sep_attr(k_sep_rows288, optin);
+    }
+    SGW_DISPATCH_SEP(n, e = sep_attr(k_sep_plane<N>, optin));
+    return e;
+}
+
+void sep_z(int n, const float2* in, float2* W, int batch, float kscale, const float2* tw, const KbReduceArgs& kr,
+           cudaStream_t st) {
+    if (batch == 0) return;
+    const float c = 0.5f * kscale / (float)n;
+    if (n == S2N) {
+        const unsigned kb = (unsigned)((kr.n_atoms + SL_NT / 32 - 1) / (SL_NT / 32));
+        k_sep_lines288<0><<<dim3((S2N / SL_TX) * S2N + kb, batch), SL_NT, sep_lines_smem(), st>>>(in, W, c, tw, kr);
+        return;
+    }
+    const unsigned kb = (unsigned)((kr.n_atoms + ZS_NT / 32 - 1) / (ZS_NT / 32));
+    SGW_DISPATCH_SEP(n, k_sep_z<N><<<dim3(ZsCfg<N>::BLOCKS + kb, batch), ZS_NT, 0, st>>>(in, W, c, tw, kr));
+}
+
+void sep_y288(const float2* in, float2* W, int batch, float kscale, const float2* tw, cudaStream_t st) {
+    if (batch == 0) return;
+    k_sep_lines288<1><<<dim3((S2N / SL_TX) * S2N, batch), SL_NT, sep_lines_smem(), st>>>(in, W, 0.5f * kscale / S2N, tw,
+                                                                                        KbReduceArgs{});
+}
+
+void sep_step(int n, const StepArgs& a, int batch, float kscale, const float2* tw, cudaStream_t st) {
+    if (batch == 0) return;
+    const float c = 0.5f * kscale / (float)n;
+    const size_t sm = sep_step_smem(n, a.kbc != nullptr ? a.max_plane_slots : 0);
+    if (n == S2N) {
+        k_sep_rows288<<<dim3(batch, S2N * S2N / SR_R), SR_NT, sm, st>>>(a, c, tw);
+        return;
+    }
+    SGW_DISPATCH_SEP(n, k_sep_plane<N><<<dim3(N, batch), SpCfg<N>::NT, sm, st>>>(a, c, tw));
+}
+
+}  // namespace sgw

@@ -88,6 +88,29 @@ struct StepArgs {
     int pf_operands;
 };
 
+// Arguments of the KB reduction kbc[b][4a + p] = E_ap dV sum_{slots of a} kbp[b][slot][p] (n_atoms 0: none)
+struct KbReduceArgs {
+    const int* atom_pos_off = nullptr;
+    const int* atom_pos = nullptr;
+    const float4* atom_e = nullptr;
+    const float2* kbp = nullptr;
+    float2* kbc = nullptr;
+    int n_atoms = 0, total_slots = 0, n_proj = 0;
+    float dV = 0.f;
+};
+
+// ---- the separable kinetic energy (kernels_sep.cu): contexts without an energy cutoff.  sep_z: W =
+// T_z in, and the KB reduction of the batch when kr.n_atoms > 0; sep_y288: W += T_y in; sep_step: the
+// rest of the fused Chebyshev step with StepArgs::W = the sum so far (Wout unused).  KB tables per
+// sep_unit_points(n) consecutive points: an xy plane, 16 x rows at 288.
+int64_t sep_unit_points(int n);
+size_t sep_step_smem(int n, int max_unit_slots);
+cudaError_t sep_init_attributes(int n);
+void sep_z(int n, const float2* in, float2* W, int batch, float kscale, const float2* tw, const KbReduceArgs& kr,
+           cudaStream_t st);
+void sep_y288(const float2* in, float2* W, int batch, float kscale, const float2* tw, cudaStream_t st);
+void sep_step(int n, const StepArgs& a, int batch, float kscale, const float2* tw, cudaStream_t st);
+
 // ---- grid kernels (kernels_grid.cu)
 bool grid_supported(int n);
 cudaError_t grid_init_attributes(int n);
@@ -126,6 +149,7 @@ void launch_plane_inv(int n, const float2* W, int batch, const float2* tw, int m
 void launch_kb_project(int n, const KBDev& kb, const float2* b1, int batch, float dV, float2* kbc,
                        cudaStream_t st);
 // kbc[b][4a + p] = E_ap dV sum over atom a's plane slots of kbp[b][slot][p]
+KbReduceArgs kb_reduce_args(const KBDev& kb, const float2* kbp, float dV, float2* kbc);
 void launch_kb_reduce(const KBDev& kb, const float2* kbp, int batch, float dV, float2* kbc, cudaStream_t st);
 // density of TDH pairs for each sample, packed as (rho - rho0) + i d rho, fwd xy transformed into Wp.
 void launch_density_fwd(int n, const float2* psi, int n_samples, int n_eta, float weight, float* rho0,

@@ -1,0 +1,96 @@
+"""The separable kinetic path (contexts without a cutoff) against the transform path: a cutoff above
+every kinetic energy selects the latter and changes no operator, so the two agree to rounding on every
+grid, batch and KB form; and a plane with more KB slots than the separable step has room for."""
+import numpy as np
+import pytest
+
+from paper_2601_21005_gb300 import build, synth
+
+import gpu_common as gc
+
+torch = pytest.importorskip('torch')
+pytestmark = pytest.mark.gpu
+
+
+def _ctx(s, batch, ecut, kb):
+    from paper_2601_21005_gb300 import sgw
+    c = sgw.Context(s['n'], s['h'], ecut=ecut, max_batch=batch)
+    c.set_potential(gc.to_dev(s['vloc'].ravel(), torch, torch.float32), s['kb_atoms'] if kb else [])
+    c.set_spectrum(float(s['vloc'].min()) - 2.0, 0.5 * 3 * (np.pi / s['h']) ** 2 + 2.0)
+    return c
+
+
+def _system(n):
+    if n == 16:
+        s = synth.wells(n=16, h=0.6)
+        # two atoms of one and two projectors whose spheres overlap and wrap around the box
+        s['kb_atoms'] = [synth.kb_projectors(16, 0.6, (0.5, 9.0, 4.8), 0.9, (1.2,), 0),
+                         synth.kb_projectors(16, 0.6, (1.7, 8.1, 4.2), 0.8, (0.7, -0.3), 1)]
+        return s
+    hp = dict(synth.H_PARAMS)
+    hp['Es'] = 0.3
+    return synth.si_cluster(n=n, h=0.5, radius=4.5, hp=hp)
+
+
+# Rounding of one H application relative to its largest element: a chain of at most 6 line transforms
+# of depth log2 n <= 9 and a few sums, each adding at most 2^-24 of a value below |T|max |b|; their
+# random sum stays below 4 sqrt(6 * 9) 2^-24 = 1.8e-6 of it.  Sixteen terms of a propagation step
+# add at most in proportion.
+TOL_H = 1.8e-6
+
+
+@pytest.mark.parametrize('n', [16, 32, 48, 64, 96, 128, 288])
+@pytest.mark.parametrize('kb', [True, False])
+def test_separable_matches_the_transform_path(n, kb):
+    assert torch.cuda.is_available()
+    build.build()
+    s = _system(n)
+    B = 3 if n < 288 else 2
+    g = torch.Generator(device='cuda').manual_seed(n)
+    x = torch.randn(B, n ** 3, dtype=torch.complex64, device='cuda', generator=g)
+    outs = []
+    for ecut in (0.0, 1e6):
+        c = _ctx(s, 4, ecut, kb)
+        y = torch.empty_like(x)
+        c.apply_h(x, y)
+        p = x.clone()
+        c.propagate(p, 2, 0.05, 16, np.array([1, -1, 1], dtype=np.int8)[:B])
+        f = torch.empty_like(x)
+        c.filter_occupied(np.array([0.3, -0.2, 0.1]), x, f)          # the shortest plans: degrees 2 and 1
+        f1 = torch.empty_like(x)
+        c.filter_occupied(np.array([0.3, -0.2]), x, f1)
+        uR = torch.empty(1, 3, n ** 3, dtype=torch.float32, device='cuda')
+        src = x[0].real.contiguous()
+        c.tdh_response((0.05 * x[:2]).contiguous(), src, 1, 2, 2, 0.05, 10, uR)
+        torch.cuda.synchronize()
+        outs.append((y, p, f, f1, uR))
+        c.close()
+    for a, b, terms in zip(outs[0], outs[1], (1, 32, 2, 1, 40)):
+        assert float((a - b).abs().max() / b.abs().max()) < TOL_H * terms
+
+
+def test_more_slots_than_the_separable_step_holds():
+    """3090 one-point atoms in one 128^2 plane: above the separable step's 3072 slots, within the
+    transform path's 3104, so the context falls back to it.  V_NL is then diagonal."""
+    from paper_2601_21005_gb300 import sgw
+    build.build()
+    n, h, na, e, beta = 128, 0.5, 3090, 0.4, 1.3
+    pts = 5 * np.arange(na)                                  # z = 0
+    atoms = [(np.array([p]), np.full((1, 1), beta), np.array([e])) for p in pts]
+    g = torch.Generator(device='cuda').manual_seed(1)
+    v = torch.randn(n ** 3, device='cuda', generator=g)
+    x = torch.randn(2, n ** 3, dtype=torch.complex64, device='cuda', generator=g)
+    a = sgw.Context(n, h, max_batch=2)
+    a.set_potential(v, atoms)
+    ya = torch.empty_like(x)
+    a.apply_h(x, ya)
+    w = v.clone()
+    w[torch.as_tensor(pts, device='cuda')] += e * beta * beta * h ** 3
+    b = sgw.Context(n, h, max_batch=2)
+    b.set_potential(w)
+    yb = torch.empty_like(x)
+    b.apply_h(x, yb)
+    assert float((ya - yb).abs().max() / yb.abs().max()) < TOL_H
+    a.set_potential(w)                                       # without the atoms the separable step is back
+    a.apply_h(x, ya)
+    assert torch.equal(ya, yb)
