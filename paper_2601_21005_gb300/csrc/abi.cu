@@ -36,7 +36,7 @@ struct sgw_ctx {
     float2* B1 = nullptr;      // [max_batch][ng]
     float2* B2 = nullptr;      // [max_batch][ng]
     sgw::VecInfo* info = nullptr;  // [max_batch]
-    float2* kbc = nullptr;     // [max_batch][n_proj]
+    float2* kbc = nullptr;     // [max_batch][total_slots][4] E-weighted projections, per slot
     float2* kbp = nullptr;     // [max_batch][total_slots][4] per-plane partial projections
     sgw::KBDev kb;
     double* scal = nullptr;    // small FP64 scratch
@@ -292,7 +292,7 @@ std::vector<Step> clenshaw_plan(const std::vector<cd>* c, const cd* phase, int K
 // Free every KB device array of the context
 void free_kb(sgw_ctx* ctx) {
     sgw::KBDev& kb = ctx->kb;
-    void* ptrs[] = {kb.atom_nproj, kb.atom_off, kb.sup_idx, kb.sup_beta, kb.atom_e, kb.plane_off, kb.slot_atom,
+    void* ptrs[] = {kb.atom_nproj, kb.atom_off, kb.sup_idx, kb.sup_beta, kb.atom_e, kb.plane_off,
                     kb.kbe_col, kb.kbe_os, kb.kbe_beta, kb.kbe_slot_beg, kb.kbe_slot_end, kb.atom_pos_off,
                     kb.atom_pos, ctx->kbc, ctx->kbp};
     for (void* p : ptrs)
@@ -315,7 +315,6 @@ void free_kb(sgw_ctx* ctx) {
 void set_kb_args(const sgw_ctx* ctx, sgw::StepArgs& a) {
     const sgw::KBDev& kb = ctx->kb;
     a.plane_off = kb.plane_off;
-    a.slot_atom = kb.slot_atom;
     a.kbe_col = kb.kbe_col;
     a.kbe_os = kb.kbe_os;
     a.kbe_beta = kb.kbe_beta;
@@ -324,7 +323,6 @@ void set_kb_args(const sgw_ctx* ctx, sgw::StepArgs& a) {
     a.max_colors = kb.max_colors;
     a.max_plane_slots = kb.max_plane_slots;
     a.total_slots = kb.total_slots;
-    a.n_proj = kb.n_proj;
 }
 
 // The fused step's arguments that do not depend on the kinetic path.
@@ -987,13 +985,9 @@ sgw_status sgw_set_potential(sgw_ctx* ctx, const float* vloc_dev, int n_atoms, c
         for (int z = 0; z < nu; ++z) plane_off[z + 1] = plane_off[z] + (int)plane_atoms[z].size();
         const int total_slots = plane_off[nu];
         if (!ctx->sep) CK(sgw::plane_step_reserve_smem(n, max_slots));
-        std::vector<int> slot_atom(std::max(total_slots, 1));
         std::vector<std::vector<int>> atom_slots(n_atoms);
         for (int z = 0; z < nu; ++z)
-            for (int k = 0; k < (int)plane_atoms[z].size(); ++k) {
-                slot_atom[plane_off[z] + k] = plane_atoms[z][k];
-                atom_slots[plane_atoms[z][k]].push_back(plane_off[z] + k);
-            }
+            for (int k = 0; k < (int)plane_atoms[z].size(); ++k) atom_slots[plane_atoms[z][k]].push_back(plane_off[z] + k);
         std::vector<int> atom_pos_off(n_atoms + 1, 0), atom_pos;
         for (int a = 0; a < n_atoms; ++a) {
             atom_pos_off[a + 1] = atom_pos_off[a] + (int)atom_slots[a].size();
@@ -1032,7 +1026,8 @@ sgw_status sgw_set_potential(sgw_ctx* ctx, const float* vloc_dev, int n_atoms, c
                     if (slot_col[plane_off[z] + k] != c) continue;
                     kbe_slot_beg[plane_off[z] + k] = (int)kbe_os.size();
                     for (int64_t i = plane_runs[z][k].first; i < plane_runs[z][k].second; ++i) {
-                        kbe_os.push_back((unsigned)(sup_idx_host[i] - z * plane_sz) | ((unsigned)k << 16));
+                        const int o = (int)(sup_idx_host[i] - z * plane_sz);
+                        kbe_os.push_back((unsigned)(ctx->sep ? sgw::sep_unit_pos(n, o) : o) | ((unsigned)k << 16));
                         kbe_beta.push_back(sup_beta[i]);
                     }
                     kbe_slot_end[plane_off[z] + k] = (int)kbe_os.size();
@@ -1045,7 +1040,6 @@ sgw_status sgw_set_potential(sgw_ctx* ctx, const float* vloc_dev, int n_atoms, c
         kb.max_plane_slots = max_slots;
         kb.max_colors = max_colors;
         kb.n_atoms = n_atoms;
-        kb.n_proj = 4 * n_atoms;
         kb.n_sup = nsup;
         const size_t ns1 = std::max<int64_t>(nsup, 1), ts1 = std::max(total_slots, 1);
         bool ok = cudaMalloc(&kb.atom_nproj, sizeof(int) * n_atoms) == cudaSuccess &&
@@ -1054,7 +1048,6 @@ sgw_status sgw_set_potential(sgw_ctx* ctx, const float* vloc_dev, int n_atoms, c
                   cudaMalloc(&kb.sup_beta, sizeof(float4) * ns1) == cudaSuccess &&
                   cudaMalloc(&kb.atom_e, sizeof(float4) * n_atoms) == cudaSuccess &&
                   cudaMalloc(&kb.plane_off, sizeof(int) * (nu + 1)) == cudaSuccess &&
-                  cudaMalloc(&kb.slot_atom, sizeof(int) * ts1) == cudaSuccess &&
                   cudaMalloc(&kb.kbe_col, sizeof(int) * kbe_col.size()) == cudaSuccess &&
                   cudaMalloc(&kb.kbe_os, sizeof(unsigned) * ns1) == cudaSuccess &&
                   cudaMalloc(&kb.kbe_beta, sizeof(float4) * ns1) == cudaSuccess &&
@@ -1062,7 +1055,7 @@ sgw_status sgw_set_potential(sgw_ctx* ctx, const float* vloc_dev, int n_atoms, c
                   cudaMalloc(&kb.kbe_slot_end, sizeof(int) * ts1) == cudaSuccess &&
                   cudaMalloc(&kb.atom_pos_off, sizeof(int) * (n_atoms + 1)) == cudaSuccess &&
                   cudaMalloc(&kb.atom_pos, sizeof(int) * ts1) == cudaSuccess &&
-                  cudaMalloc(&ctx->kbc, sizeof(float2) * (size_t)kb.n_proj * ctx->max_batch) == cudaSuccess &&
+                  cudaMalloc(&ctx->kbc, sizeof(float2) * 4 * ts1 * ctx->max_batch) == cudaSuccess &&
                   cudaMalloc(&ctx->kbp, sizeof(float2) * 4 * ts1 * ctx->max_batch) == cudaSuccess;
         if (!ok) {
             cudaGetLastError();
@@ -1075,7 +1068,6 @@ sgw_status sgw_set_potential(sgw_ctx* ctx, const float* vloc_dev, int n_atoms, c
         CK(cudaMemcpy(kb.sup_beta, sup_beta.data(), sizeof(float4) * nsup, cudaMemcpyHostToDevice));
         CK(cudaMemcpy(kb.atom_e, atom_e.data(), sizeof(float4) * n_atoms, cudaMemcpyHostToDevice));
         CK(cudaMemcpy(kb.plane_off, plane_off.data(), sizeof(int) * (nu + 1), cudaMemcpyHostToDevice));
-        CK(cudaMemcpy(kb.slot_atom, slot_atom.data(), sizeof(int) * ts1, cudaMemcpyHostToDevice));
         CK(cudaMemcpy(kb.kbe_col, kbe_col.data(), sizeof(int) * kbe_col.size(), cudaMemcpyHostToDevice));
         CK(cudaMemcpy(kb.kbe_os, kbe_os.data(), sizeof(unsigned) * nsup, cudaMemcpyHostToDevice));
         CK(cudaMemcpy(kb.kbe_beta, kbe_beta.data(), sizeof(float4) * nsup, cudaMemcpyHostToDevice));

@@ -11,11 +11,12 @@
 
 namespace sgw {
 
-constexpr int KB_B = 4;    // KB entries per lane whose loads are in flight together
+constexpr int KB_B = 3;    // KB entries per lane whose loads are in flight together
 
 // Position in shared memory of unit point o = y N + x (row y, column x) at row pitch P.  LAYOUT 0:
 // natural, y P + x.  LAYOUT 1 (N = 288, the two-stage row transforms): a row is 16 groups of 19
 // slots, column x at 19 (x mod 16) + x div 16, the order in which the 16 x 18 transforms leave it.
+// LAYOUT 2: the tables hold the positions themselves.
 template <int N, int P, int LAYOUT>
 __device__ __forceinline__ int unit_pos_yx(int y, int x) {
     if constexpr (LAYOUT == 1) {
@@ -27,12 +28,15 @@ __device__ __forceinline__ int unit_pos_yx(int y, int x) {
 }
 template <int N, int P, int LAYOUT>
 __device__ __forceinline__ int unit_pos(int o) {
-    return unit_pos_yx<N, P, LAYOUT>(o / N, o % N);
+    if constexpr (LAYOUT == 2) return o;
+    else return unit_pos_yx<N, P, LAYOUT>(o / N, o % N);
 }
 
-// kbc[b][4a + p] = E_ap dV sum_{slots of a} kbp[b][slot][p] by one warp: lane l takes projector p =
-// l % 4 of the atom's slots l / 4, l / 4 + 8, ... (in increasing unit), then the eight lanes of each p
-// are summed by a fixed shuffle tree.  The whole warp calls it with one (a, b); a >= n_atoms does nothing.
+// kbc[b][k][p] = E_ap dV sum_{slots of a} kbp[b][slot][p] for every slot k of atom a, by one warp: lane l
+// takes projector p = l % 4 of the atom's slots l / 4, l / 4 + 8, ... (in increasing unit), then the
+// eight lanes of each p are summed by a fixed shuffle tree.  The result is stored once per slot, so
+// that a unit's coefficients are one contiguous run (through the slot's atom they would be two more
+// dependent loads away).  The whole warp calls it with one (a, b); a >= n_atoms does nothing.
 __device__ __forceinline__ void kb_reduce_warp(const KbReduceArgs& kr, int a, int b, int lane) {
     if (a >= kr.n_atoms) return;
     const int p = lane & 3;
@@ -49,86 +53,167 @@ __device__ __forceinline__ void kb_reduce_warp(const KbReduceArgs& kr, int a, in
         acc.x += __shfl_xor_sync(0xffffffffu, acc.x, off);
         acc.y += __shfl_xor_sync(0xffffffffu, acc.y, off);
     }
-    if (lane < 4) {
-        const float4 e = __ldg(kr.atom_e + a);
-        const float ep = (p == 0 ? e.x : (p == 1 ? e.y : (p == 2 ? e.z : e.w))) * kr.dV;
-        kr.kbc[(size_t)b * kr.n_proj + a * 4 + p] = make_float2(ep * acc.x, ep * acc.y);
+    const float4 e = __ldg(kr.atom_e + a);
+    const float ep = (p == 0 ? e.x : (p == 1 ? e.y : (p == 2 ? e.z : e.w))) * kr.dV;
+    const float2 r = make_float2(ep * acc.x, ep * acc.y);
+    float2* kc = kr.kbc + (size_t)b * kr.total_slots * 4;
+    for (int q = q0 + (lane >> 2); q < q1; q += 8) kc[(size_t)__ldg(kr.atom_pos + q) * 4 + p] = r;
+}
+
+// What a block needs to know of its unit before it can load anything else: the unit's slots s0 .. s1
+// and the bounds of its colours, lane c of every warp holding the begin of colour c and `end` the
+// end of the last (at most 32 colours).  Loaded together, first of all.
+struct KbHead {
+    int s0 = 0, s1 = 0, col = 0, end = 0;
+    // begin of colour c (c <= max_colors); the whole warp calls it with one c
+    __device__ __forceinline__ int begin(int c, int max_colors) const {
+        const int v = __shfl_sync(0xffffffffu, col, c & 31);
+        return c >= max_colors ? end : v;
     }
+};
+__device__ __forceinline__ KbHead kb_head(const StepArgs& a, int u) {
+    KbHead h;
+    const int lane = threadIdx.x & 31;
+    const int* col = a.kbe_col + (size_t)u * (a.max_colors + 1);
+    h.s0 = __ldg(a.plane_off + u);
+    h.s1 = __ldg(a.plane_off + u + 1);
+    h.end = __ldg(col + a.max_colors);
+    h.col = __ldg(col + min(lane, a.max_colors));
+    return h;
 }
 
 // E-weighted projector coefficients of the unit's slots into shared memory: kcs[4 s + p] for the
-// unit's s-th slot and projector p.
+// unit's s-th slot and projector p (kc: the vector's coefficients, [slot][4]).
 template <int NT>
-__device__ __forceinline__ void kb_stage_coeffs(const StepArgs& a, const float2* __restrict__ kc, int u, float2* kcs) {
-    const int s0 = __ldg(a.plane_off + u), ns = __ldg(a.plane_off + u + 1) - s0;
-    for (int i = threadIdx.x; i < 4 * ns; i += NT) kcs[i] = kc[__ldg(a.slot_atom + s0 + i / 4) * 4 + (i & 3)];
+__device__ __forceinline__ void kb_stage_coeffs(const KbHead& h, const float2* __restrict__ kc, float2* kcs) {
+    const float4* src = reinterpret_cast<const float4*>(kc + (size_t)4 * h.s0);
+    for (int i = threadIdx.x; i < 2 * (h.s1 - h.s0); i += NT) reinterpret_cast<float4*>(kcs)[i] = __ldg(src + i);
 }
+
+// KB_B entries of a lane (at eb, eb + stride, ...; past e1 the last one again, to be skipped by the
+// reader), all their loads in flight at once.
+struct KbBatch {
+    unsigned os[KB_B];
+    float4 be[KB_B];
+    __device__ __forceinline__ void load(const StepArgs& a, int eb, int stride, int e1) {
+#pragma unroll
+        for (int i = 0; i < KB_B; ++i) {
+            const int e = min(eb + i * stride, e1 - 1);
+            os[i] = __ldg(a.kbe_os + e);
+            be[i] = __ldg(a.kbe_beta + e);
+        }
+    }
+};
 
 // sm += sum_ap beta_ap E_ap <beta_ap|b1> over the unit, colour by colour (slots of one colour touch
 // disjoint points, so each point is updated by one thread at a time; no atomics, fixed order).
-// Call after a barrier that made sm and kcs visible; returns after a barrier.
-template <int N, int P, int NT, int LAYOUT = 0>
-__device__ __forceinline__ void kb_apply_unit(const StepArgs& a, int u, const float2* kcs, float2* sm) {
-    const int* col = a.kbe_col + (size_t)u * (a.max_colors + 1);
-    for (int c = 0; c < a.max_colors; ++c) {
-        const int e0 = __ldg(col + c), e1 = __ldg(col + c + 1);
-        if (e0 == e1) break;                  // a unit's colours are used from 0 upwards
-        // batches of KB_B entries whose loads are all in flight at once, the last one padded: the
-        // loads' latency is paid per batch, and a remainder taken entry by entry would pay it each time
-        for (int eb = e0 + threadIdx.x; eb < e1; eb += KB_B * NT) {
-            unsigned os[KB_B];
-            float4 be[KB_B];
+// The entries' loads run one batch ahead, over the ends of the colours and past the barriers: the
+// tables come from L2, and a batch's latency would otherwise be paid once per colour and remainder.
+// (Two and three batches ahead, or larger ones, cost more registers than the latency they hid.)
+// meanwhile() runs after the first loads are on their way; a barrier before the first update of sm
+// makes its stores (and the caller's) visible; returns after a barrier.
+template <int N, int P, int NT, int LAYOUT = 0, class F>
+__device__ __forceinline__ void kb_apply_unit(const StepArgs& a, const KbHead& h, const float2* kcs, float2* sm,
+                                              F&& meanwhile) {
+    int c = 1, e0 = h.begin(0, a.max_colors), e1 = h.begin(1, a.max_colors);   // e0 .. e1 the rest of colour c - 1
+    KbBatch cur;
+    if (e0 < e1) cur.load(a, e0 + threadIdx.x, NT, e1);
+    meanwhile();
+    __syncthreads();
+    while (e0 < e1) {                     // a unit's colours are used from 0 upwards
+        KbBatch nxt;
+        const int en = e0 + KB_B * NT;
+        const bool last = en >= e1;
+        const int e2 = h.begin(c + 1, a.max_colors);
+        if (!last) nxt.load(a, en + threadIdx.x, NT, e1);
+        else if (e1 < e2) nxt.load(a, e1 + threadIdx.x, NT, e2);
 #pragma unroll
-            for (int i = 0; i < KB_B; ++i) {
-                const int e = min(eb + i * NT, e1 - 1);
-                os[i] = __ldg(a.kbe_os + e);
-                be[i] = __ldg(a.kbe_beta + e);
-            }
-#pragma unroll
-            for (int i = 0; i < KB_B; ++i) {
-                if (eb + i * NT >= e1) break;
-                const int o = (int)(os[i] & 0xffffu), sl = (int)(os[i] >> 16);
-                const float4 c01 = *reinterpret_cast<const float4*>(kcs + 4 * sl);
-                const float4 c23 = *reinterpret_cast<const float4*>(kcs + 4 * sl + 2);
-                float2& hv = sm[unit_pos<N, P, LAYOUT>(o)];
-                hv.x += be[i].x * c01.x + be[i].y * c01.z + be[i].z * c23.x + be[i].w * c23.z;
-                hv.y += be[i].x * c01.y + be[i].y * c01.w + be[i].z * c23.y + be[i].w * c23.w;
-            }
+        for (int i = 0; i < KB_B; ++i) {
+            if (e0 + (int)threadIdx.x + i * NT >= e1) break;
+            const float4 be = cur.be[i];
+            const int o = (int)(cur.os[i] & 0xffffu), sl = (int)(cur.os[i] >> 16);
+            const float4 c01 = *reinterpret_cast<const float4*>(kcs + 4 * sl);
+            const float4 c23 = *reinterpret_cast<const float4*>(kcs + 4 * sl + 2);
+            float2& hv = sm[unit_pos<N, P, LAYOUT>(o)];
+            hv.x += be.x * c01.x + be.y * c01.z + be.z * c23.x + be.w * c23.z;
+            hv.y += be.x * c01.y + be.y * c01.w + be.z * c23.y + be.w * c23.w;
         }
-        __syncthreads();
+        cur = nxt;
+        if (!last) {
+            e0 = en;
+        } else {
+            e0 = e1;
+            e1 = e2;
+            ++c;
+            __syncthreads();
+        }
     }
 }
 
-// Partial projections of the unit's values in sm (positions by unit_pos): kbp[b][slot][p] = sum over the slot's points of
-// beta_ap(r) sm(r); one warp per slot, lanes strided over the points, fixed-order warp reduction.
+// Partial projections of the unit's values in sm (positions by unit_pos): kbp[b][slot][p] = sum over the
+// slot's points of beta_ap(r) sm(r); one warp per slot, lanes strided over the points, fixed-order warp
+// reduction.  The loads run one batch ahead here too, over the ends of the slots; kb_project_begin
+// finds the warp's first two slots and can be called long before.
+struct KbSlots {
+    int k = 0, e0 = 0, e1 = 0, f0 = 0, f1 = 0;      // slot k's entries e0 .. e1, the warp's next slot's f0 .. f1
+};
+template <int NT>
+__device__ __forceinline__ KbSlots kb_project_begin(const StepArgs& a, const KbHead& h) {
+    constexpr int NW = NT / 32;
+    KbSlots s;
+    s.k = h.s0 + (threadIdx.x >> 5);
+    if (s.k < h.s1) {
+        s.e0 = __ldg(a.kbe_slot_beg + s.k);
+        s.e1 = __ldg(a.kbe_slot_end + s.k);
+        if (s.k + NW < h.s1) {
+            s.f0 = __ldg(a.kbe_slot_beg + s.k + NW);
+            s.f1 = __ldg(a.kbe_slot_end + s.k + NW);
+        }
+    }
+    return s;
+}
+// Meets a barrier before it reads sm.
 template <int N, int P, int NT, int LAYOUT = 0>
-__device__ __forceinline__ void kb_project_unit(const StepArgs& a, int u, int b, const float2* sm) {
-    const int sb = __ldg(a.plane_off + u), s1 = __ldg(a.plane_off + u + 1);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int k = sb + warp; k < s1; k += NT / 32) {
-        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        const int e1 = __ldg(a.kbe_slot_end + k);
-        for (int eb = __ldg(a.kbe_slot_beg + k) + lane; eb < e1; eb += KB_B * 32) {
-            unsigned os[KB_B];
-            float4 be[KB_B];
+__device__ __forceinline__ void kb_project_unit(const StepArgs& a, const KbHead& h, const KbSlots& sl, int b, const float2* sm) {
+    constexpr int NW = NT / 32;
+    const int s1 = h.s1, lane = threadIdx.x & 31;
+    int k = sl.k, e0 = sl.e0, e1 = sl.e1, f0 = sl.f0, f1 = sl.f1;
+    KbBatch cur;
+    if (k < s1) cur.load(a, e0 + lane, 32, e1);
+    __syncthreads();
+    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    while (k < s1) {                      // a slot has at least one entry
+        KbBatch nxt;
+        const int en = e0 + KB_B * 32;
+        const bool last = en >= e1;
+        if (!last) nxt.load(a, en + lane, 32, e1);
+        else if (k + NW < s1) nxt.load(a, f0 + lane, 32, f1);
 #pragma unroll
-            for (int i = 0; i < KB_B; ++i) {
-                const int e = min(eb + 32 * i, e1 - 1);
-                os[i] = __ldg(a.kbe_os + e);
-                be[i] = __ldg(a.kbe_beta + e);
-            }
-#pragma unroll
-            for (int i = 0; i < KB_B; ++i) {
-                if (eb + 32 * i >= e1) break;
-                const float2 v = sm[unit_pos<N, P, LAYOUT>((int)(os[i] & 0xffffu))];
-                acc[0] += be[i].x * v.x; acc[1] += be[i].x * v.y;
-                acc[2] += be[i].y * v.x; acc[3] += be[i].y * v.y;
-                acc[4] += be[i].z * v.x; acc[5] += be[i].z * v.y;
-                acc[6] += be[i].w * v.x; acc[7] += be[i].w * v.y;
-            }
+        for (int i = 0; i < KB_B; ++i) {
+            if (e0 + lane + 32 * i >= e1) break;
+            const float2 v = sm[unit_pos<N, P, LAYOUT>((int)(cur.os[i] & 0xffffu))];
+            const float4 be = cur.be[i];
+            acc[0] += be.x * v.x; acc[1] += be.x * v.y;
+            acc[2] += be.y * v.x; acc[3] += be.y * v.y;
+            acc[4] += be.z * v.x; acc[5] += be.z * v.y;
+            acc[6] += be.w * v.x; acc[7] += be.w * v.y;
+        }
+        cur = nxt;
+        if (!last) {
+            e0 = en;
+            continue;
         }
         const float r = warp_reduce_scatter8(acc, lane);
         if ((lane & 3) == 0) reinterpret_cast<float*>(a.kbp + ((size_t)b * a.total_slots + k) * 4)[lane >> 2] = r;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) acc[i] = 0.f;
+        k += NW;
+        e0 = f0;
+        e1 = f1;
+        if (k + NW < s1) {
+            f0 = __ldg(a.kbe_slot_beg + k + NW);
+            f1 = __ldg(a.kbe_slot_end + k + NW);
+        }
     }
 }
 

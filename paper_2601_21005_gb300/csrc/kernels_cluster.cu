@@ -93,8 +93,10 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(CPlaneCfg<V>::W * 3
     const size_t off = (size_t)b * NG + uoff;
     for (int i = threadIdx.x; i < CN; i += CNT) tws[i] = __ldg(tw + i);
     const VecInfo inf = a.info[b];
-    const float2* kc = a.kbc != nullptr ? a.kbc + (size_t)b * a.n_proj : nullptr;
-    if (kc != nullptr) kb_stage_coeffs<CNT>(a, kc, u, kcs);
+    const float2* kc = a.kbc != nullptr ? a.kbc + (size_t)b * a.total_slots * 4 : nullptr;
+    KbHead kh;
+    if (a.kbc != nullptr || a.kbp != nullptr) kh = kb_head(a, u);
+    if (kc != nullptr) kb_stage_coeffs<CNT>(kh, kc, kcs);
     // columns 36c .. 36c + 35 of the plane from HBM (rows of 288 bytes)
     {
         const float2* src = a.W + plane + c * CS;
@@ -130,11 +132,11 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(CPlaneCfg<V>::W * 3
         for (int k = 0; k < 9; ++k) rowb[l * PR + k + 9 * k1] = v[k];
     }
     __syncthreads();
-    if (kc != nullptr) kb_apply_unit<CN, PR, CNT>(a, u, kcs, rowb);
+    if (kc != nullptr) kb_apply_unit<CN, PR, CNT>(a, kh, kcs, rowb, [] {});
     step_pointwise<CN, CS, PR, CNT>(a, inf, off, uoff, rowb);
     cl.sync();                                             // (2) no CTA reads another's columns any more
     if (a.Wout == nullptr) return;
-    if (a.kbp != nullptr) kb_project_unit<CN, PR, CNT>(a, u, b, rowb);
+    if (a.kbp != nullptr) kb_project_unit<CN, PR, CNT>(a, kh, kb_project_begin<CNT>(a, kh), b, rowb);
     // forward FFT along x, a warp per row; point x goes to column x mod 36 of CTA x / 36
     for (int l = warp; l < CS; l += NW) {
         const int row = c * CS + l;
@@ -269,8 +271,10 @@ __global__ void __launch_bounds__(NW * 32, 2) k_rows36_step(StepArgs a, const fl
         }
     }
     for (int i = threadIdx.x; i < CN; i += CNT) tws[i] = __ldg(tw + i);
-    const float2* kc = a.kbc != nullptr ? a.kbc + (size_t)b * a.n_proj : nullptr;
-    if (kc != nullptr) kb_stage_coeffs<CNT>(a, kc, u, kcs);
+    const float2* kc = a.kbc != nullptr ? a.kbc + (size_t)b * a.total_slots * 4 : nullptr;
+    KbHead kh;
+    if (a.kbc != nullptr || a.kbp != nullptr) kh = kb_head(a, u);
+    if (kc != nullptr) kb_stage_coeffs<CNT>(kh, kc, kcs);
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
     for (int l = warp; l < CS; l += NW) {
@@ -283,7 +287,7 @@ __global__ void __launch_bounds__(NW * 32, 2) k_rows36_step(StepArgs a, const fl
         for (int k = 0; k < 9; ++k) rowb[l * PR36 + k + 9 * k1] = v[k];
     }
     __syncthreads();
-    if (kc != nullptr) kb_apply_unit<CN, PR36, CNT>(a, u, kcs, rowb);
+    if (kc != nullptr) kb_apply_unit<CN, PR36, CNT>(a, kh, kcs, rowb, [] {});
     const bool stream = (a.pf_operands & 2) != 0;
     if (stream)
         step_pointwise<CN, CS, PR36, CNT, 4, 0, true>(a, inf, off, uoff, rowb);
@@ -291,7 +295,7 @@ __global__ void __launch_bounds__(NW * 32, 2) k_rows36_step(StepArgs a, const fl
         step_pointwise<CN, CS, PR36, CNT, 4>(a, inf, off, uoff, rowb);
     if (a.Wout == nullptr) return;
     __syncthreads();
-    if (a.kbp != nullptr) kb_project_unit<CN, PR36, CNT>(a, u, b, rowb);
+    if (a.kbp != nullptr) kb_project_unit<CN, PR36, CNT>(a, kh, kb_project_begin<CNT>(a, kh), b, rowb);
     __syncthreads();
     for (int l = warp; l < CS; l += NW) {
         float2 v[9];

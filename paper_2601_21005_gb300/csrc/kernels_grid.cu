@@ -334,11 +334,11 @@ __device__ __forceinline__ void plane_step_body(const StepArgs& a, float2* sm, f
     const float* dV = (a.dvpot != nullptr && inf.dvrow >= 0) ? a.dvpot + (size_t)inf.dvrow * NG + (size_t)z * N * N
                                                                  : nullptr;
     const float2* bp = (dV != nullptr) ? a.b1 + ((size_t)inf.partner * N + z) * N * N : nullptr;
-    const float2* kc = a.kbc != nullptr ? a.kbc + (size_t)b * a.n_proj : nullptr;
+    const float2* kc = a.kbc != nullptr ? a.kbc + (size_t)b * a.total_slots * 4 : nullptr;
     const int s0 = kc != nullptr ? __ldg(a.plane_off + z) : 0;
     if (kc != nullptr) {
         const int ns = __ldg(a.plane_off + z + 1) - s0;
-        for (int i = threadIdx.x; i < 4 * ns; i += NT) kcs[i] = kc[__ldg(a.slot_atom + s0 + i / 4) * 4 + (i & 3)];
+        for (int i = threadIdx.x; i < 4 * ns; i += NT) kcs[i] = kc[4 * s0 + i];
     }
     if constexpr (IN_SMEM) {
         fft2_plane<N, NT, +1>(sm, tws);                // the plane is already in shared memory
@@ -726,11 +726,10 @@ k_kb_split(const int* __restrict__ atoms, const int64_t* __restrict__ atom_off, 
 }
 
 // ------------------------------------------------------------------ KB projection
-// kbc[b][4a + p] = E_ap * dV * sum_{r in support(a)} beta_ap(r) b1_b(r)
+// kbc[b][k][p] = E_ap * dV * sum_{r in support(a)} beta_ap(r) b1_b(r) for every slot k of atom a
 __global__ void __launch_bounds__(256)
 k_kb_project(const int64_t* __restrict__ atom_off, const int* __restrict__ sup_idx, const float4* __restrict__ sup_beta,
-             const float4* __restrict__ atom_e, const float2* __restrict__ b1, size_t ng, int n_proj, float dV,
-             float2* __restrict__ kbc) {
+             const float2* __restrict__ b1, size_t ng, KbReduceArgs kr) {
     __shared__ float red[8][8];
     const int at = blockIdx.x, b = blockIdx.y;
     const int64_t s0 = atom_off[at], s1 = atom_off[at + 1];
@@ -754,10 +753,12 @@ k_kb_project(const int64_t* __restrict__ atom_off, const int* __restrict__ sup_i
     if (threadIdx.x < 8) {
         float t = 0.f;
         for (int k = 0; k < nw; ++k) t += red[k][threadIdx.x];
-        const float4 e = __ldg(atom_e + at);
+        const float4 e = __ldg(kr.atom_e + at);
         const int p = threadIdx.x >> 1;
         const float ep = p == 0 ? e.x : (p == 1 ? e.y : (p == 2 ? e.z : e.w));
-        reinterpret_cast<float*>(kbc + (size_t)b * n_proj + at * 4)[threadIdx.x] = ep * dV * t;
+        float* kc = reinterpret_cast<float*>(kr.kbc + (size_t)b * kr.total_slots * 4);
+        for (int q = __ldg(kr.atom_pos_off + at); q < __ldg(kr.atom_pos_off + at + 1); ++q)
+            kc[(size_t)__ldg(kr.atom_pos + q) * 8 + threadIdx.x] = ep * kr.dV * t;
     }
 }
 
@@ -777,7 +778,6 @@ KbReduceArgs kb_reduce_args(const KBDev& kb, const float2* kbp, float dV, float2
     r.kbc = kbc;
     r.n_atoms = kb.n_atoms;
     r.total_slots = kb.total_slots;
-    r.n_proj = kb.n_proj;
     r.dV = dV;
     return r;
 }
@@ -1018,8 +1018,8 @@ void launch_kb_split(const int* atoms, int n_atoms_colour, const KBDev& kb, cons
 void launch_kb_project(int n, const KBDev& kb, const float2* b1, int batch, float dV, float2* kbc, cudaStream_t st) {
     if (kb.n_atoms == 0 || batch == 0) return;
     const size_t ng = (size_t)n * n * n;
-    k_kb_project<<<dim3(kb.n_atoms, batch), 256, 0, st>>>(kb.atom_off, kb.sup_idx, kb.sup_beta, kb.atom_e, b1, ng,
-                                                         kb.n_proj, dV, kbc);
+    k_kb_project<<<dim3(kb.n_atoms, batch), 256, 0, st>>>(kb.atom_off, kb.sup_idx, kb.sup_beta, b1, ng,
+                                                         kb_reduce_args(kb, nullptr, dV, kbc));
 }
 
 }  // namespace sgw

@@ -146,8 +146,10 @@ __global__ void __launch_bounds__(NW * 32, 2) k_rows36_2s(StepArgs a, const floa
         }
     }
     for (int i = threadIdx.x; i < R2N; i += CNT) tws[i] = __ldg(tw + i);
-    const float2* kc = a.kbc != nullptr ? a.kbc + (size_t)b * a.n_proj : nullptr;
-    if (kc != nullptr) kb_stage_coeffs<CNT>(a, kc, u, kcs);
+    const float2* kc = a.kbc != nullptr ? a.kbc + (size_t)b * a.total_slots * 4 : nullptr;
+    KbHead kh;
+    if (a.kbc != nullptr || a.kbp != nullptr) kh = kb_head(a, u);
+    if (kc != nullptr) kb_stage_coeffs<CNT>(kh, kc, kcs);
     __syncthreads();
     float2 v[18];
     {
@@ -173,7 +175,7 @@ __global__ void __launch_bounds__(NW * 32, 2) k_rows36_2s(StepArgs a, const floa
         for (int k2 = 0; k2 < 18; ++k2) g[k2] = v[k2];
     }
     __syncthreads();
-    if (kc != nullptr) kb_apply_unit<R2N, R2P, CNT, 1>(a, u, kcs, rowb);
+    if (kc != nullptr) kb_apply_unit<R2N, R2P, CNT, 1>(a, kh, kcs, rowb, [] {});
     const bool stream = (a.pf_operands & 2) != 0;
     if (stream)
         step_pointwise<R2N, R2S, R2P, CNT, 4, 1, true>(a, inf, off, uoff, rowb);
@@ -181,7 +183,7 @@ __global__ void __launch_bounds__(NW * 32, 2) k_rows36_2s(StepArgs a, const floa
         step_pointwise<R2N, R2S, R2P, CNT, 4, 1>(a, inf, off, uoff, rowb);
     if (a.Wout == nullptr) return;
     __syncthreads();
-    if (a.kbp != nullptr) kb_project_unit<R2N, R2P, CNT, 1>(a, u, b, rowb);
+    if (a.kbp != nullptr) kb_project_unit<R2N, R2P, CNT, 1>(a, kh, kb_project_begin<CNT>(a, kh), b, rowb);
     __syncthreads();
     for (int w = threadIdx.x; w < R2S * 16; w += CNT) {
         const int m2 = w & 15;

@@ -250,16 +250,18 @@ __global__ void __launch_bounds__(RNT) k_rows_step(StepArgs a, const float2* __r
     const size_t uoff = (size_t)u * RR * N;
     const size_t off = (size_t)b * NG + uoff;
     const VecInfo inf = a.info[b];
-    const float2* kc = a.kbc != nullptr ? a.kbc + (size_t)b * a.n_proj : nullptr;
-    if (kc != nullptr) kb_stage_coeffs<RNT>(a, kc, u, kcs);
+    const float2* kc = a.kbc != nullptr ? a.kbc + (size_t)b * a.total_slots * 4 : nullptr;
+    KbHead kh;
+    if (a.kbc != nullptr || a.kbp != nullptr) kh = kb_head(a, u);
+    if (kc != nullptr) kb_stage_coeffs<RNT>(kh, kc, kcs);
     load_rows<N>(sm, a.W + off);
     __syncthreads();
     fft_lines<N, RR, P, 1, RNT, +1>(sm, tws);
-    if (kc != nullptr) kb_apply_unit<N, P, RNT>(a, u, kcs, sm);
+    if (kc != nullptr) kb_apply_unit<N, P, RNT>(a, kh, kcs, sm, [] {});
     step_pointwise<N, RR, P, RNT>(a, inf, off, uoff, sm);
     if (a.Wout == nullptr) return;
     __syncthreads();
-    if (a.kbp != nullptr) kb_project_unit<N, P, RNT>(a, u, b, sm);
+    if (a.kbp != nullptr) kb_project_unit<N, P, RNT>(a, kh, kb_project_begin<RNT>(a, kh), b, sm);
     fft_lines<N, RR, P, 1, RNT, -1>(sm, tws);
     store_rows<N>(a.Wout + off, sm);
 }

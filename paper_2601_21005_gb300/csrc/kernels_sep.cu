@@ -14,8 +14,9 @@
 // line is held in the registers of 2 or 4 lanes (reg_dft.cuh), so a transform takes no barrier; a
 // plane's block meets one barrier per axis and per KB colour, where radix stages through shared
 // memory take two per stage.  Measured per term, the transform path -> this one (h = 0.5 clusters with
-// KB): 64^3 x 64 vectors 240 -> 203 us (z 43 us = 6.3 TB/s, planes 162 us, 129 us without KB); 64^3 x 8
-// 41 -> 36 us; 96^3 x 8 208 -> 114 us; 32^3 x 64 38 -> 32 us; 288^3 x 16 (1963 KB atoms) 8.9 -> 6.1 ms.
+// KB): 64^3 x 64 vectors 240 -> 191 us (z 43 us = 6.3 TB/s, planes 150 us, 116 us without KB); 64^3 x 8
+// 41 -> 35 us; 96^3 x 8 208 -> 108 us; 128^3 x 12 610 -> 467 us; 48^3 x 64 -> 77 us; 32^3 x 64 38 -> 31 us;
+// 288^3 x 16 (1963 KB atoms) 8.9 -> 6.0 ms.
 #include <algorithm>
 
 #include "grid_common.cuh"
@@ -45,51 +46,82 @@ __device__ __forceinline__ float axis_factor(int k1, int i, float c) {
 // The step's pointwise part on ROWS x N points of the unit at global offset `off` (unit points o = y N +
 // x at sm[y PITCH + x], which holds H b but for W and the local potential):
 //   out = cpsi psi + ch alpha (sm + W + (V - Ebar) b1 [+ dv b1_partner]) + c2 b2,
-// to global memory and back into sm.
-template <int N, int ROWS, int PITCH, int NT, int UNROLL>
-__device__ __forceinline__ void sep_pointwise(const StepArgs& a, const VecInfo& inf, size_t off, size_t uoff,
-                                              float2* sm) {
+// to global memory and back into sm.  A thread takes U pairs of points at a time and loads all their
+// operands before it uses one: absent ones are predicated off, since a branch around each would keep
+// the loads of a group from being in flight together.  REAL: ch and c2 are real (every term but the
+// last of a complex sum).
+template <int N, int ROWS, int PITCH, int NT, int U, bool TAN, bool REAL>
+__device__ __forceinline__ void sep_points(const StepArgs& a, const VecInfo& inf, size_t off, size_t uoff, float2* sm,
+                                           const float2* bs) {
     static_assert(PITCH % 2 == 0, "rows start on 16 bytes");
+    static_assert(ROWS * N / 2 % (U * NT) == 0, "whole groups");
     constexpr size_t NG = (size_t)N * N * N;
     const float* V = a.vpot + (size_t)inf.vrow * NG + uoff;
-    const float* dV = (a.dvpot != nullptr && inf.dvrow >= 0) ? a.dvpot + (size_t)inf.dvrow * NG + uoff : nullptr;
-    const float2* bp = (dV != nullptr) ? a.b1 + (size_t)inf.partner * NG + uoff : nullptr;
+    const float* dV = TAN ? a.dvpot + (size_t)inf.dvrow * NG + uoff : nullptr;
+    const float2* bp = TAN ? a.b1 + (size_t)inf.partner * NG + uoff : nullptr;
     const float2 cpsi = a.coef.cpsi[inf.cset], ch = cscale(a.coef.ch[inf.cset], a.alpha), c2 = a.coef.c2[inf.cset];
     const float ebar = a.ebar;
-#pragma unroll UNROLL
-    for (int q = threadIdx.x; q < ROWS * N / 2; q += NT) {
-        const int y = q / (N / 2), x = 2 * (q % (N / 2));
-        const int o = y * N + x, sp = y * PITCH + x;
-        const float4 bb = ld4(a.b1 + off + o), w = ldcs4(a.W + off + o);
-        const float2 v = __ldg(reinterpret_cast<const float2*>(V + o));
-        float4& sv = *reinterpret_cast<float4*>(sm + sp);
-        float2 h0 = make_float2(sv.x, sv.y), h1 = make_float2(sv.z, sv.w);
-        // the two kinetic parts first: (V - Ebar) b is the largest term, and this way one rounding of
-        // its size is made, in the multiply-add
-        h0 = make_float2(fmaf(v.x - ebar, bb.x, h0.x + w.x), fmaf(v.x - ebar, bb.y, h0.y + w.y));
-        h1 = make_float2(fmaf(v.y - ebar, bb.z, h1.x + w.z), fmaf(v.y - ebar, bb.w, h1.y + w.w));
-        if (dV != nullptr) {
-            const float2 d = __ldg(reinterpret_cast<const float2*>(dV + o));
-            const float4 pb = ld4(bp + o);
-            h0.x += d.x * pb.x;
-            h0.y += d.x * pb.y;
-            h1.x += d.y * pb.z;
-            h1.y += d.y * pb.w;
+    const bool hp = a.psi != nullptr, hb = a.b2 != nullptr;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+    for (int q0 = threadIdx.x; q0 < ROWS * N / 2; q0 += U * NT) {
+        float4 b1[U], w[U], ps[U], b2[U], pb[TAN ? U : 1];
+        float2 v[U], d[TAN ? U : 1];
+#pragma unroll
+        for (int i = 0; i < U; ++i) {
+            const int o = 2 * (q0 + i * NT);              // pairs of points are contiguous over the unit's rows
+            if (bs == nullptr) b1[i] = ld4(a.b1 + off + o);
+            w[i] = ldcs4(a.W + off + o);
+            ps[i] = hp ? ldcs4(a.psi + off + o) : zero;
+            b2[i] = hb ? ldcs4(a.b2 + off + o) : zero;
+            v[i] = __ldg(reinterpret_cast<const float2*>(V + o));
+            if constexpr (TAN) {
+                d[i] = __ldg(reinterpret_cast<const float2*>(dV + o));
+                pb[i] = ld4(bp + o);
+            }
         }
-        float2 o0 = cmul(ch, h0), o1 = cmul(ch, h1);
-        if (a.psi != nullptr) {
-            const float4 pp = ldcs4(a.psi + off + o);
-            o0 = cadd(o0, cmul(cpsi, make_float2(pp.x, pp.y)));
-            o1 = cadd(o1, cmul(cpsi, make_float2(pp.z, pp.w)));
+#pragma unroll
+        for (int i = 0; i < U; ++i) {
+            const int q = q0 + i * NT, o = 2 * q;
+            const int sp = (q / (N / 2)) * PITCH + 2 * (q % (N / 2));
+            float4& sv = *reinterpret_cast<float4*>(sm + sp);
+            if (bs != nullptr) b1[i] = *reinterpret_cast<const float4*>(bs + sp);
+            float2 h[2] = {make_float2(sv.x + w[i].x, sv.y + w[i].y), make_float2(sv.z + w[i].z, sv.w + w[i].w)};
+            const float2 bb[2] = {make_float2(b1[i].x, b1[i].y), make_float2(b1[i].z, b1[i].w)};
+            const float2 pp[2] = {make_float2(ps[i].x, ps[i].y), make_float2(ps[i].z, ps[i].w)};
+            const float2 b2v[2] = {make_float2(b2[i].x, b2[i].y), make_float2(b2[i].z, b2[i].w)};
+            const float vv[2] = {v[i].x - ebar, v[i].y - ebar};
+            float2 r[2];
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                // the kinetic parts were summed first: (V - Ebar) b is the largest term, and this way one
+                // rounding of its size is made, in the multiply-add
+                h[j] = make_float2(fmaf(vv[j], bb[j].x, h[j].x), fmaf(vv[j], bb[j].y, h[j].y));
+                if constexpr (TAN) {
+                    const float dd = j == 0 ? d[i].x : d[i].y;
+                    const float2 pbv = j == 0 ? make_float2(pb[i].x, pb[i].y) : make_float2(pb[i].z, pb[i].w);
+                    h[j] = make_float2(fmaf(dd, pbv.x, h[j].x), fmaf(dd, pbv.y, h[j].y));
+                }
+                r[j] = REAL ? cscale(h[j], ch.x) : cmul(ch, h[j]);
+                r[j] = cadd(r[j], cmul(cpsi, pp[j]));
+                r[j] = REAL ? make_float2(fmaf(c2.x, b2v[j].x, r[j].x), fmaf(c2.x, b2v[j].y, r[j].y))
+                            : cadd(r[j], cmul(c2, b2v[j]));
+            }
+            st4(a.out + off + o, r[0], r[1]);
+            sv = make_float4(r[0].x, r[0].y, r[1].x, r[1].y);
         }
-        if (a.b2 != nullptr) {
-            const float4 b2 = ldcs4(a.b2 + off + o);
-            o0 = cadd(o0, cmul(c2, make_float2(b2.x, b2.y)));
-            o1 = cadd(o1, cmul(c2, make_float2(b2.z, b2.w)));
-        }
-        st4(a.out + off + o, o0, o1);
-        sv = make_float4(o0.x, o0.y, o1.x, o1.y);
     }
+}
+
+template <int N, int ROWS, int PITCH, int NT, int U>
+__device__ __forceinline__ void sep_pointwise(const StepArgs& a, const VecInfo& inf, size_t off, size_t uoff, float2* sm,
+                                              const float2* bs = nullptr) {
+    const bool tan = a.dvpot != nullptr && inf.dvrow >= 0;
+    const bool real = a.coef.ch[inf.cset].y == 0.f && a.coef.c2[inf.cset].y == 0.f;
+    if (tan && real) sep_points<N, ROWS, PITCH, NT, U, true, true>(a, inf, off, uoff, sm, bs);
+    else if (tan) sep_points<N, ROWS, PITCH, NT, U, true, false>(a, inf, off, uoff, sm, bs);
+    else if (real) sep_points<N, ROWS, PITCH, NT, U, false, true>(a, inf, off, uoff, sm, bs);
+    else sep_points<N, ROWS, PITCH, NT, U, false, false>(a, inf, off, uoff, sm, bs);
 }
 
 // L2 prefetch of a unit's pointwise operands (one thread), PTS points at offset off
@@ -145,72 +177,117 @@ k_sep_z(const float2* __restrict__ in, float2* __restrict__ W, float c, const fl
 }
 
 // ------------------------------------------------------------------ planes, n <= 128
-// A block per plane: the plane comes into shared memory by cp.async, T_x row by row in place, the KB
-// apply, T_y of the columns (read again from L2) added, then the pointwise part.  Four lanes per
-// line: two lanes hold twice the points and half the warps, and the same pass took 195 us instead
-// of 169 at 64^3 x 64 (of one SM's four blocks the phases of the others hide one's latency).  The operands
-// of the pointwise part are asked into L2 once the plane has landed, and read evict-first: asked at
-// the block's start they were evicted before use (a third more DRAM traffic than the algorithm's).
+// A block per plane.  Up to 64^2 the plane of b is copied to shared memory beside the plane of H b: the
+// KB apply runs onto zeros while the copy is on its way, then T_x of the rows and T_y of the columns
+// are added and the pointwise part follows, all reading b from shared memory (three blocks of 256
+// threads per SM at 64^2: 5.66 TB/s without KB, 0.83 of the copy rate; with one plane in shared memory
+// and b read again from L2 for the columns and the pointwise part it was 5.0).  Two planes of 96^2 or
+// 128^2 leave room for one block at best: there the rows are transformed in place, the KB apply comes
+// after them, and b is read again from L2 (96^3 x 8: 91 us, against 102 with the KB apply first).
+// Four lanes per line: two lanes hold twice the points and half the warps, and the same pass took
+// 195 us instead of 169 at 64^3 x 64.  The operands of the pointwise part are asked into L2 once the
+// plane has landed, and read evict-first: asked at the block's start they were evicted before use (a
+// third more DRAM traffic than the algorithm's).
 template <int N> struct SpCfg {
     static constexpr int T = 4;
     static constexpr int NT = N * T;
     // row pitch of the plane in shared memory: a half-warp reads 8 rows at two neighbouring points
     // without bank conflicts, and rows start on 16 bytes
     static constexpr int PITCH = N + 2;
-    static constexpr int MINB = N == 16 ? 16 : (N == 32 ? 8 : (N == 48 ? 5 : (N == 64 ? 4 : (N == 96 ? 2 : 1))));
+    static constexpr bool KEEP = N <= 64;    // the plane of b stays in shared memory
+    static constexpr size_t POINTS = (size_t)N * PITCH * (KEEP ? 2 : 1);
+    static constexpr int MINB = N == 16 ? 16 : (N == 32 ? 8 : (N == 48 ? 5 : (N == 64 ? 3 : (N == 96 ? 2 : 1))));
 };
 
 template <int N>
 __global__ void __launch_bounds__(SpCfg<N>::NT, (SpCfg<N>::MINB)) k_sep_plane(StepArgs a, float c, const float2* __restrict__ tw) {
     constexpr int T = SpCfg<N>::T, P = N / T, CPW = 32 / T, NT = SpCfg<N>::NT, PITCH = SpCfg<N>::PITCH;
+    constexpr bool KEEP = SpCfg<N>::KEEP;
     extern __shared__ __align__(16) float2 sm[];
-    float2* tws = sm + N * PITCH;
+    float2* bs = sm + N * PITCH;
+    float2* tws = bs + (KEEP ? N * PITCH : 0);
     float2* kcs = tws + N;
     const int z = blockIdx.x, b = blockIdx.y;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const size_t uoff = (size_t)z * N * N, off = (size_t)b * N * N * N + uoff;
     const VecInfo inf = a.info[b];
-    {
+    KbHead kh;
+    if (a.kbc != nullptr || a.kbp != nullptr) kh = kb_head(a, z);
+    if constexpr (KEEP) {
+        const float2* src = a.b1 + off;
+#pragma unroll 4
+        for (int q = threadIdx.x; q < N * N / 2; q += NT) sep_cp16(bs + (q / (N / 2)) * PITCH + 2 * (q % (N / 2)), src + 2 * q);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    } else {
         const float2* src = a.b1 + off;
 #pragma unroll 4
         for (int q = threadIdx.x; q < N * N / 2; q += NT) sep_cp16(sm + (q / (N / 2)) * PITCH + 2 * (q % (N / 2)), src + 2 * q);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    if (KEEP && threadIdx.x == 0) {
+        // the plane of the block half a wave of resident blocks later, into L2 (162 -> 157 us at 64^3 x 64;
+        // at 96 and 128, with one or two blocks per SM, it gained nothing)
+        const long nxt = (long)b * N + z + SpCfg<N>::MINB * 152 / 2;
+        if (nxt < (long)gridDim.y * N) l2_prefetch(a.b1 + nxt * N * N, N * N * sizeof(float2));
     }
     for (int i = threadIdx.x; i < N; i += NT) tws[i] = __ldg(tw + i);
-    const float2* kc = a.kbc != nullptr ? a.kbc + (size_t)b * a.n_proj : nullptr;
-    if (kc != nullptr) kb_stage_coeffs<NT>(a, kc, z, kcs);
-    sep_cp_wait();
+    const float2* kc = a.kbc != nullptr ? a.kbc + (size_t)b * a.total_slots * 4 : nullptr;
+    if (kc != nullptr) {
+        if constexpr (KEEP) {
+            // V_NL b onto zeros while the plane is on its way
+            kb_apply_unit<N, PITCH, NT, 2>(a, kh, kcs, sm, [&] {
+                kb_stage_coeffs<NT>(kh, kc, kcs);
+                float4* s4 = reinterpret_cast<float4*>(sm);
+                for (int i = threadIdx.x; i < N * PITCH / 2; i += NT) s4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            });
+        } else {
+            kb_stage_coeffs<NT>(kh, kc, kcs);
+        }
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
     if (threadIdx.x == 0) sep_prefetch<N, N * N>(a, inf, off, uoff);
     const int l = warp * CPW + lane % CPW, t = lane / CPW;
     const auto f = [&](int k1, int i) { return axis_factor<N, T>(k1, i, c); };
     {
-        // T_x b of row l, in place (a lane writes the points it has read)
+        // T_x b of row l: added to V_NL b, or in place (a lane writes the points it has read)
         float2 v[P];
         float2* row = sm + l * PITCH + t;
+        const float2* src = (KEEP ? bs : sm) + l * PITCH + t;
 #pragma unroll
-        for (int i = 0; i < P; ++i) v[i] = row[T * i];
+        for (int i = 0; i < P; ++i) v[i] = src[T * i];
         line_op<N, T>(v, lane, tws, f);
+        if (KEEP && kc != nullptr) {
+#pragma unroll
+            for (int i = 0; i < P; ++i) v[i] = cadd(v[i], row[T * i]);
+        }
 #pragma unroll
         for (int i = 0; i < P; ++i) row[T * i] = v[i];
     }
-    __syncthreads();
-    if (kc != nullptr) kb_apply_unit<N, PITCH, NT>(a, z, kcs, sm);
+    if (!KEEP && kc != nullptr) kb_apply_unit<N, PITCH, NT, 2>(a, kh, kcs, sm, [] {});
+    else __syncthreads();
     {
-        // + T_y b of column l (its points come from L2: the block has just copied the plane)
+        // + T_y b of column l
         float2 v[P];
-        const float2* src = a.b1 + off + (size_t)t * N + l;
         float2* col = sm + t * PITCH + l;
+        if constexpr (KEEP) {
 #pragma unroll
-        for (int i = 0; i < P; ++i) v[i] = __ldg(src + T * i * N);
+            for (int i = 0; i < P; ++i) v[i] = bs[(t + T * i) * PITCH + l];
+        } else {
+            const float2* src = a.b1 + off + (size_t)t * N + l;
+#pragma unroll
+            for (int i = 0; i < P; ++i) v[i] = __ldg(src + T * i * N);
+        }
         line_op<N, T>(v, lane, tws, f);
 #pragma unroll
         for (int i = 0; i < P; ++i) col[T * i * PITCH] = cadd(col[T * i * PITCH], v[i]);
     }
+    KbSlots ks;
+    if (a.kbp != nullptr) ks = kb_project_begin<NT>(a, kh);
     __syncthreads();
-    sep_pointwise<N, N, PITCH, NT, 4>(a, inf, off, uoff, sm);
+    sep_pointwise<N, N, PITCH, NT, 1>(a, inf, off, uoff, sm, KEEP ? bs : nullptr);
     if (a.kbp == nullptr) return;
-    __syncthreads();
-    kb_project_unit<N, PITCH, NT>(a, z, b, sm);
+    kb_project_unit<N, PITCH, NT, 2>(a, kh, ks, b, sm);
 }
 
 // ------------------------------------------------------------------ n = 288
@@ -300,25 +377,34 @@ __global__ void __launch_bounds__(SR_NT, 4) k_sep_rows288(StepArgs a, float c, c
     const size_t uoff = (size_t)u * SR_R * S2N, off = (size_t)b * NG + uoff;
     const VecInfo inf = a.info[b];
     const int r = threadIdx.x / S2T, t = threadIdx.x % S2T;
+    KbHead kh;
+    if (a.kbc != nullptr || a.kbp != nullptr) kh = kb_head(a, u);
     float2 v[S2P];
     const float2* src = a.b1 + off + (size_t)r * S2N + t;
 #pragma unroll
     for (int i = 0; i < S2P; ++i) v[i] = __ldg(src + S2T * i);
+    if (threadIdx.x == 0) {
+        // the unit of the block half a wave later, into L2
+        const long nxt = (long)u * gridDim.x + b + 304;
+        if (nxt < (long)gridDim.x * gridDim.y)
+            l2_prefetch(a.b1 + (nxt % gridDim.x) * NG + (nxt / gridDim.x) * SR_R * S2N, SR_R * S2N * sizeof(float2));
+    }
     for (int i = threadIdx.x; i < S2N; i += SR_NT) tws[i] = __ldg(tw + i);
-    const float2* kc = a.kbc != nullptr ? a.kbc + (size_t)b * a.n_proj : nullptr;
-    if (kc != nullptr) kb_stage_coeffs<SR_NT>(a, kc, u, kcs);
+    const float2* kc = a.kbc != nullptr ? a.kbc + (size_t)b * a.total_slots * 4 : nullptr;
+    if (kc != nullptr) kb_stage_coeffs<SR_NT>(kh, kc, kcs);
     float2* row = sm + r * SR_PITCH;
     line288(v, t, c, tws, row, [](int k, int s) { return k * 13 + s; }, [] { __syncthreads(); });
     __syncthreads();
     if (threadIdx.x == 0) sep_prefetch<S2N, SR_R * S2N>(a, inf, off, uoff);
 #pragma unroll
     for (int i = 0; i < S2P; ++i) row[t + S2T * i] = v[i];
-    __syncthreads();
-    if (kc != nullptr) kb_apply_unit<S2N, SR_PITCH, SR_NT>(a, u, kcs, sm);
-    sep_pointwise<S2N, SR_R, SR_PITCH, SR_NT, 4>(a, inf, off, uoff, sm);
+    if (kc != nullptr) kb_apply_unit<S2N, SR_PITCH, SR_NT, 2>(a, kh, kcs, sm, [] {});
+    else __syncthreads();
+    KbSlots ks;
+    if (a.kbp != nullptr) ks = kb_project_begin<SR_NT>(a, kh);
+    sep_pointwise<S2N, SR_R, SR_PITCH, SR_NT, 1>(a, inf, off, uoff, sm);
     if (a.kbp == nullptr) return;
-    __syncthreads();
-    kb_project_unit<S2N, SR_PITCH, SR_NT>(a, u, b, sm);
+    kb_project_unit<S2N, SR_PITCH, SR_NT, 2>(a, kh, ks, b, sm);
 }
 
 // ------------------------------------------------------------------ launchers
@@ -333,11 +419,17 @@ __global__ void __launch_bounds__(SR_NT, 4) k_sep_rows288(StepArgs a, float c, c
         default: break;                                  \
     }
 
+int sep_unit_pos(int n, int o) {
+    int pitch = SR_PITCH;
+    SGW_DISPATCH_SEP(n, pitch = SpCfg<N>::PITCH);
+    return (o / n) * pitch + o % n;
+}
+
 int64_t sep_unit_points(int n) { return n == S2N ? (int64_t)SR_R * S2N : (int64_t)n * n; }
 
 size_t sep_step_smem(int n, int max_unit_slots) {
     size_t pts = (size_t)SR_R * SR_PITCH;
-    SGW_DISPATCH_SEP(n, pts = (size_t)N * SpCfg<N>::PITCH);
+    SGW_DISPATCH_SEP(n, pts = SpCfg<N>::POINTS);
     return sizeof(float2) * (pts + n + 4 * (size_t)max_unit_slots);
 }
 

@@ -23,7 +23,6 @@ struct StepCoef {
 
 struct KBDev {
     int n_atoms = 0;
-    int n_proj = 0;            // 4 * n_atoms (padded)
     int64_t n_sup = 0;
     int* atom_nproj = nullptr;   // [n_atoms]
     int64_t* atom_off = nullptr; // [n_atoms + 1]
@@ -32,17 +31,17 @@ struct KBDev {
     float4* atom_e = nullptr;    // [n_atoms] E_a0..3
     // per-unit partial projections (a unit is an xy plane on the plane path, 8 x rows on the row
     // path): unit z owns slots plane_off[z] .. plane_off[z+1]-1, one per atom whose support meets
-    // the unit (slot_atom[k] is that atom); atom a's slots (in increasing z) are
+    // the unit; atom a's slots (in increasing z) are
     // atom_pos[atom_pos_off[a] .. atom_pos_off[a+1]).
     int total_slots = 0;
     int max_plane_slots = 0;
     int* plane_off = nullptr;    // [units + 1]
-    int* slot_atom = nullptr;    // [total_slots]
     // plane-major entries of the fused apply and projections.  The slots of a plane are split into
     // colours whose point sets in the plane are disjoint; plane z's colour c holds the entries
     // kbe_col[z (max_colors+1) + c] .. kbe_col[z (max_colors+1) + c + 1] - 1, slot by slot
-    // (slot k: kbe_slot_beg[k] .. kbe_slot_end[k] - 1).  Entry e: kbe_os[e] = in-plane offset |
-    // (plane-local slot << 16), kbe_beta[e] = the slot atom's beta_0..3 at that point.
+    // (slot k: kbe_slot_beg[k] .. kbe_slot_end[k] - 1).  Entry e: kbe_os[e] = in-plane offset (on
+    // the separable path the point's position in the step's shared memory) | (plane-local slot << 16),
+    // kbe_beta[e] = the slot atom's beta_0..3 at that point.
     int max_colors = 0;
     int* kbe_col = nullptr;      // [units][max_colors + 1]
     unsigned* kbe_os = nullptr;  // [n_sup]
@@ -64,10 +63,9 @@ struct StepArgs {
     const float* vpot;      // [rows][ng]
     const float* dvpot;     // [rows][ng] or nullptr
     const VecInfo* info;    // [B]
-    const float2* kbc;      // [B][n_proj] E-weighted projector coefficients (nullptr: no KB)
+    const float2* kbc;      // [B][total_slots][4] E-weighted projections of each slot's atom (nullptr: no KB)
     // KB tables (see KBDev)
     const int* plane_off;
-    const int* slot_atom;
     const int* kbe_col;
     const unsigned* kbe_os;
     const float4* kbe_beta;
@@ -78,7 +76,6 @@ struct StepArgs {
     // partial projections of `out` (nullptr: skip): kbp[b][slot][4] = sum_plane beta_ap(r) out(r)
     float2* kbp;
     int total_slots;
-    int n_proj;
     float ebar, alpha;
     StepCoef coef;
     // L2 prefetch of the W plane of the block this many blocks later in launch order (0: off);
@@ -88,14 +85,15 @@ struct StepArgs {
     int pf_operands;
 };
 
-// Arguments of the KB reduction kbc[b][4a + p] = E_ap dV sum_{slots of a} kbp[b][slot][p] (n_atoms 0: none)
+// Arguments of the KB reduction kbc[b][k][p] = E_ap dV sum_{slots of a} kbp[b][slot][p], k every slot of a
+// (n_atoms 0: none)
 struct KbReduceArgs {
     const int* atom_pos_off = nullptr;
     const int* atom_pos = nullptr;
     const float4* atom_e = nullptr;
     const float2* kbp = nullptr;
     float2* kbc = nullptr;
-    int n_atoms = 0, total_slots = 0, n_proj = 0;
+    int n_atoms = 0, total_slots = 0;
     float dV = 0.f;
 };
 
@@ -104,6 +102,7 @@ struct KbReduceArgs {
 // rest of the fused Chebyshev step with StepArgs::W = the sum so far (Wout unused).  KB tables per
 // sep_unit_points(n) consecutive points: an xy plane, 16 x rows at 288.
 int64_t sep_unit_points(int n);
+int sep_unit_pos(int n, int o);    // position of unit point o in the step's shared memory
 size_t sep_step_smem(int n, int max_unit_slots);
 cudaError_t sep_init_attributes(int n);
 void sep_z(int n, const float2* in, float2* W, int batch, float kscale, const float2* tw, const KbReduceArgs& kr,
@@ -148,7 +147,6 @@ void launch_plane_inv(int n, const float2* W, int batch, const float2* tw, int m
                       float* out_re, cudaStream_t st);
 void launch_kb_project(int n, const KBDev& kb, const float2* b1, int batch, float dV, float2* kbc,
                        cudaStream_t st);
-// kbc[b][4a + p] = E_ap dV sum over atom a's plane slots of kbp[b][slot][p]
 KbReduceArgs kb_reduce_args(const KBDev& kb, const float2* kbp, float dV, float2* kbc);
 void launch_kb_reduce(const KBDev& kb, const float2* kbp, int batch, float dV, float2* kbc, cudaStream_t st);
 // density of TDH pairs for each sample, packed as (rho - rho0) + i d rho, fwd xy transformed into Wp.
