@@ -44,8 +44,8 @@ struct sgw_ctx {
     static constexpr int kWorkSlots = 11;
     void* work[kWorkSlots] = {nullptr};
     size_t work_sz[kWorkSlots] = {0};
-    float2* twM = nullptr;
-    int twM_n = 0;
+    // time-ordering matrices of the last few n_steps used (at most 8; 0.7 MB at 400 steps)
+    std::vector<std::pair<int, float2*>> to_tabs;
     std::vector<sgw::VecInfo> info_host;
     // instrumentation: launch counter and CUDA-event timing per kernel kind
     int64_t launches = 0;
@@ -613,9 +613,10 @@ void sgw_destroy(sgw_ctx* ctx) {
     cudaSetDevice(ctx->device);
     if (ctx->stream) cudaStreamSynchronize(ctx->stream);
     free_kb(ctx);
-    void* ptrs[] = {ctx->tw, ctx->vloc, ctx->W, ctx->B1, ctx->B2, ctx->info, ctx->scal, ctx->twM};
+    void* ptrs[] = {ctx->tw, ctx->vloc, ctx->W, ctx->B1, ctx->B2, ctx->info, ctx->scal};
     for (void* p : ptrs)
         if (p) cudaFree(p);
+    for (auto& t : ctx->to_tabs) cudaFree(t.second);
     for (int i = 0; i < sgw_ctx::kWorkSlots; ++i)
         if (ctx->work[i]) cudaFree(ctx->work[i]);
     for (int k = 0; k < SGW_PROF_KINDS; ++k)
@@ -1597,18 +1598,38 @@ sgw_status sgw_time_order_points(sgw_ctx* ctx, const float* uR_dev, void* u_dev,
     int M = 4;                                    // the smallest power of two >= 4 (n_steps + 1)
     while (M < 4 * (n_steps + 1)) M *= 2;
     if (M > 4096) return fail(ctx, SGW_EINVAL, "n_steps too large for the time-ordering FFT (M <= 4096)");
-    if (ctx->twM_n != M) {
-        if (ctx->twM) cudaFree(ctx->twM);
-        ctx->twM = nullptr;
-        ctx->twM_n = 0;
-        CK(cudaMalloc(&ctx->twM, sizeof(float2) * M));
-        auto t = twiddles(M);
-        CK(cudaMemcpy(ctx->twM, t.data(), sizeof(float2) * M, cudaMemcpyHostToDevice));
-        ctx->twM_n = M;
+    const float2* g = nullptr;
+    for (auto& t : ctx->to_tabs)
+        if (t.first == n_steps) g = t.second;
+    if (!g) {
+        // built by a kernel, once: during a stream capture it would be recorded, not run
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        CK(cudaStreamIsCapturing(ctx->stream, &cap));
+        if (cap != cudaStreamCaptureStatusNone)
+            return fail(ctx, SGW_ESTATE, "the first time ordering of this n_steps must come before any stream capture");
+        if (ctx->to_tabs.size() >= 8) {
+            CK(cudaStreamSynchronize(ctx->stream));
+            cudaFree(ctx->to_tabs.front().second);
+            ctx->to_tabs.erase(ctx->to_tabs.begin());
+        }
+        float2* t = nullptr;
+        if (cudaMalloc(&t, sgw::time_order_matrix_bytes(n_steps)) != cudaSuccess) {
+            cudaGetLastError();
+            return fail(ctx, SGW_ENOMEM, "time-ordering matrix allocation failed");
+        }
+        sgw::launch_time_order_matrix(n_steps, M, t, ctx->stream);
+        cudaError_t e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);       // later calls may use another stream
+        if (e != cudaSuccess) {
+            cudaFree(t);
+            return fail(ctx, SGW_ECUDA, std::string("time-ordering matrix: ") + cudaGetErrorString(e));
+        }
+        ctx->to_tabs.push_back({n_steps, t});
+        g = t;
     }
     {
         Launch L(ctx, SGW_PROF_TIME_ORDER, 1, (double)n_points * n_samples * (n_steps + 1) * 12.0);
-        sgw::launch_time_order(n_points, uR_dev, (float2*)u_dev, n_samples, n_steps, M, ctx->twM, ctx->stream);
+        sgw::launch_time_order(n_points, uR_dev, (float2*)u_dev, n_samples, n_steps, g, ctx->stream);
         CKL();
     }
     return SGW_OK;

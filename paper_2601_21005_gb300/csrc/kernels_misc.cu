@@ -1,5 +1,5 @@
 // Non-FFT kernels of the sGW hot path: Philox white noise, the TDH kick, power-iteration
-// reductions, the Sigma(t) reductions (Eq. 5), time ordering of u^R (FFT over t), the
+// reductions, the Sigma(t) reductions (Eq. 5), time ordering of u^R, the
 // damped transform (Eq. 7) and the QP root (Eq. 6).
 #include <cmath>
 #include <mutex>
@@ -423,105 +423,209 @@ void launch_sigma_reduce(const double2* partial, int n_samples, int n_steps, int
 }
 
 // ------------------------------------------------------------------ time ordering
-// One CTA per (GP grid points, sample).  Lines are padded to M + 1 complex.
-template <int M, int GP, int NT>
-__global__ void __launch_bounds__(NT)
-k_time_order(int64_t ng, const float* __restrict__ uR, float2* __restrict__ u, int n_steps, const float2* __restrict__ tw) {
-    extern __shared__ float2 sm[];
-    constexpr int LS = M + 1;
-    constexpr int NP = GP / 2;           // packed lines
-    const int s = blockIdx.y;
-    const int64_t g0 = (int64_t)blockIdx.x * GP;
-    const int nt = n_steps + 1;
-    const float* src = uR + (size_t)s * nt * ng;
-    // 1. pack two real grid points per complex line (point 2l in .x, 2l+1 in .y), zero padded;
-    //    reads run along the grid index so that each time row is one contiguous segment.
-    for (int q = threadIdx.x; q < NP * (M - nt); q += NT) {
-        const int l = q / (M - nt), t = nt + q % (M - nt);
-        sm[l * LS + t] = make_float2(0.f, 0.f);
-    }
-    float* smf = reinterpret_cast<float*>(sm);
-    for (int q = threadIdx.x; q < nt * GP; q += NT) {
-        const int t = q / GP, p = q % GP;
-        const int64_t g = g0 + p;
-        smf[2 * ((p >> 1) * LS + t) + (p & 1)] = g < ng ? src[(size_t)t * ng + g] : 0.f;
-    }
-    __syncthreads();
-    // 2. transform with e^{+i omega t}
-    fft_lines<M, NP, LS, 1, NT, +1>(sm, tw);
-    // 3. unpack: X_a = (Z_m + conj Z_-m)/2, X_b = -i (Z_m - conj Z_-m)/2; take the even extension of
-    //    the non-negative frequencies (the negative half becomes the conjugate) -> lines 2l, 2l+1.
-    constexpr int HALF = M / 2 + 1;
-    constexpr int PER = (NP * HALF + NT - 1) / NT;
-    float2 ya[PER], yb[PER];
-#pragma unroll
-    for (int p = 0; p < PER; ++p) {
-        const int q = threadIdx.x + p * NT;
-        if (q < NP * HALF) {
-            const int l = q / HALF, m = q % HALF;
-            const float2 zm = sm[l * LS + m];
-            const float2 zn = sm[l * LS + ((M - m) & (M - 1))];
-            ya[p] = make_float2(0.5f * (zm.x + zn.x), 0.5f * (zm.y - zn.y));
-            yb[p] = make_float2(0.5f * (zm.y + zn.y), -0.5f * (zm.x - zn.x));
+// u of one point is y_t = (1/M) sum_m X_|m| e^{-2 pi i t m / M} with X the length-M transform (e^{+}) of
+// its real, causal, zero-padded u^R.  The real part of X is the transform of u^R's even part, so
+//   Re y_0 = x_0, Re y_t = x_t / 2   (t > 0; the padding keeps t and -t apart),
+// and the odd imaginary part, made even, gives
+//   Im y_t = sum_j G(t, j) x_j, G(t, j) = (g(j + t) + g(j - t)) / M, g(n) = cot(pi n / M) for odd n, 0 for
+// even n.  G couples times of opposite parity only, so the ordering of all points is two real matrix
+// products with half the times each: 80 k multiply-adds per point at 400 steps, fewer operations than
+// the point's three length-2048 transforms, in one pass over u^R and u and without their 9 KB of
+// shared memory per point.  Bound by FP32 multiply-adds and the shared-memory reads that feed them.
+// Measured at 64^3 points x 401 times: 4.72 ms by transforms, 1.24 ms (34 T multiply-add operations/s,
+// 0.42 of the FP32 rate; smaller tiles of 7 or 10 rows a warp 1.42-1.50 ms, 4 rows 1.71).
+// Sums run over chunks of CH terms whose totals are added up, which keeps the rounding below the
+// transforms' (8e-8 against 1.0e-7 relative at 400 steps; one long sum would have 2.2e-7).
+constexpr int TO_BK = 16, TO_BN = 128, TO_NT = 128, TO_STAGES = 3;
+constexpr int TO_R = TO_NT / 32;     // a warp's lanes take 4 points each and share their rows
+
+// Row tiles: TO_R warps of TM rows each, held in TMP = TM rounded up to even slots.
+struct ToShape {
+    int tm, tiles, kpad;      // TM, row tiles per parity, padded K
+};
+static ToShape to_shape(int n_steps) {
+    const int rows = n_steps / 2 + 1;                 // the even times; the odd ones are at most as many
+    const int cand[] = {1, 2, 4, 7, 10, 13};
+    ToShape s;
+    s.tiles = (rows + TO_R * 13 - 1) / (TO_R * 13);
+    s.tm = 13;
+    for (int c : cand)
+        if (TO_R * c * s.tiles >= rows) {
+            s.tm = c;
+            break;
         }
+    s.kpad = (rows + TO_BK - 1) / TO_BK * TO_BK;
+    return s;
+}
+static int to_tmp(int tm) { return (tm + 1) & ~1; }
+
+size_t time_order_matrix_bytes(int n_steps) {
+    const ToShape s = to_shape(n_steps);
+    return sizeof(float2) * 2 * (size_t)s.tiles * s.kpad * TO_R * to_tmp(s.tm);
+}
+
+// G in the order the product reads it, each value twice (the packed multiply-adds take pairs):
+// [parity of t][tile][k][warp][slot], row t = 2 (TO_R TM tile + TM warp + slot) + parity, column
+// j = 2 k + 1 - parity; 0 outside the times.
+__global__ void k_time_order_matrix(int n_steps, int M, int tm, int tmp, int tiles, int kpad, float2* __restrict__ G) {
+    const int total = 2 * tiles * kpad * TO_R * tmp;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+        const int slot = i % tmp, row = (i / tmp) % TO_R, k = (i / (TO_R * tmp)) % kpad,
+                  tile = (i / (TO_R * tmp * kpad)) % tiles, par = i / (TO_R * tmp * kpad * tiles);
+        const int t = 2 * (TO_R * tm * tile + tm * row + slot) + par, j = 2 * k + 1 - par;
+        double v = 0.0;
+        if (slot < tm && t <= n_steps && j <= n_steps) {
+            const double a = (double)(j + t) / M, b = (double)(j - t) / M;      // j + t and j - t are odd
+            v = (cospi(a) / sinpi(a) + cospi(b) / sinpi(b)) / M;
+        }
+        G[i] = make_float2((float)v, (float)v);
     }
-    __syncthreads();
+}
+
+__device__ __forceinline__ void to_cp(void* smem, const void* gmem, int bytes, int valid) {
+    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+    if (bytes == 16) asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(s), "l"(gmem), "r"(valid) : "memory");
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(s), "l"(gmem), "r"(valid) : "memory");
+}
+// Pairs of floats in 64-bit registers, for the packed operations (one instruction issued for two)
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 a) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
+    return r;
+}
+
+// One (parity, row tile) of 128 points of a sample.  Warp tm: rows TM tm .. + TM; lane tn: points 4 tn .. + 4.
+// VEC: rows of u^R and u start on 16 bytes (the number of points is a multiple of 4).
+template <int TM, bool VEC>
+__global__ void __launch_bounds__(TO_NT, 3)
+k_time_order(int64_t np, const float* __restrict__ uR, float2* __restrict__ u, int n_steps, int tiles, int kpad, int ch,
+             const float2* __restrict__ G) {
+    constexpr int TMP = (TM + 1) & ~1, AM = TO_R * TMP;
+    extern __shared__ __align__(16) unsigned char to_sm[];
+    float2* As = reinterpret_cast<float2*>(to_sm);                                  // [stage][k][TO_R][TMP]
+    float* Bs = reinterpret_cast<float*>(As + TO_STAGES * TO_BK * AM);              // [stage][k][TO_BN]
+    // the blocks of one group of points run together: they read the same rows of u^R
+    const int which = blockIdx.x % (2 * tiles), par = which / tiles, tile = which % tiles;
+    const int64_t p0 = (int64_t)(blockIdx.x / (2 * tiles)) * TO_BN;
+    const size_t row0 = (size_t)blockIdx.y * (n_steps + 1);
+    const int tn = threadIdx.x % 32, tm = threadIdx.x / 32;
+    const float2* A = G + ((size_t)par * tiles + tile) * kpad * AM;
+    const int nk = kpad / TO_BK;
+    const auto load = [&](int s, int kt) {
+        const float2* a = A + (size_t)kt * TO_BK * AM;
+        float2* as = As + s * TO_BK * AM;
+        for (int i = threadIdx.x; i < TO_BK * AM / 2; i += TO_NT) to_cp(as + 2 * i, a + 2 * i, 16, 16);
+        float* bs = Bs + s * TO_BK * TO_BN;
+        constexpr int V = VEC ? 4 : 1;
+        for (int i = threadIdx.x; i < TO_BK * TO_BN / V; i += TO_NT) {
+            const int k = i / (TO_BN / V), p = i % (TO_BN / V) * V;
+            const int j = 2 * (kt * TO_BK + k) + 1 - par;
+            const bool ok = j <= n_steps && p0 + p < np;
+            to_cp(bs + k * TO_BN + p, ok ? uR + (row0 + j) * np + p0 + p : uR, 4 * V, ok ? 4 * V : 0);
+        }
+    };
+    f32x2 acc[TM][2], tot[TM][2];
 #pragma unroll
-    for (int p = 0; p < PER; ++p) {
-        const int q = threadIdx.x + p * NT;
-        if (q < NP * HALF) {
-            const int l = q / HALF, m = q % HALF;
-            sm[(2 * l) * LS + m] = ya[p];
-            sm[(2 * l + 1) * LS + m] = yb[p];
-            if (m > 0 && m < M / 2) {
-                sm[(2 * l) * LS + M - m] = ya[p];
-                sm[(2 * l + 1) * LS + M - m] = yb[p];
+    for (int i = 0; i < TM; ++i) acc[i][0] = acc[i][1] = tot[i][0] = tot[i][1] = 0ull;
+#pragma unroll
+    for (int s = 0; s < TO_STAGES - 1; ++s) {
+        if (s < nk) load(s, s);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    for (int kt = 0; kt < nk; ++kt) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(TO_STAGES - 2) : "memory");
+        __syncthreads();                                  // stage kt has landed; stage kt - 1 is free
+        if (kt + TO_STAGES - 1 < nk) load((kt + TO_STAGES - 1) % TO_STAGES, kt + TO_STAGES - 1);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        const ulonglong2* as = reinterpret_cast<const ulonglong2*>(As + (kt % TO_STAGES) * TO_BK * AM + tm * TMP);
+        const float* bs = Bs + (kt % TO_STAGES) * TO_BK * TO_BN + 4 * tn;
+#pragma unroll
+        for (int k = 0; k < TO_BK; ++k) {
+            const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(bs + k * TO_BN);
+#pragma unroll
+            for (int i = 0; i < TMP / 2; ++i) {
+                const ulonglong2 a = as[k * (AM / 2) + i];
+                acc[2 * i][0] = fma2(a.x, b.x, acc[2 * i][0]);
+                acc[2 * i][1] = fma2(a.x, b.y, acc[2 * i][1]);
+                if (2 * i + 1 < TM) {
+                    acc[(2 * i + 1) % TM][0] = fma2(a.y, b.x, acc[(2 * i + 1) % TM][0]);
+                    acc[(2 * i + 1) % TM][1] = fma2(a.y, b.y, acc[(2 * i + 1) % TM][1]);
+                }
             }
         }
+        if (((kt + 1) * TO_BK) % ch == 0) {
+#pragma unroll
+            for (int i = 0; i < TM; ++i)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    tot[i][h] = add2(tot[i][h], acc[i][h]);
+                    acc[i][h] = 0ull;
+                }
+        }
     }
-    __syncthreads();
-    // 4. inverse transform e^{-i omega t} / M
-    fft_lines<M, GP, LS, 1, NT, -1>(sm, tw);
-    const float inv = 1.0f / (float)M;
-    float2* dst = u + (size_t)s * nt * ng;
-    for (int q = threadIdx.x; q < GP * nt; q += NT) {
-        const int t = q / GP, l = q % GP;
-        const int64_t g = g0 + l;
-        if (g < ng) dst[(size_t)t * ng + g] = cscale(sm[l * LS + t], inv);
+    const int64_t p = p0 + 4 * tn;
+#pragma unroll
+    for (int i = 0; i < TM; ++i) {
+        const int t = 2 * (TO_R * TM * tile + TM * tm + i) + par;
+        if (t > n_steps || p >= np) continue;
+        const float* x = uR + (row0 + t) * np + p;
+        float2* y = u + (row0 + t) * np + p;
+        const float half = t == 0 ? 1.f : 0.5f;
+        const float2 i0 = unpack2(add2(tot[i][0], acc[i][0])), i1 = unpack2(add2(tot[i][1], acc[i][1]));
+        const float im[4] = {i0.x, i0.y, i1.x, i1.y};
+        if constexpr (VEC) {
+            const float4 r = __ldg(reinterpret_cast<const float4*>(x));
+            reinterpret_cast<float4*>(y)[0] = make_float4(half * r.x, im[0], half * r.y, im[1]);
+            reinterpret_cast<float4*>(y)[1] = make_float4(half * r.z, im[2], half * r.w, im[3]);
+        } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (p + q < np) y[q] = make_float2(half * __ldg(x + q), im[q]);
+        }
     }
 }
 
-int time_order_threads(int M) { return M <= 1024 ? 256 : 512; }
-
-template <int M> static void tlaunch(int64_t ng, const float* uR, float2* u, int n_samples, int n_steps,
-                                     const float2* tw, cudaStream_t st) {
-    constexpr int GP = M <= 2048 ? 8 : 4;
-    constexpr int NT = M <= 1024 ? 256 : 512;
-    const size_t smem = sizeof(float2) * GP * (M + 1);
-    static bool attr = false;
-    if (!attr) {
-        cudaFuncSetAttribute(k_time_order<M, GP, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        attr = true;
+template <int TM> static void tlaunch(int64_t np, const float* uR, float2* u, int n_samples, int n_steps, const ToShape& s,
+                                      const float2* G, cudaStream_t st) {
+    constexpr int TMP = (TM + 1) & ~1;
+    const size_t smem = TO_STAGES * TO_BK * (sizeof(float2) * TO_R * TMP + sizeof(float) * TO_BN);
+    const dim3 grid((unsigned)(2 * s.tiles * ((np + TO_BN - 1) / TO_BN)), n_samples);
+    // chunks of 16 terms, 32 above 256: as many chunks as terms in one, about
+    const int ch = s.kpad > 256 ? 2 * TO_BK : TO_BK;
+    if (np % 4 == 0) {
+        cudaFuncSetAttribute(k_time_order<TM, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        k_time_order<TM, true><<<grid, TO_NT, smem, st>>>(np, uR, u, n_steps, s.tiles, s.kpad, ch, G);
+    } else {
+        cudaFuncSetAttribute(k_time_order<TM, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        k_time_order<TM, false><<<grid, TO_NT, smem, st>>>(np, uR, u, n_steps, s.tiles, s.kpad, ch, G);
     }
-    const dim3 grid((unsigned)((ng + GP - 1) / GP), n_samples);
-    k_time_order<M, GP, NT><<<grid, NT, smem, st>>>(ng, uR, u, n_steps, tw);
 }
 
-void launch_time_order(int ng, const float* uR, float2* u, int n_samples, int n_steps, int M, const float2* twM,
-                       cudaStream_t st) {
-    switch (M) {
-        case 4: tlaunch<4>(ng, uR, u, n_samples, n_steps, twM, st); break;
-        case 8: tlaunch<8>(ng, uR, u, n_samples, n_steps, twM, st); break;
-        case 16: tlaunch<16>(ng, uR, u, n_samples, n_steps, twM, st); break;
-        case 32: tlaunch<32>(ng, uR, u, n_samples, n_steps, twM, st); break;
-        case 64: tlaunch<64>(ng, uR, u, n_samples, n_steps, twM, st); break;
-        case 128: tlaunch<128>(ng, uR, u, n_samples, n_steps, twM, st); break;
-        case 256: tlaunch<256>(ng, uR, u, n_samples, n_steps, twM, st); break;
-        case 512: tlaunch<512>(ng, uR, u, n_samples, n_steps, twM, st); break;
-        case 1024: tlaunch<1024>(ng, uR, u, n_samples, n_steps, twM, st); break;
-        case 2048: tlaunch<2048>(ng, uR, u, n_samples, n_steps, twM, st); break;
-        case 4096: tlaunch<4096>(ng, uR, u, n_samples, n_steps, twM, st); break;
-        default: break;
+void launch_time_order_matrix(int n_steps, int M, float2* G, cudaStream_t st) {
+    const ToShape s = to_shape(n_steps);
+    k_time_order_matrix<<<152, 256, 0, st>>>(n_steps, M, s.tm, to_tmp(s.tm), s.tiles, s.kpad, G);
+}
+
+void launch_time_order(int np, const float* uR, float2* u, int n_samples, int n_steps, const float2* G, cudaStream_t st) {
+    const ToShape s = to_shape(n_steps);
+    switch (s.tm) {
+        case 1: tlaunch<1>(np, uR, u, n_samples, n_steps, s, G, st); break;
+        case 2: tlaunch<2>(np, uR, u, n_samples, n_steps, s, G, st); break;
+        case 4: tlaunch<4>(np, uR, u, n_samples, n_steps, s, G, st); break;
+        case 7: tlaunch<7>(np, uR, u, n_samples, n_steps, s, G, st); break;
+        case 10: tlaunch<10>(np, uR, u, n_samples, n_steps, s, G, st); break;
+        default: tlaunch<13>(np, uR, u, n_samples, n_steps, s, G, st); break;
     }
 }
 

@@ -226,14 +226,15 @@ void launch_sigma_accum_xi(const float2* zeta, const float* phi, const float2* U
                            float c, int fp64, double2* partial, int nblk, cudaStream_t st);
 void launch_sigma_reduce(const double2* partial, int n_samples, int n_steps, int nblk, double dV, int fp64,
                          double* sigma, cudaStream_t st);
-void launch_time_order(int ng, const float* uR, float2* u, int n_samples, int n_steps, int M,
-                       const float2* twM, cudaStream_t st);
+// time ordering as a product with the matrix of n_steps (transform length M), which the caller keeps
+size_t time_order_matrix_bytes(int n_steps);
+void launch_time_order_matrix(int n_steps, int M, float2* G, cudaStream_t st);
+void launch_time_order(int np, const float* uR, float2* u, int n_samples, int n_steps, const float2* G, cudaStream_t st);
 void launch_sigma_omega(const double* sigma, int n_samples, int n_steps, double dt, double gamma,
                         const double* omega, int n_omega, int fp64, double* out, cudaStream_t st);
 void launch_qp(const double* sigma, const double* x, int n_samples, int n_steps, double dt, double gamma,
                double eps_ks, double vxc, double window, double step, int fp64, double* scan,
                int n_scan, double* result, cudaStream_t st);
-int time_order_threads(int M);
 void set_global_error(const char* msg);
 // control variate (kernels_mlp.cu)
 void launch_cv_source(int64_t ng, const float2* zb, int64_t stride, const float* phi, int n_samples, float2* out,

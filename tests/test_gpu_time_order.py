@@ -1,0 +1,63 @@
+"""The time ordering as a matrix product, against the oracle's transforms at the edges of its tiles (64
+points, 104 times per parity, 16 terms per stage), for point counts that are and are not a multiple of 4."""
+import numpy as np
+import pytest
+
+from oracle import sgw as osgw
+from paper_2601_21005_gb300 import build
+
+torch = pytest.importorskip('torch')
+pytestmark = pytest.mark.gpu
+
+
+def _abs_matrix(n):
+    """|G(t, j)| of Im u(t) = sum_j G(t, j) u^R(t_j) (zero for equal parities)."""
+    M = osgw.time_order_length(n)
+    t = np.arange(n + 1)
+    g = np.zeros((n + 1, n + 1))
+    odd = (t[:, None] + t[None, :]) % 2 == 1
+    s, d = (t[:, None] + t[None, :])[odd], (t[:, None] - t[None, :])[odd]
+    g[odd] = (1 / np.tan(np.pi * s / M) - 1 / np.tan(np.pi * d / M)) / M
+    return np.abs(g)
+
+
+@pytest.mark.parametrize('n,points', [(0, 5), (1, 64), (2, 63), (3, 1), (15, 66), (16, 65), (31, 128), (63, 7), (111, 68),
+                                      (206, 130), (207, 64), (208, 61), (400, 193), (401, 192), (513, 64), (1023, 67)])
+def test_time_order_matrix_product(n, points):
+    assert torch.cuda.is_available()
+    build.build()
+    from paper_2601_21005_gb300 import sgw
+    r = np.random.default_rng(n)
+    x = r.normal(size=(2, n + 1, points)).astype(np.float32)
+    c = sgw.Context(16, 0.5)
+    u = torch.full((2, n + 1, points), float('nan'), dtype=torch.complex64, device='cuda')
+    xd = torch.as_tensor(x).cuda()
+    c.time_order_points(xd, u, 2, n, points)
+    got = u.cpu().numpy()
+    A = _abs_matrix(n)
+    for s in range(2):
+        ref = osgw.time_order(x[s].astype(np.float64))
+        # a chunk of up to 32 terms, up to 17 chunk totals, G itself and the store: at most 52 roundings
+        # of 2^-24 on the sum of the magnitudes; the real part is x or x / 2 exactly
+        bound = 52 * 2.0 ** -24 * (A @ np.abs(x[s].astype(np.float64))) + 1e-30
+        assert np.all(np.abs(got[s].imag - ref.imag) <= bound + 1e-12)
+        assert np.all(np.abs(got[s].real - ref.real) <= 1e-12 * np.max(np.abs(x)))
+    u2 = torch.empty_like(u)
+    c.time_order_points(xd, u2, 2, n, points)                 # the kept matrix gives the same bits
+    assert torch.equal(u, u2)
+
+
+def test_many_step_counts_in_one_context():
+    """More step counts than matrices are kept, and back to the first."""
+    build.build()
+    from paper_2601_21005_gb300 import sgw
+    c = sgw.Context(16, 0.5)
+    x = torch.randn(1, 41, 70, device='cuda')
+    first = None
+    for n in list(range(20, 41)) + [20]:
+        u = torch.empty(1, n + 1, 70, dtype=torch.complex64, device='cuda')
+        c.time_order_points(x[:, :n + 1].contiguous(), u, 1, n, 70)
+        if n == 20:
+            if first is not None:
+                assert torch.equal(u, first)
+            first = u
