@@ -598,6 +598,7 @@ sgw_status sgw_setup_grid(sgw_ctx** out, int nx, int ny, int nz, double h, doubl
     e = cudaMemcpy(ctx->tw, tw.data(), sizeof(float2) * nx, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = sgw::grid_init_attributes(nx);
     if (e == cudaSuccess && ctx->sep) e = sgw::sep_init_attributes(nx);
+    if (e == cudaSuccess && ctx->sep && !sgw::rows_path(nx)) e = sgw::sep_split_init_attributes(nx);
     if (e == cudaSuccess) e = cudaMemset(ctx->vloc, 0, sizeof(float) * ctx->ng);
     if (e != cudaSuccess) {
         std::string m = std::string("setup: ") + cudaGetErrorString(e);
@@ -758,8 +759,8 @@ static sgw_status build_split_tables(sgw_ctx* ctx, int n_atoms, const int* nproj
     return SGW_OK;
 }
 
-// F_a(tau) = e^{-i tau M_a} - 1 for tau = dt/2 (set 0) and -dt/2 (set 1): the device table of this
-// dt (built and uploaded on its first use) in *out
+// F_a(tau) = e^{-i tau M_a} - 1 for tau = dt/2, -dt/2, dt and -dt (sets 0 .. 3): the device table of
+// this dt (built and uploaded on its first use) in *out
 static sgw_status split_factors(sgw_ctx* ctx, double dt, const float2** out) {
     const int na = ctx->kb.n_atoms;
     *out = nullptr;
@@ -771,18 +772,18 @@ static sgw_status split_factors(sgw_ctx* ctx, double dt, const float2** out) {
             *out = t.second;
             return SGW_OK;
         }
-    std::vector<float2> F((size_t)na * 32);
+    std::vector<float2> F((size_t)na * 64);
     for (int a = 0; a < na; ++a) {
         double lam[4], w[16];
         jacobi_eig(4, &ctx->kb_m[(size_t)a * 16], lam, w);
-        for (int set = 0; set < 2; ++set) {
-            const double tau = (set == 0 ? 0.5 : -0.5) * dt;
+        for (int set = 0; set < 4; ++set) {
+            const double tau = (set & 1 ? -0.5 : 0.5) * (set & 2 ? 2.0 : 1.0) * dt;
             for (int i = 0; i < 4; ++i)
                 for (int j = 0; j < 4; ++j) {
                     std::complex<double> f = 0.0;
                     for (int k = 0; k < 4; ++k)
                         f += w[i * 4 + k] * (std::exp(std::complex<double>(0.0, -tau * lam[k])) - 1.0) * w[j * 4 + k];
-                    F[((size_t)a * 2 + set) * 16 + i * 4 + j] = make_float2((float)f.real(), (float)f.imag());
+                    F[((size_t)a * 4 + set) * 16 + i * 4 + j] = make_float2((float)f.real(), (float)f.imag());
                 }
         }
     }
@@ -1370,51 +1371,74 @@ sgw_status sgw_propagate(sgw_ctx* ctx, void* psi_dev, int batch, int n_steps, do
     });
 }
 
-// One split-operator step of a batch in place (ctx->info: per-vector direction, potential row,
-// tangent row and partner); split_factors(ctx, dt) must have run.
-static sgw_status split_step_batch(sgw_ctx* ctx, float2* psi, int batch, const float* vpot, const float* dvpot,
-                                   double dt, const float2* F) {
+// Colours c0, c0 + dir, .. (count of them) of the split KB factor on a batch; full: e^{-i dt V_a} instead of
+// the half-step's e^{-i (dt/2) V_a}.
+static sgw_status split_kb(sgw_ctx* ctx, float2* psi, int batch, const float2* F, int c0, int count, int dir, bool full) {
+    const double kb_bytes = (double)ctx->kb.n_sup * batch * 24.0;     // gather + write back + Q per point
+    for (int i = 0; i < count; ++i) {
+        const int c = c0 + dir * i, a0 = ctx->acol_off[c], na = ctx->acol_off[c + 1] - a0;
+        Launch L(ctx, SGW_PROF_KB, 1, kb_bytes * na / std::max(ctx->kb.n_atoms, 1));
+        sgw::launch_kb_split(ctx->acol_atoms + a0, na, ctx->kb, ctx->kbq, F, full ? 1 : 0, ctx->info, psi, batch,
+                             (size_t)ctx->ng, ctx->stream);
+        CKL();
+    }
+    return SGW_OK;
+}
+
+// The local and kinetic factors e^{-i V dt/2} e^{-i T dt} e^{-i V dt/2} of a split-operator step, in place
+// (ctx->info: per-vector direction, potential row, tangent row and partner).  Without a cutoff the
+// half-step phases of the potential rows come from the table split_phases left in ctx->B1.
+static sgw_status split_core(sgw_ctx* ctx, float2* psi, int batch, const float* vpot, const float* dvpot, double dt) {
     const int n = ctx->n;
     const float kscale = (float)std::pow(2.0 * M_PI / ctx->L, 2);
-    const int nc = (int)ctx->acol_off.size() - 1;
     const double vb = (double)ctx->ng * batch;
-    const double kb_bytes = (double)ctx->kb.n_sup * batch * 24.0;     // gather + write back + Q per point
-    auto kb_half = [&](bool descending) -> sgw_status {
-        for (int i = 0; i < nc; ++i) {
-            const int c = descending ? nc - 1 - i : i;
-            const int a0 = ctx->acol_off[c], na = ctx->acol_off[c + 1] - a0;
-            Launch L(ctx, SGW_PROF_KB, 1, kb_bytes * na / std::max(ctx->kb.n_atoms, 1));
-            sgw::launch_kb_split(ctx->acol_atoms + a0, na, ctx->kb, ctx->kbq, F, ctx->info, psi, batch,
-                                 (size_t)ctx->ng, ctx->stream);
+    if (!(ctx->ecut > 0)) {
+        Launch L(ctx, SGW_PROF_PLANE_FWD, 2, (dvpot ? 40.0 : 32.0) * vb + 16.0 * ctx->ng);
+        sgw::sep_split_core(n, psi, ctx->B1, dvpot, ctx->info, (float)dt, kscale, ctx->W, batch, ctx->tw, ctx->stream);
+        CKL();
+    } else {
+        {
+            Launch L(ctx, SGW_PROF_PLANE_FWD, 1, (dvpot ? 24.0 : 16.0) * vb + 8.0 * ctx->ng);
+            sgw::launch_plane_fwd_phase(n, psi, vpot, dvpot, ctx->info, (float)dt, ctx->W, batch, ctx->tw, ctx->stream);
             CKL();
         }
-        return SGW_OK;
-    };
-    sgw_status r;
-    if (ctx->kb.n_atoms > 0 && (r = kb_half(false))) return r;
-    {
-        Launch L(ctx, SGW_PROF_PLANE_FWD, 1, (dvpot ? 24.0 : 16.0) * vb + 8.0 * ctx->ng);
-        sgw::launch_plane_fwd_phase(n, psi, vpot, dvpot, ctx->info, (float)dt, ctx->W, batch, ctx->tw, ctx->stream);
-        CKL();
-    }
-    {
-        Launch L(ctx, SGW_PROF_PENCIL, 1, 16.0 * vb);
-        sgw::launch_pencil(n, ctx->W, batch, 2, kscale, (float)ctx->ecut, ctx->tw, ctx->stream,
-                           ctx->tune[SGW_TUNE_PENCIL_LOOKAHEAD], ctx->info, (float)dt);
-        CKL();
-    }
-    {
-        Launch L(ctx, SGW_PROF_SPLIT_INV, 1, 16.0 * vb + 4.0 * ctx->ng);
-        sgw::launch_plane_inv_phase(n, ctx->W, vpot, ctx->info, (float)dt, psi, batch, ctx->tw, ctx->stream);
-        CKL();
+        {
+            Launch L(ctx, SGW_PROF_PENCIL, 1, 16.0 * vb);
+            sgw::launch_pencil(n, ctx->W, batch, 2, kscale, (float)ctx->ecut, ctx->tw, ctx->stream,
+                               ctx->tune[SGW_TUNE_PENCIL_LOOKAHEAD], ctx->info, (float)dt);
+            CKL();
+        }
+        {
+            Launch L(ctx, SGW_PROF_SPLIT_INV, 1, 16.0 * vb + 4.0 * ctx->ng);
+            sgw::launch_plane_inv_phase(n, ctx->W, vpot, ctx->info, (float)dt, psi, batch, ctx->tw, ctx->stream);
+            CKL();
+        }
     }
     if (dvpot != nullptr) {
         Launch L(ctx, SGW_PROF_OTHER, 1, 14.0 * vb);     // tangent halves: own + partner + dv
         sgw::launch_split_tangent(psi, dvpot, ctx->info, (float)dt, batch, ctx->ng, ctx->stream);
         CKL();
     }
-    if (ctx->kb.n_atoms > 0 && (r = kb_half(true))) return r;
     return SGW_OK;
+}
+
+// The half-step phases of `rows` potential rows into ctx->B1 (which no split-operator call uses otherwise)
+static sgw_status split_phases(sgw_ctx* ctx, const float* vpot, int rows, double dt) {
+    if (ctx->ecut > 0) return SGW_OK;
+    Launch L(ctx, SGW_PROF_OTHER, 1, 12.0 * (double)ctx->ng * rows);
+    sgw::sep_split_phase(ctx->ng * rows, vpot, (float)dt, ctx->B1, ctx->stream);
+    CKL();
+    return SGW_OK;
+}
+
+// One split-operator step of a batch in place; split_factors(ctx, dt) and split_phases must have run.
+static sgw_status split_step_batch(sgw_ctx* ctx, float2* psi, int batch, const float* vpot, const float* dvpot,
+                                   double dt, const float2* F) {
+    const int nc = ctx->kb.n_atoms > 0 ? (int)ctx->acol_off.size() - 1 : 0;
+    sgw_status r;
+    if ((r = split_kb(ctx, psi, batch, F, 0, nc, 1, false))) return r;
+    if ((r = split_core(ctx, psi, batch, vpot, dvpot, dt))) return r;
+    return split_kb(ctx, psi, batch, F, nc - 1, nc, -1, false);
 }
 
 sgw_status sgw_propagate_split(sgw_ctx* ctx, void* psi_dev, int batch, int n_steps, double dt,
@@ -1437,10 +1461,21 @@ sgw_status sgw_propagate_split(sgw_ctx* ctx, void* psi_dev, int batch, int n_ste
     float2* psi = (float2*)psi_dev;
     std::vector<uint64_t> key = {7, (uint64_t)batch, (uint64_t)n_steps, bits(dt), (uint64_t)psi,
                                  fnv(info.data(), sizeof(sgw::VecInfo) * info.size())};
-    return graphed(ctx, key, [&]() {
-        for (int j = 0; j < n_steps; ++j)
-            if (sgw_status r = split_step_batch(ctx, psi, batch, ctx->vloc, nullptr, dt, F)) return r;
-        return SGW_OK;
+    return graphed(ctx, key, [&]() -> sgw_status {
+        // between two steps the last factor of the one and the first of the next are the same colour's:
+        // one full factor instead of two halves
+        const int nc = ctx->kb.n_atoms > 0 ? (int)ctx->acol_off.size() - 1 : 0;
+        sgw_status r;
+        if ((r = split_phases(ctx, ctx->vloc, 1, dt))) return r;
+        if ((r = split_kb(ctx, psi, batch, F, 0, nc, 1, false))) return r;
+        for (int j = 0; j < n_steps; ++j) {
+            if ((r = split_core(ctx, psi, batch, ctx->vloc, nullptr, dt))) return r;
+            if (j + 1 == n_steps || nc == 0) continue;
+            if ((r = split_kb(ctx, psi, batch, F, nc - 1, nc - 1, -1, false))) return r;
+            if ((r = split_kb(ctx, psi, batch, F, 0, 1, 1, true))) return r;
+            if ((r = split_kb(ctx, psi, batch, F, 1, nc - 1, 1, false))) return r;
+        }
+        return split_kb(ctx, psi, batch, F, nc - 1, nc, -1, false);
     });
 }
 
@@ -1558,6 +1593,7 @@ static sgw_status tdh_run(sgw_ctx* ctx, const void* eta_dev, const float* source
             CKL();
             if (j == n_steps) break;
             if (cheb_deg == 0) {
+                if (sgw_status s2 = split_phases(ctx, vtot, n_samples, dt)) return s2;
                 if (sgw_status s2 = split_step_batch(ctx, psi, B, vtot, dv, dt, F)) return s2;
             } else if (sgw_status s2 = run_series(ctx, plan, psi, psi, B, vtot, dv, ctx->info, j > 0, true, n_samples)) {
                 return s2;
@@ -1678,6 +1714,8 @@ static sgw_status sigma_run(sgw_ctx* ctx, void* zeta_dev, const float* phi_dev, 
                                (uint64_t)xi->K, (uint64_t)xi->L});
     }
     return graphed(ctx, key, [&]() -> sgw_status {
+    if (cheb_deg == 0 && n_steps > 0)
+        if (sgw_status s2 = split_phases(ctx, ctx->vloc, 1, dt)) return s2;
     for (int j = 0; j <= n_steps; ++j) {
         {
             if (xi) {

@@ -20,6 +20,7 @@ __device__ __forceinline__ void st4(float2* p, float2 a, float2 b) {
 // they displace neither the operands prefetched into L2 for later blocks nor the data shared by
 // the vectors of one unit.
 __device__ __forceinline__ float4 ldcs4(const float2* p) { return __ldcs(reinterpret_cast<const float4*>(p)); }
+__device__ __forceinline__ float2 ldcs2(const float2* p) { return __ldcs(p); }
 __device__ __forceinline__ void stcs4(float2* p, float2 a, float2 b) {
     __stcs(reinterpret_cast<float4*>(p), make_float4(a.x, a.y, b.x, b.y));
 }

@@ -669,59 +669,74 @@ k_split_tangent(float2* __restrict__ psi, const float* __restrict__ dvpot, const
 // One colour of the split KB factor: block (i, b) applies e^{-i tau V_a} = 1 + Q_a F_a Q_a^T to
 // vector b for atom a = atoms[i]: c = Q_a^T x over the atom's support (fixed-order block sum),
 // d = F c with F the 4 x 4 complex factor of the vector's direction, x += Q_a d.  Atoms of one
-// colour have disjoint supports, so the blocks of a launch touch disjoint points.
+// colour have disjoint supports, so the blocks of a launch touch disjoint points.  Latency-bound (index,
+// then point, then the block's sum): the support's loads are all in flight at once and its points
+// stay in registers for the update, up to KBS_R per thread (2048 points; the supports of the
+// cluster at h = 0.5 have 1557); what a larger support has beyond that is read again.
+constexpr int KBS_R = 8;
 __global__ void __launch_bounds__(256)
 k_kb_split(const int* __restrict__ atoms, const int64_t* __restrict__ atom_off, const int* __restrict__ sup_idx,
-           const float4* __restrict__ q4, const float2* __restrict__ F /*[n_atoms][2][16]*/,
+           const float4* __restrict__ q4, const float2* __restrict__ F /*[n_atoms][4][16]*/, int full,
            const VecInfo* __restrict__ info, float2* __restrict__ x, size_t ng) {
     __shared__ float red[8][8];
     __shared__ float2 d[4];
     const int a = __ldg(atoms + blockIdx.x), b = blockIdx.y;
     const int64_t s0 = __ldg(atom_off + a), s1 = __ldg(atom_off + a + 1);
     float2* v = x + (size_t)b * ng;
-    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    for (int64_t s = s0 + threadIdx.x; s < s1; s += blockDim.x) {
-        const float2 p = v[__ldg(sup_idx + s)];
-        const float4 q = __ldg(q4 + s);
-        acc[0] += q.x * p.x; acc[1] += q.x * p.y;
-        acc[2] += q.y * p.x; acc[3] += q.y * p.y;
-        acc[4] += q.z * p.x; acc[5] += q.z * p.y;
-        acc[6] += q.w * p.x; acc[7] += q.w * p.y;
-    }
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    int g[KBS_R];
+    float4 q[KBS_R];
+    float2 p[KBS_R];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        for (int o = 16; o > 0; o >>= 1) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], o);
-        if (lane == 0) red[w][i] = acc[i];
+    for (int i = 0; i < KBS_R; ++i) {
+        const int64_t s = s0 + threadIdx.x + 256 * i;
+        g[i] = s < s1 ? __ldg(sup_idx + s) : -1;
+        q[i] = s < s1 ? __ldg(q4 + s) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
+#pragma unroll
+    for (int i = 0; i < KBS_R; ++i) p[i] = g[i] >= 0 ? v[g[i]] : make_float2(0.f, 0.f);
+    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    const auto add = [&](float4 qq, float2 pp) {
+        acc[0] += qq.x * pp.x; acc[1] += qq.x * pp.y;
+        acc[2] += qq.y * pp.x; acc[3] += qq.y * pp.y;
+        acc[4] += qq.z * pp.x; acc[5] += qq.z * pp.y;
+        acc[6] += qq.w * pp.x; acc[7] += qq.w * pp.y;
+    };
+#pragma unroll
+    for (int i = 0; i < KBS_R; ++i) add(q[i], p[i]);
+    for (int64_t s = s0 + threadIdx.x + 256 * KBS_R; s < s1; s += 256) add(__ldg(q4 + s), v[__ldg(sup_idx + s)]);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const float r = warp_reduce_scatter8(acc, lane);
+    if ((lane & 3) == 0) red[w][lane >> 2] = r;
     __syncthreads();
     if (threadIdx.x < 4) {
-        const int p = threadIdx.x;
-        const float2* f = F + ((size_t)a * 2 + (info[b].cset == 0 ? 0 : 1)) * 16 + p * 4;
-        float2 c[4];
+        const int pr = threadIdx.x;
+        const float2* f = F + ((size_t)a * 4 + 2 * full + (info[b].cset == 0 ? 0 : 1)) * 16 + pr * 4;
+        float2 o = make_float2(0.f, 0.f);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             float re = 0.f, im = 0.f;
+#pragma unroll
             for (int ww = 0; ww < 8; ++ww) {
                 re += red[ww][2 * k];
                 im += red[ww][2 * k + 1];
             }
-            c[k] = make_float2(re, im);
+            o = cadd(o, cmul(__ldg(f + k), make_float2(re, im)));
         }
-        float2 o = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) o = cadd(o, cmul(__ldg(f + k), c[k]));
-        d[p] = o;
+        d[pr] = o;
     }
     __syncthreads();
     const float2 d0 = d[0], d1 = d[1], d2 = d[2], d3 = d[3];
-    for (int64_t s = s0 + threadIdx.x; s < s1; s += blockDim.x) {
-        const int g = __ldg(sup_idx + s);
-        const float4 q = __ldg(q4 + s);
-        float2 p = v[g];
-        p.x += q.x * d0.x + q.y * d1.x + q.z * d2.x + q.w * d3.x;
-        p.y += q.x * d0.y + q.y * d1.y + q.z * d2.y + q.w * d3.y;
-        v[g] = p;
+    const auto upd = [&](float4 qq, float2 pp) {
+        pp.x += qq.x * d0.x + qq.y * d1.x + qq.z * d2.x + qq.w * d3.x;
+        pp.y += qq.x * d0.y + qq.y * d1.y + qq.z * d2.y + qq.w * d3.y;
+        return pp;
+    };
+#pragma unroll
+    for (int i = 0; i < KBS_R; ++i)
+        if (g[i] >= 0) v[g[i]] = upd(q[i], p[i]);
+    for (int64_t s = s0 + threadIdx.x + 256 * KBS_R; s < s1; s += 256) {
+        const int gi = __ldg(sup_idx + s);
+        v[gi] = upd(__ldg(q4 + s), v[gi]);
     }
 }
 
@@ -1009,10 +1024,10 @@ void launch_split_tangent(float2* psi, const float* dvpot, const VecInfo* info, 
     k_split_tangent<<<dim3(bx, batch), 256, 0, st>>>(psi, dvpot, info, dt, ng);
 }
 
-void launch_kb_split(const int* atoms, int n_atoms_colour, const KBDev& kb, const float4* q4, const float2* F,
+void launch_kb_split(const int* atoms, int n_atoms_colour, const KBDev& kb, const float4* q4, const float2* F, int full,
                      const VecInfo* info, float2* x, int batch, size_t ng, cudaStream_t st) {
     if (n_atoms_colour == 0 || batch == 0) return;
-    k_kb_split<<<dim3(n_atoms_colour, batch), 256, 0, st>>>(atoms, kb.atom_off, kb.sup_idx, q4, F, info, x, ng);
+    k_kb_split<<<dim3(n_atoms_colour, batch), 256, 0, st>>>(atoms, kb.atom_off, kb.sup_idx, q4, F, full, info, x, ng);
 }
 
 void launch_kb_project(int n, const KBDev& kb, const float2* b1, int batch, float dV, float2* kbc, cudaStream_t st) {

@@ -290,6 +290,127 @@ __global__ void __launch_bounds__(SpCfg<N>::NT, (SpCfg<N>::MINB)) k_sep_plane(St
     kb_project_unit<N, PITCH, NT, 2>(a, kh, ks, b, sm);
 }
 
+// ------------------------------------------------------------------ split-operator passes
+// e^{-i T dt} is a product over the axes: planes W = e^{-i (T_x + T_y) dt} e^{-i V dt/2} psi (16 B per
+// vector-point), then z lines psi = e^{-i V dt/2} e^{-i T_z dt} W (16 B), where the 3D transform took three
+// passes.  The half-step phases e^{-i V dt/2} come from a table per potential row, which the vectors
+// share (backward vectors take the conjugate); the factors along an axis depend on |m| only and are
+// computed once per block.  Along an axis the line gains IDFT((e^{-i T_a dt} - 1) DFT(line)): the rounding
+// of the transforms and of the factor, which is the same in every step, is then in proportion to what
+// the step changes (three factors of modulus 1 +- 2^-25 would add up over the steps).
+// Measured, ten steps of 27 vectors at 64^3 with KB: 1.40 -> 1.00 ms, of which the two passes 0.66 (at two
+// blocks of 256 threads per SM; three or four spill the second line operation: 1.03, 1.04); the error
+// against 64 bits went from 1.3e-6 to 3.7e-7.
+template <int N>
+__device__ __forceinline__ void axis_phases(float2* ph, float ks, float dt, int nt) {
+    for (int m = threadIdx.x; m <= N / 2; m += nt) {
+        float sn, cs;                          // e^{-i w} - 1 = -2 sin^2(w/2) - 2 i sin(w/2) cos(w/2), over N
+        sincosf(0.25f * ks * (float)(m * m) * dt, &sn, &cs);
+        ph[m] = make_float2(sn * sn * (-2.0f / N), sn * cs * (-2.0f / N));
+    }
+}
+template <int N, int T>
+__device__ __forceinline__ float2 axis_phase(const float2* ph, int k1, int i) {
+    return ph[abs(k1 + (N / T) * i - (2 * i >= T ? N : 0))];
+}
+
+template <int N>
+__global__ void __launch_bounds__(SpCfg<N>::NT, (N == 128 ? 1 : (N == 64 ? 2 : 8)))
+k_split_plane(const float2* __restrict__ psi, const float2* __restrict__ phase, const float* __restrict__ dvpot,
+              const VecInfo* __restrict__ info, float dt, float ks, float2* __restrict__ W, const float2* __restrict__ tw) {
+    constexpr int T = SpCfg<N>::T, P = N / T, CPW = 32 / T, NT = SpCfg<N>::NT, PITCH = SpCfg<N>::PITCH;
+    constexpr size_t NG = (size_t)N * N * N;
+    extern __shared__ __align__(16) float2 sm[];
+    float2* tws = sm + N * PITCH;
+    float2* ph = tws + N;
+    const int z = blockIdx.x, b = blockIdx.y;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const size_t uoff = (size_t)z * N * N, off = (size_t)b * NG + uoff;
+    const VecInfo inf = info[b];
+    const float sg = inf.cset == 0 ? 1.f : -1.f;
+    const float2* E = phase + (size_t)inf.vrow * NG + uoff;
+    const bool tan = dvpot != nullptr && inf.dvrow >= 0;
+    const float* dV = tan ? dvpot + (size_t)inf.dvrow * NG + uoff : nullptr;
+    const float2* pp = tan ? psi + (size_t)inf.partner * NG + uoff : nullptr;
+#pragma unroll 2
+    for (int q = threadIdx.x; q < N * N / 2; q += NT) {
+        const int o = 2 * q;
+        const float4 v = ld4(psi + off + o), e = ld4(E + o);
+        float2 a0 = make_float2(v.x, v.y), a1 = make_float2(v.z, v.w);
+        if (tan) {
+            // the derivative of the half-step along V -> V + lam dv: psi - i s (dt/2) dv psi_partner
+            const float4 pa = ld4(pp + o);
+            const float2 d = __ldg(reinterpret_cast<const float2*>(dV + o));
+            const float h = 0.5f * sg * dt;
+            a0 = make_float2(a0.x + h * d.x * pa.y, a0.y - h * d.x * pa.x);
+            a1 = make_float2(a1.x + h * d.y * pa.w, a1.y - h * d.y * pa.z);
+        }
+        a0 = cmul(a0, make_float2(e.x, sg * e.y));
+        a1 = cmul(a1, make_float2(e.z, sg * e.w));
+        *reinterpret_cast<float4*>(sm + (q / (N / 2)) * PITCH + 2 * (q % (N / 2))) = make_float4(a0.x, a0.y, a1.x, a1.y);
+    }
+    for (int i = threadIdx.x; i < N; i += NT) tws[i] = __ldg(tw + i);
+    axis_phases<N>(ph, ks, sg * dt, NT);
+    __syncthreads();
+    const int l = warp * CPW + lane % CPW, t = lane / CPW;
+    const auto f = [&](int k1, int i) { return axis_phase<N, T>(ph, k1, i); };
+    float2 v[P];
+    float2* row = sm + l * PITCH + t;
+#pragma unroll
+    for (int i = 0; i < P; ++i) v[i] = row[T * i];
+    line_op<N, T>(v, lane, tws, f);
+    asm volatile("" ::: "memory");           // the line is read again, not held in registers meanwhile
+#pragma unroll
+    for (int i = 0; i < P; ++i) row[T * i] = cadd(row[T * i], v[i]);
+    __syncthreads();
+    const float2* col = sm + t * PITCH + l;
+#pragma unroll
+    for (int i = 0; i < P; ++i) v[i] = col[T * i * PITCH];
+    line_op<N, T>(v, lane, tws, f);
+    asm volatile("" ::: "memory");
+    float2* dst = W + off + (size_t)t * N + l;
+#pragma unroll
+    for (int i = 0; i < P; ++i) dst[T * i * N] = cadd(col[T * i * PITCH], v[i]);
+}
+
+template <int N>
+__global__ void __launch_bounds__(ZS_NT, 4)
+k_split_z(const float2* __restrict__ W, const float2* __restrict__ phase, const VecInfo* __restrict__ info, float dt,
+          float ks, float2* __restrict__ psi, const float2* __restrict__ tw) {
+    constexpr int T = ZsCfg<N>::T, P = N / T, CPW = 32 / T;
+    constexpr size_t NG = (size_t)N * N * N, NN = (size_t)N * N;
+    __shared__ float2 tws[N], ph[N / 2 + 1];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int b = gridDim.y - 1 - blockIdx.y;       // the last vectors' W is still in L2
+    const VecInfo inf = info[b];
+    const float sg = inf.cset == 0 ? 1.f : -1.f;
+    for (int i = threadIdx.x; i < N; i += ZS_NT) tws[i] = __ldg(tw + i);
+    const size_t at = (blockIdx.x * (ZS_NT / 32) + warp) * CPW + lane % CPW + (size_t)(lane / CPW) * NN;
+    const float2* src = W + (size_t)b * NG + at;
+    float2 v[P];
+#pragma unroll
+    for (int a = 0; a < P; ++a) v[a] = __ldg(src + (size_t)(T * a) * NN);
+    axis_phases<N>(ph, ks, sg * dt, ZS_NT);
+    __syncthreads();
+    line_op<N, T>(v, lane, tws, [&](int k1, int i) { return axis_phase<N, T>(ph, k1, i); });
+    const float2* E = phase + (size_t)inf.vrow * NG + at;
+    float2* dst = psi + (size_t)b * NG + at;
+#pragma unroll
+    for (int a = 0; a < P; ++a) {
+        const float2 e = __ldg(E + (size_t)(T * a) * NN), w = __ldg(src + (size_t)(T * a) * NN);
+        dst[(size_t)(T * a) * NN] = cmul(cadd(w, v[a]), make_float2(e.x, sg * e.y));
+    }
+}
+
+// e^{-i V dt/2} of `count` potential values
+__global__ void __launch_bounds__(256) k_split_phase(int64_t count, const float* __restrict__ V, float hdt, float2* __restrict__ e) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
+        float sn, cs;
+        sincosf(__ldg(V + i) * hdt, &sn, &cs);
+        e[i] = make_float2(cs, -sn);
+    }
+}
+
 // ------------------------------------------------------------------ n = 288
 // A 288-point line in the registers of 12 threads, 24 points each: x[t + 12 a] -> DFT24 over a,
 // exchange through shared memory, two DFT12 over t for k1 = t' + 12 i (times W288^(t k1) on the way
@@ -419,6 +540,15 @@ __global__ void __launch_bounds__(SR_NT, 4) k_sep_rows288(StepArgs a, float c, c
         default: break;                                  \
     }
 
+#define SGW_DISPATCH_SPLIT(n, ...)                       \
+    switch (n) {                                         \
+        case 16: { constexpr int N = 16; __VA_ARGS__; } break;   \
+        case 32: { constexpr int N = 32; __VA_ARGS__; } break;   \
+        case 64: { constexpr int N = 64; __VA_ARGS__; } break;   \
+        case 128: { constexpr int N = 128; __VA_ARGS__; } break; \
+        default: break;                                  \
+    }
+
 int sep_unit_pos(int n, int o) {
     int pitch = SR_PITCH;
     SGW_DISPATCH_SEP(n, pitch = SpCfg<N>::PITCH);
@@ -485,6 +615,32 @@ void sep_step(int n, const StepArgs& a, int batch, float kscale, const float2* t
         return;
     }
     SGW_DISPATCH_SEP(n, k_sep_plane<N><<<dim3(N, batch), SpCfg<N>::NT, sm, st>>>(a, c, tw));
+}
+
+static size_t split_plane_smem(int n) {
+    size_t pts = 0;
+    SGW_DISPATCH_SEP(n, pts = (size_t)N * SpCfg<N>::PITCH);
+    return sizeof(float2) * (pts + n + n / 2 + 1);
+}
+
+cudaError_t sep_split_init_attributes(int n) {
+    cudaError_t e = cudaSuccess;
+    SGW_DISPATCH_SPLIT(n, e = sep_attr(k_split_plane<N>, (int)split_plane_smem(n)));
+    return e;
+}
+
+void sep_split_phase(int64_t count, const float* V, float dt, float2* phase, cudaStream_t st) {
+    k_split_phase<<<(unsigned)std::min<int64_t>((count + 255) / 256, 152 * 16), 256, 0, st>>>(count, V, 0.5f * dt, phase);
+}
+
+void sep_split_core(int n, float2* psi, const float2* phase, const float* dvpot, const VecInfo* info, float dt, float kscale,
+                    float2* W, int batch, const float2* tw, cudaStream_t st) {
+    if (batch == 0) return;
+    SGW_DISPATCH_SPLIT(n, {
+        k_split_plane<N><<<dim3(N, batch), SpCfg<N>::NT, split_plane_smem(n), st>>>(psi, phase, dvpot, info, dt, kscale, W,
+                                                                                   tw);
+        k_split_z<N><<<dim3(ZsCfg<N>::BLOCKS, batch), ZS_NT, 0, st>>>(W, phase, info, dt, kscale, psi, tw);
+    });
 }
 
 }  // namespace sgw

@@ -109,6 +109,12 @@ void sep_z(int n, const float2* in, float2* W, int batch, float kscale, const fl
            cudaStream_t st);
 void sep_y288(const float2* in, float2* W, int batch, float kscale, const float2* tw, cudaStream_t st);
 void sep_step(int n, const StepArgs& a, int batch, float kscale, const float2* tw, cudaStream_t st);
+// split operator (power-of-two grids): phase = e^{-i V dt/2} of `count` values; the core
+// psi <- e^{-i V dt/2} e^{-i T dt} e^{-i V dt/2} psi (tangent source of the first half included) of a batch
+cudaError_t sep_split_init_attributes(int n);
+void sep_split_phase(int64_t count, const float* V, float dt, float2* phase, cudaStream_t st);
+void sep_split_core(int n, float2* psi, const float2* phase, const float* dvpot, const VecInfo* info, float dt, float kscale,
+                    float2* W, int batch, const float2* tw, cudaStream_t st);
 
 // ---- grid kernels (kernels_grid.cu)
 bool grid_supported(int n);
@@ -131,7 +137,8 @@ void launch_split_tangent(float2* psi, const float* dvpot, const VecInfo* info, 
                           cudaStream_t st);
 void launch_plane_inv_phase(int n, const float2* W, const float* vloc, const VecInfo* info, float dt, float2* psi,
                             int batch, const float2* tw, cudaStream_t st);
-void launch_kb_split(const int* atoms, int n_atoms_colour, const KBDev& kb, const float4* q4, const float2* F,
+// F: [n_atoms][4 sets][16], set = 2 full + (backward vector ? 1 : 0)
+void launch_kb_split(const int* atoms, int n_atoms_colour, const KBDev& kb, const float4* q4, const float2* F, int full,
                      const VecInfo* info, float2* x, int batch, size_t ng, cudaStream_t st);
 // exchange energy: acc[b / per] += (dV / N) sum_k v(k) |F(k)|^2 after the z transform
 int pencil_blocks(int n);

@@ -94,3 +94,34 @@ def test_more_slots_than_the_separable_step_holds():
     a.set_potential(w)                                       # without the atoms the separable step is back
     a.apply_h(x, ya)
     assert torch.equal(ya, yb)
+
+
+@pytest.mark.parametrize('n', [16, 32, 64, 128])
+def test_split_steps_match_the_transform_path(n):
+    """Propagation, TDH and Sigma(t) by split-operator steps with and without a (never reached) cutoff, and
+    one call of three steps against three calls of one (merged colours against halves)."""
+    build.build()
+    s = _system(n)
+    B = 3
+    g = torch.Generator(device='cuda').manual_seed(n)
+    x = torch.randn(B, n ** 3, dtype=torch.complex64, device='cuda', generator=g)
+    outs = []
+    for ecut in (0.0, 1e6):
+        c = _ctx(s, 4, ecut, True)
+        dirs = np.array([1, -1, 1], dtype=np.int8)
+        p, q = x.clone(), x.clone()
+        c.propagate_split(p, 3, 0.05, dirs)
+        for _ in range(3):
+            c.propagate_split(q, 1, 0.05, dirs)
+        uR = torch.empty(1, 3, n ** 3, dtype=torch.float32, device='cuda')
+        c.tdh_response((0.05 * x[:2]).contiguous(), x[0].real.contiguous(), 1, 2, 2, 0.05, 0, uR)
+        z = x[:2].clone()
+        sig = torch.empty(1, 5, dtype=torch.complex128, device='cuda')
+        c.sigma_c(z, x[2].real.contiguous(), x[:3].reshape(1, 3, -1).contiguous(), 1, 2, 0.05, 0, sig)
+        torch.cuda.synchronize()
+        assert float((p - q).abs().max() / q.abs().max()) < 3 * 4 * TOL_H
+        outs.append((p, uR, z))
+        c.close()
+    # a step is 6 line transforms and the phases, twice the chain of one H application
+    for a, b, steps in zip(outs[0], outs[1], (3, 6, 2)):
+        assert float((a - b).abs().max() / b.abs().max()) < 4 * TOL_H * steps
