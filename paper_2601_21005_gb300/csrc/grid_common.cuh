@@ -20,9 +20,27 @@ __device__ __forceinline__ void st4(float2* p, float2 a, float2 b) {
 // they displace neither the operands prefetched into L2 for later blocks nor the data shared by
 // the vectors of one unit.
 __device__ __forceinline__ float4 ldcs4(const float2* p) { return __ldcs(reinterpret_cast<const float4*>(p)); }
-__device__ __forceinline__ float2 ldcs2(const float2* p) { return __ldcs(p); }
 __device__ __forceinline__ void stcs4(float2* p, float2 a, float2 b) {
     __stcs(reinterpret_cast<float4*>(p), make_float4(a.x, a.y, b.x, b.y));
+}
+
+// Loads of data that the kernel before this one writes, after a wait for it inside this kernel
+// (programmatic launches): neither the read-only path, whose data must not change while the kernel
+// runs, nor an intrinsic that the compiler may move above the wait.
+__device__ __forceinline__ float2 ld2_written(const float2* p) {
+    float2 v;
+    asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float4 ld4_written(const float2* p) {
+    float4 v;
+    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float4 ldcs4_written(const float2* p) {
+    float4 v;
+    asm volatile("ld.global.cs.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
 }
 
 // Sum 8 per-lane values over a warp by halving exchanges at lane distances 16, 8, 4 (each lane keeps

@@ -44,7 +44,7 @@ __device__ __forceinline__ void kb_reduce_warp(const KbReduceArgs& kr, int a, in
     const float2* kb = kr.kbp + (size_t)b * kr.total_slots * 4;
     float2 acc = make_float2(0.f, 0.f);
     for (int q = q0 + (lane >> 2); q < q1; q += 8) {
-        const float2 v = __ldg(kb + (size_t)__ldg(kr.atom_pos + q) * 4 + p);
+        const float2 v = ld2_written(kb + (size_t)__ldg(kr.atom_pos + q) * 4 + p);
         acc.x += v.x;
         acc.y += v.y;
     }
@@ -85,9 +85,9 @@ __device__ __forceinline__ KbHead kb_head(const StepArgs& a, int u) {
 // E-weighted projector coefficients of the unit's slots into shared memory: kcs[4 s + p] for the
 // unit's s-th slot and projector p (kc: the vector's coefficients, [slot][4]).
 template <int NT>
-__device__ __forceinline__ void kb_stage_coeffs(const KbHead& h, const float2* __restrict__ kc, float2* kcs) {
-    const float4* src = reinterpret_cast<const float4*>(kc + (size_t)4 * h.s0);
-    for (int i = threadIdx.x; i < 2 * (h.s1 - h.s0); i += NT) reinterpret_cast<float4*>(kcs)[i] = __ldg(src + i);
+__device__ __forceinline__ void kb_stage_coeffs(const KbHead& h, const float2* kc, float2* kcs) {
+    const float2* src = kc + (size_t)4 * h.s0;
+    for (int i = threadIdx.x; i < 2 * (h.s1 - h.s0); i += NT) reinterpret_cast<float4*>(kcs)[i] = ld4_written(src + 2 * i);
 }
 
 // KB_B entries of a lane (at eb, eb + stride, ...; past e1 the last one again, to be skipped by the
