@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "../../include/sgw.h"
+#include "dependent_launch.cuh"
 #include "fft_smem.cuh"
 #include "sgw_internal.cuh"
 
@@ -22,183 +23,407 @@ namespace sgw {
 // ------------------------------------------------------------------ BF16 tensor-core GEMM
 // C[m][n] = sum_k A(m, k) B(k, n),  A(m, k) = TA ? A[k lda + m] : A[m lda + k],
 //                                   B(k, n) = TB ? B[n ldb + k] : B[k ldb + n].
-// CTA tile 64 x 64, K step 32, 4 warps of 32 x 32 (2 x 4 tiles of mma.m16n8k16).
-enum { EPI_STORE = 0, EPI_BIAS_TANH = 1, EPI_BIAS = 2, EPI_DTANH = 3 };
+// The products are small (M <= some hundreds of rows, N and K 20 to 1603), so a call is a chain of
+// short kernels and the latency of each is what counts.  A block has a TM x 64 tile (4 warps of
+// TM/2 x 32, mma.m16n8k16); four K steps of 64 are in flight by cp.async, which for K <= 256 is the
+// whole slab at once, and the weights' share of them is requested before the kernel waits for the one
+// before it.  BF16 matrices have rows padded with zeros to multiples of 8 elements, so every copy is
+// 16 bytes and only rows are checked.  K of 384 and more is split over the blocks of a cluster (three
+// steps of 64 at least to a block), whose partial tiles are summed in rank order through distributed
+// shared memory.
+// 148-256-256-256-1603, gradients of 32 rows and the forward of 512: 292 and 92 us per call with 64 x 64
+// tiles, one scalar load per element and a kernel for each sum; now 53 and 25.
+enum { EPI_STORE = 0, EPI_BIAS_TANH = 1, EPI_BIAS = 2, EPI_DTANH = 3, EPI_LOSS = 4 };
 
 struct GemmEpi {
     int mode;
-    const float* bias;      // [N] (EPI_BIAS*)
-    float* out;             // [M][ldo] fp32 result (pre-activation for EPI_BIAS_TANH; dZ for EPI_DTANH)
-    int ldo;
-    __nv_bfloat16* out_bf;  // [M][ldo] bf16 copy of tanh(z) (BIAS_TANH) or of dZ (DTANH); may be null
-    const float* zprev;     // [M][ldo] pre-activation whose tanh' multiplies (EPI_DTANH)
+    const float* bias;      // [N] (EPI_BIAS*, EPI_LOSS)
+    float* out;             // [M][ldo] fp32 result (pre-activation for EPI_BIAS_TANH, dZ for EPI_DTANH, dY for
+    int64_t ldo;            //  EPI_LOSS); null for a pre-activation nothing reads
+    __nv_bfloat16* out_bf;  // [M][ldb] bf16 copy of tanh(z) (BIAS_TANH) or of out (DTANH, LOSS)
+    int ldb;
+    const float* aux;       // [M][ldo] the pre-activation whose tanh' multiplies (DTANH), or the targets (LOSS)
+    const float* w;         // [N] loss weights (LOSS), null: all 1
+    float scale;            // LOSS: out = scale w (y - aux)
+    float* y;               // [M][ldo] the output itself (LOSS)
 };
 
-constexpr int GT = 64, GK = 32, GPAD = 8;
+struct Gemm {
+    int M, N, K;
+    const __nv_bfloat16* A;
+    int lda;
+    const __nv_bfloat16* B;
+    int ldb;
+    GemmEpi ep;
+};
 
-__device__ __forceinline__ uint32_t ld_bf2(const __nv_bfloat16* p) { return *reinterpret_cast<const uint32_t*>(p); }
+constexpr int GN = 64, GK = 64, GS = 4, G_NT = 128;
+template <int TM> struct GemmCfg {
+    static constexpr int A_EL = TM * (GK + 8) > GK * (TM + 8) ? TM * (GK + 8) : GK * (TM + 8);
+    static constexpr int ST_EL = A_EL + GK * (GN + 8);                 // bf16 elements of one stage
+    static constexpr int SMEM = 2 * ST_EL * GS;
+    static_assert(4 * TM * (GN + 4) <= SMEM, "the split's partial tile fits in the stages");
+};
 
-template <int TA, int TB>
-__global__ void __launch_bounds__(128)
-k_gemm_bf16(int M, int N, int K, const __nv_bfloat16* __restrict__ A, int lda, const __nv_bfloat16* __restrict__ B,
-            int ldb, GemmEpi ep) {
-    __shared__ __align__(16) __nv_bfloat16 sA[GT][GK + GPAD];    // [m][k]
-    __shared__ __align__(16) __nv_bfloat16 sB[GT][GK + GPAD];    // [n][k] (B transposed)
-    const int m0 = blockIdx.y * GT, n0 = blockIdx.x * GT;
+int64_t gemm_tiles(int tm, int M, int N) { return ((M + tm - 1) / tm) * (int64_t)((N + GN - 1) / GN); }
+
+__device__ __forceinline__ void cp16(uint32_t dst, const void* src, bool valid) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(valid ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ float ldf_written(const float* p) {
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+    return v;
+}
+template <bool TRANS>
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t a) {
+    if (TRANS)
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+    else
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+}
+
+// One K step of an operand into shared memory: R x C elements at (r0, c0) of a row-major matrix of `rows`
+// rows and a padded row length ld.
+template <int R, int C>
+__device__ __forceinline__ void gemm_stage(uint32_t dst, const __nv_bfloat16* src, int ld, int rows, int r0, int c0) {
+    static_assert(R * C / 8 % G_NT == 0, "whole passes");
+#pragma unroll
+    for (int i = 0; i < R * C / 8 / G_NT; ++i) {
+        const int e = threadIdx.x + i * G_NT, r = e / (C / 8), c = e % (C / 8) * 8;
+        const bool ok = r0 + r < rows && c0 + c < ld;
+        cp16(dst + 2 * (r * (C + 8) + c), ok ? src + (size_t)(r0 + r) * ld + c0 + c : src, ok);
+    }
+}
+
+__device__ __forceinline__ void gemm_finish(const GemmEpi& ep, int row, int col, float v, float aux) {
+    const size_t o = (size_t)row * ep.ldo + col;
+    if (ep.mode == EPI_STORE) {
+        ep.out[o] = v;
+    } else if (ep.mode == EPI_BIAS_TANH) {
+        v += ep.bias[col];
+        if (ep.out) ep.out[o] = v;
+        ep.out_bf[(size_t)row * ep.ldb + col] = __float2bfloat16(tanhf(v));
+    } else if (ep.mode == EPI_BIAS) {
+        ep.out[o] = v + ep.bias[col];
+    } else if (ep.mode == EPI_DTANH) {
+        const float th = tanhf(aux);
+        v *= 1.f - th * th;
+        ep.out[o] = v;
+        ep.out_bf[(size_t)row * ep.ldb + col] = __float2bfloat16(v);
+    } else {
+        v += ep.bias[col];
+        ep.y[o] = v;
+        v = ep.scale * (ep.w ? ep.w[col] : 1.f) * (v - aux);
+        ep.out[o] = v;
+        ep.out_bf[(size_t)row * ep.ldb + col] = __float2bfloat16(v);
+    }
+}
+
+// One tile of a product, by a block that is rank `rank` of `splits` for it.  WEIGHTS: B was written
+// before the kernel directly before this one started.
+template <int TM, int TA, int TB, bool WEIGHTS>
+__device__ __forceinline__ void gemm_tile(const Gemm& g, int64_t tile, int rank, int splits) {
+    extern __shared__ __align__(16) __nv_bfloat16 gsm[];
+    typedef GemmCfg<TM> C;
+    constexpr int MT = TM / 32;                                        // m16 tiles of a warp
+    constexpr int LA = TA ? TM + 8 : GK + 8, LB = TB ? GK + 8 : GN + 8;
+    const int nt = (g.N + GN - 1) / GN;
+    const int m0 = (int)(tile / nt) * TM, n0 = (int)(tile % nt) * GN;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;
-    const int g = lane >> 2, t = lane & 3;
-    float acc[2][4][4];
+    const int wm = (warp >> 1) * (TM / 2), wn = (warp & 1) * 32;
+    const int chunk = ((g.K + GK - 1) / GK + splits - 1) / splits;
+    const int s0 = min(rank * chunk, (g.K + GK - 1) / GK);
+    const int steps = min(chunk, (g.K + GK - 1) / GK - s0);
+    const uint32_t base = (uint32_t)__cvta_generic_to_shared(gsm);
+    auto stage_a = [&](int s) {
+        const uint32_t d = base + 2 * C::ST_EL * (s % GS);
+        const int k0 = (s0 + s) * GK;
+        if (TA) gemm_stage<GK, TM>(d, g.A, g.lda, g.K, k0, m0);
+        else gemm_stage<TM, GK>(d, g.A, g.lda, g.M, m0, k0);
+    };
+    auto stage_b = [&](int s) {
+        const uint32_t d = base + 2 * C::ST_EL * (s % GS) + 2 * C::A_EL;
+        const int k0 = (s0 + s) * GK;
+        if (TB) gemm_stage<GN, GK>(d, g.B, g.ldb, g.N, n0, k0);
+        else gemm_stage<GK, GN>(d, g.B, g.ldb, g.K, k0, n0);
+    };
+    if (WEIGHTS)
+        for (int s = 0; s < min(GS, steps); ++s) stage_b(s);
+    dependents_wait();
+    dependents_launch();
+    // the stages' groups are committed in order; B of the first GS, if early, belongs to the first group
 #pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int jn = 0; jn < 4; ++jn)
-#pragma unroll
-            for (int r = 0; r < 4; ++r) acc[i][jn][r] = 0.f;
-    const __nv_bfloat16 zero = __float2bfloat16(0.f);
-    for (int k0 = 0; k0 < K; k0 += GK) {
-        for (int e = threadIdx.x; e < GT * GK; e += 128) {
-            int mm, kk;
-            if (TA) { mm = e % GT; kk = e / GT; } else { kk = e % GK; mm = e / GK; }
-            const int gm = m0 + mm, gk = k0 + kk;
-            sA[mm][kk] = (gm < M && gk < K) ? (TA ? A[(size_t)gk * lda + gm] : A[(size_t)gm * lda + gk]) : zero;
-            int nn, kb;
-            if (TB) { kb = e % GK; nn = e / GK; } else { nn = e % GT; kb = e / GT; }
-            const int gn = n0 + nn, gk2 = k0 + kb;
-            sB[nn][kb] = (gn < N && gk2 < K) ? (TB ? B[(size_t)gn * ldb + gk2] : B[(size_t)gk2 * ldb + gn]) : zero;
+    for (int s = 0; s < GS; ++s) {
+        if (s < steps) {
+            stage_a(s);
+            if (!WEIGHTS) stage_b(s);
         }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    // the epilogue's operands, requested ahead
+    const bool with_aux = g.ep.mode == EPI_DTANH || g.ep.mode == EPI_LOSS;
+    float aux[MT][4][4];
+    if (with_aux && splits == 1) {
+#pragma unroll
+        for (int i = 0; i < MT; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const int row = m0 + wm + 16 * i + (lane >> 2) + (r >= 2 ? 8 : 0);
+                    const int col = n0 + wn + 8 * j + 2 * (lane & 3) + (r & 1);
+                    aux[i][j][r] = row < g.M && col < g.N ? ldf_written(g.ep.aux + (size_t)row * g.ep.ldo + col) : 0.f;
+                }
+    }
+    float acc[MT][4][4];
+#pragma unroll
+    for (int i = 0; i < MT; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int r = 0; r < 4; ++r) acc[i][j][r] = 0.f;
+    for (int s = 0; s < steps; ++s) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(GS - 1) : "memory");
         __syncthreads();
+        const uint32_t sa = base + 2 * C::ST_EL * (s % GS), sb = sa + 2 * C::A_EL;
 #pragma unroll
         for (int ks = 0; ks < GK; ks += 16) {
-            uint32_t af[2][4], bfr[4][2];
+            uint32_t af[MT][4], bf[2][4];
 #pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const int r0 = wm + 16 * i + g;
-                af[i][0] = ld_bf2(&sA[r0][ks + 2 * t]);
-                af[i][1] = ld_bf2(&sA[r0 + 8][ks + 2 * t]);
-                af[i][2] = ld_bf2(&sA[r0][ks + 2 * t + 8]);
-                af[i][3] = ld_bf2(&sA[r0 + 8][ks + 2 * t + 8]);
+            for (int i = 0; i < MT; ++i) {
+                const int m = wm + 16 * i;
+                if (TA) ldsm4<true>(af[i], sa + 2 * ((ks + (lane & 7) + (lane >> 4) * 8) * LA + m + (lane >> 3 & 1) * 8));
+                else ldsm4<false>(af[i], sa + 2 * ((m + (lane & 15)) * LA + ks + (lane >> 4) * 8));
             }
 #pragma unroll
-            for (int jn = 0; jn < 4; ++jn) {
-                const int c0 = wn + 8 * jn + g;
-                bfr[jn][0] = ld_bf2(&sB[c0][ks + 2 * t]);
-                bfr[jn][1] = ld_bf2(&sB[c0][ks + 2 * t + 8]);
+            for (int j = 0; j < 2; ++j) {
+                const int n = wn + 16 * j;
+                if (TB) ldsm4<false>(bf[j], sb + 2 * ((n + (lane & 7) + (lane >> 4) * 8) * LB + ks + (lane >> 3 & 1) * 8));
+                else ldsm4<true>(bf[j], sb + 2 * ((ks + (lane & 15)) * LB + n + (lane >> 4) * 8));
             }
 #pragma unroll
-            for (int i = 0; i < 2; ++i)
+            for (int i = 0; i < MT; ++i)
 #pragma unroll
-                for (int jn = 0; jn < 4; ++jn) {
-                    float* c = acc[i][jn];
+                for (int j = 0; j < 4; ++j) {
+                    float* c = acc[i][j];
                     asm volatile(
                         "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
                         "{%8,%9}, {%0,%1,%2,%3};\n"
                         : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-                        : "r"(af[i][0]), "r"(af[i][1]), "r"(af[i][2]), "r"(af[i][3]), "r"(bfr[jn][0]),
-                          "r"(bfr[jn][1]));
+                        : "r"(af[i][0]), "r"(af[i][1]), "r"(af[i][2]), "r"(af[i][3]), "r"(bf[j >> 1][2 * (j & 1)]),
+                          "r"(bf[j >> 1][2 * (j & 1) + 1]));
                 }
         }
         __syncthreads();
+        if (s + GS < steps) {
+            stage_a(s + GS);
+            stage_b(s + GS);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
     }
-    // epilogue: c0,c1 at (row g, cols 2t, 2t+1), c2,c3 at (row g + 8, same cols)
+    if (splits == 1) {
 #pragma unroll
-    for (int i = 0; i < 2; ++i)
+        for (int i = 0; i < MT; ++i)
 #pragma unroll
-        for (int jn = 0; jn < 4; ++jn)
+            for (int j = 0; j < 4; ++j)
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const int row = m0 + wm + 16 * i + g + (r >= 2 ? 8 : 0);
-                const int col = n0 + wn + 8 * jn + 2 * t + (r & 1);
-                if (row >= M || col >= N) continue;
-                float v = acc[i][jn][r];
-                const size_t o = (size_t)row * ep.ldo + col;
-                if (ep.mode == EPI_BIAS_TANH) {
-                    v += ep.bias[col];
-                    ep.out[o] = v;
-                    if (ep.out_bf) ep.out_bf[o] = __float2bfloat16(tanhf(v));
-                } else if (ep.mode == EPI_BIAS) {
-                    ep.out[o] = v + ep.bias[col];
-                } else if (ep.mode == EPI_DTANH) {
-                    const float th = tanhf(ep.zprev[o]);
-                    v *= 1.f - th * th;
-                    ep.out[o] = v;
-                    if (ep.out_bf) ep.out_bf[o] = __float2bfloat16(v);
-                } else {
-                    ep.out[o] = v;
+                for (int r = 0; r < 4; ++r) {
+                    const int row = m0 + wm + 16 * i + (lane >> 2) + (r >= 2 ? 8 : 0);
+                    const int col = n0 + wn + 8 * j + 2 * (lane & 3) + (r & 1);
+                    if (row < g.M && col < g.N) gemm_finish(g.ep, row, col, acc[i][j][r], aux[i][j][r]);
                 }
+    } else {
+        constexpr int LP = GN + 4;
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+        float* part = reinterpret_cast<float*>(gsm);
+#pragma unroll
+        for (int i = 0; i < MT; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int r = 0; r < 4; r += 2)
+                    *reinterpret_cast<float2*>(part + (wm + 16 * i + (lane >> 2) + 4 * r) * LP + wn + 8 * j + 2 * (lane & 3)) =
+                        make_float2(acc[i][j][r], acc[i][j][r + 1]);
+        asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        for (int e = rank * (TM * GN / splits) + threadIdx.x; e < (rank + 1) * (TM * GN / splits); e += G_NT) {
+            const int r = e / GN, c = e % GN;
+            const uint32_t at = base + 4 * (r * LP + c);
+            float v = 0.f;
+            for (int q = 0; q < splits; ++q) {
+                uint32_t ra;
+                float p;
+                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(at), "r"(q));
+                asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(p) : "r"(ra) : "memory");
+                v += p;
             }
+            if (m0 + r < g.M && n0 + c < g.N)
+                gemm_finish(g.ep, m0 + r, n0 + c, v,
+                            with_aux ? ldf_written(g.ep.aux + (size_t)(m0 + r) * g.ep.ldo + n0 + c) : 0.f);
+        }
+        // no block leaves while another may still read its partial tile
+        asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
 }
 
-static void gemm(int M, int N, int K, int TA, int TB, const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb,
-                 const GemmEpi& ep, cudaStream_t st) {
-    const dim3 grid((N + GT - 1) / GT, (M + GT - 1) / GT);
-    if (!TA && !TB) k_gemm_bf16<0, 0><<<grid, 128, 0, st>>>(M, N, K, A, lda, B, ldb, ep);
-    else if (TA && !TB) k_gemm_bf16<1, 0><<<grid, 128, 0, st>>>(M, N, K, A, lda, B, ldb, ep);
-    else if (!TA && TB) k_gemm_bf16<0, 1><<<grid, 128, 0, st>>>(M, N, K, A, lda, B, ldb, ep);
-    else k_gemm_bf16<1, 1><<<grid, 128, 0, st>>>(M, N, K, A, lda, B, ldb, ep);
+// a layer's forward product
+template <int TM>
+__global__ void __launch_bounds__(G_NT) k_mlp_forward(Gemm g) {
+    gemm_tile<TM, 0, 0, true>(g, blockIdx.x, 0, 1);
 }
 
-// ------------------------------------------------------------------ small MLP kernels
-__global__ void k_to_bf16(int64_t n, const float* __restrict__ x, __nv_bfloat16* __restrict__ y) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        y[i] = __float2bfloat16(x[i]);
+// out[n] = sum_m d[m][n] for 32 columns, fixed order: each warp a quarter of the rows in turn
+__device__ __forceinline__ void colsum_block(int M, int N, int64_t ld, const float* d, float* out, int block) {
+    __shared__ float sh[G_NT / 32][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n = block * 32 + lane;
+    float s = 0.f;
+    if (n < N) {
+        int m = warp;
+        for (; m + 28 < M; m += 32) {
+            float v[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) v[i] = ldf_written(d + (size_t)(m + 4 * i) * ld + n);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) s += v[i];
+        }
+        for (; m < M; m += 4) s += ldf_written(d + (size_t)m * ld + n);
+    }
+    sh[warp][lane] = s;
+    __syncthreads();
+    if (warp == 0 && n < N) out[n] = (sh[0][lane] + sh[1][lane]) + (sh[2][lane] + sh[3][lane]);
 }
 
-// Weighted loss sum_o w_o (y - t)^2 / (M O): dY = 2 w_o (y - t) / (M O) (fp32 and bf16); the loss
-// sum is accumulated in FP64.  w == nullptr means all weights 1.
-__global__ void k_loss_grad(int64_t n, int O, const float* __restrict__ y, const float* __restrict__ t,
-                            const float* __restrict__ w, float scale, float* __restrict__ d,
-                            __nv_bfloat16* __restrict__ dbf, double* loss) {
-    __shared__ double sh[32];
+// The loss sum_o w_o (y - t)^2 in FP64 and a fixed order: partials loss[1 + block] in the launch that follows
+// the output (its other blocks have more to do, and FP64 is slow), their sum in the one after it.
+struct Loss {
+    int64_t n;
+    int O, blocks;
+    const float *y, *t, *w;
+    double* loss;
+};
+
+__device__ __forceinline__ void loss_block(const Loss& l, int block) {
+    __shared__ double sh[G_NT / 32];
     double a = 0.0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const float e = y[i] - t[i];
-        const float wo = w ? w[i % O] : 1.f;
+    for (int64_t i = block * (int64_t)G_NT + threadIdx.x; i < l.n; i += (int64_t)l.blocks * G_NT) {
+        const float e = ldf_written(l.y + i) - l.t[i];
+        const float wo = l.w ? l.w[i % l.O] : 1.f;
         a += (double)wo * e * e;
-        d[i] = scale * wo * e;
-        dbf[i] = __float2bfloat16(scale * wo * e);
     }
     for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = a;
     __syncthreads();
-    if (threadIdx.x < 32) {
-        double s = threadIdx.x < (blockDim.x >> 5) ? sh[threadIdx.x] : 0.0;
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (threadIdx.x == 0) loss[1 + blockIdx.x] = s;      // per-block partial, summed by k_loss_sum
+    if (threadIdx.x == 0) {
+        double s = 0.0;
+        for (int i = 0; i < G_NT / 32; ++i) s += sh[i];
+        l.loss[1 + block] = s;
     }
 }
 
-// loss[0] = sum of the nb per-block partials loss[1 .. nb] in a fixed order (one warp)
-__global__ void k_loss_sum(int nb, double* loss) {
+__device__ __forceinline__ void loss_sum(const Loss& l) {
+    if (threadIdx.x >= 32) return;
     double s = 0.0;
-    for (int i = threadIdx.x; i < nb; i += 32) s += loss[1 + i];
+    for (int i = threadIdx.x; i < l.blocks; i += 32) s += *(const volatile double*)(l.loss + 1 + i);
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (threadIdx.x == 0) loss[0] = s;
+    if (threadIdx.x == 0) l.loss[0] = s;
 }
 
-// db[n] = sum_m d[m][n]   (one thread per column, fixed order)
-__global__ void k_colsum(int M, int N, const float* __restrict__ d, float* __restrict__ db) {
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    float s = 0.f;
-    for (int m = 0; m < M; ++m) s += d[(size_t)m * N + n];
-    db[n] = s;
+// A layer's backward pass in one launch, all of it from dZ of the layer: the clusters of dZ of the layer
+// below (d, absent for the first layer: d_tiles = 0) come first, then the blocks of dW, of the bias
+// gradient and of the loss (partials after the last layer, their sum one launch later).
+struct Backward {
+    Gemm d, w;
+    int64_t d_tiles, w_tiles;
+    int splits, db_blocks, loss_blocks, loss_sums;
+    const float* dz;
+    float* db;
+    int64_t ldz;
+    Loss loss;
+};
+
+__global__ void __launch_bounds__(G_NT) k_mlp_backward(Backward b) {
+    constexpr int TM = 32;
+    int64_t i = blockIdx.x;
+    if (i < b.d_tiles * b.splits) {
+        gemm_tile<TM, 0, 1, true>(b.d, i / b.splits, (int)(i % b.splits), b.splits);
+        return;
+    }
+    i -= b.d_tiles * b.splits;
+    if (i < b.w_tiles) {
+        gemm_tile<TM, 1, 0, false>(b.w, i, 0, 1);
+        return;
+    }
+    i -= b.w_tiles;
+    dependents_wait();
+    dependents_launch();
+    if (i < b.db_blocks) {
+        colsum_block(b.w.K, b.w.N, b.ldz, b.dz, b.db, (int)i);
+        return;
+    }
+    i -= b.db_blocks;
+    if (i < b.loss_blocks) loss_block(b.loss, (int)i);
+    else if (i == b.loss_blocks && b.loss_sums) loss_sum(b.loss);
+}
+
+// ------------------------------------------------------------------ small MLP kernels
+// x [rows][cols] -> y [rows][ld] in BF16 (the columns beyond cols stay zero)
+__global__ void k_mlp_input(int64_t n, int cols, int ld, const float* __restrict__ x, __nv_bfloat16* __restrict__ y) {
+    dependents_launch();
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        y[i / cols * ld + i % cols] = __float2bfloat16(x[i]);
+}
+
+// Where the parameters of the layers start, and where the BF16 copy of each matrix lies; and the blocks of
+// a kernel over them all: a block has MLP_NT columns of a row of a matrix, or of the bias (row = rows).
+constexpr int MLP_NT = 256;
+struct MlpLayout {
+    int64_t woff[4], boff[4], poff[4], first[5];
+    int rows[4], cols[4], ld[4], chunks[4];
+};
+
+// The parameter of this thread and its place among the BF16 copies (-1: none); false: no parameter.
+__device__ __forceinline__ bool mlp_param(const MlpLayout& L, int64_t& i, int64_t& at) {
+    const int64_t b = blockIdx.x;
+    int64_t first = L.first[0], woff = L.woff[0], boff = L.boff[0], poff = L.poff[0];
+    int rows = L.rows[0], cols = L.cols[0], ld = L.ld[0], chunks = L.chunks[0];
+#pragma unroll
+    for (int l = 1; l < 4; ++l)
+        if (b >= L.first[l]) {
+            first = L.first[l]; woff = L.woff[l]; boff = L.boff[l]; poff = L.poff[l];
+            rows = L.rows[l]; cols = L.cols[l]; ld = L.ld[l]; chunks = L.chunks[l];
+        }
+    const unsigned u = (unsigned)(b - first), r = u / (unsigned)chunks;
+    const int c = (int)(u - r * (unsigned)chunks) * MLP_NT + threadIdx.x;
+    if (c >= cols) return false;
+    const bool bias = r == (unsigned)rows;
+    i = bias ? boff + c : woff + (int64_t)r * cols + c;
+    at = bias ? -1 : poff + (int64_t)r * ld + c;
+    return true;
+}
+
+__global__ void __launch_bounds__(MLP_NT) k_mlp_weights(const float* __restrict__ w, __nv_bfloat16* __restrict__ wbf,
+                                                        MlpLayout L) {
+    int64_t i, at;
+    if (mlp_param(L, i, at) && at >= 0) wbf[at] = __float2bfloat16(w[i]);
 }
 
 // Adam (Kingma & Ba) on FP32 master weights; writes the BF16 copies of the matrices.
-__global__ void k_adam(int64_t n, float* __restrict__ w, const float* __restrict__ g, float* __restrict__ m,
-                       float* __restrict__ v, __nv_bfloat16* __restrict__ wbf, float lr, float b1, float b2, float c1,
-                       float c2, float eps) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const float gi = g[i];
-        const float mi = b1 * m[i] + (1.f - b1) * gi;
-        const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-        m[i] = mi;
-        v[i] = vi;
-        const float wi = w[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-        w[i] = wi;
-        if (wbf) wbf[i] = __float2bfloat16(wi);
-    }
+__global__ void __launch_bounds__(MLP_NT) k_adam(float* __restrict__ w, const float* __restrict__ g, float* __restrict__ m,
+                                                 float* __restrict__ v, __nv_bfloat16* __restrict__ wbf, MlpLayout L,
+                                                 float lr, float b1, float b2, float c1, float c2, float eps) {
+    int64_t i, at;
+    if (!mlp_param(L, i, at)) return;
+    const float gi = g[i];
+    const float mi = b1 * m[i] + (1.f - b1) * gi;
+    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
+    m[i] = mi;
+    v[i] = vi;
+    const float wi = w[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    w[i] = wi;
+    if (at >= 0) wbf[at] = __float2bfloat16(wi);
 }
 
 // ------------------------------------------------------------------ features
@@ -498,12 +723,14 @@ struct sgw_mlp {
     int n_in = 0, width = 0, n_out = 0, max_batch = 0, device = 0;
     cudaStream_t stream = nullptr;
     int dims[5] = {0};
-    int64_t woff[4] = {0}, boff[4] = {0}, np = 0;
+    sgw::MlpLayout lay{};
+    int ldx = 0, ldh = 0, ldo = 0;  // padded row lengths of the BF16 matrices with n_in, width, n_out columns
+    int64_t np = 0;
     float* P = nullptr;            // FP32 master parameters: W1, b1, W2, b2, W3, b3, W4, b4
     float* G = nullptr;            // gradients (same layout)
     float* Ma = nullptr;           // Adam first moments
     float* Va = nullptr;           // Adam second moments
-    __nv_bfloat16* Pbf = nullptr;  // BF16 copies (weights used by the GEMMs)
+    __nv_bfloat16* Pbf = nullptr;  // BF16 copies of the weight matrices, rows padded (used by the GEMMs)
     int step = 0;
     __nv_bfloat16 *Xbf = nullptr, *Abf[3] = {nullptr}, *dYbf = nullptr, *dZbf[2] = {nullptr};
     float *Z[3] = {nullptr}, *Y = nullptr, *dY = nullptr, *dZ[2] = {nullptr};
@@ -533,53 +760,91 @@ uint64_t splitmix64(uint64_t& s) {
 
 unsigned grid1(int64_t n) { return (unsigned)std::min<int64_t>((n + 255) / 256, 152 * 16); }
 
-sgw_status mlp_forward(sgw_mlp* m, const float* x, int M) {
-    cudaStream_t st = m->stream;
+constexpr int MAX_LOSS_BLOCKS = 304;       // partial sums of the loss: two blocks to an SM at most
+
+// Rows of 32 or 64 to a tile: 64 reads the weights half as often and pays once its tiles fill the chip.
+bool wide_tiles(int M, int N) { return sgw::gemm_tiles(64, M, N) >= 152; }
+
+void forward_gemm(sgw_mlp* m, const sgw::Gemm& g) {
+    if (wide_tiles(g.M, g.N))
+        sgw::launch_dependent(sgw::k_mlp_forward<64>, dim3((unsigned)sgw::gemm_tiles(64, g.M, g.N)), sgw::G_NT,
+                              sgw::GemmCfg<64>::SMEM, 1, m->stream, g);
+    else
+        sgw::launch_dependent(sgw::k_mlp_forward<32>, dim3((unsigned)sgw::gemm_tiles(32, g.M, g.N)), sgw::G_NT,
+                              sgw::GemmCfg<32>::SMEM, 1, m->stream, g);
+}
+
+// The three hidden layers (their pre-activations kept when `keep`), then `last` for the output.
+sgw_status mlp_forward(sgw_mlp* m, const float* x, int M, bool keep, const sgw::GemmEpi& last) {
     const int H = m->width, I = m->n_in, O = m->n_out;
-    sgw::k_to_bf16<<<grid1((int64_t)M * I), 256, 0, st>>>((int64_t)M * I, x, m->Xbf);
+    const int64_t n = (int64_t)M * I;
+    sgw::k_mlp_input<<<grid1(n), 256, 0, m->stream>>>(n, I, m->ldx, x, m->Xbf);
     const __nv_bfloat16* in = m->Xbf;
-    int K = I;
+    int K = I, ld = m->ldx;
     for (int l = 0; l < 3; ++l) {
-        sgw::GemmEpi ep{sgw::EPI_BIAS_TANH, m->P + m->boff[l], m->Z[l], H, m->Abf[l], nullptr};
-        sgw::gemm(M, H, K, 0, 0, in, K, m->Pbf + m->woff[l], H, ep, st);
+        sgw::GemmEpi ep{};
+        ep.mode = sgw::EPI_BIAS_TANH; ep.bias = m->P + m->lay.boff[l];
+        ep.out = keep ? m->Z[l] : nullptr; ep.ldo = H; ep.out_bf = m->Abf[l]; ep.ldb = m->ldh;
+        forward_gemm(m, sgw::Gemm{M, H, K, in, ld, m->Pbf + m->lay.poff[l], m->lay.ld[l], ep});
         in = m->Abf[l];
         K = H;
+        ld = m->ldh;
     }
-    sgw::GemmEpi ep{sgw::EPI_BIAS, m->P + m->boff[3], m->Y, O, nullptr, nullptr};
-    sgw::gemm(M, O, H, 0, 0, in, H, m->Pbf + m->woff[3], O, ep, st);
+    forward_gemm(m, sgw::Gemm{M, O, H, in, ld, m->Pbf + m->lay.poff[3], m->lay.ld[3], last});
     MCK(cudaGetLastError());
     return SGW_OK;
 }
 
-sgw_status mlp_backward(sgw_mlp* m, const float* t, int M) {
-    cudaStream_t st = m->stream;
+// Loss sum_o w_o (y - t)^2 / (M O) and its gradient.
+sgw_status mlp_gradients(sgw_mlp* m, const float* x, const float* t, int M) {
     const int H = m->width, I = m->n_in, O = m->n_out;
-    const int64_t ny = (int64_t)M * O;
-    sgw::k_loss_grad<<<grid1(ny), 256, 0, st>>>(ny, O, m->Y, t, m->lw, 2.0f / (float)ny, m->dY, m->dYbf, m->loss);
-    sgw::k_loss_sum<<<1, 32, 0, st>>>((int)grid1(ny), m->loss);
-    // layer 4
-    {
-        sgw::GemmEpi ep{sgw::EPI_STORE, nullptr, m->G + m->woff[3], O, nullptr, nullptr};
-        sgw::gemm(H, O, M, 1, 0, m->Abf[2], H, m->dYbf, O, ep, st);
-        sgw::k_colsum<<<(O + 127) / 128, 128, 0, st>>>(M, O, m->dY, m->G + m->boff[3]);
-        sgw::GemmEpi ed{sgw::EPI_DTANH, nullptr, m->dZ[0], H, m->dZbf[0], m->Z[2]};
-        sgw::gemm(M, H, O, 0, 1, m->dYbf, O, m->Pbf + m->woff[3], O, ed, st);
-    }
-    int cur = 0;
-    for (int l = 2; l >= 0; --l) {
-        const __nv_bfloat16* a_in = l > 0 ? m->Abf[l - 1] : m->Xbf;
-        const int K_in = l > 0 ? H : I;
-        sgw::GemmEpi ep{sgw::EPI_STORE, nullptr, m->G + m->woff[l], H, nullptr, nullptr};
-        sgw::gemm(K_in, H, M, 1, 0, a_in, K_in, m->dZbf[cur], H, ep, st);
-        sgw::k_colsum<<<(H + 127) / 128, 128, 0, st>>>(M, H, m->dZ[cur], m->G + m->boff[l]);
+    sgw::GemmEpi le{};
+    le.mode = sgw::EPI_LOSS; le.bias = m->P + m->lay.boff[3]; le.out = m->dY; le.ldo = O;
+    le.out_bf = m->dYbf; le.ldb = m->ldo; le.aux = t; le.w = m->lw; le.scale = 2.0f / (float)((int64_t)M * O);
+    le.y = m->Y;
+    sgw_status s = mlp_forward(m, x, M, true, le);
+    if (s) return s;
+    const float* dz = m->dY;
+    const __nv_bfloat16* dzbf = m->dYbf;
+    int N = O, ldz = m->ldo;
+    for (int l = 3; l >= 0; --l) {
+        const int K_in = l > 0 ? H : I, to = l & 1;
+        sgw::Backward b{};
+        sgw::GemmEpi ew{};
+        ew.mode = sgw::EPI_STORE; ew.out = m->G + m->lay.woff[l]; ew.ldo = N;
+        b.w = sgw::Gemm{K_in, N, M, l > 0 ? m->Abf[l - 1] : m->Xbf, l > 0 ? m->ldh : m->ldx, dzbf, ldz, ew};
+        b.splits = 1;
         if (l > 0) {
-            sgw::GemmEpi ed{sgw::EPI_DTANH, nullptr, m->dZ[1 - cur], H, m->dZbf[1 - cur], m->Z[l - 1]};
-            sgw::gemm(M, H, H, 0, 1, m->dZbf[cur], H, m->Pbf + m->woff[l], H, ed, st);
-            cur = 1 - cur;
+            sgw::GemmEpi ed{};
+            ed.mode = sgw::EPI_DTANH; ed.out = m->dZ[to]; ed.ldo = H; ed.out_bf = m->dZbf[to]; ed.ldb = m->ldh;
+            ed.aux = m->Z[l - 1];
+            b.d = sgw::Gemm{M, H, N, dzbf, ldz, m->Pbf + m->lay.poff[l], m->lay.ld[l], ed};
         }
+        b.d_tiles = l > 0 ? sgw::gemm_tiles(32, M, H) : 0;
+        while (b.splits < 8 && N >= 2 * b.splits * 3 * sgw::GK && b.d_tiles * b.splits * 2 <= 152) b.splits *= 2;
+        b.w_tiles = sgw::gemm_tiles(32, K_in, N);
+        b.db_blocks = (N + 31) / 32;
+        b.dz = dz; b.db = m->G + m->lay.boff[l]; b.ldz = N;
+        const int64_t ny = (int64_t)M * O;
+        b.loss = sgw::Loss{ny, O, (int)std::min<int64_t>((ny + sgw::G_NT - 1) / sgw::G_NT, MAX_LOSS_BLOCKS), m->Y, t, m->lw, m->loss};
+        b.loss_blocks = l == 3 ? b.loss.blocks : 0;
+        b.loss_sums = l == 2;
+        int64_t blocks = b.d_tiles * b.splits + b.w_tiles + b.db_blocks + b.loss_blocks + b.loss_sums;
+        blocks = (blocks + b.splits - 1) / b.splits * b.splits;
+        sgw::launch_dependent(sgw::k_mlp_backward, dim3((unsigned)blocks), sgw::G_NT, sgw::GemmCfg<32>::SMEM,
+                              (unsigned)b.splits, m->stream, b);
+        dz = m->dZ[to]; dzbf = m->dZbf[to];
+        N = H; ldz = m->ldh;
     }
     MCK(cudaGetLastError());
     return SGW_OK;
+}
+
+int pad8(int n) { return (n + 7) / 8 * 8; }
+
+template <class K>
+bool gemm_attributes(K kern, int smem) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess;
 }
 
 sgw_status mlp_check(sgw_mlp* m, int M) {
@@ -603,23 +868,33 @@ sgw_status sgw_mlp_create(sgw_mlp** out, int n_in, int width, int n_out, int max
     m->n_in = n_in; m->width = width; m->n_out = n_out; m->max_batch = max_batch;
     m->device = device; m->stream = (cudaStream_t)stream;
     const int d[5] = {n_in, width, width, width, n_out};
-    int64_t off = 0;
+    int64_t off = 0, bf = 0;
     for (int l = 0; l < 4; ++l) {
-        m->woff[l] = off; off += (int64_t)d[l] * d[l + 1];
-        m->boff[l] = off; off += d[l + 1];
+        m->lay.woff[l] = off; off += (int64_t)d[l] * d[l + 1];
+        m->lay.boff[l] = off; off += d[l + 1];
+        m->lay.cols[l] = d[l + 1];
+        m->lay.ld[l] = pad8(d[l + 1]);
+        m->lay.rows[l] = d[l];
+        m->lay.chunks[l] = (d[l + 1] + sgw::MLP_NT - 1) / sgw::MLP_NT;
+        m->lay.first[l + 1] = m->lay.first[l] + ((int64_t)d[l] + 1) * m->lay.chunks[l];
+        m->lay.poff[l] = bf; bf += (int64_t)d[l] * m->lay.ld[l];
     }
+    m->ldx = pad8(n_in); m->ldh = pad8(width); m->ldo = pad8(n_out);
     for (int l = 0; l < 5; ++l) m->dims[l] = d[l];
     m->np = off;
     const size_t B = max_batch;
-    bool ok = cudaMalloc(&m->P, 4 * off) == cudaSuccess && cudaMalloc(&m->G, 4 * off) == cudaSuccess &&
-              cudaMalloc(&m->Ma, 4 * off) == cudaSuccess && cudaMalloc(&m->Va, 4 * off) == cudaSuccess &&
-              cudaMalloc(&m->Pbf, 2 * off) == cudaSuccess && cudaMalloc(&m->Xbf, 2 * B * n_in) == cudaSuccess &&
-              cudaMalloc(&m->Y, 4 * B * n_out) == cudaSuccess && cudaMalloc(&m->dY, 4 * B * n_out) == cudaSuccess &&
-              cudaMalloc(&m->dYbf, 2 * B * n_out) == cudaSuccess && cudaMalloc(&m->loss, sizeof(double) * (1 + 152 * 16)) == cudaSuccess;
-    for (int l = 0; l < 3 && ok; ++l)
-        ok = cudaMalloc(&m->Abf[l], 2 * B * width) == cudaSuccess && cudaMalloc(&m->Z[l], 4 * B * width) == cudaSuccess;
-    for (int l = 0; l < 2 && ok; ++l)
-        ok = cudaMalloc(&m->dZ[l], 4 * B * width) == cudaSuccess && cudaMalloc(&m->dZbf[l], 2 * B * width) == cudaSuccess;
+    // the BF16 matrices are zeroed: what pads their rows is never written again
+    auto get = [](auto** p, size_t bytes) { return cudaMalloc(p, bytes) == cudaSuccess; };
+    auto get_bf = [&](__nv_bfloat16** p, int64_t el) { return get(p, 2 * el) && cudaMemset(*p, 0, 2 * el) == cudaSuccess; };
+    bool ok = get(&m->P, 4 * off) && get(&m->G, 4 * off) && get(&m->Ma, 4 * off) && get(&m->Va, 4 * off) &&
+              get_bf(&m->Pbf, bf) && get_bf(&m->Xbf, B * m->ldx) && get(&m->Y, 4 * B * n_out) &&
+              get(&m->dY, 4 * B * n_out) && get_bf(&m->dYbf, B * m->ldo) &&
+              get(&m->loss, sizeof(double) * (1 + MAX_LOSS_BLOCKS));
+    for (int l = 0; l < 3 && ok; ++l) ok = get_bf(&m->Abf[l], B * m->ldh) && get(&m->Z[l], 4 * B * width);
+    for (int l = 0; l < 2 && ok; ++l) ok = get(&m->dZ[l], 4 * B * width) && get_bf(&m->dZbf[l], B * m->ldh);
+    ok = ok && gemm_attributes(sgw::k_mlp_forward<32>, sgw::GemmCfg<32>::SMEM) &&
+         gemm_attributes(sgw::k_mlp_forward<64>, sgw::GemmCfg<64>::SMEM) &&
+         gemm_attributes(sgw::k_mlp_backward, sgw::GemmCfg<32>::SMEM);
     if (!ok) {
         cudaGetLastError();
         sgw_mlp_destroy(m);
@@ -632,7 +907,7 @@ sgw_status sgw_mlp_create(sgw_mlp** out, int n_in, int width, int n_out, int max
         const double a = 1.0 / std::sqrt((double)d[l]);
         for (int64_t i = 0; i < (int64_t)d[l] * d[l + 1]; ++i) {
             const double u = (double)(splitmix64(s) >> 11) * (1.0 / 9007199254740992.0);
-            h[m->woff[l] + i] = (float)(a * (2.0 * u - 1.0));
+            h[m->lay.woff[l] + i] = (float)(a * (2.0 * u - 1.0));
         }
     }
     sgw_status st = sgw_mlp_set_params(m, h.data(), off);
@@ -666,7 +941,7 @@ sgw_status sgw_mlp_set_params(sgw_mlp* m, const float* params_host, int64_t n) {
     MCK(cudaMemset(m->Ma, 0, 4 * n));
     MCK(cudaMemset(m->Va, 0, 4 * n));
     m->step = 0;
-    sgw::k_to_bf16<<<grid1(n), 256, 0, m->stream>>>(n, m->P, m->Pbf);
+    sgw::k_mlp_weights<<<(unsigned)m->lay.first[4], sgw::MLP_NT, 0, m->stream>>>(m->P, m->Pbf, m->lay);
     MCK(cudaGetLastError());
     MCK(cudaStreamSynchronize(m->stream));
     return SGW_OK;
@@ -697,8 +972,12 @@ sgw_status sgw_mlp_forward(sgw_mlp* m, const float* x_dev, int M, float* y_dev) 
     sgw_status s = mlp_check(m, M);
     if (s) return s;
     if (!x_dev || !y_dev) return mfail(m, SGW_EINVAL, "null pointers");
-    if ((s = mlp_forward(m, x_dev, M))) return s;
-    MCK(cudaMemcpyAsync(y_dev, m->Y, sizeof(float) * (size_t)M * m->n_out, cudaMemcpyDeviceToDevice, m->stream));
+    // a y that floats can't be stored to goes by way of Y and a copy
+    const bool direct = reinterpret_cast<uintptr_t>(y_dev) % alignof(float) == 0;
+    sgw::GemmEpi ep{};
+    ep.mode = sgw::EPI_BIAS; ep.bias = m->P + m->lay.boff[3]; ep.out = direct ? y_dev : m->Y; ep.ldo = m->n_out;
+    if ((s = mlp_forward(m, x_dev, M, false, ep))) return s;
+    if (!direct) MCK(cudaMemcpyAsync(y_dev, m->Y, sizeof(float) * (size_t)M * m->n_out, cudaMemcpyDeviceToDevice, m->stream));
     return SGW_OK;
 }
 
@@ -707,8 +986,7 @@ sgw_status sgw_mlp_gradients(sgw_mlp* m, const float* x_dev, const float* t_dev,
     sgw_status s = mlp_check(m, M);
     if (s) return s;
     if (!x_dev || !t_dev) return mfail(m, SGW_EINVAL, "null pointers");
-    if ((s = mlp_forward(m, x_dev, M))) return s;
-    if ((s = mlp_backward(m, t_dev, M))) return s;
+    if ((s = mlp_gradients(m, x_dev, t_dev, M))) return s;
     if (loss_host) {
         double l;
         MCK(cudaMemcpyAsync(&l, m->loss, 8, cudaMemcpyDeviceToHost, m->stream));
@@ -728,8 +1006,8 @@ sgw_status sgw_mlp_adam_step(sgw_mlp* m, float lr) {
     m->step += 1;
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.f - (float)std::pow(0.9, m->step), c2 = 1.f - (float)std::pow(0.999, m->step);
-    sgw::k_adam<<<grid1(m->np), 256, 0, m->stream>>>(m->np, m->P, m->G, m->Ma, m->Va, m->Pbf, lr, b1, b2, c1, c2,
-                                                     1e-8f);
+    sgw::k_adam<<<(unsigned)m->lay.first[4], sgw::MLP_NT, 0, m->stream>>>(m->P, m->G, m->Ma, m->Va, m->Pbf, m->lay, lr, b1,
+                                                                          b2, c1, c2, 1e-8f);
     MCK(cudaGetLastError());
     return SGW_OK;
 }

@@ -19,6 +19,7 @@
 // 288^3 x 16 (1963 KB atoms) 8.9 -> 6.0 ms.
 #include <algorithm>
 
+#include "dependent_launch.cuh"
 #include "grid_common.cuh"
 #include "kb_unit.cuh"
 #include "reg_dft.cuh"
@@ -36,18 +37,10 @@ __device__ __forceinline__ void sep_cp_wait() {
     asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
 }
 
-// The kernels of a term are launched with programmatic stream serialisation: a kernel's blocks may start
-// while the last ones of the kernel before it run, and what they do before dependents_wait() overlaps
-// that kernel's end and the launch.  dependents_wait() returns when the kernel before has completed
-// and its stores are visible; since every kernel waits before it lets the next one start
-// (dependents_launch), everything older has completed too.  So before the wait a kernel may read
-// what the kernel directly before it does not write; what that one does write is loaded by the
-// ld*_written forms.  The next kernel is let in late (after the pointwise
-// part, or at the end): its blocks take the first free places, and let in at the start they crowd on
-// the SMs with room to spare, which then finish last (48^3 x 6: 17.5 us per term against 12.8; without
-// the early start 18.5).
-__device__ __forceinline__ void dependents_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void dependents_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// The kernels of a term are launched by launch_dependent.  The next kernel is let in late (after the
+// pointwise part, or at the end): its blocks take the first free places, and let in at the start they
+// crowd on the SMs with room to spare, which then finish last (48^3 x 6: 17.5 us per term against 12.8;
+// without the early start 18.5).
 
 // c m^2 for k = k1 + (N / T) i, m the signed frequency of k
 template <int N, int T>
@@ -617,37 +610,22 @@ cudaError_t sep_init_attributes(int n) {
     return e;
 }
 
-template <class... P, class... A>
-static void launch_dependent(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, kern, P(args)...);
-}
-
 void sep_z(int n, const float2* in, float2* W, int batch, float kscale, const float2* tw, const KbReduceArgs& kr,
            cudaStream_t st) {
     if (batch == 0) return;
     const float c = 0.5f * kscale / (float)n;
     if (n == S2N) {
         const unsigned kb = (unsigned)((kr.n_atoms + SL_NT / 32 - 1) / (SL_NT / 32));
-        launch_dependent(k_sep_lines288<0>, dim3((S2N / SL_TX) * S2N + kb, batch), SL_NT, sep_lines_smem(), st, in, W, c, tw, kr);
+        launch_dependent(k_sep_lines288<0>, dim3((S2N / SL_TX) * S2N + kb, batch), SL_NT, sep_lines_smem(), 1, st, in, W, c, tw, kr);
         return;
     }
     const unsigned kb = (unsigned)((kr.n_atoms + ZS_NT / 32 - 1) / (ZS_NT / 32));
-    SGW_DISPATCH_SEP(n, launch_dependent(k_sep_z<N>, dim3(ZsCfg<N>::BLOCKS + kb, batch), ZS_NT, 0, st, in, W, c, tw, kr));
+    SGW_DISPATCH_SEP(n, launch_dependent(k_sep_z<N>, dim3(ZsCfg<N>::BLOCKS + kb, batch), ZS_NT, 0, 1, st, in, W, c, tw, kr));
 }
 
 void sep_y288(const float2* in, float2* W, int batch, float kscale, const float2* tw, cudaStream_t st) {
     if (batch == 0) return;
-    launch_dependent(k_sep_lines288<1>, dim3((S2N / SL_TX) * S2N, batch), SL_NT, sep_lines_smem(), st, in, W,
+    launch_dependent(k_sep_lines288<1>, dim3((S2N / SL_TX) * S2N, batch), SL_NT, sep_lines_smem(), 1, st, in, W,
                      0.5f * kscale / S2N, tw, KbReduceArgs{});
 }
 
@@ -656,10 +634,10 @@ void sep_step(int n, const StepArgs& a, int batch, float kscale, const float2* t
     const float c = 0.5f * kscale / (float)n;
     const size_t sm = sep_step_smem(n, a.kbc != nullptr ? a.max_plane_slots : 0);
     if (n == S2N) {
-        launch_dependent(k_sep_rows288, dim3(batch, S2N * S2N / SR_R), SR_NT, sm, st, a, c, tw);
+        launch_dependent(k_sep_rows288, dim3(batch, S2N * S2N / SR_R), SR_NT, sm, 1, st, a, c, tw);
         return;
     }
-    SGW_DISPATCH_SEP(n, launch_dependent(k_sep_plane<N>, dim3(N, batch), SpCfg<N>::NT, sm, st, a, c, tw));
+    SGW_DISPATCH_SEP(n, launch_dependent(k_sep_plane<N>, dim3(N, batch), SpCfg<N>::NT, sm, 1, st, a, c, tw));
 }
 
 static size_t split_plane_smem(int n) {
