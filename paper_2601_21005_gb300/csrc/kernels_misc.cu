@@ -227,6 +227,54 @@ void launch_power_update(int ng, const float2* w, float2* v, const double* scal,
 // ------------------------------------------------------------------ Sigma(t) accumulation (Eq. 5)
 // zeta: [n_samples][2] (occ, unocc).  partial[((s*(n_steps+1) + j)*2 + pm) * nblk + blk]:
 // pm = 0: sum phi zeta_unocc u ; pm = 1: sum phi zeta_occ u.
+
+// A sum kept as three floats, s0 + s1 + s2: what rounding s0 loses goes to s1 without loss, what s1 loses
+// to s2.  72 bits to FP64's 53.
+struct Sum3 {
+    float s0 = 0.f, s1 = 0.f, s2 = 0.f;
+    static __device__ __forceinline__ float two_sum(float& s, float x) {     // s + x exactly: the new s and what is returned
+        const float t = __fadd_rn(s, x), z = __fsub_rn(t, s);
+        const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(x, z));
+        s = t;
+        return e;
+    }
+    // adds x (h + l), h + l a product's two halves; m: the largest leading product so far
+    __device__ __forceinline__ void add(float x, float h, float l, float& m) {
+        const float a = __fmul_rn(x, h), b = __fmaf_rn(x, h, -a);
+        m = fmaxf(m, fabsf(a));
+        const float e = two_sum(s0, a);
+        const float e1 = two_sum(s1, b), e2 = two_sum(s1, __fmul_rn(x, l)), e3 = two_sum(s1, e);
+        s2 = __fadd_rn(s2, __fadd_rn(__fadd_rn(e1, e2), e3));
+    }
+    __device__ __forceinline__ void add(const Sum3& o) {
+        const float e = two_sum(s0, o.s0), e1 = two_sum(s1, o.s1), e2 = two_sum(s1, e);
+        s2 = __fadd_rn(s2, __fadd_rn(o.s2, __fadd_rn(e1, e2)));
+    }
+    __device__ __forceinline__ double value() const { return (double)s0 + ((double)s1 + (double)s2); }
+};
+
+// f zeta u summed over this thread's points (complex products, no conjugation) in T
+template <typename T>
+__device__ __forceinline__ void sigma_points(int64_t ng, const float2* zu, const float2* zo, const float* phi,
+                                             const float2* uj, T (&a)[4]) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < ng; i += (int64_t)gridDim.x * blockDim.x) {
+        const float f = phi[i];
+        const float2 uu = uj[i];
+        const float2 p = zu[i], m = zo[i];
+        const T ur = (T)uu.x * f, ui = (T)uu.y * f;
+        a[0] += (T)p.x * ur - (T)p.y * ui;
+        a[1] += (T)p.x * ui + (T)p.y * ur;
+        a[2] += (T)m.x * ur - (T)m.y * ui;
+        a[3] += (T)m.x * ui + (T)m.y * ur;
+    }
+}
+
+// T = double: the FP64 units do one or two operations a clock and SM, and the 17 that a point takes and
+// those of the block's sums made this 58 us at 64^3 x 4 (0.45 TB/s).  Threads and warps sum instead as
+// Sum3 on the FP32 units, 280 operations a point, with less rounding than FP64's: 20 us.  The
+// halves of the products are exact while they are normal numbers, so a block whose largest product lies
+// outside 2^-90 .. 2^100 (their errors would be above 2^-56 of it), or whose sums are not numbers, does
+// its points again in FP64.
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_sigma_accum(int64_t ng, const float2* __restrict__ zeta, const float* __restrict__ phi, const float2* __restrict__ u,
@@ -236,22 +284,67 @@ k_sigma_accum(int64_t ng, const float2* __restrict__ zeta, const float* __restri
     const float2* zo = zeta + (size_t)(2 * s) * ng;
     const float2* zu = zeta + (size_t)(2 * s + 1) * ng;
     const float2* uj = u + (size_t)s * u_ss + (size_t)j * ng;
+    const size_t base = ((size_t)s * (n_steps + 1) + j) * 2;
     T a[4] = {0, 0, 0, 0};
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < ng; i += (int64_t)gridDim.x * blockDim.x) {
-        const float f = phi[i];
-        const float2 uu = uj[i];
-        const float2 p = zu[i], m = zo[i];
-        // f * zeta * u  (complex product, no conjugation)
-        const T ur = (T)uu.x * f, ui = (T)uu.y * f;
-        a[0] += (T)p.x * ur - (T)p.y * ui;
-        a[1] += (T)p.x * ui + (T)p.y * ur;
-        a[2] += (T)m.x * ur - (T)m.y * ui;
-        a[3] += (T)m.x * ui + (T)m.y * ur;
+    if constexpr (sizeof(T) == 8) {
+        __shared__ double w[8][4];
+        __shared__ float wbig[8];
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        Sum3 q[4];
+        float big = 0.f;
+        for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < ng; i += (int64_t)gridDim.x * blockDim.x) {
+            const float f = phi[i];
+            const float2 uu = uj[i];
+            const float2 p = zu[i], m = zo[i];
+            const float rh = __fmul_rn(uu.x, f), rl = __fmaf_rn(uu.x, f, -rh);
+            const float ih = __fmul_rn(uu.y, f), il = __fmaf_rn(uu.y, f, -ih);
+            q[0].add(p.x, rh, rl, big); q[0].add(-p.y, ih, il, big);
+            q[1].add(p.x, ih, il, big); q[1].add(p.y, rh, rl, big);
+            q[2].add(m.x, rh, rl, big); q[2].add(-m.y, ih, il, big);
+            q[3].add(m.x, ih, il, big); q[3].add(m.y, rh, rl, big);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            big = fmaxf(big, __shfl_xor_sync(0xffffffffu, big, o));
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                Sum3 x;
+                x.s0 = __shfl_down_sync(0xffffffffu, q[k].s0, o);
+                x.s1 = __shfl_down_sync(0xffffffffu, q[k].s1, o);
+                x.s2 = __shfl_down_sync(0xffffffffu, q[k].s2, o);
+                q[k].add(x);
+            }
+        }
+        if (lane == 0) {
+            bool finite = true;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                w[warp][k] = q[k].value();
+                finite = finite && fabsf(q[k].s0) <= 0x1p120f;
+            }
+            wbig[warp] = finite ? big : __int_as_float(0x7f800000);
+        }
+        __syncthreads();
+        big = 0.f;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) big = fmaxf(big, wbig[i]);
+        if (big >= 0x1p-90f && big <= 0x1p100f) {
+            if (threadIdx.x < 2) {
+                double re = 0, im = 0;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    re += w[i][2 * threadIdx.x];
+                    im += w[i][2 * threadIdx.x + 1];
+                }
+                partial[(base + threadIdx.x) * gridDim.x + blockIdx.x] = make_double2(re, im);
+            }
+            return;
+        }
     }
+    sigma_points<T>(ng, zu, zo, phi, uj, a);
     if constexpr (sizeof(T) == 8) block_sum<4>(a, sh);
     else block_sumf<4>(a, sh);
     if (threadIdx.x == 0) {
-        const size_t base = ((size_t)s * (n_steps + 1) + j) * 2;
         partial[(base + 0) * gridDim.x + blockIdx.x] = make_double2((double)a[0], (double)a[1]);
         partial[(base + 1) * gridDim.x + blockIdx.x] = make_double2((double)a[2], (double)a[3]);
     }
@@ -383,43 +476,43 @@ void launch_sigma_accum_xi(const float2* zeta, const float* phi, const float2* U
 }
 
 // sigma[s][n + j] = dV S+ ; sigma[s][n - j] = -dV S- ; sigma[s][n] = (dV S+ - dV S-)/2 at j = 0.
-// The cross-block sums run in the accumulation precision (fp64 flag).
-__global__ void k_sigma_reduce(const double2* __restrict__ partial, int n_samples, int n_steps, int nblk, double dV,
-                               int fp64, double2* __restrict__ sigma) {
-    const int total = n_samples * (n_steps + 1);
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
-        const int s = t / (n_steps + 1), j = t % (n_steps + 1);
-        double2 r[2];
-        for (int pm = 0; pm < 2; ++pm) {
-            const double2* p = partial + ((size_t)t * 2 + pm) * nblk;
-            if (fp64) {
-                double x = 0, y = 0;
-                for (int b = 0; b < nblk; ++b) { x += p[b].x; y += p[b].y; }
-                r[pm] = make_double2(x, y);
-            } else {
-                float x = 0, y = 0;
-                for (int b = 0; b < nblk; ++b) { x += (float)p[b].x; y += (float)p[b].y; }
-                r[pm] = make_double2(x, y);
-            }
-        }
-        double2* row = sigma + (size_t)s * (2 * n_steps + 1);
-        const double2 sp = make_double2(dV * r[0].x, dV * r[0].y);
-        const double2 sm = make_double2(-dV * r[1].x, -dV * r[1].y);
-        if (j == 0) {
-            row[n_steps] = make_double2(0.5 * (sp.x + sm.x), 0.5 * (sp.y + sm.y));
-        } else {
-            row[n_steps + j] = sp;
-            row[n_steps - j] = sm;
-        }
+// The cross-block sums run in the accumulation precision, one warp to a time (one thread to a time waited
+// for 128 loads in turn: 37 us at 13 times, now 5).
+constexpr int SR_RED_NT = 128;
+template <typename T>
+__global__ void __launch_bounds__(SR_RED_NT)
+k_sigma_reduce(const double2* __restrict__ partial, int n_samples, int n_steps, int nblk, double dV,
+               double2* __restrict__ sigma) {
+    const int t = (int)((blockIdx.x * (int64_t)SR_RED_NT + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (t >= n_samples * (n_steps + 1)) return;
+    const int s = t / (n_steps + 1), j = t % (n_steps + 1);
+    T r[4] = {0, 0, 0, 0};
+    for (int b = lane; b < nblk; b += 32) {
+        const double2 p = partial[(size_t)t * 2 * nblk + b], m = partial[((size_t)t * 2 + 1) * nblk + b];
+        r[0] += (T)p.x; r[1] += (T)p.y; r[2] += (T)m.x; r[3] += (T)m.y;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        for (int o = 16; o > 0; o >>= 1) r[k] += __shfl_xor_sync(0xffffffffu, r[k], o);
+    if (lane != 0) return;
+    double2* row = sigma + (size_t)s * (2 * n_steps + 1);
+    const double2 sp = make_double2(dV * r[0], dV * r[1]);
+    const double2 sm = make_double2(-dV * r[2], -dV * r[3]);
+    if (j == 0) {
+        row[n_steps] = make_double2(0.5 * (sp.x + sm.x), 0.5 * (sp.y + sm.y));
+    } else {
+        row[n_steps + j] = sp;
+        row[n_steps - j] = sm;
     }
 }
 
 void launch_sigma_reduce(const double2* partial, int n_samples, int n_steps, int nblk, double dV, int fp64,
                             double* sigma, cudaStream_t st) {
-    const int total = n_samples * (n_steps + 1);
-    const int blocks = (total + 127) / 128;
-    k_sigma_reduce<<<blocks, 128, 0, st>>>(partial, n_samples, n_steps, nblk, dV, fp64,
-                                           reinterpret_cast<double2*>(sigma));
+    const int64_t total = (int64_t)n_samples * (n_steps + 1);
+    const unsigned blocks = (unsigned)((total * 32 + SR_RED_NT - 1) / SR_RED_NT);
+    double2* out = reinterpret_cast<double2*>(sigma);
+    if (fp64) k_sigma_reduce<double><<<blocks, SR_RED_NT, 0, st>>>(partial, n_samples, n_steps, nblk, dV, out);
+    else k_sigma_reduce<float><<<blocks, SR_RED_NT, 0, st>>>(partial, n_samples, n_steps, nblk, dV, out);
 }
 
 // ------------------------------------------------------------------ time ordering
@@ -691,99 +784,129 @@ __global__ void k_qp_damped(const double2* __restrict__ sigma, int n_samples, in
     damped[jj] = make_double2((double)re, (double)im);
 }
 
+// Re Sigma(w) over the times +-dt j, j = j0, j0 + js, ...: a pair has one sine and cosine.
 template <typename T>
 __device__ __forceinline__ T re_sigma_at(const double2* __restrict__ damped, int n_steps, double dt, T w, int j0, int js) {
     T acc = 0;
-    for (int jj = j0; jj <= 2 * n_steps; jj += js) {
-        const T t = (T)(dt * (jj - n_steps));
+    for (int j = j0; j <= n_steps; j += js) {
+        const T t = (T)(dt * j);
         T sn, cs;
         sincos(w * t, &sn, &cs);
-        acc += (T)damped[jj].x * cs - (T)damped[jj].y * sn;
+        const double2 p = damped[n_steps + j], m = damped[n_steps - j];
+        acc += (T)p.x * cs - (T)p.y * sn;
+        if (j > 0) acc += (T)m.x * cs + (T)m.y * sn;
     }
     return acc;
 }
 
-// scan[i] = f(w_i) = w_i - eps - X - Re Sigma(w_i) + vxc, w_i = eps - window + i step
+// scan[i] = f(w_i) = w_i - eps - X - Re Sigma(w_i) + vxc, w_i = eps - window + i step.  Bound by the latency
+// and then the rate of FP64 sines: QP_SCAN_L lanes share a point's times, in blocks of one warp, so that every
+// SM has some (4001 points x 25 times: 31 us with one thread to a point in 32 blocks, now 9.6).
+constexpr int QP_SCAN_L = 4, QP_SCAN_P = 32 / QP_SCAN_L;
 template <typename T>
-__global__ void k_qp_scan(const double2* __restrict__ damped, int n_steps, double dt, double eps,
-                          const double* __restrict__ x, int n_samples, double vxc, double window, double step,
-                          int n_scan, double* __restrict__ scan) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_scan) return;
+__global__ void __launch_bounds__(32)
+k_qp_scan(const double2* __restrict__ damped, int n_steps, double dt, double eps, const double* __restrict__ x,
+          int n_samples, double vxc, double window, double step, int n_scan, double* __restrict__ scan) {
+    const int i = blockIdx.x * QP_SCAN_P + threadIdx.x / QP_SCAN_L;
+    const double w = eps - window + step * i;
+    double r = (double)re_sigma_at<T>(damped, n_steps, dt, (T)w, threadIdx.x % QP_SCAN_L, QP_SCAN_L);
+    for (int o = QP_SCAN_L / 2; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+    if (i >= n_scan || threadIdx.x % QP_SCAN_L != 0) return;
     double xm = 0.0;
+#pragma unroll 8
     for (int s = 0; s < n_samples; ++s) xm += x[s];
     xm /= n_samples;
-    const double w = eps - window + step * i;
-    scan[i] = w - eps - xm - (double)re_sigma_at<T>(damped, n_steps, dt, (T)w, 0, 1) + vxc;
+    scan[i] = w - eps - xm - r + vxc;
 }
 
+// Re Sigma(w) by the block: one barrier, the warps' sums in two halves of sh[2 * 8] in turn
+constexpr int QP_NT = 256;
 template <typename T>
-__device__ double block_re_sigma(const double2* damped, int n_steps, double dt, double w, double* sh) {
-    double v[1] = {(double)re_sigma_at<T>(damped, n_steps, dt, (T)w, threadIdx.x, blockDim.x)};
+__device__ __forceinline__ double block_re_sigma(const double2* damped, int n_steps, double dt, double w, double* sh,
+                                                 int& turn) {
+    double v = (double)re_sigma_at<T>(damped, n_steps, dt, (T)w, threadIdx.x, QP_NT);
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    double* h = sh + (turn ^= QP_NT / 32);
+    if ((threadIdx.x & 31) == 0) h[threadIdx.x >> 5] = v;
     __syncthreads();
-    block_sum<1>(v, sh);
-    __syncthreads();
-    if (threadIdx.x == 0) sh[64] = v[0];
-    __syncthreads();
-    const double r = sh[64];
-    __syncthreads();
+    double r = 0.0;
+#pragma unroll
+    for (int i = 0; i < QP_NT / 32; ++i) r += h[i];
     return r;
 }
 
-// Single CTA: bracket nearest eps, bisection to 1e-10, standard error with the Z factor.
-// result = (eps_qp, se, Re Sigma(eps_qp), Z); status[0] = 0 ok, 1 no root.
+// One block: bracket nearest eps, bisection to 1e-10, standard error with the Z factor.  It is a chain of
+// some 30 sums over the times, so what counts is the latency of each: the bracket is searched by all
+// threads (one thread walking the 4001 points of the default scan took most of 1417 us at 25 times;
+// now 93 us in all), a sum has one barrier, and the samples of the standard error go to the warps.
+// result = (eps_qp, se, Re Sigma(eps_qp), Z); all NaN: no root.
 template <typename T>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(QP_NT)
 k_qp_solve(const double2* __restrict__ sigma, const double* __restrict__ x, const double2* __restrict__ damped,
            int n_samples, int n_steps, double dt, double gamma, double eps, double vxc, double window, double step,
            const double* __restrict__ scan, int n_scan, double* __restrict__ result) {
-    __shared__ double sh[96];
-    __shared__ int best;
-    __shared__ double xm_s;
+    constexpr int NW = QP_NT / 32;
+    __shared__ double sh[2 * NW], bds[NW], xm_s;
+    __shared__ int bis[NW];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         double xs = 0;
+#pragma unroll 8
         for (int s = 0; s < n_samples; ++s) xs += x[s];
         xm_s = xs / n_samples;
-        // bracket whose midpoint is nearest eps (first on ties)
-        int bi = -1;
-        double bd = 1e300;
-        for (int i = 0; i + 1 < n_scan; ++i) {
-            const double a = scan[i], b = scan[i + 1];
-            const int sa = (a > 0) - (a < 0), sb = (b > 0) - (b < 0);
-            if (sa * sb <= 0) {
-                const double mid = 0.5 * ((eps - window + step * i) + (eps - window + step * (i + 1)));
-                const double d = fabs(mid - eps);
-                if (d < bd) { bd = d; bi = i; }
-            }
-        }
-        best = bi;
     }
+    // bracket whose midpoint is nearest eps (first on ties)
+    int best = -1;
+    double bd = 1e300;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < n_scan - 1; i += QP_NT) {
+        const double a = scan[i], b = scan[i + 1];
+        const int sa = (a > 0) - (a < 0), sb = (b > 0) - (b < 0);
+        if (sa * sb <= 0) {
+            const double mid = 0.5 * ((eps - window + step * i) + (eps - window + step * (i + 1)));
+            const double d = fabs(mid - eps);
+            if (d < bd) { bd = d; best = i; }
+        }
+    }
+    auto nearer = [&](double d, int i) {
+        if (i >= 0 && (best < 0 || d < bd || (d == bd && i < best))) { bd = d; best = i; }
+    };
+    for (int o = 16; o > 0; o >>= 1) {
+        const double d = __shfl_xor_sync(0xffffffffu, bd, o);
+        const int i = __shfl_xor_sync(0xffffffffu, best, o);
+        nearer(d, i);
+    }
+    if (lane == 0) { bds[warp] = bd; bis[warp] = best; }
     __syncthreads();
+    best = -1;
+    bd = 1e300;
+    for (int i = 0; i < NW; ++i) nearer(bds[i], bis[i]);
     if (best < 0) {
         if (threadIdx.x == 0) { result[0] = nan(""); result[1] = nan(""); result[2] = nan(""); result[3] = nan(""); }
         return;
     }
     const double xm = xm_s;
+    int turn = 0;
     double a = eps - window + step * best, b = eps - window + step * (best + 1);
     double fa = scan[best];
     while (b - a > 1e-10) {
         const double c = 0.5 * (a + b);
-        const double fc = c - eps - xm - block_re_sigma<T>(damped, n_steps, dt, c, sh) + vxc;
+        const double fc = c - eps - xm - block_re_sigma<T>(damped, n_steps, dt, c, sh, turn) + vxc;
         const int sfc = (fc > 0) - (fc < 0), sfa = (fa > 0) - (fa < 0);
         if (sfc == sfa && fc != 0.0) { a = c; fa = fc; }
         else b = c;
     }
     const double e = 0.5 * (a + b);
-    const double rs = block_re_sigma<T>(damped, n_steps, dt, e, sh);
+    const double rs = block_re_sigma<T>(damped, n_steps, dt, e, sh, turn);
     const double d = 1e-4;
-    const double slope = (block_re_sigma<T>(damped, n_steps, dt, e + d, sh) -
-                          block_re_sigma<T>(damped, n_steps, dt, e - d, sh)) / (2 * d);
+    const double slope = (block_re_sigma<T>(damped, n_steps, dt, e + d, sh, turn) -
+                          block_re_sigma<T>(damped, n_steps, dt, e - d, sh, turn)) / (2 * d);
     const double z = 1.0 / (1.0 - slope);
     // per-sample X_i + Re Sigma_i(e): Sigma_i(t) damped the same way (no sample mean)
     double m1 = 0, m2 = 0;
-    for (int s = 0; s < n_samples; ++s) {
+    for (int s = warp; s < n_samples; s += NW) {
         double acc = 0;
-        for (int jj = threadIdx.x; jj <= 2 * n_steps; jj += blockDim.x) {
+        for (int jj = lane; jj <= 2 * n_steps; jj += 32) {
             const int j = jj - n_steps;
             const T t = (T)(dt * j);
             const T w = (jj == 0 || jj == 2 * n_steps) ? (T)0.5 : (T)1.0;
@@ -793,17 +916,17 @@ k_qp_solve(const double2* __restrict__ sigma, const double* __restrict__ x, cons
             sincos((T)e * t, &sn, &cs);
             acc += (double)(((T)v.x * cs - (T)v.y * sn) * damp);
         }
-        double vv[1] = {acc};
-        __syncthreads();
-        block_sum<1>(vv, sh);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            const double per = x[s] + vv[0];
-            m1 += per;
-            m2 += per * per;
-        }
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        const double per = x[s] + acc;
+        m1 += per;
+        m2 += per * per;
     }
+    __syncthreads();
+    if (lane == 0) { sh[warp] = m1; sh[NW + warp] = m2; }
+    __syncthreads();
     if (threadIdx.x == 0) {
+        m1 = m2 = 0;
+        for (int i = 0; i < NW; ++i) { m1 += sh[i]; m2 += sh[NW + i]; }
         double se = nan("");
         if (n_samples > 1) {
             const double mean = m1 / n_samples;
@@ -826,15 +949,15 @@ void launch_qp(const double* sigma, const double* x, int n_samples, int n_steps,
     const int nt = 2 * n_steps + 1;
     if (fp64) {
         k_qp_damped<double><<<(nt + 127) / 128, 128, 0, st>>>(sg, n_samples, n_steps, dt, gamma, damped);
-        k_qp_scan<double><<<(n_scan + 127) / 128, 128, 0, st>>>(damped, n_steps, dt, eps_ks, x, n_samples, vxc, window,
+        k_qp_scan<double><<<(n_scan + QP_SCAN_P - 1) / QP_SCAN_P, 32, 0, st>>>(damped, n_steps, dt, eps_ks, x, n_samples, vxc, window,
                                                               step, n_scan, scan);
-        k_qp_solve<double><<<1, 256, 0, st>>>(sg, x, damped, n_samples, n_steps, dt, gamma, eps_ks, vxc, window, step,
+        k_qp_solve<double><<<1, QP_NT, 0, st>>>(sg, x, damped, n_samples, n_steps, dt, gamma, eps_ks, vxc, window, step,
                                               scan, n_scan, result);
     } else {
         k_qp_damped<float><<<(nt + 127) / 128, 128, 0, st>>>(sg, n_samples, n_steps, dt, gamma, damped);
-        k_qp_scan<float><<<(n_scan + 127) / 128, 128, 0, st>>>(damped, n_steps, dt, eps_ks, x, n_samples, vxc, window,
+        k_qp_scan<float><<<(n_scan + QP_SCAN_P - 1) / QP_SCAN_P, 32, 0, st>>>(damped, n_steps, dt, eps_ks, x, n_samples, vxc, window,
                                                              step, n_scan, scan);
-        k_qp_solve<float><<<1, 256, 0, st>>>(sg, x, damped, n_samples, n_steps, dt, gamma, eps_ks, vxc, window, step,
+        k_qp_solve<float><<<1, QP_NT, 0, st>>>(sg, x, damped, n_samples, n_steps, dt, gamma, eps_ks, vxc, window, step,
                                              scan, n_scan, result);
     }
 }
