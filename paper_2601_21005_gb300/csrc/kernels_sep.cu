@@ -37,10 +37,13 @@ __device__ __forceinline__ void sep_cp_wait() {
     asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
 }
 
-// The kernels of a term are launched by launch_dependent.  The next kernel is let in late (after the
-// pointwise part, or at the end): its blocks take the first free places, and let in at the start they
-// crowd on the SMs with room to spare, which then finish last (48^3 x 6: 17.5 us per term against 12.8;
-// without the early start 18.5).
+// The kernels of a term are launched by launch_dependent.  The z lines let the planes in at once: those load
+// b and transform their rows and columns beside them, and wait only for the KB coefficients and W
+// (per term, with the launches of a term in order, overlapped at their ends only, and so: 16^3 x 2 8.3, 3.9,
+// 3.3 us; 32^3 x 12 16.5, 9.9, 8.5; 48^3 x 6 18.5, 12.8, 11.7; 64^3 x 8 36.1, 31.0, 29.2; 64^3 x 64 195, 188,
+// 182).
+// The plane pass lets the next term in after the pointwise part: at its start the z lines' blocks, which can
+// do nothing yet, would take the places of planes.
 
 // c m^2 for k = k1 + (N / T) i, m the signed frequency of k
 template <int N, int T>
@@ -130,12 +133,11 @@ __device__ __forceinline__ void sep_pointwise(const StepArgs& a, const VecInfo& 
     else sep_points<N, ROWS, PITCH, NT, U, false, false>(a, inf, off, uoff, sm, bs);
 }
 
-// L2 prefetch of a unit's pointwise operands (one thread), PTS points at offset off
+// L2 prefetch of a unit's pointwise operands but W (one thread), PTS points at offset off
 template <int N, int PTS>
 __device__ __forceinline__ void sep_prefetch(const StepArgs& a, const VecInfo& inf, size_t off, size_t uoff) {
     constexpr size_t NG = (size_t)N * N * N;
     constexpr unsigned CB = PTS * sizeof(float2), VB = PTS * sizeof(float);
-    l2_prefetch(a.W + off, CB);
     if (a.psi != nullptr) l2_prefetch(a.psi + off, CB);
     if (a.b2 != nullptr) l2_prefetch(a.b2 + off, CB);
     l2_prefetch(a.vpot + (size_t)inf.vrow * NG + uoff, VB);
@@ -176,6 +178,7 @@ k_sep_z(const float2* in, float2* W, float c, const float2* __restrict__ tw, KbR
     const int t = lane / CPW;
     const size_t off = (size_t)b * N * N * N + (blockIdx.x * (ZS_NT / 32) + warp) * CPW + lane % CPW + (size_t)t * N * N;
     dependents_wait();                       // the step before wrote `in`
+    dependents_launch();
     float2 v[P];
 #pragma unroll
     for (int a = 0; a < P; ++a) v[a] = ld2_written(in + off + (size_t)(T * a) * N * N);
@@ -186,13 +189,11 @@ k_sep_z(const float2* in, float2* W, float c, const float2* __restrict__ tw, KbR
 }
 
 // ------------------------------------------------------------------ planes, n <= 128
-// A block per plane.  Up to 64^2 the plane of b is copied to shared memory beside the plane of H b: the
-// KB apply runs onto zeros while the copy is on its way, then T_x of the rows and T_y of the columns
-// are added and the pointwise part follows, all reading b from shared memory (three blocks of 256
-// threads per SM at 64^2: 5.66 TB/s without KB, 0.83 of the copy rate; with one plane in shared memory
-// and b read again from L2 for the columns and the pointwise part it was 5.0).  Two planes of 96^2 or
+// A block per plane.  Up to 64^2 the plane of b is copied to shared memory and T_x of the rows and T_y of
+// the columns go to a second plane; the KB apply and the pointwise part follow on that one (64^3 x 36: 111 us
+// per term with the KB apply first, which then waits for the z lines, and 106 so).  Two planes of 96^2 or
 // 128^2 leave room for one block at best: there the rows are transformed in place, the KB apply comes
-// after them, and b is read again from L2 (96^3 x 8: 91 us, against 102 with the KB apply first).
+// before the columns, and b is read again from L2 (96^3 x 8: 91 us, against 102 with the KB apply first).
 // Four lanes per line: two lanes hold twice the points and half the warps, and the same pass took
 // 195 us instead of 169 at 64^3 x 64.  The operands of the pointwise part are asked into L2 once the
 // plane has landed, and read evict-first: asked at the block's start they were evicted before use (a
@@ -241,46 +242,36 @@ __global__ void __launch_bounds__(SpCfg<N>::NT, (SpCfg<N>::MINB)) k_sep_plane(St
     }
     for (int i = threadIdx.x; i < N; i += NT) tws[i] = __ldg(tw + i);
     const float2* kc = a.kbc != nullptr ? a.kbc + (size_t)b * a.total_slots * 4 : nullptr;
-    if (kc != nullptr) {
-        if constexpr (KEEP) {
-            // V_NL b onto zeros while the plane is on its way
-            kb_apply_unit<N, PITCH, NT, 2>(a, kh, kcs, sm, [&] {
-                float4* s4 = reinterpret_cast<float4*>(sm);
-                for (int i = threadIdx.x; i < N * PITCH / 2; i += NT) s4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-                dependents_wait();           // the z lines wrote W and the coefficients
-                kb_stage_coeffs<NT>(kh, kc, kcs);
-            });
-        }
-    } else if (KEEP) {
-        dependents_wait();
-    }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
     if (KEEP && threadIdx.x == 0) sep_prefetch<N, N * N>(a, inf, off, uoff);
     const int l = warp * CPW + lane % CPW, t = lane / CPW;
     const auto f = [&](int k1, int i) { return axis_factor<N, T>(k1, i, c); };
     {
-        // T_x b of row l: added to V_NL b, or in place (a lane writes the points it has read)
+        // T_x b of row l, in place in the one-plane form (a lane writes the points it has read)
         float2 v[P];
         float2* row = sm + l * PITCH + t;
         const float2* src = (KEEP ? bs : sm) + l * PITCH + t;
 #pragma unroll
         for (int i = 0; i < P; ++i) v[i] = src[T * i];
         line_op<N, T>(v, lane, tws, f);
-        if (KEEP && kc != nullptr) {
-#pragma unroll
-            for (int i = 0; i < P; ++i) v[i] = cadd(v[i], row[T * i]);
-        }
 #pragma unroll
         for (int i = 0; i < P; ++i) row[T * i] = v[i];
     }
-    if constexpr (!KEEP) {
-        dependents_wait();
-        if (threadIdx.x == 0) sep_prefetch<N, N * N>(a, inf, off, uoff);
+    const auto staged = [&] {
+        dependents_wait();                   // the z lines wrote W and the coefficients
+        if (threadIdx.x == 0) {
+            if (!KEEP) sep_prefetch<N, N * N>(a, inf, off, uoff);
+            l2_prefetch(a.W + off, N * N * sizeof(float2));
+        }
         if (kc != nullptr) kb_stage_coeffs<NT>(kh, kc, kcs);
+    };
+    if (!KEEP && kc != nullptr) {
+        kb_apply_unit<N, PITCH, NT, 2>(a, kh, kcs, sm, staged);
+    } else {
+        if (!KEEP) staged();
+        __syncthreads();
     }
-    if (!KEEP && kc != nullptr) kb_apply_unit<N, PITCH, NT, 2>(a, kh, kcs, sm, [] {});
-    else __syncthreads();
     {
         // + T_y b of column l
         float2 v[P];
@@ -296,6 +287,10 @@ __global__ void __launch_bounds__(SpCfg<N>::NT, (SpCfg<N>::MINB)) k_sep_plane(St
         line_op<N, T>(v, lane, tws, f);
 #pragma unroll
         for (int i = 0; i < P; ++i) col[T * i * PITCH] = cadd(col[T * i * PITCH], v[i]);
+    }
+    if constexpr (KEEP) {
+        if (kc != nullptr) kb_apply_unit<N, PITCH, NT, 2>(a, kh, kcs, sm, staged);
+        else staged();
     }
     KbSlots ks;
     if (a.kbp != nullptr) ks = kb_project_begin<NT>(a, kh);
@@ -539,7 +534,10 @@ __global__ void __launch_bounds__(SR_NT, 4) k_sep_rows288(StepArgs a, float c, c
 #pragma unroll
     for (int i = 0; i < S2P; ++i) row[t + S2T * i] = v[i];
     dependents_wait();                       // the y lines wrote W, and the coefficients are older
-    if (threadIdx.x == 0) sep_prefetch<S2N, SR_R * S2N>(a, inf, off, uoff);
+    if (threadIdx.x == 0) {
+        sep_prefetch<S2N, SR_R * S2N>(a, inf, off, uoff);
+        l2_prefetch(a.W + off, SR_R * S2N * sizeof(float2));
+    }
     if (kc != nullptr) kb_stage_coeffs<SR_NT>(kh, kc, kcs);
     if (kc != nullptr) kb_apply_unit<S2N, SR_PITCH, SR_NT, 2>(a, kh, kcs, sm, [] {});
     else __syncthreads();
@@ -596,6 +594,11 @@ template <class K> static cudaError_t sep_attr(K kern, int bytes) {
     return e != cudaSuccess ? e : cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 
+template <class K>
+static cudaError_t sep_carveout(K kern) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+}
+
 cudaError_t sep_init_attributes(int n) {
     int dev = 0, optin = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -607,6 +610,11 @@ cudaError_t sep_init_attributes(int n) {
         return sep_attr(k_sep_rows288, optin);
     }
     SGW_DISPATCH_SEP(n, e = sep_attr(k_sep_plane<N>, optin));
+    // Small planes' blocks start beside the z lines' (see spread_smem), and an SM that changes between the two
+    // kernels' shares of shared memory and L1 has to run dry first: both take the largest share (48^3 x 6:
+    // 11.8 -> 11.4 us per term; above, where the z lines use L1, it cost 1 to 4 %).
+    if (e == cudaSuccess && n <= 48)
+        SGW_DISPATCH_SEP(n, e = sep_carveout(k_sep_plane<N>); if (e == cudaSuccess) e = sep_carveout(k_sep_z<N>));
     return e;
 }
 
@@ -629,6 +637,17 @@ void sep_y288(const float2* in, float2* W, int batch, float kscale, const float2
                      0.5f * kscale / S2N, tw, KbReduceArgs{});
 }
 
+// Shared memory for a block of the plane pass.  The z lines let the planes in early, and blocks take the
+// first free places: without a limit up to MINB crowd on the SMs that run few z lines, and these finish
+// last.  A grid of less than MINB blocks to an SM asks for so much that only an even share fits (32^3 x 12:
+// 13.2 us per term without, 9.2 with; 48^3 x 6: 17.7, 11.8).
+template <int N>
+static size_t spread_smem(size_t sm, long blocks) {
+    const long per = (blocks + 151) / 152;
+    if (per >= SpCfg<N>::MINB) return sm;
+    return std::max(sm, ((size_t)228 * 1024 / (per + 1) - 1024 + 255) / 128 * 128);
+}
+
 void sep_step(int n, const StepArgs& a, int batch, float kscale, const float2* tw, cudaStream_t st) {
     if (batch == 0) return;
     const float c = 0.5f * kscale / (float)n;
@@ -637,7 +656,8 @@ void sep_step(int n, const StepArgs& a, int batch, float kscale, const float2* t
         launch_dependent(k_sep_rows288, dim3(batch, S2N * S2N / SR_R), SR_NT, sm, 1, st, a, c, tw);
         return;
     }
-    SGW_DISPATCH_SEP(n, launch_dependent(k_sep_plane<N>, dim3(N, batch), SpCfg<N>::NT, sm, 1, st, a, c, tw));
+    SGW_DISPATCH_SEP(n, launch_dependent(k_sep_plane<N>, dim3(N, batch), SpCfg<N>::NT, spread_smem<N>(sm, (long)N * batch), 1, st,
+                                         a, c, tw));
 }
 
 static size_t split_plane_smem(int n) {
