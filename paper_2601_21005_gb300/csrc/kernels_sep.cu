@@ -309,9 +309,10 @@ __global__ void __launch_bounds__(SpCfg<N>::NT, (SpCfg<N>::MINB)) k_sep_plane(St
 // computed once per block.  Along an axis the line gains IDFT((e^{-i T_a dt} - 1) DFT(line)): the rounding
 // of the transforms and of the factor, which is the same in every step, is then in proportion to what
 // the step changes (three factors of modulus 1 +- 2^-25 would add up over the steps).
-// Measured, ten steps of 27 vectors at 64^3 with KB: 1.40 -> 1.00 ms, of which the two passes 0.66 (at two
+// Measured, ten steps of 27 vectors at 64^3 with KB: 1.40 -> 0.94 ms, of which the two passes 0.66 (at two
 // blocks of 256 threads per SM; three or four spill the second line operation: 1.03, 1.04); the error
-// against 64 bits went from 1.3e-6 to 3.7e-7.
+// against 64 bits went from 1.3e-6 to 3.7e-7.  Started early as the kernels of a term are, the two passes
+// were slower (1.01 ms): they have little to do before they wait.
 template <int N>
 __device__ __forceinline__ void axis_phases(float2* ph, float ks, float dt, int nt) {
     for (int m = threadIdx.x; m <= N / 2; m += nt) {
@@ -461,10 +462,12 @@ __device__ __forceinline__ void line288(float2 (&v)[S2P], int t, float c, const 
 }
 
 // z lines (AXIS 0: W = T_z b) and y lines (AXIS 1: W += T_y b) of tiles of 16 x-columns; AXIS 0's
-// blocks past the columns' reduce the KB partials.
+// blocks past the columns' reduce the KB partials.  Five blocks to an SM at 64 registers (8 vectors, z and y:
+// 645 and 876 us, 4.76 and 5.24 TB/s; four at 80 registers 681 and 911; tiles of 8 columns, which are two
+// sectors to a row, 828 and 1284, of 32 columns 707 and 893).
 constexpr int SL_TX = 16, SL_NT = SL_TX * S2T;
 template <int AXIS>
-__global__ void __launch_bounds__(SL_NT, 4)
+__global__ void __launch_bounds__(SL_NT, 5)
 k_sep_lines288(const float2* in, float2* W, float c, const float2* __restrict__ tw, KbReduceArgs kr) {
     constexpr int NXT = S2N / SL_TX, BLOCKS = NXT * S2N;
     constexpr size_t NN = (size_t)S2N * S2N, ST = AXIS == 0 ? NN : S2N;
