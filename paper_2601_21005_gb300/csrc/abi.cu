@@ -398,8 +398,11 @@ sgw_status run_series(sgw_ctx* ctx, const std::vector<Step>& plan, const float2*
         sgw::launch_plane_fwd(n, psi_in, ctx->W, batch, ctx->tw, st);
         CKL();
     }
+    // A plan of one step (degree 1) reads b_1 = psi, and a tangent vector its partner's as well: in place it
+    // would read what the partner's blocks of the same launch have overwritten.
+    float2* const last = dvpot != nullptr && plan.size() == 1 && out == psi_in ? ctx->B1 : out;
     auto buf = [&](int id) -> float2* {
-        return id == 0 ? const_cast<float2*>(psi_in) : (id == 1 ? ctx->B1 : (id == 2 ? ctx->B2 : out));
+        return id == 0 ? const_cast<float2*>(psi_in) : (id == 1 ? ctx->B1 : (id == 2 ? ctx->B2 : last));
     };
     for (size_t i = 0; i < plan.size(); ++i) {
         const Step& s = plan[i];
@@ -461,6 +464,7 @@ sgw_status run_series(sgw_ctx* ctx, const std::vector<Step>& plan, const float2*
             }
         }
     }
+    if (last != out) CK(cudaMemcpyAsync(out, last, sizeof(float2) * ctx->ng * batch, cudaMemcpyDeviceToDevice, st));
     return SGW_OK;
 }
 

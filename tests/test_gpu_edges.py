@@ -1,11 +1,12 @@
 """Edge and degenerate cases of the entry points on the GPU: empty batches and sample counts,
-zero time steps, the largest batch a context takes (and one more, refused), a degree-0 filter,
+zero time steps, TDH steps of degree 1 and 2, the largest batch a context takes (and one more, refused), a degree-0 filter,
 dt = 0 propagation (identity for both steppers), zero vectors, and a QP window without a root."""
 import numpy as np
 import pytest
 
 from oracle import chebyshev as cheb
 from oracle import hamiltonian as ham
+from oracle import sgw as osgw
 from paper_2601_21005_gb300 import build, synth
 
 import gpu_common as gc
@@ -119,3 +120,31 @@ def test_qp_window_without_a_root_reports_no_convergence(ctx):
     x = torch.full((3,), 5.0, dtype=torch.float64, device='cuda')
     with pytest.raises(RuntimeError):
         c.qp_energy(sig, x, 3, 10, 0.05, 1.0, -0.2, 0.0, 1.0, 1e-3, 1)
+
+
+@pytest.mark.parametrize('n,ecut', [(32, 0.0), (32, 1e6), (48, 0.0), (48, 1e6)])
+@pytest.mark.parametrize('deg', [1, 2])
+def test_tdh_at_the_lowest_degrees(n, ecut, deg):
+    """A series of one term runs in place and reads psi both as b_1 and, for a tangent vector, through
+    its partner.  Tolerance: that of the TDH parity tests at degree 16, which has more terms to round."""
+    from paper_2601_21005_gb300 import sgw
+    build.build()
+    s = gc.small_cluster(n)
+    g = ham.Grid(s['n'], s['h'])
+    lo, hi = float(s['vloc'].min()) - 2.0, 0.5 * 3 * (np.pi / s['h']) ** 2 + 2.0
+    r = np.random.default_rng(deg)
+    n_s, n_eta, N = 2, 3, 2
+    shape = (n_s, n_eta) + g.shape()
+    eta = (0.05 * (r.normal(size=shape) + 1j * r.normal(size=shape))).astype(np.complex64)
+    src = r.normal(size=(n_s,) + g.shape()).astype(np.float32)
+    c = sgw.Context(n, s['h'], ecut=ecut, max_batch=2 * n_s * n_eta)
+    c.set_potential(gc.to_dev(s['vloc'].ravel(), torch, torch.float32), s['kb_atoms'])
+    c.set_spectrum(lo, hi)
+    uR = torch.empty(n_s, N + 1, g.ng, dtype=torch.float32, device='cuda')
+    c.tdh_response(gc.to_dev(eta.reshape(n_s * n_eta, -1), torch, torch.complex64),
+                   gc.to_dev(src.reshape(n_s, -1), torch, torch.float32), n_s, n_eta, N, 0.05, deg, uR)
+    got = uR.cpu().numpy().reshape((n_s, N + 1) + g.shape())
+    prob = osgw.Problem(g, s['vloc'], ham.KB(s['kb_atoms']), lo, hi, 0, 0, np.zeros(g.shape()))
+    for si in range(n_s):
+        ref = osgw.tdh_response_tangent(prob, eta[si].astype(np.complex128), src[si].astype(np.float64), N, 0.05, deg)
+        assert gc.rel_err(got[si], ref) < 2e-4
