@@ -1375,6 +1375,12 @@ sgw_status sgw_propagate(sgw_ctx* ctx, void* psi_dev, int batch, int n_steps, do
     });
 }
 
+// Colours of the split KB factor: none without projectors, nor where sgw_set_potential refused them (their
+// factors were not built, and the steps leave them out)
+static int split_colours(const sgw_ctx* ctx) {
+    return ctx->kb.n_atoms > 0 && !ctx->acol_off.empty() ? (int)ctx->acol_off.size() - 1 : 0;
+}
+
 // Colours c0, c0 + dir, .. (count of them) of the split KB factor on a batch; full: e^{-i dt V_a} instead of
 // the half-step's e^{-i (dt/2) V_a}.
 static sgw_status split_kb(sgw_ctx* ctx, float2* psi, int batch, const float2* F, int c0, int count, int dir, bool full) {
@@ -1438,7 +1444,7 @@ static sgw_status split_phases(sgw_ctx* ctx, const float* vpot, int rows, double
 // One split-operator step of a batch in place; split_factors(ctx, dt) and split_phases must have run.
 static sgw_status split_step_batch(sgw_ctx* ctx, float2* psi, int batch, const float* vpot, const float* dvpot,
                                    double dt, const float2* F) {
-    const int nc = ctx->kb.n_atoms > 0 ? (int)ctx->acol_off.size() - 1 : 0;
+    const int nc = split_colours(ctx);
     sgw_status r;
     if ((r = split_kb(ctx, psi, batch, F, 0, nc, 1, false))) return r;
     if ((r = split_core(ctx, psi, batch, vpot, dvpot, dt))) return r;
@@ -1468,7 +1474,7 @@ sgw_status sgw_propagate_split(sgw_ctx* ctx, void* psi_dev, int batch, int n_ste
     return graphed(ctx, key, [&]() -> sgw_status {
         // between two steps the last factor of the one and the first of the next are the same colour's:
         // one full factor instead of two halves
-        const int nc = ctx->kb.n_atoms > 0 ? (int)ctx->acol_off.size() - 1 : 0;
+        const int nc = split_colours(ctx);
         sgw_status r;
         if ((r = split_phases(ctx, ctx->vloc, 1, dt))) return r;
         if ((r = split_kb(ctx, psi, batch, F, 0, nc, 1, false))) return r;

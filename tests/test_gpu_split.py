@@ -134,3 +134,27 @@ def test_split_pipeline_tracks_the_chebyshev_pipeline():
     assert np.array_equal(a[1], b[1])                       # the exchange does not propagate
     assert np.linalg.norm(a[0] - b[0]) < 2e-2 * np.linalg.norm(a[0])
     assert abs(a[2] - b[2]) * 27.2114 < 0.05
+
+
+def test_split_after_refused_projectors():
+    """An atom with dependent projectors is refused; a context that goes on steps without a KB factor,
+    in a call of several steps (whose colours are merged) as in calls of one."""
+    build.build()
+    s = synth.wells()
+    one = synth.kb_projectors(s['n'], s['h'], (4.0, 4.0, 4.0), 0.9, (1.2,), 0)
+    bad = (one[0], np.concatenate([one[1], 0 * one[1]]), np.array([0.5, 0.5]))
+    v = gc.to_dev(s['vloc'].ravel(), torch, torch.float32)
+    x = torch.randn(2, s['n'] ** 3, dtype=torch.complex64, device='cuda')
+    outs = []
+    for refused in (True, False):
+        c = _ctx(s, 2)
+        if refused:
+            with pytest.raises(RuntimeError):
+                c.set_potential(v, [bad])
+        a, b = x.clone(), x.clone()
+        c.propagate_split(a, 2, 0.05)
+        for _ in range(2):
+            c.propagate_split(b, 1, 0.05)
+        assert torch.equal(a, b)
+        outs.append(a)
+    assert torch.equal(outs[0], outs[1])
