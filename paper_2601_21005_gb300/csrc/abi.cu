@@ -44,8 +44,14 @@ struct sgw_ctx {
     static constexpr int kWorkSlots = 11;
     void* work[kWorkSlots] = {nullptr};
     size_t work_sz[kWorkSlots] = {0};
-    // time-ordering matrices of the last few n_steps used (at most 8; 0.7 MB at 400 steps)
-    std::vector<std::pair<int, float2*>> to_tabs;
+    // time-ordering matrices by n_steps, least recently used first (0.7 MB at 400 steps): those that a stream
+    // capture has recorded stay, its graph holds the address; of the others at most 8 are kept
+    struct ToTab {
+        int n_steps;
+        float2* G;
+        bool captured;
+    };
+    std::vector<ToTab> to_tabs;
     std::vector<sgw::VecInfo> info_host;
     // instrumentation: launch counter and CUDA-event timing per kernel kind
     int64_t launches = 0;
@@ -621,7 +627,7 @@ void sgw_destroy(sgw_ctx* ctx) {
     void* ptrs[] = {ctx->tw, ctx->vloc, ctx->W, ctx->B1, ctx->B2, ctx->info, ctx->scal};
     for (void* p : ptrs)
         if (p) cudaFree(p);
-    for (auto& t : ctx->to_tabs) cudaFree(t.second);
+    for (auto& t : ctx->to_tabs) cudaFree(t.G);
     for (int i = 0; i < sgw_ctx::kWorkSlots; ++i)
         if (ctx->work[i]) cudaFree(ctx->work[i]);
     for (int k = 0; k < SGW_PROF_KINDS; ++k)
@@ -1644,19 +1650,23 @@ sgw_status sgw_time_order_points(sgw_ctx* ctx, const float* uR_dev, void* u_dev,
     int M = 4;                                    // the smallest power of two >= 4 (n_steps + 1)
     while (M < 4 * (n_steps + 1)) M *= 2;
     if (M > 4096) return fail(ctx, SGW_EINVAL, "n_steps too large for the time-ordering FFT (M <= 4096)");
-    const float2* g = nullptr;
-    for (auto& t : ctx->to_tabs)
-        if (t.first == n_steps) g = t.second;
-    if (!g) {
+    // (the query fails where the stream may not be used just now; the launch below says so)
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(ctx->stream, &cap) != cudaSuccess) cudaGetLastError();
+    const bool capturing = cap != cudaStreamCaptureStatusNone;
+    auto& tabs = ctx->to_tabs;
+    const auto same = [&](const sgw_ctx::ToTab& t) { return t.n_steps == n_steps; };
+    auto tab = std::find_if(tabs.begin(), tabs.end(), same);
+    if (tab == tabs.end()) {
         // built by a kernel, once: during a stream capture it would be recorded, not run
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        CK(cudaStreamIsCapturing(ctx->stream, &cap));
-        if (cap != cudaStreamCaptureStatusNone)
+        if (capturing)
             return fail(ctx, SGW_ESTATE, "the first time ordering of this n_steps must come before any stream capture");
-        if (ctx->to_tabs.size() >= 8) {
+        const auto free_to_go = [](const sgw_ctx::ToTab& t) { return !t.captured; };
+        if (std::count_if(tabs.begin(), tabs.end(), free_to_go) >= 8) {
+            auto old = std::find_if(tabs.begin(), tabs.end(), free_to_go);
             CK(cudaStreamSynchronize(ctx->stream));
-            cudaFree(ctx->to_tabs.front().second);
-            ctx->to_tabs.erase(ctx->to_tabs.begin());
+            cudaFree(old->G);
+            tabs.erase(old);
         }
         float2* t = nullptr;
         if (cudaMalloc(&t, sgw::time_order_matrix_bytes(n_steps)) != cudaSuccess) {
@@ -1670,9 +1680,12 @@ sgw_status sgw_time_order_points(sgw_ctx* ctx, const float* uR_dev, void* u_dev,
             cudaFree(t);
             return fail(ctx, SGW_ECUDA, std::string("time-ordering matrix: ") + cudaGetErrorString(e));
         }
-        ctx->to_tabs.push_back({n_steps, t});
-        g = t;
+        tabs.push_back({n_steps, t, false});
+    } else {
+        std::rotate(tab, tab + 1, tabs.end());                              // the most recently used is the last
     }
+    tabs.back().captured |= capturing;
+    const float2* g = tabs.back().G;
     {
         Launch L(ctx, SGW_PROF_TIME_ORDER, 1, (double)n_points * n_samples * (n_steps + 1) * 12.0);
         sgw::launch_time_order(n_points, uR_dev, (float2*)u_dev, n_samples, n_steps, g, ctx->stream);

@@ -61,3 +61,31 @@ def test_many_step_counts_in_one_context():
             if first is not None:
                 assert torch.equal(u, first)
             first = u
+
+
+def test_captured_orderings_outlive_other_step_counts():
+    """A caller's graph keeps the matrix it was captured with, whatever the context orders afterwards; and the
+    step count in constant use stays among those kept."""
+    build.build()
+    from paper_2601_21005_gb300 import sgw
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        c = sgw.Context(16, 0.5, stream=st.cuda_stream)
+        x = torch.randn(1, 61, 70, device='cuda')
+        order = lambda n, u: c.time_order_points(x[:, :n + 1].contiguous(), u, 1, n, 70)
+        out = lambda n: torch.empty(1, n + 1, 70, dtype=torch.complex64, device='cuda')
+        xs = x[:, :21].contiguous()
+        u, want = out(20), out(20)
+        c.time_order_points(xs, want, 1, 20, 70)
+        st.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=st):
+            c.time_order_points(xs, u, 1, 20, 70)
+        junk = []
+        for n in range(21, 45):
+            order(n, out(n))
+            order(50, out(50))
+            junk.append(torch.full((1 << 18,), float('nan'), device='cuda'))    # would land in memory given back
+        g.replay()
+    st.synchronize()
+    assert torch.equal(u, want)
