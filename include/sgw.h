@@ -294,6 +294,8 @@ sgw_status sgw_tdh_response(sgw_ctx* ctx, const void* eta_dev, const float* sour
  * and sample: zero-pad to M (the smallest power of two >= 4 (n_steps + 1), M <= 4096),
  * FFT with e^{+i omega t}, replace the negative-frequency half by its complex conjugate,
  * inverse FFT.  uR_dev: [n_samples][n_steps+1][N_g] float; u_dev: same shape, c64.
+ * The first call for each M prepares tables and may not come in a stream capture (SGW_ESTATE); the tables
+ * that a capture has recorded live until sgw_destroy.
  */
 sgw_status sgw_time_order(sgw_ctx* ctx, const float* uR_dev, void* u_dev, int n_samples,
                           int n_steps);

@@ -44,12 +44,14 @@ struct sgw_ctx {
     static constexpr int kWorkSlots = 11;
     void* work[kWorkSlots] = {nullptr};
     size_t work_sz[kWorkSlots] = {0};
-    // time-ordering matrices by n_steps, least recently used first (0.7 MB at 400 steps): those that a stream
-    // capture has recorded stay, its graph holds the address; of the others at most 8 are kept
+    // time-ordering matrices by n_steps, least recently used first (0.7 MB at 400 steps).  Those that stay:
+    // the first of a transform length, with the length's longest in the same allocation, which serves the
+    // other step counts of the length in a stream capture; and what a capture has recorded, since its graph
+    // holds the address.  Of the others at most 8 are kept.
     struct ToTab {
         int n_steps;
         float2* G;
-        bool captured;
+        bool stays, owned;     // owned: G is the start of an allocation
     };
     std::vector<ToTab> to_tabs;
     std::vector<sgw::VecInfo> info_host;
@@ -627,7 +629,8 @@ void sgw_destroy(sgw_ctx* ctx) {
     void* ptrs[] = {ctx->tw, ctx->vloc, ctx->W, ctx->B1, ctx->B2, ctx->info, ctx->scal};
     for (void* p : ptrs)
         if (p) cudaFree(p);
-    for (auto& t : ctx->to_tabs) cudaFree(t.G);
+    for (auto& t : ctx->to_tabs)
+        if (t.owned) cudaFree(t.G);
     for (int i = 0; i < sgw_ctx::kWorkSlots; ++i)
         if (ctx->work[i]) cudaFree(ctx->work[i]);
     for (int k = 0; k < SGW_PROF_KINDS; ++k)
@@ -1655,40 +1658,51 @@ sgw_status sgw_time_order_points(sgw_ctx* ctx, const float* uR_dev, void* u_dev,
     if (cudaStreamIsCapturing(ctx->stream, &cap) != cudaSuccess) cudaGetLastError();
     const bool capturing = cap != cudaStreamCaptureStatusNone;
     auto& tabs = ctx->to_tabs;
-    const auto same = [&](const sgw_ctx::ToTab& t) { return t.n_steps == n_steps; };
-    auto tab = std::find_if(tabs.begin(), tabs.end(), same);
+    const auto find = [&](int steps) {
+        return std::find_if(tabs.begin(), tabs.end(), [&](const sgw_ctx::ToTab& t) { return t.n_steps == steps; });
+    };
+    const int longest = M / 4 - 1;                // the most steps of this transform length
+    auto tab = find(n_steps);
+    if (tab == tabs.end() && capturing) {
+        // a kernel would be recorded here, not run: the length's longest matrix holds this one's values
+        tab = find(longest);
+        if (tab == tabs.end())
+            return fail(ctx, SGW_ESTATE, "the first time ordering of a transform length must come before any stream capture");
+    }
     if (tab == tabs.end()) {
-        // built by a kernel, once: during a stream capture it would be recorded, not run
-        if (capturing)
-            return fail(ctx, SGW_ESTATE, "the first time ordering of this n_steps must come before any stream capture");
-        const auto free_to_go = [](const sgw_ctx::ToTab& t) { return !t.captured; };
-        if (std::count_if(tabs.begin(), tabs.end(), free_to_go) >= 8) {
-            auto old = std::find_if(tabs.begin(), tabs.end(), free_to_go);
+        // built by a kernel, once; the first of its length brings the longest with it
+        const bool first = find(longest) == tabs.end(), two = first && n_steps != longest;
+        const auto may_go = [](const sgw_ctx::ToTab& t) { return !t.stays; };
+        if (!first && std::count_if(tabs.begin(), tabs.end(), may_go) >= 8) {
+            auto old = std::find_if(tabs.begin(), tabs.end(), may_go);
             CK(cudaStreamSynchronize(ctx->stream));
             cudaFree(old->G);
             tabs.erase(old);
         }
+        const size_t own = sgw::time_order_matrix_bytes(n_steps), both = own + (two ? sgw::time_order_matrix_bytes(longest) : 0);
         float2* t = nullptr;
-        if (cudaMalloc(&t, sgw::time_order_matrix_bytes(n_steps)) != cudaSuccess) {
+        if (cudaMalloc(&t, both) != cudaSuccess) {
             cudaGetLastError();
             return fail(ctx, SGW_ENOMEM, "time-ordering matrix allocation failed");
         }
         sgw::launch_time_order_matrix(n_steps, M, t, ctx->stream);
+        if (two) sgw::launch_time_order_matrix(longest, M, t + own / sizeof(float2), ctx->stream);
         cudaError_t e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);       // later calls may use another stream
         if (e != cudaSuccess) {
             cudaFree(t);
             return fail(ctx, SGW_ECUDA, std::string("time-ordering matrix: ") + cudaGetErrorString(e));
         }
-        tabs.push_back({n_steps, t, false});
+        if (two) tabs.push_back({longest, t + own / sizeof(float2), true, false});
+        tabs.push_back({n_steps, t, first, true});
     } else {
         std::rotate(tab, tab + 1, tabs.end());                              // the most recently used is the last
     }
-    tabs.back().captured |= capturing;
-    const float2* g = tabs.back().G;
+    tabs.back().stays |= capturing;
+    const sgw_ctx::ToTab g = tabs.back();
     {
         Launch L(ctx, SGW_PROF_TIME_ORDER, 1, (double)n_points * n_samples * (n_steps + 1) * 12.0);
-        sgw::launch_time_order(n_points, uR_dev, (float2*)u_dev, n_samples, n_steps, g, ctx->stream);
+        sgw::launch_time_order(n_points, uR_dev, (float2*)u_dev, n_samples, n_steps, g.G, g.n_steps, ctx->stream);
         CKL();
     }
     return SGW_OK;

@@ -531,6 +531,7 @@ void launch_sigma_reduce(const double2* partial, int n_samples, int n_steps, int
 // transforms' (8e-8 against 1.0e-7 relative at 400 steps; one long sum would have 2.2e-7).
 constexpr int TO_BK = 16, TO_BN = 128, TO_NT = 128, TO_STAGES = 3;
 constexpr int TO_R = TO_NT / 32;     // a warp's lanes take 4 points each and share their rows
+constexpr int TO_TM = 13;            // rows of a warp at most
 
 // Row tiles: TO_R warps of TM rows each, held in TMP = TM rounded up to even slots.
 struct ToShape {
@@ -538,10 +539,10 @@ struct ToShape {
 };
 static ToShape to_shape(int n_steps) {
     const int rows = n_steps / 2 + 1;                 // the even times; the odd ones are at most as many
-    const int cand[] = {1, 2, 4, 7, 10, 13};
+    const int cand[] = {1, 2, 4, 7, 10, TO_TM};
     ToShape s;
-    s.tiles = (rows + TO_R * 13 - 1) / (TO_R * 13);
-    s.tm = 13;
+    s.tiles = (rows + TO_R * TO_TM - 1) / (TO_R * TO_TM);
+    s.tm = TO_TM;
     for (int c : cand)
         if (TO_R * c * s.tiles >= rows) {
             s.tm = c;
@@ -559,19 +560,25 @@ size_t time_order_matrix_bytes(int n_steps) {
 
 // G in the order the product reads it, each value twice (the packed multiply-adds take pairs):
 // [parity of t][tile][k][warp][slot], row t = 2 (TO_R TM tile + TM warp + slot) + parity, column
-// j = 2 k + 1 - parity; 0 outside the times.
-__global__ void k_time_order_matrix(int n_steps, int M, int tm, int tmp, int tiles, int kpad, float2* __restrict__ G) {
-    const int total = 2 * tiles * kpad * TO_R * tmp;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-        const int slot = i % tmp, row = (i / tmp) % TO_R, k = (i / (TO_R * tmp)) % kpad,
-                  tile = (i / (TO_R * tmp * kpad)) % tiles, par = i / (TO_R * tmp * kpad * tiles);
-        const int t = 2 * (TO_R * tm * tile + tm * row + slot) + par, j = 2 * k + 1 - par;
-        double v = 0.0;
-        if (slot < tm && t <= n_steps && j <= n_steps) {
-            const double a = (double)(j + t) / M, b = (double)(j - t) / M;      // j + t and j - t are odd
-            v = (cospi(a) / sinpi(a) + cospi(b) / sinpi(b)) / M;
-        }
-        G[i] = make_float2((float)v, (float)v);
+// j = 2 k + 1 - parity; 0 outside the times.  A block has TO_BK columns of a tile, whose j + t and j - t
+// take as many values as it has rows and columns: so many FP64 cotangents it computes.
+__global__ void __launch_bounds__(TO_NT)
+k_time_order_matrix(int n_steps, int M, int tm, int tmp, int tiles, int kpad, float2* __restrict__ G) {
+    __shared__ double cs[TO_R * TO_TM + TO_BK], cd[TO_R * TO_TM + TO_BK];        // cot(pi (j + t) / M), cot(pi (j - t) / M)
+    const int nk = kpad / TO_BK, k0 = (int)(blockIdx.x % nk) * TO_BK, tile = (int)(blockIdx.x / nk) % tiles;
+    const int par = (int)(blockIdx.x / nk) / tiles, R = TO_R * tm, r0 = R * tile;
+    for (int i = threadIdx.x; i < R + TO_BK - 1; i += TO_NT) {
+        const double a = (double)(2 * (k0 + r0 + i) + 1) / M, b = (double)(2 * (k0 - r0 + i - (R - 1)) + 1 - 2 * par) / M;
+        cs[i] = cospi(a) / sinpi(a);                                             // j + t and j - t are odd
+        cd[i] = cospi(b) / sinpi(b);
+    }
+    __syncthreads();
+    float2* g = G + (((size_t)par * tiles + tile) * kpad + k0) * TO_R * tmp;
+    for (int i = threadIdx.x; i < TO_BK * TO_R * tmp; i += TO_NT) {
+        const int slot = i % tmp, r = tm * (i / tmp % TO_R) + slot, q = i / (TO_R * tmp);
+        const bool in = slot < tm && 2 * (r0 + r) + par <= n_steps && 2 * (k0 + q) + 1 - par <= n_steps;
+        const float v = in ? (float)((cs[q + r] + cd[q - r + R - 1]) / M) : 0.f;
+        g[i] = make_float2(v, v);
     }
 }
 
@@ -602,8 +609,8 @@ __device__ __forceinline__ float2 unpack2(f32x2 a) {
 // VEC: rows of u^R and u start on 16 bytes (the number of points is a multiple of 4).
 template <int TM, bool VEC>
 __global__ void __launch_bounds__(TO_NT, 3)
-k_time_order(int64_t np, const float* __restrict__ uR, float2* __restrict__ u, int n_steps, int tiles, int kpad, int ch,
-             const float2* __restrict__ G) {
+k_time_order(int64_t np, const float* __restrict__ uR, float2* __restrict__ u, int n_steps, int tiles, int nk, int ch,
+             const float2* __restrict__ G, int g_tiles, int g_kpad) {
     constexpr int TMP = (TM + 1) & ~1, AM = TO_R * TMP;
     extern __shared__ __align__(16) unsigned char to_sm[];
     float2* As = reinterpret_cast<float2*>(to_sm);                                  // [stage][k][TO_R][TMP]
@@ -613,8 +620,7 @@ k_time_order(int64_t np, const float* __restrict__ uR, float2* __restrict__ u, i
     const int64_t p0 = (int64_t)(blockIdx.x / (2 * tiles)) * TO_BN;
     const size_t row0 = (size_t)blockIdx.y * (n_steps + 1);
     const int tn = threadIdx.x % 32, tm = threadIdx.x / 32;
-    const float2* A = G + ((size_t)par * tiles + tile) * kpad * AM;
-    const int nk = kpad / TO_BK;
+    const float2* A = G + ((size_t)par * g_tiles + tile) * g_kpad * AM;
     const auto load = [&](int s, int kt) {
         const float2* a = A + (size_t)kt * TO_BK * AM;
         float2* as = As + s * TO_BK * AM;
@@ -689,36 +695,38 @@ k_time_order(int64_t np, const float* __restrict__ uR, float2* __restrict__ u, i
     }
 }
 
-template <int TM> static void tlaunch(int64_t np, const float* uR, float2* u, int n_samples, int n_steps, const ToShape& s,
+template <int TM> static void tlaunch(int64_t np, const float* uR, float2* u, int n_samples, int n_steps, const ToShape& g,
                                       const float2* G, cudaStream_t st) {
     constexpr int TMP = (TM + 1) & ~1;
     const size_t smem = TO_STAGES * TO_BK * (sizeof(float2) * TO_R * TMP + sizeof(float) * TO_BN);
-    const dim3 grid((unsigned)(2 * s.tiles * ((np + TO_BN - 1) / TO_BN)), n_samples);
+    const int rows = n_steps / 2 + 1, tiles = (rows + TO_R * TM - 1) / (TO_R * TM), nk = (rows + TO_BK - 1) / TO_BK;
+    const dim3 grid((unsigned)(2 * tiles * ((np + TO_BN - 1) / TO_BN)), n_samples);
     // chunks of 16 terms, 32 above 256: as many chunks as terms in one, about
-    const int ch = s.kpad > 256 ? 2 * TO_BK : TO_BK;
+    const int ch = nk * TO_BK > 256 ? 2 * TO_BK : TO_BK;
     if (np % 4 == 0) {
         cudaFuncSetAttribute(k_time_order<TM, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_time_order<TM, true><<<grid, TO_NT, smem, st>>>(np, uR, u, n_steps, s.tiles, s.kpad, ch, G);
+        k_time_order<TM, true><<<grid, TO_NT, smem, st>>>(np, uR, u, n_steps, tiles, nk, ch, G, g.tiles, g.kpad);
     } else {
         cudaFuncSetAttribute(k_time_order<TM, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_time_order<TM, false><<<grid, TO_NT, smem, st>>>(np, uR, u, n_steps, s.tiles, s.kpad, ch, G);
+        k_time_order<TM, false><<<grid, TO_NT, smem, st>>>(np, uR, u, n_steps, tiles, nk, ch, G, g.tiles, g.kpad);
     }
 }
 
 void launch_time_order_matrix(int n_steps, int M, float2* G, cudaStream_t st) {
     const ToShape s = to_shape(n_steps);
-    k_time_order_matrix<<<152, 256, 0, st>>>(n_steps, M, s.tm, to_tmp(s.tm), s.tiles, s.kpad, G);
+    k_time_order_matrix<<<2 * s.tiles * (s.kpad / TO_BK), TO_NT, 0, st>>>(n_steps, M, s.tm, to_tmp(s.tm), s.tiles, s.kpad, G);
 }
 
-void launch_time_order(int np, const float* uR, float2* u, int n_samples, int n_steps, const float2* G, cudaStream_t st) {
-    const ToShape s = to_shape(n_steps);
+void launch_time_order(int np, const float* uR, float2* u, int n_samples, int n_steps, const float2* G, int g_steps,
+                       cudaStream_t st) {
+    const ToShape s = to_shape(g_steps);
     switch (s.tm) {
         case 1: tlaunch<1>(np, uR, u, n_samples, n_steps, s, G, st); break;
         case 2: tlaunch<2>(np, uR, u, n_samples, n_steps, s, G, st); break;
         case 4: tlaunch<4>(np, uR, u, n_samples, n_steps, s, G, st); break;
         case 7: tlaunch<7>(np, uR, u, n_samples, n_steps, s, G, st); break;
         case 10: tlaunch<10>(np, uR, u, n_samples, n_steps, s, G, st); break;
-        default: tlaunch<13>(np, uR, u, n_samples, n_steps, s, G, st); break;
+        default: tlaunch<TO_TM>(np, uR, u, n_samples, n_steps, s, G, st); break;
     }
 }
 

@@ -233,10 +233,12 @@ void launch_sigma_accum_xi(const float2* zeta, const float* phi, const float2* U
                            float c, int fp64, double2* partial, int nblk, cudaStream_t st);
 void launch_sigma_reduce(const double2* partial, int n_samples, int n_steps, int nblk, double dV, int fp64,
                          double* sigma, cudaStream_t st);
-// time ordering as a product with the matrix of n_steps (transform length M), which the caller keeps
+// time ordering as a product with the matrix G of g_steps >= n_steps (same transform length M), which the
+// caller keeps
 size_t time_order_matrix_bytes(int n_steps);
 void launch_time_order_matrix(int n_steps, int M, float2* G, cudaStream_t st);
-void launch_time_order(int np, const float* uR, float2* u, int n_samples, int n_steps, const float2* G, cudaStream_t st);
+void launch_time_order(int np, const float* uR, float2* u, int n_samples, int n_steps, const float2* G, int g_steps,
+                       cudaStream_t st);
 void launch_sigma_omega(const double* sigma, int n_samples, int n_steps, double dt, double gamma,
                         const double* omega, int n_omega, int fp64, double* out, cudaStream_t st);
 void launch_qp(const double* sigma, const double* x, int n_samples, int n_steps, double dt, double gamma,

@@ -89,3 +89,25 @@ def test_captured_orderings_outlive_other_step_counts():
         g.replay()
     st.synchronize()
     assert torch.equal(u, want)
+
+
+@pytest.mark.parametrize('kept,captured', [(8, 12), (64, 100), (300, 400), (16, 31)])
+def test_step_counts_of_one_length_share_a_capture(kept, captured):
+    """A first ordering of one step count lets a capture record any other of the same padded length
+    (64, 512, 2048, 128 here), with the bits that the step count's own matrix gives."""
+    build.build()
+    from paper_2601_21005_gb300 import sgw
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        c = sgw.Context(16, 0.5, stream=st.cuda_stream)
+        x = torch.randn(1, captured + 1, 70, device='cuda')
+        u = [torch.empty(1, captured + 1, 70, dtype=torch.complex64, device='cuda') for _ in range(2)]
+        c.time_order_points(x[:, :kept + 1].contiguous(), u[0][:, :kept + 1].contiguous(), 1, kept, 70)
+        st.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=st):
+            c.time_order_points(x, u[0], 1, captured, 70)
+        g.replay()
+        c.time_order_points(x, u[1], 1, captured, 70)
+    st.synchronize()
+    assert torch.equal(u[0], u[1])
