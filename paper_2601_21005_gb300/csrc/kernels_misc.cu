@@ -272,9 +272,11 @@ __device__ __forceinline__ void sigma_points(int64_t ng, const float2* zu, const
 // T = double: the FP64 units do one or two operations a clock and SM, and the 17 that a point takes and
 // those of the block's sums made this 58 us at 64^3 x 4 (0.45 TB/s).  Threads and warps sum instead as
 // Sum3 on the FP32 units, 280 operations a point, with less rounding than FP64's: 20 us.  The
-// halves of the products are exact while they are normal numbers, so a block whose largest product lies
-// outside 2^-90 .. 2^100 (their errors would be above 2^-56 of it), or whose sums are not numbers, does
-// its points again in FP64.
+// halves of the products are exact while they are normal numbers: each product may lose 2^-149 where they
+// are not, and |x| 2^-150 with x = zeta, whose factor u phi has halves of its own.  A block has at most 2^18
+// points and a sum two products of each, so the losses stay below 2^-53 of the largest product while that is
+// above 2^-76 and above 2^-77 |x|.  A block where it is not, or is above 2^100, or whose sums are not numbers,
+// does its points again in FP64.
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_sigma_accum(int64_t ng, const float2* __restrict__ zeta, const float* __restrict__ phi, const float2* __restrict__ u,
@@ -288,14 +290,15 @@ k_sigma_accum(int64_t ng, const float2* __restrict__ zeta, const float* __restri
     T a[4] = {0, 0, 0, 0};
     if constexpr (sizeof(T) == 8) {
         __shared__ double w[8][4];
-        __shared__ float wbig[8];
+        __shared__ float wbig[8], wx[8];
         const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
         Sum3 q[4];
-        float big = 0.f;
+        float big = 0.f, xs = 0.f;           // the largest product's and the largest zeta's magnitude
         for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < ng; i += (int64_t)gridDim.x * blockDim.x) {
             const float f = phi[i];
             const float2 uu = uj[i];
             const float2 p = zu[i], m = zo[i];
+            xs = fmaxf(fmaxf(xs, fmaxf(fabsf(p.x), fabsf(p.y))), fmaxf(fabsf(m.x), fabsf(m.y)));
             const float rh = __fmul_rn(uu.x, f), rl = __fmaf_rn(uu.x, f, -rh);
             const float ih = __fmul_rn(uu.y, f), il = __fmaf_rn(uu.y, f, -ih);
             q[0].add(p.x, rh, rl, big); q[0].add(-p.y, ih, il, big);
@@ -306,6 +309,7 @@ k_sigma_accum(int64_t ng, const float2* __restrict__ zeta, const float* __restri
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             big = fmaxf(big, __shfl_xor_sync(0xffffffffu, big, o));
+            xs = fmaxf(xs, __shfl_xor_sync(0xffffffffu, xs, o));
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 Sum3 x;
@@ -323,12 +327,16 @@ k_sigma_accum(int64_t ng, const float2* __restrict__ zeta, const float* __restri
                 finite = finite && fabsf(q[k].s0) <= 0x1p120f;
             }
             wbig[warp] = finite ? big : __int_as_float(0x7f800000);
+            wx[warp] = xs;
         }
         __syncthreads();
-        big = 0.f;
+        big = xs = 0.f;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) big = fmaxf(big, wbig[i]);
-        if (big >= 0x1p-90f && big <= 0x1p100f) {
+        for (int i = 0; i < 8; ++i) {
+            big = fmaxf(big, wbig[i]);
+            xs = fmaxf(xs, wx[i]);
+        }
+        if (big >= 0x1p-76f && big >= 0x1p-77f * xs && big <= 0x1p100f) {
             if (threadIdx.x < 2) {
                 double re = 0, im = 0;
 #pragma unroll

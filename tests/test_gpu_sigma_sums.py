@@ -26,21 +26,24 @@ def _ctx(n, batch):
     return c
 
 
-@pytest.mark.parametrize('n,scale,spread,fp64', [
-    (16, 1.0, 0.0, 1), (64, 1.0, 0.0, 1),
-    (32, 1.0, 12.0, 1),              # magnitudes over 24 decades, as in a cluster's tails
-    (32, 2.0 ** -110, 0.0, 1),       # products below what FP32 halves hold exactly
-    (32, 2.0 ** -100, 6.0, 1),       # some threads on either side of that line
-    (32, 2.0 ** 110, 0.0, 1),        # products beyond FP32
-    (48, 1.0, 4.0, 0),
+@pytest.mark.parametrize('n,scale,spread,fp64,zscale', [
+    (16, 1.0, 0.0, 1, 1.0), (64, 1.0, 0.0, 1, 1.0),
+    (32, 1.0, 12.0, 1, 1.0),              # magnitudes over 24 decades, as in a cluster's tails
+    (32, 2.0 ** -110, 0.0, 1, 1.0),       # products below what FP32 halves hold exactly
+    (32, 2.0 ** -100, 6.0, 1, 1.0),       # some threads on either side of that line
+    (32, 2.0 ** 110, 0.0, 1, 1.0),        # products beyond FP32
+    (48, 1.0, 4.0, 0, 1.0),
+    (32, 2.0 ** -120, 0.0, 1, 2.0 ** 40),     # products well in range, of factors u phi that are not
+    (32, 2.0 ** -130, 0.0, 1, 2.0 ** 60),     # and of subnormal u
+    (32, 2.0 ** -85, 3.0, 1, 2.0 ** 12),      # blocks on either side of the line for zeta
 ])
-def test_sums_against_wide_arithmetic(n, scale, spread, fp64):
+def test_sums_against_wide_arithmetic(n, scale, spread, fp64, zscale):
     ns, steps, ng = 2, 1, n ** 3
     rng = np.random.default_rng(n + int(spread))
     mag = 10.0 ** (spread * (rng.random(ng) - 0.5) * 2)
     phi = (rng.normal(size=ng) * mag).astype(np.float32)
     u = (scale * (rng.normal(size=(ns, steps + 1, ng)) + 1j * rng.normal(size=(ns, steps + 1, ng)))).astype(np.complex64)
-    z = (rng.normal(size=(ns, 2, ng)) + 1j * rng.normal(size=(ns, 2, ng))).astype(np.complex64)
+    z = (zscale * (rng.normal(size=(ns, 2, ng)) + 1j * rng.normal(size=(ns, 2, ng)))).astype(np.complex64)
     sig = torch.empty(ns, 2 * steps + 1, dtype=torch.complex128, device='cuda')
     c = _ctx(n, 2 * ns)
     c.sigma_c(gc.to_dev(z, torch, torch.complex64), gc.to_dev(phi, torch, torch.float32),
