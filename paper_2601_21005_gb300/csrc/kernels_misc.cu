@@ -229,7 +229,7 @@ void launch_power_update(int ng, const float2* w, float2* v, const double* scal,
 // pm = 0: sum phi zeta_unocc u ; pm = 1: sum phi zeta_occ u.
 
 // A sum kept as three floats, s0 + s1 + s2: what rounding s0 loses goes to s1 without loss, what s1 loses
-// to s2.  72 bits to FP64's 53.
+// to s2 (Knuth's two-sum).  72 bits to FP64's 53.
 struct Sum3 {
     float s0 = 0.f, s1 = 0.f, s2 = 0.f;
     static __device__ __forceinline__ float two_sum(float& s, float x) {     // s + x exactly: the new s and what is returned
@@ -240,11 +240,11 @@ struct Sum3 {
     }
     // adds x (h + l), h + l a product's two halves; m: the largest leading product so far
     __device__ __forceinline__ void add(float x, float h, float l, float& m) {
-        const float a = __fmul_rn(x, h), b = __fmaf_rn(x, h, -a);
+        const float a = __fmul_rn(x, h), b = __fmaf_rn(x, h, -a), c = __fmul_rn(x, l), d = __fmaf_rn(x, l, -c);
         m = fmaxf(m, fabsf(a));
         const float e = two_sum(s0, a);
-        const float e1 = two_sum(s1, b), e2 = two_sum(s1, __fmul_rn(x, l)), e3 = two_sum(s1, e);
-        s2 = __fadd_rn(s2, __fadd_rn(__fadd_rn(e1, e2), e3));
+        const float e1 = two_sum(s1, b), e2 = two_sum(s1, c), e3 = two_sum(s1, e);
+        s2 = __fadd_rn(s2, __fadd_rn(__fadd_rn(e1, e2), __fadd_rn(e3, d)));
     }
     __device__ __forceinline__ void add(const Sum3& o) {
         const float e = two_sum(s0, o.s0), e1 = two_sum(s1, o.s1), e2 = two_sum(s1, e);
@@ -271,7 +271,7 @@ __device__ __forceinline__ void sigma_points(int64_t ng, const float2* zu, const
 
 // T = double: the FP64 units do one or two operations a clock and SM, and the 17 that a point takes and
 // those of the block's sums made this 58 us at 64^3 x 4 (0.45 TB/s).  Threads and warps sum instead as
-// Sum3 on the FP32 units, 280 operations a point, with less rounding than FP64's: 20 us.  The
+// Sum3 on the FP32 units, 300 operations a point, with less rounding than FP64's: 20 us.  The
 // halves of the products are exact while they are normal numbers: each product may lose 2^-149 where they
 // are not, and |x| 2^-150 with x = zeta, whose factor u phi has halves of its own.  A block has at most 2^18
 // points and a sum two products of each, so the losses stay below 2^-53 of the largest product while that is

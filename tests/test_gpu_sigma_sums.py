@@ -59,6 +59,32 @@ def test_sums_against_wide_arithmetic(n, scale, spread, fp64, zscale):
         assert abs(complex(got[s]) - complex(want)) <= 64 * eps * float(size)
 
 
+def test_one_point_keeps_fp64_precision():
+    """With one point in the grid a sum is a single complex product of three.  FP64 rounds each part of it four
+    times at most (u phi is exact): 2 * 2^-53 of its terms' magnitudes, and dV and the halving are exact."""
+    n, ns = 16, 64
+    ng = n ** 3
+    rng = np.random.default_rng(7)
+    c = _ctx(n, 2 * ns)
+    for _ in range(8):
+        at = rng.integers(0, ng, ns)
+        z, u = (rng.normal(size=(ns, 2)).astype(np.float32) for _ in range(2))
+        phi = rng.normal(size=ng).astype(np.float32)
+        f = phi[at]
+        zd = np.zeros((ns, 2, ng), np.complex64)
+        ud = np.zeros((ns, 1, ng), np.complex64)
+        zd[np.arange(ns), 1, at] = z[:, 0] + 1j * z[:, 1]
+        ud[np.arange(ns), 0, at] = u[:, 0] + 1j * u[:, 1]
+        sig = torch.empty(ns, 1, dtype=torch.complex128, device='cuda')
+        c.sigma_c(gc.to_dev(zd, torch, torch.complex64), gc.to_dev(phi, torch, torch.float32),
+                  gc.to_dev(ud, torch, torch.complex64), ns, 0, 0.05, 8, sig, 1)
+        got = sig.cpu().numpy()[:, 0]
+        zl, ul, fl = z.astype(np.longdouble), u.astype(np.longdouble), f.astype(np.longdouble)
+        re, im = [zl[:, 0] * fl * ul[:, 0], -zl[:, 1] * fl * ul[:, 1]], [zl[:, 0] * fl * ul[:, 1], zl[:, 1] * fl * ul[:, 0]]
+        for part, (a, b) in ((got.real, re), (got.imag, im)):
+            assert np.all(np.abs(part - (a + b) / 16) <= 2 * 2.0 ** -53 * (np.abs(a) + np.abs(b)) / 16)
+
+
 def test_sums_pass_infinities_and_nan_on():
     n, ng = 16, 16 ** 3
     c = _ctx(n, 2)
