@@ -749,7 +749,7 @@ static sgw_status build_split_tables(sgw_ctx* ctx, int n_atoms, const int* nproj
         for (int64_t i = sup_off[a]; i < sup_off[a + 1]; ++i) used |= mask[sup_idx[i]];
         int c = 0;
         while (c < 32 && (used >> c & 1u)) ++c;
-        if (c == 32) return fail(ctx, SGW_EINVAL, "more than 32 projector supports overlap at a point");
+        if (c == 32) return fail(ctx, SGW_EINVAL, "the overlapping projector supports need more than 32 colours");
         for (int64_t i = sup_off[a]; i < sup_off[a + 1]; ++i) mask[sup_idx[i]] |= 1u << c;
         col[a] = c;
         nc = std::max(nc, c + 1);
@@ -954,9 +954,9 @@ sgw_status sgw_set_potential(sgw_ctx* ctx, const float* vloc_dev, int n_atoms, c
                 sup_beta[i] = b;
             }
         }
-        // slots: one per (unit, atom) pair where the atom's support meets the unit (a unit is an xy
-        // plane on the plane path, 8 x rows on the row path: unit_points consecutive points); atom a's
-        // points in unit z are one contiguous run of its sorted support: [run_beg, run_end)
+        // slots: one per (unit, atom) pair where the atom's support meets the unit (unit_points or, without a
+        // cutoff, sep_unit_points consecutive points: an xy plane or some x rows); atom a's points in unit z
+        // are one contiguous run of its sorted support: [run_beg, run_end)
         const int n = ctx->n;
         int optin = 0;
         CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device));
@@ -983,16 +983,41 @@ sgw_status sgw_set_potential(sgw_ctx* ctx, const float* vloc_dev, int n_atoms, c
             }
             for (int z = 0; z < nu; ++z) max_slots = std::max(max_slots, (int)plane_atoms[z].size());
         };
+        // the slots of each unit coloured greedily (lowest colour not used by an overlapping slot); false: more
+        // than 32 colours
+        std::vector<std::vector<int>> slot_col;
+        int max_colors = 0;
+        auto build_colors = [&]() -> bool {
+            slot_col.assign(nu, {});
+            max_colors = 0;
+            std::vector<uint32_t> mask(plane_sz);
+            for (int z = 0; z < nu; ++z) {
+                std::fill(mask.begin(), mask.end(), 0u);
+                for (const auto& run : plane_runs[z]) {
+                    uint32_t used = 0;
+                    for (int64_t i = run.first; i < run.second; ++i) used |= mask[sup_idx_host[i] - z * plane_sz];
+                    int c = 0;
+                    while (c < 32 && (used >> c & 1u)) ++c;
+                    if (c == 32) return false;
+                    for (int64_t i = run.first; i < run.second; ++i) mask[sup_idx_host[i] - z * plane_sz] |= 1u << c;
+                    slot_col[z].push_back(c);
+                    max_colors = std::max(max_colors, c + 1);
+                }
+            }
+            return true;
+        };
         if (ctx->sep) {
             build_slots(sgw::sep_unit_points(n));
-            // more slots than a plane's block has room for: the transform path's smaller units may fit
-            ctx->sep = sgw::sep_step_smem(n, max_slots) <= (size_t)optin;
+            // more slots than a plane's block has room for, or more colours: the transform path's smaller
+            // units may do
+            ctx->sep = sgw::sep_step_smem(n, max_slots) <= (size_t)optin && build_colors();
         }
         if (!ctx->sep) {
             build_slots(sgw::unit_points(n));
             if (sgw::plane_step_smem(n, max_slots) > (size_t)optin ||
                 (sgw::plane_pipe_supported(n) && sgw::plane_pipe_smem(n, max_slots) > (size_t)optin))
                 return fail(ctx, SGW_EINVAL, "the projector slots of one plane do not fit in shared memory");
+            if (!build_colors()) return fail(ctx, SGW_EINVAL, "the overlapping projector supports need more than 32 colours");
         }
         if (plane_sz > 65536) return fail(ctx, SGW_EINVAL, "in-unit offsets must fit 16 bits");
         if (max_slots >= 65536) return fail(ctx, SGW_EINVAL, "too many projector supports meet one plane");
@@ -1008,25 +1033,6 @@ sgw_status sgw_set_potential(sgw_ctx* ctx, const float* vloc_dev, int n_atoms, c
             atom_pos_off[a + 1] = atom_pos_off[a] + (int)atom_slots[a].size();
             atom_pos.insert(atom_pos.end(), atom_slots[a].begin(), atom_slots[a].end());
         }
-        // colour the slots of each unit greedily (lowest colour not used by an overlapping slot)
-        std::vector<int> slot_col(std::max(total_slots, 1), 0);
-        int max_colors = 0;
-        std::vector<uint32_t> mask(plane_sz);
-        for (int z = 0; z < nu; ++z) {
-            std::fill(mask.begin(), mask.end(), 0u);
-            for (int k = 0; k < (int)plane_atoms[z].size(); ++k) {
-                uint32_t used = 0;
-                for (int64_t i = plane_runs[z][k].first; i < plane_runs[z][k].second; ++i)
-                    used |= mask[sup_idx_host[i] - z * plane_sz];
-                int c = 0;
-                while (c < 32 && (used >> c & 1u)) ++c;
-                if (c == 32) return fail(ctx, SGW_EINVAL, "more than 32 projector supports overlap at a point");
-                for (int64_t i = plane_runs[z][k].first; i < plane_runs[z][k].second; ++i)
-                    mask[sup_idx_host[i] - z * plane_sz] |= 1u << c;
-                slot_col[plane_off[z] + k] = c;
-                max_colors = std::max(max_colors, c + 1);
-            }
-        }
         // unit-major, colour-major, slot-major entry table
         std::vector<int> kbe_col((size_t)nu * (max_colors + 1), 0);
         std::vector<unsigned> kbe_os;
@@ -1038,7 +1044,7 @@ sgw_status sgw_set_potential(sgw_ctx* ctx, const float* vloc_dev, int n_atoms, c
             for (int c = 0; c < max_colors; ++c) {
                 kbe_col[(size_t)z * (max_colors + 1) + c] = (int)kbe_os.size();
                 for (int k = 0; k < (int)plane_atoms[z].size(); ++k) {
-                    if (slot_col[plane_off[z] + k] != c) continue;
+                    if (slot_col[z][k] != c) continue;
                     kbe_slot_beg[plane_off[z] + k] = (int)kbe_os.size();
                     for (int64_t i = plane_runs[z][k].first; i < plane_runs[z][k].second; ++i) {
                         const int o = (int)(sup_idx_host[i] - z * plane_sz);

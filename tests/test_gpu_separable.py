@@ -1,9 +1,10 @@
 """The separable kinetic path (contexts without a cutoff) against the transform path: a cutoff above
 every kinetic energy selects the latter and changes no operator, so the two agree to rounding on every
-grid, batch and KB form; and a plane with more KB slots than the separable step has room for."""
+grid, batch and KB form; and planes with more KB slots or colours than the separable step has room for."""
 import numpy as np
 import pytest
 
+from oracle import hamiltonian as ham
 from paper_2601_21005_gb300 import build, synth
 
 import gpu_common as gc
@@ -94,6 +95,52 @@ def test_more_slots_than_the_separable_step_holds():
     a.set_potential(w)                                       # without the atoms the separable step is back
     a.apply_h(x, ya)
     assert torch.equal(ya, yb)
+
+
+def _colours(atoms, unit, ng):
+    """Most colours that first-fit colouring of the atoms takes in a unit of `unit` points."""
+    most = 0
+    for u in range(ng // unit):
+        used = {}
+        for idx, _, _ in atoms:
+            pts = idx[(idx >= u * unit) & (idx < (u + 1) * unit)]
+            taken = set().union(*[used.get(p, set()) for p in pts]) if len(pts) else set()
+            c = next(i for i in range(len(atoms)) if i not in taken)
+            for p in pts:
+                used.setdefault(p, set()).add(c)
+            most = max(most, c + 1) if len(pts) else most
+    return most
+
+
+def test_more_colours_than_the_separable_step_holds():
+    """33 pairs of atoms a_i, b_i where a_i and b_j share a point of one 48^2 plane for all i != j: first-fit
+    colouring in the order a_0 b_0 a_1 ... takes 33 colours in the plane, but few in units of 8 rows, which
+    the transform path has.  (a_0 and b_0 share a point elsewhere, so the atoms as a whole take 2.)"""
+    from paper_2601_21005_gb300 import sgw
+    build.build()
+    n, h, m = 48, 0.5, 33
+    r = np.random.default_rng(3)
+    pairs = [(i, j) for i in range(m) for j in range(m) if i != j]
+    pts = {p: int(q) for p, q in zip(pairs, r.permutation(n * n))}
+    atoms = []
+    for i in range(m):
+        for own in ([pts[i, j] for j in range(m) if j != i], [pts[j, i] for j in range(m) if j != i]):
+            idx = np.sort(np.array(own + ([n * n] if i == 0 else [])))
+            atoms.append((idx, r.uniform(0.3, 1.0, (1, len(idx))), np.array([r.uniform(-1, 1)])))
+    assert _colours(atoms, n * n, 2 * n * n) == 33 and _colours(atoms, 8 * n, 2 * n * n) <= 32
+    assert _colours(atoms, 2 * n * n, 2 * n * n) == 2
+    v = r.normal(size=(n, n, n)).astype(np.float32)
+    x = (r.normal(size=(2, n, n, n)) + 1j * r.normal(size=(2, n, n, n))).astype(np.complex64)
+    c = sgw.Context(n, h, max_batch=2)
+    c.set_potential(gc.to_dev(v.ravel(), torch, torch.float32), atoms)
+    xd = gc.to_dev(x.reshape(2, -1), torch, torch.complex64)
+    y = torch.empty_like(xd)
+    c.apply_h(xd, y)
+    ref = ham.apply_h(x.astype(np.complex128), ham.Grid(n, h), v.astype(np.float64), ham.KB(atoms))
+    assert gc.rel_err(y.cpu().numpy().reshape(ref.shape), ref) < TOL_H
+    # 33 atoms at one point are refused on every path
+    with pytest.raises(RuntimeError):
+        c.set_potential(gc.to_dev(v.ravel(), torch, torch.float32), [(np.array([5]), np.ones((1, 1)), np.ones(1))] * 33)
 
 
 @pytest.mark.parametrize('n', [16, 32, 64, 128])
