@@ -92,8 +92,9 @@ sgw_status sgw_set_graph_mode(sgw_ctx* ctx, int enable);
 /*
  * Launch tuning (the paper's GPU port batches all vectors of a step into each launch, Sec. 2.3;
  * these keys refine how those launches use the memory system).  Every key is a performance hint:
- * no result depends on it.  They act on the passes of contexts with an energy cutoff; without one
- * the kernels take no launch hints, the keys are accepted and the autotuner keeps their values.
+ * no result depends on it beyond FP32 rounding.  They act on the passes of contexts with an energy
+ * cutoff.  Without one only SGW_TUNE_LINE_FORM acts, at n = 288 on the Coulomb z lines of TDH (form 4
+ * as 3); the other keys are accepted and the autotuner keeps their values.
  *   SGW_TUNE_PLANE_OPERANDS   : bit 0 (1) = each xy-plane pass block starts by prefetching into L2
  *                               the operands of its pointwise step (b_{k+1}, psi, b_{k+2},
  *                               potential rows), so they arrive while its inverse transform runs;
@@ -146,7 +147,8 @@ sgw_status sgw_get_tuning(sgw_ctx* ctx, int key, int* value_host);
  * 2 waves of resident blocks from the occupancy of this GPU, then the line form 0-4 at n = 288), keep
  * the fastest per key, each key timed with the
  * choices already made for the keys before it, and write the chosen values to chosen_host
- * [SGW_TUNE_KEYS] (may be NULL).  Needs sgw_set_potential and a spectral interval (SGW_ESTATE
+ * [SGW_TUNE_KEYS] (may be NULL).  Without a cutoff only the line form at n = 288 is timed, 0-3, on
+ * the Coulomb lines of one vector.  Needs sgw_set_potential and a spectral interval (SGW_ESTATE
  * otherwise); 1 <= batch <= max_batch and reps >= 1 (SGW_EINVAL otherwise).  Uses a context work
  * area of 2 batch-sized complex arrays (SGW_ENOMEM if it cannot grow).  Synchronises; must not be
  * called inside a stream capture.

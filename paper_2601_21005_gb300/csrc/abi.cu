@@ -858,11 +858,22 @@ sgw_status sgw_autotune(sgw_ctx* ctx, int batch, int reps, int* chosen_host) {
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
+    // The separable kernels take no launch hints: without a cutoff what a key acts on is the Coulomb z lines of
+    // TDH, which go over one vector per sample.
+    auto body = [&]() -> sgw_status {
+        if (!ctx->sep) return run_series(ctx, plan, psi, out, batch, ctx->vloc, nullptr, ctx->info, false, false);
+        sgw::launch_pencil(ctx->n, out, 1, 1, (float)std::pow(2.0 * M_PI / ctx->L, 2), 0.f, ctx->tw, ctx->stream, 0, nullptr,
+                           0.f, ctx->tune[SGW_TUNE_LINE_FORM]);
+        CKL();
+        return SGW_OK;
+    };
     auto timed = [&](float* best_ms) -> sgw_status {
         *best_ms = 1e30f;
         for (int r = 0; r <= reps; ++r) {          // the first run warms up
+            if (ctx->sep)
+                CK(cudaMemcpyAsync(out, psi, sizeof(float2) * ctx->ng, cudaMemcpyDeviceToDevice, ctx->stream));
             cudaEventRecord(e0, ctx->stream);
-            sgw_status q = run_series(ctx, plan, psi, out, batch, ctx->vloc, nullptr, ctx->info, false, false);
+            sgw_status q = body();
             if (q) return q;
             cudaEventRecord(e1, ctx->stream);
             if (cudaEventSynchronize(e1) != cudaSuccess) return fail(ctx, SGW_ECUDA, "autotune timing failed");
@@ -890,7 +901,10 @@ sgw_status sgw_autotune(sgw_ctx* ctx, int batch, int reps, int* chosen_host) {
         else if (key == SGW_TUNE_PLANE_VARIANT && sgw::cluster_plane(ctx->n)) cand = {0, 1, 2};
         else if (key == SGW_TUNE_PLANE_OPERANDS && sgw::cluster_plane(ctx->n)) cand = {0, 1, 2, 3};
         else if (sgw::rows_path(ctx->n)) cand = {ctx->tune[key]};   // the row kernels take no other launch hints
-        if (ctx->sep) cand = {ctx->tune[key]};                      // the separable kernels take no launch hints
+        if (ctx->sep) {                                             // (lines of form 4 are those of 3)
+            if (key == SGW_TUNE_LINE_FORM && sgw::cluster_plane(ctx->n)) cand = {0, 1, 2, 3};
+            else cand = {ctx->tune[key]};
+        }
         if (cand.size() == 1 && cand[0] == ctx->tune[key]) continue;
         int best_v = 0;
         float best = 1e30f;

@@ -125,3 +125,26 @@ def test_cluster_launch_choices_and_batches_are_bit_identical(large288):
     one = gc.to_dev(x[1].reshape(1, -1), torch, torch.complex64)
     c.propagate(one, 1, 0.05, 8)
     assert torch.equal(one[0], ref[1])
+
+
+def test_line_form_without_a_cutoff(large288):
+    """Without a cutoff the line form chooses the Coulomb lines of TDH (4 being 3 there), and the autotuner
+    times it and leaves the other keys.  The forms' transforms agree to FP32 rounding, some 1e-6; u^R after
+    one step is what is left of a response whose parts cancel (it vanishes before the first), so that shows
+    enlarged, as all rounding does in u^R: the bar is the TDH parity tests', 2e-4."""
+    s, g, kb, _, c = large288
+    x = gc.to_dev(0.05 * np.stack([_vec(g, 7).reshape(-1)]), torch, torch.complex64)
+    src = (x[0].real * 1e3).contiguous()
+    outs = []
+    for form in (0, 1, 2, 3, 4):
+        c.set_tuning(c.TUNE_LINE_FORM, form)
+        uR = torch.empty(1, 2, g.ng, dtype=torch.float32, device='cuda')
+        c.tdh_response(x, src, 1, 1, 1, 0.05, 8, uR)
+        outs.append(uR)
+    assert torch.equal(outs[3], outs[4]) and float(outs[0].abs().max()) > 0
+    for o in outs[1:]:
+        assert float((o - outs[0]).abs().max()) < 2e-4 * float(outs[0].abs().max())
+    before = [c.get_tuning(k) for k in range(c.TUNE_KEYS)]
+    chosen = c.autotune(2, reps=1)
+    assert chosen[:4] == before[:4] and chosen[4] in (0, 1, 2, 3)
+    c.set_tuning(c.TUNE_LINE_FORM, 0)
