@@ -11,7 +11,7 @@
 
 namespace sgw {
 
-constexpr int KB_B = 3;    // KB entries per lane whose loads are in flight together
+constexpr int KB_B = 3;    // KB entries per lane whose loads are in flight together, in units of a plane or many rows
 
 // Position in shared memory of unit point o = y N + x (row y, column x) at row pitch P.  LAYOUT 0:
 // natural, y P + x.  LAYOUT 1 (N = 288, the two-stage row transforms): a row is 16 groups of 19
@@ -90,14 +90,15 @@ __device__ __forceinline__ void kb_stage_coeffs(const KbHead& h, const float2* k
     for (int i = threadIdx.x; i < 2 * (h.s1 - h.s0); i += NT) reinterpret_cast<float4*>(kcs)[i] = ld4_written(src + 2 * i);
 }
 
-// KB_B entries of a lane (at eb, eb + stride, ...; past e1 the last one again, to be skipped by the
+// B entries of a lane (at eb, eb + stride, ...; past e1 the last one again, to be skipped by the
 // reader), all their loads in flight at once.
+template <int B>
 struct KbBatch {
-    unsigned os[KB_B];
-    float4 be[KB_B];
+    unsigned os[B];
+    float4 be[B];
     __device__ __forceinline__ void load(const StepArgs& a, int eb, int stride, int e1) {
 #pragma unroll
-        for (int i = 0; i < KB_B; ++i) {
+        for (int i = 0; i < B; ++i) {
             const int e = min(eb + i * stride, e1 - 1);
             os[i] = __ldg(a.kbe_os + e);
             be[i] = __ldg(a.kbe_beta + e);
@@ -112,23 +113,23 @@ struct KbBatch {
 // (Two and three batches ahead, or larger ones, cost more registers than the latency they hid.)
 // meanwhile() runs after the first loads are on their way; a barrier before the first update of sm
 // makes its stores (and the caller's) visible; returns after a barrier.
-template <int N, int P, int NT, int LAYOUT = 0, class F>
+template <int N, int P, int NT, int LAYOUT = 0, int B = KB_B, class F>
 __device__ __forceinline__ void kb_apply_unit(const StepArgs& a, const KbHead& h, const float2* kcs, float2* sm,
                                               F&& meanwhile) {
     int c = 1, e0 = h.begin(0, a.max_colors), e1 = h.begin(1, a.max_colors);   // e0 .. e1 the rest of colour c - 1
-    KbBatch cur;
+    KbBatch<B> cur;
     if (e0 < e1) cur.load(a, e0 + threadIdx.x, NT, e1);
     meanwhile();
     __syncthreads();
     while (e0 < e1) {                     // a unit's colours are used from 0 upwards
-        KbBatch nxt;
-        const int en = e0 + KB_B * NT;
+        KbBatch<B> nxt;
+        const int en = e0 + B * NT;
         const bool last = en >= e1;
         const int e2 = h.begin(c + 1, a.max_colors);
         if (!last) nxt.load(a, en + threadIdx.x, NT, e1);
         else if (e1 < e2) nxt.load(a, e1 + threadIdx.x, NT, e2);
 #pragma unroll
-        for (int i = 0; i < KB_B; ++i) {
+        for (int i = 0; i < B; ++i) {
             if (e0 + (int)threadIdx.x + i * NT >= e1) break;
             const float4 be = cur.be[i];
             const int o = (int)(cur.os[i] & 0xffffu), sl = (int)(cur.os[i] >> 16);
@@ -173,23 +174,23 @@ __device__ __forceinline__ KbSlots kb_project_begin(const StepArgs& a, const KbH
     return s;
 }
 // Meets a barrier before it reads sm.
-template <int N, int P, int NT, int LAYOUT = 0>
+template <int N, int P, int NT, int LAYOUT = 0, int B = KB_B>
 __device__ __forceinline__ void kb_project_unit(const StepArgs& a, const KbHead& h, const KbSlots& sl, int b, const float2* sm) {
     constexpr int NW = NT / 32;
     const int s1 = h.s1, lane = threadIdx.x & 31;
     int k = sl.k, e0 = sl.e0, e1 = sl.e1, f0 = sl.f0, f1 = sl.f1;
-    KbBatch cur;
+    KbBatch<B> cur;
     if (k < s1) cur.load(a, e0 + lane, 32, e1);
     __syncthreads();
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     while (k < s1) {                      // a slot has at least one entry
-        KbBatch nxt;
-        const int en = e0 + KB_B * 32;
+        KbBatch<B> nxt;
+        const int en = e0 + B * 32;
         const bool last = en >= e1;
         if (!last) nxt.load(a, en + lane, 32, e1);
         else if (k + NW < s1) nxt.load(a, f0 + lane, 32, f1);
 #pragma unroll
-        for (int i = 0; i < KB_B; ++i) {
+        for (int i = 0; i < B; ++i) {
             if (e0 + lane + 32 * i >= e1) break;
             const float2 v = sm[unit_pos<N, P, LAYOUT>((int)(cur.os[i] & 0xffffu))];
             const float4 be = cur.be[i];

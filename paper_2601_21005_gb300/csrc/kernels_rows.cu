@@ -239,8 +239,11 @@ __global__ void __launch_bounds__(RNT) k_rows_density(const float2* __restrict__
 // lines): inverse x transform of W -> KB apply colour by colour (unit tables, projections staged
 // in shared memory) -> + (V - Ebar) b1 (+ dv b1_partner for tangents) -> combine with psi and b2 ->
 // write out -> per-slot partial projections of out -> forward x transform -> Wout.
+// A unit of 8 rows has few KB entries to a colour: batches of one per lane, and with them 6 blocks to an SM at
+// 48^3 (6 vectors, H psi and a term: 43.3 and 41.4 us with batches of 3, which leave 4 blocks, now 41.5 and 39.6).
+constexpr int RKB = 1;
 template <int N>
-__global__ void __launch_bounds__(RNT) k_rows_step(StepArgs a, const float2* __restrict__ tw) {
+__global__ void __launch_bounds__(RNT, N == 48 ? 6 : 4) k_rows_step(StepArgs a, const float2* __restrict__ tw) {
     extern __shared__ float2 sm[];
     constexpr int P = N + 1;
     constexpr size_t NG = (size_t)N * N * N;
@@ -257,11 +260,11 @@ __global__ void __launch_bounds__(RNT) k_rows_step(StepArgs a, const float2* __r
     load_rows<N>(sm, a.W + off);
     __syncthreads();
     fft_lines<N, RR, P, 1, RNT, +1>(sm, tws);
-    if (kc != nullptr) kb_apply_unit<N, P, RNT>(a, kh, kcs, sm, [] {});
+    if (kc != nullptr) kb_apply_unit<N, P, RNT, 0, RKB>(a, kh, kcs, sm, [] {});
     step_pointwise<N, RR, P, RNT>(a, inf, off, uoff, sm);
     if (a.Wout == nullptr) return;
     __syncthreads();
-    if (a.kbp != nullptr) kb_project_unit<N, P, RNT>(a, kh, kb_project_begin<RNT>(a, kh), b, sm);
+    if (a.kbp != nullptr) kb_project_unit<N, P, RNT, 0, RKB>(a, kh, kb_project_begin<RNT>(a, kh), b, sm);
     fft_lines<N, RR, P, 1, RNT, -1>(sm, tws);
     store_rows<N>(a.Wout + off, sm);
 }
