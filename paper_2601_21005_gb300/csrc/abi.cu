@@ -1128,6 +1128,11 @@ sgw_status sgw_apply_h(sgw_ctx* ctx, const void* in_dev, void* out_dev, int batc
     std::vector<sgw::VecInfo> info(batch, sgw::VecInfo{0, -1, -1, 0});
     if ((s = upload_info(ctx, info))) return s;
     const float2* in = (const float2*)in_dev;
+    if (!ctx->sep) {         // first: it leaves vectors in L2 for the projections
+        Launch L(ctx, SGW_PROF_PLANE_FWD);
+        sgw::launch_plane_fwd(ctx->n, in, ctx->W, batch, ctx->tw, ctx->stream);
+        CKL();
+    }
     if (ctx->kb.n_atoms > 0) {
         Launch L(ctx, SGW_PROF_KB);
         sgw::launch_kb_project(ctx->n, ctx->kb, in, batch, (float)ctx->dV, ctx->kbc, ctx->stream);
@@ -1142,11 +1147,6 @@ sgw_status sgw_apply_h(sgw_ctx* ctx, const void* in_dev, void* out_dev, int batc
     a.ebar = 0.f;
     a.alpha = 1.f;
     if (ctx->sep) return sep_term(ctx, a, batch, false, 1);
-    {
-        Launch L(ctx, SGW_PROF_PLANE_FWD);
-        sgw::launch_plane_fwd(ctx->n, in, ctx->W, batch, ctx->tw, ctx->stream);
-        CKL();
-    }
     {
         Launch L(ctx, SGW_PROF_PENCIL);
         sgw::launch_pencil(ctx->n, ctx->W, batch, 0, (float)std::pow(2.0 * M_PI / ctx->L, 2), (float)ctx->ecut, ctx->tw,

@@ -754,6 +754,9 @@ k_kb_project(const int64_t* __restrict__ atom_off, const int* __restrict__ sup_i
     const int at = blockIdx.x, b = blockIdx.y;
     const int64_t s0 = atom_off[at], s1 = atom_off[at + 1];
     const float2* v = b1 + (size_t)b * ng;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int q1 = __ldg(kr.atom_pos_off + at + 1);
+    int q0 = __ldg(kr.atom_pos_off + at);
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     for (int64_t s = s0 + threadIdx.x; s < s1; s += blockDim.x) {
         const float2 p = __ldg(v + __ldg(sup_idx + s));
@@ -763,23 +766,28 @@ k_kb_project(const int64_t* __restrict__ atom_off, const int* __restrict__ sup_i
         acc[4] += be.z * p.x; acc[5] += be.z * p.y;
         acc[6] += be.w * p.x; acc[7] += be.w * p.y;
     }
+    // the first warp stores the result to the atom's slots, four at a time; their numbers come in beside the sums (one
+    // slot after another, each number waited for: H psi at 16^3 x 2 20.6 us with a cutoff and 10.3 without, now
+    // 18.6 and 8.4; the numbers waited for before the sums: 128^3 x 12 574.1 -> 580.2)
+    const float4 e = __ldg(kr.atom_e + at);
+    int slot = w == 0 && q0 + lane < q1 ? __ldg(kr.atom_pos + q0 + lane) : 0;
 #pragma unroll
     for (int i = 0; i < 8; ++i)
         for (int o = 16; o > 0; o >>= 1) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], o);
-    const int w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    if ((threadIdx.x & 31) == 0)
+    if (lane == 0)
         for (int i = 0; i < 8; ++i) red[w][i] = acc[i];
     __syncthreads();
-    if (threadIdx.x < 8) {
-        float t = 0.f;
-        for (int k = 0; k < nw; ++k) t += red[k][threadIdx.x];
-        const float4 e = __ldg(kr.atom_e + at);
-        const int p = threadIdx.x >> 1;
-        const float ep = p == 0 ? e.x : (p == 1 ? e.y : (p == 2 ? e.z : e.w));
-        float* kc = reinterpret_cast<float*>(kr.kbc + (size_t)b * kr.total_slots * 4);
-        for (int q = __ldg(kr.atom_pos_off + at); q < __ldg(kr.atom_pos_off + at + 1); ++q)
-            kc[(size_t)__ldg(kr.atom_pos + q) * 8 + threadIdx.x] = ep * kr.dV * t;
-    }
+    if (w != 0) return;
+    const int c = lane & 7;
+    float t = 0.f;
+    for (int k = 0; k < nw; ++k) t += red[k][c];
+    t *= (c < 2 ? e.x : (c < 4 ? e.y : (c < 6 ? e.z : e.w))) * kr.dV;
+    float* kc = reinterpret_cast<float*>(kr.kbc + (size_t)b * kr.total_slots * 4);
+    for (; q0 < q1; q0 += 32, slot = q0 + lane < q1 ? __ldg(kr.atom_pos + q0 + lane) : 0)
+        for (int i = 0; i < min(q1 - q0, 32); i += 4) {
+            const int k = __shfl_sync(0xffffffffu, slot, i + (lane >> 3));
+            if (q0 + i + (lane >> 3) < q1) kc[(size_t)k * 8 + c] = t;
+        }
 }
 
 // One warp per (b, a), see kb_reduce_warp.
