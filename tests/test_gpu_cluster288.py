@@ -4,7 +4,9 @@ s/p KB projectors, 11 M support points, so every 36-row unit carries many slots 
 H psi element by element, one degree-16 Chebyshev propagation step, reversibility of a
 forward-backward pair, and the results under every plane-pass and line form (bit-identical where
 only the thread that computes a butterfly changes, within FP32 rounding where warp FFTs replace
-radix stages) and any batch composition."""
+radix stages) and any batch composition.  Those forms are the transform path's, which a context takes
+with a cutoff; one above every kinetic energy changes no operator.  Contexts without a cutoff take the
+kernels of kernels_sep.cu, which go through the oracle tests as well."""
 import numpy as np
 import pytest
 
@@ -29,11 +31,27 @@ def large288():
     # and the KB energies (projectors normalised, |E| <= 1.2)
     lo = float(s['vloc'].min()) - 2.0
     hi = float(s['vloc'].max()) + 1.5 * (np.pi / s['h']) ** 2 + 8.0
+    return s, g, kb, (lo, hi), {}
+
+
+NO_CUT, CUT = 0.0, 1e6
+# every line form of the transform path's, and the axis kernels, which take none
+FORMS = [(NO_CUT, 0), (CUT, 0), (CUT, 3), (CUT, 4)]
+
+
+def _ctx(large288, ecut):
+    """The context with this cutoff, one at a time on the device."""
     from paper_2601_21005_gb300 import sgw
-    c = sgw.Context(s['n'], s['h'], max_batch=3)
-    c.set_potential(gc.to_dev(s['vloc'].ravel(), torch, torch.float32), s['kb_atoms'])
-    c.set_spectrum(lo, hi)
-    return s, g, kb, (lo, hi), c
+    s, _, _, (lo, hi), kept = large288
+    if ecut not in kept:
+        for c in kept.values():
+            c.close()
+        kept.clear()
+        c = sgw.Context(s['n'], s['h'], ecut=ecut, max_batch=3)
+        c.set_potential(gc.to_dev(s['vloc'].ravel(), torch, torch.float32), s['kb_atoms'])
+        c.set_spectrum(lo, hi)
+        kept[ecut] = c
+    return kept[ecut]
 
 
 _ORACLE = {}          # oracle results shared by the parametrised cases
@@ -51,9 +69,10 @@ def _vec(g, seed):
     return (x / np.sqrt(np.sum(np.abs(x) ** 2))).astype(np.complex64)
 
 
-@pytest.mark.parametrize('line_form', [0, 3, 4])
-def test_cluster_apply_h_288_large_cluster(large288, line_form):
-    s, g, kb, _, c = large288
+@pytest.mark.parametrize('ecut,line_form', FORMS)
+def test_cluster_apply_h_288_large_cluster(large288, ecut, line_form):
+    s, g, kb, _, _ = large288
+    c = _ctx(large288, ecut)
     x = np.stack([_vec(g, 1), _vec(g, 2)])
     xd = gc.to_dev(x.reshape(2, -1), torch, torch.complex64)
     yd = torch.empty_like(xd)
@@ -65,9 +84,10 @@ def test_cluster_apply_h_288_large_cluster(large288, line_form):
     assert gc.rel_err(got[1].reshape(g.shape()), ref) < 2e-5
 
 
-@pytest.mark.parametrize('line_form', [0, 3, 4])
-def test_cluster_propagate_288_large_cluster(large288, line_form):
-    s, g, kb, (lo, hi), c = large288
+@pytest.mark.parametrize('ecut,line_form', FORMS)
+def test_cluster_propagate_288_large_cluster(large288, ecut, line_form):
+    s, g, kb, (lo, hi), _ = large288
+    c = _ctx(large288, ecut)
     x0 = _vec(g, 3)
     x = np.stack([x0, x0])
     xd = gc.to_dev(x.reshape(2, -1), torch, torch.complex64)
@@ -88,7 +108,8 @@ def test_cluster_propagate_288_large_cluster(large288, line_form):
 
 
 def test_cluster_launch_choices_and_batches_are_bit_identical(large288):
-    s, g, kb, _, c = large288
+    s, g, kb, _, _ = large288
+    c = _ctx(large288, CUT)
     x = np.stack([_vec(g, 4), _vec(g, 5), _vec(g, 6)])
     ref = None
     outs = {}
@@ -111,6 +132,8 @@ def test_cluster_launch_choices_and_batches_are_bit_identical(large288):
         # transform (form 3: z lines and the row form's y lines; form 4: its rows too) order the
         # sums differently from the radix stages: equal to FP32 rounding
         assert gc.rel_err(xd.cpu().numpy(), ref.cpu().numpy()) < 1e-5, (variant, form)
+    # (and do differ in some bits: another kernel ran)
+    assert not any(torch.equal(outs[k], ref) for k in ((0, 3), (0, 4), (1, 0)))
     c.set_tuning(c.TUNE_PLANE_VARIANT, 0)
     # the operand hints (L2 prefetch, streaming cache policy) change no arithmetic: the same bits
     for form in (0, 4):
@@ -127,12 +150,39 @@ def test_cluster_launch_choices_and_batches_are_bit_identical(large288):
     assert torch.equal(one[0], ref[1])
 
 
+def test_axis_kernels_take_any_batch(large288):
+    s, g, kb, _, _ = large288
+    c = _ctx(large288, NO_CUT)
+    x = gc.to_dev(np.stack([_vec(g, i).reshape(-1) for i in (4, 5, 6)]), torch, torch.complex64)
+    one = x[1:2].clone()
+    c.propagate(x, 1, 0.05, 8)
+    c.propagate(one, 1, 0.05, 8)
+    assert torch.equal(one[0], x[1])
+
+
+def test_autotune_with_a_cutoff(large288):
+    """The search over the 288^3 forms picks among those there are, and what it picks changes no result."""
+    s, g, kb, _, _ = large288
+    c = _ctx(large288, CUT)
+    x0 = gc.to_dev(_vec(g, 8).reshape(1, -1), torch, torch.complex64)
+    x, y = x0.clone(), x0.clone()
+    c.propagate(x, 1, 0.05, 8)
+    chosen = c.autotune(2, reps=1)
+    assert chosen[c.TUNE_PLANE_OPERANDS] in range(4) and chosen[c.TUNE_PLANE_VARIANT] in range(3)
+    assert chosen[c.TUNE_LINE_FORM] in range(5) and [c.get_tuning(k) for k in range(c.TUNE_KEYS)] == chosen
+    c.propagate(y, 1, 0.05, 8)
+    assert gc.rel_err(x.cpu().numpy(), y.cpu().numpy()) < 1e-5
+    for k, v in enumerate((1, 0, 0, 0, 0)):
+        c.set_tuning(k, v)
+
+
 def test_line_form_without_a_cutoff(large288):
     """Without a cutoff the line form chooses the Coulomb lines of TDH (4 being 3 there), and the autotuner
     times it and leaves the other keys.  The forms' transforms agree to FP32 rounding, some 1e-6; u^R after
     one step is what is left of a response whose parts cancel (it vanishes before the first), so that shows
     enlarged, as all rounding does in u^R: the bar is the TDH parity tests', 2e-4."""
-    s, g, kb, _, c = large288
+    s, g, kb, _, _ = large288
+    c = _ctx(large288, NO_CUT)
     x = gc.to_dev(0.05 * np.stack([_vec(g, 7).reshape(-1)]), torch, torch.complex64)
     src = (x[0].real * 1e3).contiguous()
     outs = []

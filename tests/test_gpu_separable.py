@@ -4,7 +4,9 @@ grid, batch and KB form; and planes with more KB slots or colours than the separ
 import numpy as np
 import pytest
 
+from oracle import chebyshev as cheb
 from oracle import hamiltonian as ham
+from oracle import splitop
 from paper_2601_21005_gb300 import build, synth
 
 import gpu_common as gc
@@ -68,6 +70,36 @@ def test_separable_matches_the_transform_path(n, kb):
         c.close()
     for a, b, terms in zip(outs[0], outs[1], (1, 32, 2, 1, 40)):
         assert float((a - b).abs().max() / b.abs().max()) < TOL_H * terms
+
+
+@pytest.mark.parametrize('n', [16, 32, 48, 64, 96])
+def test_cutoff_that_binds(n):
+    """A cutoff below the largest kinetic energy of one axis caps T(k), which is then no sum over the axes:
+    H psi, a propagation step and a split-operator step against the oracle with the same cap.  (Rounding of
+    H psi as above; a step's as in the parity tests.)"""
+    build.build()
+    s = _system(n)
+    ecut = 0.3 * 0.5 * (np.pi / s['h']) ** 2
+    g, kb = ham.Grid(n, s['h'], ecut), ham.KB(s['kb_atoms'])
+    lo, hi = float(s['vloc'].min()) - 2.0, ecut + 4.0
+    r = np.random.default_rng(n)
+    x = (r.normal(size=(2,) + g.shape()) + 1j * r.normal(size=(2,) + g.shape())).astype(np.complex64)
+    c = _ctx(s, 2, ecut, True)
+    c.set_spectrum(lo, hi)
+    xd = gc.to_dev(x.reshape(2, -1), torch, torch.complex64)
+    y, p = torch.empty_like(xd), xd.clone()
+    c.apply_h(xd, y)
+    c.propagate(p, 1, 0.05, 12, np.array([1, -1], dtype=np.int8))
+    h = lambda v: ham.apply_h(v, g, s['vloc'], kb)
+    assert gc.rel_err(y.cpu().numpy().reshape(x.shape), h(x.astype(np.complex128))) < TOL_H
+    for b, d in enumerate((1, -1)):
+        ref = cheb.propagate_step(h, x[b].astype(np.complex128), lo, hi, 0.05 * d, 12)
+        assert gc.rel_err(p[b].cpu().numpy().reshape(g.shape()), ref) < 1e-5
+    if n in (16, 32, 64):
+        q = xd.clone()
+        c.propagate_split(q, 1, 0.05)
+        ref = splitop.split_propagate(x[0].astype(np.complex128), g, s['vloc'], splitop.KBSplit(s['kb_atoms'], g), 0.05, 1)
+        assert gc.rel_err(q[0].cpu().numpy().reshape(g.shape()), ref) < 1e-5
 
 
 def test_more_slots_than_the_separable_step_holds():

@@ -1,5 +1,7 @@
 """Launch tuning: the L2 prefetch hints and the autotuner change no result (bit-identical
-propagation and TDH response under every setting), and bad keys or values are rejected."""
+propagation and TDH response under every setting), and bad keys or values are rejected.  The settings act
+on the transform path, so on contexts with a cutoff (one above every kinetic energy changes no operator);
+without one they are accepted and do nothing."""
 import numpy as np
 import pytest
 
@@ -11,9 +13,9 @@ torch = pytest.importorskip('torch')
 pytestmark = pytest.mark.gpu
 
 
-def _ctx(s, mb):
+def _ctx(s, mb, ecut):
     from paper_2601_21005_gb300 import sgw
-    c = sgw.Context(s['n'], s['h'], max_batch=mb)
+    c = sgw.Context(s['n'], s['h'], ecut=ecut, max_batch=mb)
     c.set_potential(gc.to_dev(s['vloc'].ravel(), torch, torch.float32), s['kb_atoms'])
     c.set_spectrum(float(s['vloc'].min()) - 2.0, 0.5 * 3 * (np.pi / s['h']) ** 2 + 2.0)
     return c
@@ -32,11 +34,12 @@ def _run(c, s):
     return x, uR
 
 
-def test_tuning_is_only_a_hint():
+@pytest.mark.parametrize('ecut', [1e6, 0.0])
+def test_tuning_is_only_a_hint(ecut):
     assert torch.cuda.is_available()
     build.build()
     s = gc.small_cluster()
-    c = _ctx(s, 16)
+    c = _ctx(s, 16, ecut)
     assert [c.get_tuning(k) for k in range(c.TUNE_KEYS)] == [1, 0, 0, 0, 0]
     ref = _run(c, s)
     for setting in ((0, 0, 0, 0), (1, 7, 0, 1), (0, 0, 13, 0), (1, 100000, 100000, 1), (1, 0, 0, 2),
@@ -56,7 +59,7 @@ def test_tuning_is_only_a_hint():
 def test_tuning_rejects_bad_keys_and_values():
     build.build()
     s = gc.small_cluster()
-    c = _ctx(s, 4)
+    c = _ctx(s, 4, 1e6)
     for key, val in ((5, 0), (-1, 0), (0, 4), (1, -5), (2, -1), (3, 3), (4, 5), (4, -1)):
         with pytest.raises(RuntimeError):
             c.set_tuning(key, val)
