@@ -1,8 +1,9 @@
-"""GPU parity of the row path (grids of side 2^a 3^b: 48, 96 and 288, whose planes are split into
-units of 8 x rows plus y- and z-line passes) against the FP64 oracle: H psi, the occupied filter,
-the propagator, a whole MC sample through the pipeline (filter, TDH, time ordering, Sigma(t),
-exchange) on a small KB cluster at 48^3, H psi at 96^3 and on the 288^3 large-cluster grid, and
-the split operator refused there.  Tolerances as on the plane path (FP32 arithmetic)."""
+"""GPU parity on grids of side 2^a 3^b (48, 96 and 288) against the FP64 oracle: H psi, the occupied
+filter, the propagator, TDH and Sigma(t) on a small KB cluster at 48^3, H psi at 96^3 and on the 288^3
+large-cluster grid, each axis by axis (no cutoff) and on the row path (planes split into units of 8 x
+rows plus y- and z-line passes), which a cutoff above every kinetic energy selects; a whole MC sample
+through the pipeline, the exchange, and the split operator refused there.  Tolerances as on the plane
+path (FP32 arithmetic)."""
 import numpy as np
 import pytest
 
@@ -38,8 +39,11 @@ def cluster48():
     return s, g, kb, (lo, hi)
 
 
-def _ctx(s, max_batch, spectrum=None):
-    c = _sgw().Context(s['n'], s['h'], max_batch=max_batch)
+both_paths = pytest.mark.parametrize('ecut', [0.0, 1e6], ids=['axes', 'rows'])
+
+
+def _ctx(s, max_batch, spectrum=None, ecut=0.0):
+    c = _sgw().Context(s['n'], s['h'], ecut=ecut, max_batch=max_batch)
     c.set_potential(gc.to_dev(s['vloc'].ravel(), torch, torch.float32), s['kb_atoms'])
     if spectrum is not None:
         c.set_spectrum(*spectrum)
@@ -51,9 +55,9 @@ def _rand_c(shape, seed):
     return r.normal(size=shape) + 1j * r.normal(size=shape)
 
 
-def _apply_h_check(s, g, kb, B, seed, tol):
+def _apply_h_check(s, g, kb, B, seed, tol, ecut):
     x = _rand_c((B,) + g.shape(), seed)
-    c = _ctx(s, B)
+    c = _ctx(s, B, ecut=ecut)
     xd = gc.to_dev(x.reshape(B, -1), torch, torch.complex64)
     yd = torch.empty_like(xd)
     c.apply_h(xd, yd)
@@ -64,20 +68,22 @@ def _apply_h_check(s, g, kb, B, seed, tol):
     return c, xd, yd
 
 
-def test_rows_apply_h_48(cluster48):
+@both_paths
+def test_rows_apply_h_48(cluster48, ecut):
     s, g, kb, _ = cluster48
-    c, xd, yd = _apply_h_check(s, g, kb, 3, 1, 1e-5)
+    c, xd, yd = _apply_h_check(s, g, kb, 3, 1, 1e-5, ecut)
     # vector by vector: a ragged batch gives the same vectors
     y1 = torch.empty_like(xd[1:2])
     c.apply_h(xd[1:2].contiguous(), y1)
     assert torch.equal(y1[0], yd[1])
 
 
-def test_rows_filter_48(cluster48):
+@both_paths
+def test_rows_filter_48(cluster48, ecut):
     s, g, kb, (lo, hi) = cluster48
     N, B = 100, 3
     a = cheb.gapped_filter_coeffs(-0.3, -0.1, lo, hi, N)
-    c = _ctx(s, B, (lo, hi))
+    c = _ctx(s, B, (lo, hi), ecut)
     noise = torch.empty(B, g.ng, dtype=torch.complex64, device='cuda')
     c.white_noise(5, 1, 0, 1, B, noise)
     out = torch.empty_like(noise)
@@ -89,13 +95,14 @@ def test_rows_filter_48(cluster48):
         assert gc.rel_err(got[b], ref[b]) < 2e-6 * N
 
 
-def test_rows_propagate_48(cluster48):
+@both_paths
+def test_rows_propagate_48(cluster48, ecut):
     s, g, kb, (lo, hi) = cluster48
     B = 4
     x = _rand_c((B,) + g.shape(), 3)
     x /= np.sqrt(np.sum(np.abs(x) ** 2, axis=(1, 2, 3), keepdims=True))
     dirs = np.array([1, -1, 1, -1], dtype=np.int8)
-    c = _ctx(s, B, (lo, hi))
+    c = _ctx(s, B, (lo, hi), ecut)
     h = lambda v: ham.apply_h(v, g, s['vloc'], kb)
     xd = gc.to_dev(x.reshape(B, -1), torch, torch.complex64)
     ref = x.astype(np.complex64).astype(np.complex128)
@@ -138,18 +145,20 @@ def test_rows_whole_sample_48(cluster48, ks48):
     assert abs(x[0].item() - xr) < 1e-4 * abs(xr)
 
 
-def test_rows_apply_h_96():
+@both_paths
+def test_rows_apply_h_96(ecut):
     s = synth.si_cluster(n=96, h=0.5, radius=6.0)
     g = ham.Grid(s['n'], s['h'])
-    _apply_h_check(s, g, ham.KB(s['kb_atoms']), 2, 4, 1e-5)
+    _apply_h_check(s, g, ham.KB(s['kb_atoms']), 2, 4, 1e-5, ecut)
 
 
-def test_rows_apply_h_288():
+@both_paths
+def test_rows_apply_h_288(ecut):
     """The 288^3 grid of the large cluster (23.9 M points, 191 MB per vector), one vector with the
     KB part of a small cluster at the box centre, every element against the oracle."""
     s = synth.si_cluster(n=288, h=0.5, radius=4.5)
     g = ham.Grid(s['n'], s['h'])
-    _apply_h_check(s, g, ham.KB(s['kb_atoms']), 1, 5, 2e-5)
+    _apply_h_check(s, g, ham.KB(s['kb_atoms']), 1, 5, 2e-5, ecut)
 
 
 def test_rows_split_operator_refused(cluster48):
@@ -180,15 +189,16 @@ def test_rows_exchange_48(cluster48):
         assert abs(x[si].item() - ref) < 1e-5 * abs(ref)
 
 
+@both_paths
 @pytest.mark.parametrize('with_kb', [False, True])
-def test_rows_tdh_48(cluster48, with_kb):
+def test_rows_tdh_48(cluster48, with_kb, ecut):
     s, g, kb, (lo, hi) = cluster48
     n_s, n_eta, N = 2, 2, 3
     eta = (0.05 * _rand_c((n_s, n_eta) + g.shape(), 8)).astype(np.complex64)
     phi = _phi48(g)
     r = np.random.default_rng(9)
     src = (np.sign(r.normal(size=(n_s,) + g.shape())) * phi).astype(np.float32)
-    c = _sgw().Context(s['n'], s['h'], max_batch=2 * n_s * n_eta)
+    c = _sgw().Context(s['n'], s['h'], ecut=ecut, max_batch=2 * n_s * n_eta)
     c.set_potential(gc.to_dev(s['vloc'].ravel(), torch, torch.float32), s['kb_atoms'] if with_kb else [])
     c.set_spectrum(lo, hi)
     uR = torch.empty(n_s, N + 1, g.ng, dtype=torch.float32, device='cuda')
@@ -201,13 +211,14 @@ def test_rows_tdh_48(cluster48, with_kb):
         assert gc.rel_err(got[si], ref) < 2e-4, (si, [gc.rel_err(got[si, j], ref[j]) for j in range(N + 1)])
 
 
-def test_rows_sigma_48(cluster48):
+@both_paths
+def test_rows_sigma_48(cluster48, ecut):
     s, g, kb, (lo, hi) = cluster48
     n_s, N = 2, 3
     zeta = _rand_c((n_s, 2) + g.shape(), 5).astype(np.complex64)
     u = (0.3 * _rand_c((n_s, N + 1) + g.shape(), 6)).astype(np.complex64)
     phi = _phi48(g)
-    c = _ctx(s, 2 * n_s, (lo, hi))
+    c = _ctx(s, 2 * n_s, (lo, hi), ecut)
     sig = torch.empty(n_s, 2 * N + 1, dtype=torch.complex128, device='cuda')
     c.sigma_c(gc.to_dev(zeta.reshape(2 * n_s, -1), torch, torch.complex64), gc.to_dev(phi.ravel(), torch, torch.float32),
               gc.to_dev(u.reshape(n_s, N + 1, -1), torch, torch.complex64), n_s, N, 0.05, 16, sig, 1)

@@ -2,7 +2,7 @@
 same atom colours): 32^3 cluster with KB projectors in both directions, 16^3 wells, sampled
 vectors of a 64-vector batch at 64^3; unitarity, time reversibility and graph replay.
 
-Tolerance: each step is two FP32 xy transforms and one z transform (relative ~ log2(N_g) 2^-24)
+Tolerance: each step is an FP32 transform pair along every axis (relative ~ log2(N_g) 2^-24)
 plus FP32 phases and KB factors; 1e-5 per step, so 3e-5 for three steps."""
 import numpy as np
 import pytest

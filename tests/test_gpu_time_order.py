@@ -1,5 +1,5 @@
-"""The time ordering as a matrix product, against the oracle's transforms at the edges of its tiles (64
-points, 104 times per parity, 16 terms per stage), for point counts that are and are not a multiple of 4."""
+"""The time ordering as a matrix product, against the oracle's transforms at the edges of its tiles (128
+points, up to 52 times per parity, 16 terms per stage), for point counts that are and are not a multiple of 4."""
 import numpy as np
 import pytest
 
@@ -21,8 +21,8 @@ def _abs_matrix(n):
     return np.abs(g)
 
 
-@pytest.mark.parametrize('n,points', [(0, 5), (1, 64), (2, 63), (3, 1), (15, 66), (16, 65), (31, 128), (63, 7), (111, 68),
-                                      (206, 130), (207, 64), (208, 61), (400, 193), (401, 192), (513, 64), (1023, 67)])
+@pytest.mark.parametrize('n,points', [(0, 5), (1, 64), (2, 63), (3, 1), (15, 66), (16, 65), (31, 128), (63, 7), (103, 127),
+                                      (104, 129), (111, 68), (206, 130), (207, 64), (208, 61), (400, 193), (401, 192), (513, 64), (1023, 67)])
 def test_time_order_matrix_product(n, points):
     assert torch.cuda.is_available()
     build.build()
