@@ -73,7 +73,7 @@ struct sgw_ctx {
     std::vector<GraphEntry> graphs;
     // split-operator KB factors: orthonormalised projectors per support point (atom-major, like
     // kb.sup_idx), atoms grouped by 3D colour, per-atom M_a = R E R^T (host, 4 x 4), and the
-    // complex factors e^{-i tau M_a} - 1 for tau = +dt/2 and -dt/2 of the last dt
+    // complex factors e^{-i tau M_a} - 1 for tau = dt/2, -dt/2, dt and -dt
     float4* kbq = nullptr;
     int* acol_atoms = nullptr;
     std::vector<int> acol_off;

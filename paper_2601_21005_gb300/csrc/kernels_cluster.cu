@@ -14,7 +14,8 @@
 //   FFT x (outputs into the cluster), FFT y]
 // i.e. the two passes of the plane path (Sec. 2.2: the cost of an H application is dominated by
 // the FFTs; the potential multiply and the KB apply are fused into them).  The KB tables are per
-// unit of 36 rows (a CTA's rows of a plane).
+// unit of 36 rows (a CTA's rows of a plane).  Terms go this way in contexts with a cutoff (and see
+// kernels_grid.cu); the z lines also solve Poisson's equation in every context.
 #include <cooperative_groups.h>
 
 #include "fft_smem.cuh"

@@ -8,6 +8,9 @@
 //   Chebyshev recurrence combine, write; xy fwd of the result for the next term].
 // so one Chebyshev term costs two HBM passes over the batch (Sec. 2.2: the cost of each
 // H application is dominated by the FFTs; the potential multiply is fused into them).
+// Terms go this way, the transform path, in contexts with an energy cutoff, and where the KB slots or colours
+// are too many for the separable path (kernels_sep.cu).  Densities, Poisson solves and the exchange
+// use the plane and pencil passes in every context.
 #include "fft_smem.cuh"
 #include "dependent_launch.cuh"
 #include "grid_common.cuh"

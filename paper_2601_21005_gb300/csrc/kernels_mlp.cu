@@ -28,9 +28,10 @@ namespace sgw {
 // TM/2 x 32, mma.m16n8k16); four K steps of 64 are in flight by cp.async, which for K <= 256 is the
 // whole slab at once, and the weights' share of them is requested before the kernel waits for the one
 // before it.  BF16 matrices have rows padded with zeros to multiples of 8 elements, so every copy is
-// 16 bytes and only rows are checked.  K of 384 and more is split over the blocks of a cluster (three
-// steps of 64 at least to a block), whose partial tiles are summed in rank order through distributed
-// shared memory.
+// 16 bytes and only rows are checked.  Where the backward pass's dZ has a K of 384 and more and few tiles, its K is
+// split over the blocks of a cluster: up to eight, as long as three steps of 64 are left to each on
+// average (a rank has a whole number of them, the last ones fewer or none: 26 steps over 8 ranks are
+// 4 4 4 4 4 4 2 0).  The partial tiles are summed in rank order through distributed shared memory.
 // 148-256-256-256-1603, gradients of 32 rows and the forward of 512: 292 and 92 us per call with 64 x 64
 // tiles, one scalar load per element and a kernel for each sum; now 53 and 25.
 enum { EPI_STORE = 0, EPI_BIAS_TANH = 1, EPI_BIAS = 2, EPI_DTANH = 3, EPI_LOSS = 4 };
@@ -722,7 +723,6 @@ void launch_cv_lin_rows(int mc, int n, int p, int o, const double* m, const floa
 struct sgw_mlp {
     int n_in = 0, width = 0, n_out = 0, max_batch = 0, device = 0;
     cudaStream_t stream = nullptr;
-    int dims[5] = {0};
     sgw::MlpLayout lay{};
     int ldx = 0, ldh = 0, ldo = 0;  // padded row lengths of the BF16 matrices with n_in, width, n_out columns
     int64_t np = 0;
@@ -880,7 +880,6 @@ sgw_status sgw_mlp_create(sgw_mlp** out, int n_in, int width, int n_out, int max
         m->lay.poff[l] = bf; bf += (int64_t)d[l] * m->lay.ld[l];
     }
     m->ldx = pad8(n_in); m->ldh = pad8(width); m->ldo = pad8(n_out);
-    for (int l = 0; l < 5; ++l) m->dims[l] = d[l];
     m->np = off;
     const size_t B = max_batch;
     // the BF16 matrices are zeroed: what pads their rows is never written again

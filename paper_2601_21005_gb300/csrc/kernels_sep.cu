@@ -13,10 +13,10 @@
 // Traffic bounds both passes at batches larger than L2; below that the planes' serial phases.  Every
 // line is held in the registers of 2 or 4 lanes (reg_dft.cuh), so a transform takes no barrier; a
 // plane's block meets one barrier per axis and per KB colour, where radix stages through shared
-// memory take two per stage.  Measured per term, the transform path -> this one (h = 0.5 clusters with
-// KB): 64^3 x 64 vectors 240 -> 191 us (z 43 us = 6.3 TB/s, planes 150 us, 116 us without KB); 64^3 x 8
-// 41 -> 35 us; 96^3 x 8 208 -> 108 us; 128^3 x 12 610 -> 467 us; 48^3 x 64 -> 77 us; 32^3 x 64 38 -> 31 us;
-// 288^3 x 16 (1963 KB atoms) 8.9 -> 6.0 ms.
+// memory take two per stage.  Measured per term of a degree-16 step with the KB parts of h = 0.5 clusters, the
+// transform path -> this one: 64^3 x 64 240 -> 181 us (without KB 213 -> 148; the kernels by themselves, not
+// overlapped: z lines 44 us, planes 148, 118 without KB), 64^3 x 8 40 -> 29 us, 96^3 x 8 218 -> 108 us, 128^3 x 12
+// 594 -> 452 us, 48^3 x 64 213 -> 79 us, 32^3 x 64 38 -> 24 us, 288^3 x 16 (1963 KB atoms) 9.4 -> 6.6 ms.
 #include <algorithm>
 
 #include "dependent_launch.cuh"
@@ -32,9 +32,6 @@ namespace sgw {
 __device__ __forceinline__ void sep_cp16(void* smem, const void* gmem) {
     const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(s), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void sep_cp_wait() {
-    asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
 }
 
 // The kernels of a term are launched by launch_dependent.  The z lines let the planes in at once: those load
@@ -193,7 +190,7 @@ k_sep_z(const float2* in, float2* W, float c, const float2* __restrict__ tw, KbR
 // the columns go to a second plane; the KB apply and the pointwise part follow on that one (64^3 x 36: 111 us
 // per term with the KB apply first, which then waits for the z lines, and 106 so).  Two planes of 96^2 or
 // 128^2 leave room for one block at best: there the rows are transformed in place, the KB apply comes
-// before the columns, and b is read again from L2 (96^3 x 8: 91 us, against 102 with the KB apply first).
+// before the columns, and b is read again from L2 (96^3 x 7: 91 us, against 102 with the KB apply first).
 // Four lanes per line: two lanes hold twice the points and half the warps, and the same pass took
 // 195 us instead of 169 at 64^3 x 64.  The operands of the pointwise part are asked into L2 once the
 // plane has landed, and read evict-first: asked at the block's start they were evicted before use (a

@@ -29,8 +29,8 @@ struct KBDev {
     int* sup_idx = nullptr;      // [n_sup]
     float4* sup_beta = nullptr;  // [n_sup]   beta_a0..3 at each support point
     float4* atom_e = nullptr;    // [n_atoms] E_a0..3
-    // per-unit partial projections (a unit is an xy plane on the plane path, 8 x rows on the row
-    // path): unit z owns slots plane_off[z] .. plane_off[z+1]-1, one per atom whose support meets
+    // per-unit partial projections (a unit is sep_unit_points consecutive points on the separable path,
+    // unit_points on the transform path: an xy plane or some x rows): unit z owns slots plane_off[z] .. plane_off[z+1]-1, one per atom whose support meets
     // the unit; atom a's slots (in increasing z) are
     // atom_pos[atom_pos_off[a] .. atom_pos_off[a+1]).
     int total_slots = 0;
@@ -162,7 +162,7 @@ void launch_density_fwd(int n, const float2* psi, int n_samples, int n_eta, floa
 
 // ---- row path (kernels_rows.cu): grids of side 2^a 3^b (48, 96, 288) whose planes are split into
 // units of 8 x rows; the launchers above dispatch to it for those sizes.  KB tables, slots and
-// colours are per unit (unit_points(n) consecutive points: n^2 on the plane path, 8 n here).
+// colours are per unit (unit_points(n) consecutive points: n^2 on the plane path, 8 n here, 36 n at 288).
 bool rows_path(int n);
 int64_t unit_points(int n);
 int rows_units(int n);
