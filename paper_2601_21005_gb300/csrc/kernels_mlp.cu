@@ -377,54 +377,76 @@ __global__ void k_mlp_input(int64_t n, int cols, int ld, const float* __restrict
         y[i / cols * ld + i % cols] = __float2bfloat16(x[i]);
 }
 
-// Where the parameters of the layers start, and where the BF16 copy of each matrix lies; and the blocks of
-// a kernel over them all: a block has MLP_NT columns of a row of a matrix, or of the bias (row = rows).
-constexpr int MLP_NT = 256;
+// Where the parameters of the layers start, and where the BF16 copy of each matrix lies, as a kernel over
+// them all wants it: in rows, of which a block takes a piece of MLP_PC elements, MLP_U to a thread.  A matrix
+// whose copy is padded has its rows and then the bias; one whose copy is not is a single row with the bias at
+// its end.  Bound by the blocks' latency and L2 traffic: 64-1024-1024-1024-64 14.9 us with an element to a
+// thread, 2000-64-64-64-64 6.7 with its short rows by themselves; with four and flat rows 10.4 and 4.3;
+// 16-2048-2048-2048-16 59.5 -> 41 us, 148-256-256-256-1603 6.3 either way.
+constexpr int MLP_NT = 256, MLP_U = 4, MLP_PC = MLP_NT * MLP_U;
 struct MlpLayout {
-    int64_t woff[4], boff[4], poff[4], first[5];
-    int rows[4], cols[4], ld[4], chunks[4];
+    int64_t woff[4], poff[4], mat[4], first[5];     // mat: elements of the matrix; first: of the layer's blocks
+    int len[4], ld[4], pieces[4];                   // len: of a row; ld: of the copy's; pieces: of a row
 };
 
-// The parameter of this thread and its place among the BF16 copies (-1: none); false: no parameter.
-__device__ __forceinline__ bool mlp_param(const MlpLayout& L, int64_t& i, int64_t& at) {
+// The elements of this block: i, i + 1, .. below i + n (the first parameter's index), of which those before
+// i + copied have a BF16 copy, from at on.
+struct MlpPiece {
+    int64_t i, at;
+    int n, copied;
+};
+__device__ __forceinline__ MlpPiece mlp_piece(const MlpLayout& L) {
     const int64_t b = blockIdx.x;
-    int64_t first = L.first[0], woff = L.woff[0], boff = L.boff[0], poff = L.poff[0];
-    int rows = L.rows[0], cols = L.cols[0], ld = L.ld[0], chunks = L.chunks[0];
+    int64_t first = L.first[0], woff = L.woff[0], poff = L.poff[0], mat = L.mat[0];
+    int len = L.len[0], ld = L.ld[0], pieces = L.pieces[0];
 #pragma unroll
     for (int l = 1; l < 4; ++l)
         if (b >= L.first[l]) {
-            first = L.first[l]; woff = L.woff[l]; boff = L.boff[l]; poff = L.poff[l];
-            rows = L.rows[l]; cols = L.cols[l]; ld = L.ld[l]; chunks = L.chunks[l];
+            first = L.first[l]; woff = L.woff[l]; poff = L.poff[l]; mat = L.mat[l];
+            len = L.len[l]; ld = L.ld[l]; pieces = L.pieces[l];
         }
-    const unsigned u = (unsigned)(b - first), r = u / (unsigned)chunks;
-    const int c = (int)(u - r * (unsigned)chunks) * MLP_NT + threadIdx.x;
-    if (c >= cols) return false;
-    const bool bias = r == (unsigned)rows;
-    i = bias ? boff + c : woff + (int64_t)r * cols + c;
-    at = bias ? -1 : poff + (int64_t)r * ld + c;
-    return true;
+    const unsigned u = (unsigned)(b - first), r = u / (unsigned)pieces;
+    const int c = (int)(u - r * (unsigned)pieces) * MLP_PC;
+    const int64_t k = (int64_t)r * len + c;
+    MlpPiece p;
+    p.i = woff + k;
+    p.at = poff + (int64_t)r * ld + c;
+    p.n = min(len - c, MLP_PC);
+    p.copied = (int)min((int64_t)p.n, max(mat - k, (int64_t)0));
+    return p;
 }
 
 __global__ void __launch_bounds__(MLP_NT) k_mlp_weights(const float* __restrict__ w, __nv_bfloat16* __restrict__ wbf,
                                                         MlpLayout L) {
-    int64_t i, at;
-    if (mlp_param(L, i, at) && at >= 0) wbf[at] = __float2bfloat16(w[i]);
+    const MlpPiece p = mlp_piece(L);
+    for (int c = threadIdx.x; c < p.copied; c += MLP_NT) wbf[p.at + c] = __float2bfloat16(w[p.i + c]);
 }
 
 // Adam (Kingma & Ba) on FP32 master weights; writes the BF16 copies of the matrices.
 __global__ void __launch_bounds__(MLP_NT) k_adam(float* __restrict__ w, const float* __restrict__ g, float* __restrict__ m,
                                                  float* __restrict__ v, __nv_bfloat16* __restrict__ wbf, MlpLayout L,
                                                  float lr, float b1, float b2, float c1, float c2, float eps) {
-    int64_t i, at;
-    if (!mlp_param(L, i, at)) return;
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.f - b1) * gi;
-    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    const float wi = w[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-    w[i] = wi;
-    if (at >= 0) wbf[at] = __float2bfloat16(wi);
+    const MlpPiece p = mlp_piece(L);
+    g += p.i; m += p.i; v += p.i; w += p.i; wbf += p.at;
+    float g0[MLP_U], m0[MLP_U], v0[MLP_U], w0[MLP_U];
+#pragma unroll
+    for (int q = 0; q < MLP_U; ++q) {
+        const int c = threadIdx.x + q * MLP_NT;
+        if (c < p.n) { g0[q] = g[c]; m0[q] = m[c]; v0[q] = v[c]; w0[q] = w[c]; }
+    }
+#pragma unroll
+    for (int q = 0; q < MLP_U; ++q) {
+        const int c = threadIdx.x + q * MLP_NT;
+        if (c >= p.n) break;
+        const float gi = g0[q];
+        const float mi = b1 * m0[q] + (1.f - b1) * gi;
+        const float vi = b2 * v0[q] + (1.f - b2) * gi * gi;
+        m[c] = mi;
+        v[c] = vi;
+        const float wi = w0[q] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+        w[c] = wi;
+        if (c < p.copied) wbf[c] = __float2bfloat16(wi);
+    }
 }
 
 // ------------------------------------------------------------------ features
@@ -724,6 +746,8 @@ struct sgw_mlp {
     int n_in = 0, width = 0, n_out = 0, max_batch = 0, device = 0;
     cudaStream_t stream = nullptr;
     sgw::MlpLayout lay{};
+    int64_t boff[4] = {0};          // where the biases start
+    int ldw[4] = {0};               // padded row lengths of the BF16 weight matrices
     int ldx = 0, ldh = 0, ldo = 0;  // padded row lengths of the BF16 matrices with n_in, width, n_out columns
     int64_t np = 0;
     float* P = nullptr;            // FP32 master parameters: W1, b1, W2, b2, W3, b3, W4, b4
@@ -783,14 +807,14 @@ sgw_status mlp_forward(sgw_mlp* m, const float* x, int M, bool keep, const sgw::
     int K = I, ld = m->ldx;
     for (int l = 0; l < 3; ++l) {
         sgw::GemmEpi ep{};
-        ep.mode = sgw::EPI_BIAS_TANH; ep.bias = m->P + m->lay.boff[l];
+        ep.mode = sgw::EPI_BIAS_TANH; ep.bias = m->P + m->boff[l];
         ep.out = keep ? m->Z[l] : nullptr; ep.ldo = H; ep.out_bf = m->Abf[l]; ep.ldb = m->ldh;
-        forward_gemm(m, sgw::Gemm{M, H, K, in, ld, m->Pbf + m->lay.poff[l], m->lay.ld[l], ep});
+        forward_gemm(m, sgw::Gemm{M, H, K, in, ld, m->Pbf + m->lay.poff[l], m->ldw[l], ep});
         in = m->Abf[l];
         K = H;
         ld = m->ldh;
     }
-    forward_gemm(m, sgw::Gemm{M, O, H, in, ld, m->Pbf + m->lay.poff[3], m->lay.ld[3], last});
+    forward_gemm(m, sgw::Gemm{M, O, H, in, ld, m->Pbf + m->lay.poff[3], m->ldw[3], last});
     MCK(cudaGetLastError());
     return SGW_OK;
 }
@@ -799,7 +823,7 @@ sgw_status mlp_forward(sgw_mlp* m, const float* x, int M, bool keep, const sgw::
 sgw_status mlp_gradients(sgw_mlp* m, const float* x, const float* t, int M) {
     const int H = m->width, I = m->n_in, O = m->n_out;
     sgw::GemmEpi le{};
-    le.mode = sgw::EPI_LOSS; le.bias = m->P + m->lay.boff[3]; le.out = m->dY; le.ldo = O;
+    le.mode = sgw::EPI_LOSS; le.bias = m->P + m->boff[3]; le.out = m->dY; le.ldo = O;
     le.out_bf = m->dYbf; le.ldb = m->ldo; le.aux = t; le.w = m->lw; le.scale = 2.0f / (float)((int64_t)M * O);
     le.y = m->Y;
     sgw_status s = mlp_forward(m, x, M, true, le);
@@ -818,13 +842,13 @@ sgw_status mlp_gradients(sgw_mlp* m, const float* x, const float* t, int M) {
             sgw::GemmEpi ed{};
             ed.mode = sgw::EPI_DTANH; ed.out = m->dZ[to]; ed.ldo = H; ed.out_bf = m->dZbf[to]; ed.ldb = m->ldh;
             ed.aux = m->Z[l - 1];
-            b.d = sgw::Gemm{M, H, N, dzbf, ldz, m->Pbf + m->lay.poff[l], m->lay.ld[l], ed};
+            b.d = sgw::Gemm{M, H, N, dzbf, ldz, m->Pbf + m->lay.poff[l], m->ldw[l], ed};
         }
         b.d_tiles = l > 0 ? sgw::gemm_tiles(32, M, H) : 0;
         while (b.splits < 8 && N >= 2 * b.splits * 3 * sgw::GK && b.d_tiles * b.splits * 2 <= 152) b.splits *= 2;
         b.w_tiles = sgw::gemm_tiles(32, K_in, N);
         b.db_blocks = (N + 31) / 32;
-        b.dz = dz; b.db = m->G + m->lay.boff[l]; b.ldz = N;
+        b.dz = dz; b.db = m->G + m->boff[l]; b.ldz = N;
         const int64_t ny = (int64_t)M * O;
         b.loss = sgw::Loss{ny, O, (int)std::min<int64_t>((ny + sgw::G_NT - 1) / sgw::G_NT, MAX_LOSS_BLOCKS), m->Y, t, m->lw, m->loss};
         b.loss_blocks = l == 3 ? b.loss.blocks : 0;
@@ -870,14 +894,17 @@ sgw_status sgw_mlp_create(sgw_mlp** out, int n_in, int width, int n_out, int max
     const int d[5] = {n_in, width, width, width, n_out};
     int64_t off = 0, bf = 0;
     for (int l = 0; l < 4; ++l) {
-        m->lay.woff[l] = off; off += (int64_t)d[l] * d[l + 1];
-        m->lay.boff[l] = off; off += d[l + 1];
-        m->lay.cols[l] = d[l + 1];
-        m->lay.ld[l] = pad8(d[l + 1]);
-        m->lay.rows[l] = d[l];
-        m->lay.chunks[l] = (d[l + 1] + sgw::MLP_NT - 1) / sgw::MLP_NT;
-        m->lay.first[l + 1] = m->lay.first[l] + ((int64_t)d[l] + 1) * m->lay.chunks[l];
-        m->lay.poff[l] = bf; bf += (int64_t)d[l] * m->lay.ld[l];
+        const int ld = pad8(d[l + 1]);
+        const bool one = ld == d[l + 1] && (d[l] + (int64_t)1) * d[l + 1] < (1 << 30);     // (a row's length is an int)
+        m->ldw[l] = ld;
+        m->lay.woff[l] = off;
+        m->lay.mat[l] = (int64_t)d[l] * d[l + 1]; off += m->lay.mat[l];
+        m->boff[l] = off; off += d[l + 1];
+        m->lay.poff[l] = bf; bf += (int64_t)d[l] * ld;
+        m->lay.len[l] = one ? (d[l] + 1) * d[l + 1] : d[l + 1];
+        m->lay.ld[l] = ld;
+        m->lay.pieces[l] = (m->lay.len[l] + sgw::MLP_PC - 1) / sgw::MLP_PC;
+        m->lay.first[l + 1] = m->lay.first[l] + (int64_t)(one ? 1 : d[l] + 1) * m->lay.pieces[l];
     }
     m->ldx = pad8(n_in); m->ldh = pad8(width); m->ldo = pad8(n_out);
     m->np = off;
@@ -974,7 +1001,7 @@ sgw_status sgw_mlp_forward(sgw_mlp* m, const float* x_dev, int M, float* y_dev) 
     // a y that floats can't be stored to goes by way of Y and a copy
     const bool direct = reinterpret_cast<uintptr_t>(y_dev) % alignof(float) == 0;
     sgw::GemmEpi ep{};
-    ep.mode = sgw::EPI_BIAS; ep.bias = m->P + m->lay.boff[3]; ep.out = direct ? y_dev : m->Y; ep.ldo = m->n_out;
+    ep.mode = sgw::EPI_BIAS; ep.bias = m->P + m->boff[3]; ep.out = direct ? y_dev : m->Y; ep.ldo = m->n_out;
     if ((s = mlp_forward(m, x_dev, M, false, ep))) return s;
     if (!direct) MCK(cudaMemcpyAsync(y_dev, m->Y, sizeof(float) * (size_t)M * m->n_out, cudaMemcpyDeviceToDevice, m->stream));
     return SGW_OK;
