@@ -68,9 +68,9 @@ CONFIGS = {
 # capture of the kernel source whose sha256 prefix is given; a roofline line reports `traffic`
 # only while that source is unchanged.
 TRAFFIC = {
-    # k_sep_rows288, third term of a 4-vector kernel_bench step: 3.768 GB read + 0.753 GB written
+    # k_sep_rows288, third term of a 4-vector kernel_bench step: 3.767 GB read + 0.753 GB written
     # against 4.138 GB algorithmic
-    ('plane_step', 288): dict(ratio=(3.768 + 0.753) / 4.138, sha='2e42d0b63d6875c0', capture='4-vector launch',
+    ('plane_step', 288): dict(ratio=(3.767 + 0.753) / 4.138, sha='58d1414003c4ff45', capture='4-vector launch',
                               source=('kernels_sep.cu', 'kb_unit.cuh', 'grid_common.cuh', 'reg_dft.cuh')),
 }
 

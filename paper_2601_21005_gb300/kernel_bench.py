@@ -1,10 +1,11 @@
 """Micro-benchmark of the propagation kernels on one batch (also the small case for ncu).
 
-    python -m paper_2601_21005_gb300.kernel_bench [--n 64] [--batch 64] [--steps 2] [--deg 16]
+    python -m paper_2601_21005_gb300.kernel_bench [--n 64] [--batch 64] [--steps 2] [--deg 16] [--ecut 0]
 
 Sets up the Si35H36 cluster (local + KB potentials) on an n^3 grid, fills a batch of
 complex vectors with Philox noise and propagates it n_steps steps with the degree-`deg`
-Chebyshev expansion through the C ABI, timing each kernel kind with CUDA events.  Device
+Chebyshev expansion through the C ABI, timing each kernel kind with CUDA events.  With a cutoff (1e6
+is above every kinetic energy) the terms take the transform path.  Device
 memory: four batch-sized complex arrays (0.5 GB at 64^3 x 64).
 """
 import argparse
@@ -24,6 +25,7 @@ def main():
     ap.add_argument('--no-kb', action='store_true')
     ap.add_argument('--radius', type=float, default=None,
                     help='cluster radius in bohr (default 10.5 = Si35H36; 28.0 = Si657H300 at n = 128)')
+    ap.add_argument('--ecut', type=float, default=0.0, help='energy cutoff in Ha; the tuning keys act with one only')
     ap.add_argument('--tune', default=None,
                     help='semicolon-separated settings "operands,plane_lookahead,pencil_lookahead,variant,line_tile" '
                          '(a prefix of the tuning keys) to time in turn')
@@ -33,7 +35,7 @@ def main():
     build.build()
     radius = args.radius if args.radius is not None else (10.5 if args.n >= 64 else 4.5)
     s = synth.si_cluster(n=args.n, h=0.5, radius=radius)
-    ctx = sgw.Context(args.n, 0.5, max_batch=args.batch)
+    ctx = sgw.Context(args.n, 0.5, ecut=args.ecut, max_batch=args.batch)
     ctx.set_potential(torch.as_tensor(s['vloc'].reshape(-1).astype(np.float32)).cuda(),
                       [] if args.no_kb else s['kb_atoms'])
     ctx.set_spectrum(float(s['vloc'].min()) - 1.0, 0.5 * 3 * (np.pi / 0.5) ** 2 + 3.0)
