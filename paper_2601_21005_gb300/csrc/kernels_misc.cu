@@ -614,11 +614,12 @@ __device__ __forceinline__ float2 unpack2(f32x2 a) {
 }
 
 // One (parity, row tile) of 128 points of a sample.  Warp tm: rows TM tm .. + TM; lane tn: points 4 tn .. + 4.
-// VEC: rows of u^R and u start on 16 bytes (the number of points is a multiple of 4).
+// VEC: rows of u^R and u start on 16 bytes (the number of points is a multiple of 4).  G may be the matrix of more
+// steps, which has a parity every g_par elements and a tile every g_tile of it; K is padded to kpad here.
 template <int TM, bool VEC>
 __global__ void __launch_bounds__(TO_NT, 3)
-k_time_order(int64_t np, const float* __restrict__ uR, float2* __restrict__ u, int n_steps, int tiles, int nk, int ch,
-             const float2* __restrict__ G, int g_tiles, int g_kpad) {
+k_time_order(int64_t np, const float* __restrict__ uR, float2* __restrict__ u, int n_steps, int tiles, int kpad, int ch,
+             const float2* __restrict__ G, int g_par, int g_tile) {
     constexpr int TMP = (TM + 1) & ~1, AM = TO_R * TMP;
     extern __shared__ __align__(16) unsigned char to_sm[];
     float2* As = reinterpret_cast<float2*>(to_sm);                                  // [stage][k][TO_R][TMP]
@@ -628,7 +629,8 @@ k_time_order(int64_t np, const float* __restrict__ uR, float2* __restrict__ u, i
     const int64_t p0 = (int64_t)(blockIdx.x / (2 * tiles)) * TO_BN;
     const size_t row0 = (size_t)blockIdx.y * (n_steps + 1);
     const int tn = threadIdx.x % 32, tm = threadIdx.x / 32;
-    const float2* A = G + ((size_t)par * g_tiles + tile) * g_kpad * AM;
+    const float2* A = G + (par * g_par + tile * g_tile);
+    const int nk = kpad / TO_BK;
     const auto load = [&](int s, int kt) {
         const float2* a = A + (size_t)kt * TO_BK * AM;
         float2* as = As + s * TO_BK * AM;
@@ -711,12 +713,13 @@ template <int TM> static void tlaunch(int64_t np, const float* uR, float2* u, in
     const dim3 grid((unsigned)(2 * tiles * ((np + TO_BN - 1) / TO_BN)), n_samples);
     // chunks of 16 terms, 32 above 256: as many chunks as terms in one, about
     const int ch = nk * TO_BK > 256 ? 2 * TO_BK : TO_BK;
+    const int kpad = nk * TO_BK, g_tile = g.kpad * TO_R * TMP, g_par = g.tiles * g_tile;
     if (np % 4 == 0) {
         cudaFuncSetAttribute(k_time_order<TM, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_time_order<TM, true><<<grid, TO_NT, smem, st>>>(np, uR, u, n_steps, tiles, nk, ch, G, g.tiles, g.kpad);
+        k_time_order<TM, true><<<grid, TO_NT, smem, st>>>(np, uR, u, n_steps, tiles, kpad, ch, G, g_par, g_tile);
     } else {
         cudaFuncSetAttribute(k_time_order<TM, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_time_order<TM, false><<<grid, TO_NT, smem, st>>>(np, uR, u, n_steps, tiles, nk, ch, G, g.tiles, g.kpad);
+        k_time_order<TM, false><<<grid, TO_NT, smem, st>>>(np, uR, u, n_steps, tiles, kpad, ch, G, g_par, g_tile);
     }
 }
 
