@@ -613,28 +613,39 @@ __device__ __forceinline__ float2 unpack2(f32x2 a) {
     return r;
 }
 
-// One (parity, row tile) of 128 points of a sample.  Warp tm: rows TM tm .. + TM; lane tn: points 4 tn .. + 4.
+// One (parity, row tile) of 128 points of a sample.  Warp tm: rows TM tm .. + TM, of which the block takes TS (all,
+// or an even number of slots: a tile has NSUB blocks then); lane tn: points 4 tn .. + 4.
 // VEC: rows of u^R and u start on 16 bytes (the number of points is a multiple of 4).  G may be the matrix of more
 // steps, which has a parity every g_par elements and a tile every g_tile of it; K is padded to kpad here.
-template <int TM, bool VEC>
+template <int TM, int TS, bool VEC>
 __global__ void __launch_bounds__(TO_NT, 3)
 k_time_order(int64_t np, const float* __restrict__ uR, float2* __restrict__ u, int n_steps, int tiles, int kpad, int ch,
              const float2* __restrict__ G, int g_par, int g_tile) {
-    constexpr int TMP = (TM + 1) & ~1, AM = TO_R * TMP;
+    constexpr int TMP = (TM + 1) & ~1, NSUB = (TM + TS - 1) / TS, TSP = (TS + 1) & ~1, AM = TO_R * TSP;
+    static_assert(NSUB == 1 || TS % 2 == 0, "slots are copied in pairs");
     extern __shared__ __align__(16) unsigned char to_sm[];
-    float2* As = reinterpret_cast<float2*>(to_sm);                                  // [stage][k][TO_R][TMP]
+    float2* As = reinterpret_cast<float2*>(to_sm);                                  // [stage][k][TO_R][TSP]
     float* Bs = reinterpret_cast<float*>(As + TO_STAGES * TO_BK * AM);              // [stage][k][TO_BN]
     // the blocks of one group of points run together: they read the same rows of u^R
-    const int which = blockIdx.x % (2 * tiles), par = which / tiles, tile = which % tiles;
-    const int64_t p0 = (int64_t)(blockIdx.x / (2 * tiles)) * TO_BN;
+    const int which = blockIdx.x / NSUB % (2 * tiles), par = which / tiles, tile = which % tiles;
+    const int slot0 = TS * (blockIdx.x % NSUB);
+    const int64_t p0 = (int64_t)(blockIdx.x / (2 * NSUB * tiles)) * TO_BN;
     const size_t row0 = (size_t)blockIdx.y * (n_steps + 1);
     const int tn = threadIdx.x % 32, tm = threadIdx.x / 32;
-    const float2* A = G + (par * g_par + tile * g_tile);
+    const float2* A = G + (par * g_par + tile * g_tile) + slot0;
     const int nk = kpad / TO_BK;
     const auto load = [&](int s, int kt) {
-        const float2* a = A + (size_t)kt * TO_BK * AM;
+        const float2* a = A + (size_t)kt * TO_BK * TO_R * TMP;
         float2* as = As + s * TO_BK * AM;
-        for (int i = threadIdx.x; i < TO_BK * AM / 2; i += TO_NT) to_cp(as + 2 * i, a + 2 * i, 16, 16);
+        for (int i = threadIdx.x; i < TO_BK * AM / 2; i += TO_NT) {
+            if constexpr (NSUB == 1) {
+                to_cp(as + 2 * i, a + 2 * i, 16, 16);
+            } else {
+                const int row = i / (TSP / 2), slot = i % (TSP / 2) * 2;
+                const bool ok = slot0 + slot < TMP;
+                to_cp(as + 2 * i, ok ? a + row * TMP + slot : a, 16, ok ? 16 : 0);
+            }
+        }
         float* bs = Bs + s * TO_BK * TO_BN;
         constexpr int V = VEC ? 4 : 1;
         for (int i = threadIdx.x; i < TO_BK * TO_BN / V; i += TO_NT) {
@@ -644,9 +655,9 @@ k_time_order(int64_t np, const float* __restrict__ uR, float2* __restrict__ u, i
             to_cp(bs + k * TO_BN + p, ok ? uR + (row0 + j) * np + p0 + p : uR, 4 * V, ok ? 4 * V : 0);
         }
     };
-    f32x2 acc[TM][2], tot[TM][2];
+    f32x2 acc[TS][2], tot[TS][2];
 #pragma unroll
-    for (int i = 0; i < TM; ++i) acc[i][0] = acc[i][1] = tot[i][0] = tot[i][1] = 0ull;
+    for (int i = 0; i < TS; ++i) acc[i][0] = acc[i][1] = tot[i][0] = tot[i][1] = 0ull;
 #pragma unroll
     for (int s = 0; s < TO_STAGES - 1; ++s) {
         if (s < nk) load(s, s);
@@ -657,25 +668,25 @@ k_time_order(int64_t np, const float* __restrict__ uR, float2* __restrict__ u, i
         __syncthreads();                                  // stage kt has landed; stage kt - 1 is free
         if (kt + TO_STAGES - 1 < nk) load((kt + TO_STAGES - 1) % TO_STAGES, kt + TO_STAGES - 1);
         asm volatile("cp.async.commit_group;" ::: "memory");
-        const ulonglong2* as = reinterpret_cast<const ulonglong2*>(As + (kt % TO_STAGES) * TO_BK * AM + tm * TMP);
+        const ulonglong2* as = reinterpret_cast<const ulonglong2*>(As + (kt % TO_STAGES) * TO_BK * AM + tm * TSP);
         const float* bs = Bs + (kt % TO_STAGES) * TO_BK * TO_BN + 4 * tn;
 #pragma unroll
         for (int k = 0; k < TO_BK; ++k) {
             const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(bs + k * TO_BN);
 #pragma unroll
-            for (int i = 0; i < TMP / 2; ++i) {
+            for (int i = 0; i < TSP / 2; ++i) {
                 const ulonglong2 a = as[k * (AM / 2) + i];
                 acc[2 * i][0] = fma2(a.x, b.x, acc[2 * i][0]);
                 acc[2 * i][1] = fma2(a.x, b.y, acc[2 * i][1]);
-                if (2 * i + 1 < TM) {
-                    acc[(2 * i + 1) % TM][0] = fma2(a.y, b.x, acc[(2 * i + 1) % TM][0]);
-                    acc[(2 * i + 1) % TM][1] = fma2(a.y, b.y, acc[(2 * i + 1) % TM][1]);
+                if (2 * i + 1 < TS) {
+                    acc[(2 * i + 1) % TS][0] = fma2(a.y, b.x, acc[(2 * i + 1) % TS][0]);
+                    acc[(2 * i + 1) % TS][1] = fma2(a.y, b.y, acc[(2 * i + 1) % TS][1]);
                 }
             }
         }
         if (((kt + 1) * TO_BK) % ch == 0) {
 #pragma unroll
-            for (int i = 0; i < TM; ++i)
+            for (int i = 0; i < TS; ++i)
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     tot[i][h] = add2(tot[i][h], acc[i][h]);
@@ -685,9 +696,9 @@ k_time_order(int64_t np, const float* __restrict__ uR, float2* __restrict__ u, i
     }
     const int64_t p = p0 + 4 * tn;
 #pragma unroll
-    for (int i = 0; i < TM; ++i) {
-        const int t = 2 * (TO_R * TM * tile + TM * tm + i) + par;
-        if (t > n_steps || p >= np) continue;
+    for (int i = 0; i < TS; ++i) {
+        const int t = 2 * (TO_R * TM * tile + TM * tm + slot0 + i) + par;
+        if (t > n_steps || p >= np || (NSUB > 1 && slot0 + i >= TM)) continue;
         const float* x = uR + (row0 + t) * np + p;
         float2* y = u + (row0 + t) * np + p;
         const float half = t == 0 ? 1.f : 0.5f;
@@ -705,22 +716,31 @@ k_time_order(int64_t np, const float* __restrict__ uR, float2* __restrict__ u, i
     }
 }
 
+template <int TM, int TS, bool VEC>
+static void tlaunch(int64_t np, const float* uR, float2* u, int n_samples, int n_steps, int tiles, const ToShape& g,
+                    const float2* G, cudaStream_t st) {
+    constexpr int TMP = (TM + 1) & ~1, TSP = (TS + 1) & ~1, NSUB = (TM + TS - 1) / TS;
+    const size_t smem = TO_STAGES * TO_BK * (sizeof(float2) * TO_R * TSP + sizeof(float) * TO_BN);
+    const dim3 grid((unsigned)(2 * NSUB * tiles * ((np + TO_BN - 1) / TO_BN)), n_samples);
+    const int kpad = (n_steps / 2 + TO_BK) / TO_BK * TO_BK;
+    // chunks of 16 terms, 32 above 256: as many chunks as terms in one, about
+    const int ch = kpad > 256 ? 2 * TO_BK : TO_BK;
+    const int g_tile = g.kpad * TO_R * TMP, g_par = g.tiles * g_tile;
+    cudaFuncSetAttribute(k_time_order<TM, TS, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k_time_order<TM, TS, VEC><<<grid, TO_NT, smem, st>>>(np, uR, u, n_steps, tiles, kpad, ch, G, g_par, g_tile);
+}
+// Few points leave most of the chip idle: below a tile to every other SM a block takes four of its warps' TM rows.
+// (100 steps of 1000 points, 16 tiles: 11.0 -> 6.9 us; 400 of 1000, 64: 22.9 -> 17.1; 400 of 2000, 128: 22.9 with
+// whole tiles, 27.5 so.)
 template <int TM> static void tlaunch(int64_t np, const float* uR, float2* u, int n_samples, int n_steps, const ToShape& g,
                                       const float2* G, cudaStream_t st) {
-    constexpr int TMP = (TM + 1) & ~1;
-    const size_t smem = TO_STAGES * TO_BK * (sizeof(float2) * TO_R * TMP + sizeof(float) * TO_BN);
-    const int rows = n_steps / 2 + 1, tiles = (rows + TO_R * TM - 1) / (TO_R * TM), nk = (rows + TO_BK - 1) / TO_BK;
-    const dim3 grid((unsigned)(2 * tiles * ((np + TO_BN - 1) / TO_BN)), n_samples);
-    // chunks of 16 terms, 32 above 256: as many chunks as terms in one, about
-    const int ch = nk * TO_BK > 256 ? 2 * TO_BK : TO_BK;
-    const int kpad = nk * TO_BK, g_tile = g.kpad * TO_R * TMP, g_par = g.tiles * g_tile;
-    if (np % 4 == 0) {
-        cudaFuncSetAttribute(k_time_order<TM, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_time_order<TM, true><<<grid, TO_NT, smem, st>>>(np, uR, u, n_steps, tiles, kpad, ch, G, g_par, g_tile);
-    } else {
-        cudaFuncSetAttribute(k_time_order<TM, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_time_order<TM, false><<<grid, TO_NT, smem, st>>>(np, uR, u, n_steps, tiles, kpad, ch, G, g_par, g_tile);
-    }
+    constexpr int TS = TM > 4 ? 4 : TM;
+    const int tiles = (n_steps / 2 + TO_R * TM) / (TO_R * TM);
+    const bool few = 2 * tiles * ((np + TO_BN - 1) / TO_BN) * n_samples < 76;
+    if (np % 4 == 0) few ? tlaunch<TM, TS, true>(np, uR, u, n_samples, n_steps, tiles, g, G, st)
+                         : tlaunch<TM, TM, true>(np, uR, u, n_samples, n_steps, tiles, g, G, st);
+    else few ? tlaunch<TM, TS, false>(np, uR, u, n_samples, n_steps, tiles, g, G, st)
+             : tlaunch<TM, TM, false>(np, uR, u, n_samples, n_steps, tiles, g, G, st);
 }
 
 void launch_time_order_matrix(int n_steps, int M, float2* G, cudaStream_t st) {

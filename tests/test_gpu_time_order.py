@@ -111,3 +111,20 @@ def test_step_counts_of_one_length_share_a_capture(kept, captured):
         c.time_order_points(x, u[1], 1, captured, 70)
     st.synchronize()
     assert torch.equal(u[0], u[1])
+
+
+@pytest.mark.parametrize('n,points', [(50, 1), (63, 127), (79, 300), (103, 1000), (206, 999), (400, 1024), (401, 1001),
+                                      (1000, 384)])
+def test_few_points_give_the_bits_of_many(n, points):
+    """Calls of few points give a tile's rows to several blocks (odd and even numbers of rows to a warp here); a
+    point's sums have the same order either way."""
+    build.build()
+    from paper_2601_21005_gb300 import sgw
+    c = sgw.Context(16, 0.5)
+    many = 40000
+    x = torch.randn(1, n + 1, many, device='cuda')
+    u = torch.empty(1, n + 1, many, dtype=torch.complex64, device='cuda')
+    c.time_order_points(x, u, 1, n, many)
+    few = torch.full((1, n + 1, points), float('nan'), dtype=torch.complex64, device='cuda')
+    c.time_order_points(x[..., :points].contiguous(), few, 1, n, points)
+    assert torch.equal(few, u[..., :points])
